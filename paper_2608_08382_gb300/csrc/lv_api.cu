@@ -15,6 +15,7 @@
 #include "lv_fit.cuh"
 #include "lv_kernels.cuh"
 #include "lv_metrics.cuh"
+#include "lv_tile.cuh"
 #include "lv_warp.cuh"
 #include "lv_whatif.cuh"
 
@@ -27,6 +28,8 @@ struct lv_ctx {
   int *d_status = nullptr;
   TilePart *d_tiles = nullptr;
   int64_t tiles_cap = 0;
+  int64_t *d_bound = nullptr;  // first batch of each tile (k_tiles)
+  int64_t bound_cap = 0;
   unsigned long long *d_ctr = nullptr;  // [0] warp tiles handed out, [1] jumbo batches queued
   int64_t *d_jumbo = nullptr;
   int64_t jumbo_cap = 0;
@@ -64,7 +67,7 @@ struct lv_tenant_acc {
 
 namespace {
 
-constexpr int kKTableN = 4096;
+constexpr int kKTableN = kTabN;
 
 #define LV_CUDA(call)                          \
   do {                                         \
@@ -383,7 +386,7 @@ lv_status ensure_sched(lv_ctx *ctx, int64_t jumbo_cap) {
 int64_t jumbo_bound(int64_t n_req) { return n_req / (kJumbo + 1) + 1; }
 
 // Partition + warp and jumbo kernels for the given batches.
-lv_status run_tiles(lv_ctx *ctx, TileArgs &a, int mode, cudaStream_t stream) {
+lv_status run_fit_tiles(lv_ctx *ctx, TileArgs &a, cudaStream_t stream) {
   ctx->last_grid = 0;
   const int64_t units = a.n_batch + a.n_req;
   // larger tiles fill the per-lane batch groups better and cost fewer tile
@@ -410,15 +413,120 @@ lv_status run_tiles(lv_ctx *ctx, TileArgs &a, int mode, cudaStream_t stream) {
   LV_CUDA(cudaGetLastError());
   int64_t *g = &ctx->last_grid;
   const int sms = ctx->sms;
+  return launch_warps_mode<M_FEAT | M_FIT>(ctx, sms, a, stream, g);
+}
+
+// Tiles of the batches: D merge positions each, so that the warps' rounds of
+// tiles come out even (a last round with few tiles would leave warps idle).
+struct TilePlan {
+  int64_t n_tiles;
+  uint64_t magic;
+};
+
+TilePlan plan_tiles(int64_t n_batch, int64_t n_req, int64_t warps) {
+  const int64_t units = kTW * n_batch + n_req;
+  const int64_t rounds = (units + warps * kTDMax - 1) / (warps * kTDMax);
+  int64_t D = (units + warps * rounds - 1) / (warps * rounds);
+  D = std::min<int64_t>(kTDMax, std::max<int64_t>(kTDMin, (D + 7) & ~(int64_t)7));
+  TilePlan p;
+  p.n_tiles = (units + D - 1) / D;
+  p.magic = UINT64_MAX / (uint64_t)D + 1;
+  return p;
+}
+
+// Kernel attributes and CTAs per SM of k_tiles<MODE>, once per (context or,
+// without one, process; shared-memory size).
+template <int MODE>
+lv_status tiles_occupancy(lv_ctx *ctx, size_t smem, int *per_sm) {
+  const uint64_t key = ((uint64_t)(MODE | 1 << 16) << 32) | smem;
+  *per_sm = 0;
+  if (ctx) {
+    for (const auto &e : ctx->occ)
+      if (e.first == key) *per_sm = e.second;
+  } else {
+    std::lock_guard<std::mutex> lock(free_occ_mu<MODE>());
+    for (const auto &e : free_occ<MODE>())
+      if (e.first == key) *per_sm = e.second;
+  }
+  if (*per_sm) return LV_OK;
+  LV_CUDA(cudaFuncSetAttribute(k_tiles<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)(sizeof(TSmem) + ((MODE & M_TEN) ? sizeof(TenSmem) : 0))));
+  LV_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_tiles<MODE>, kTThreads, smem));
+  if (*per_sm < 1) *per_sm = 1;
+  if (ctx) {
+    ctx->occ.emplace_back(key, *per_sm);
+  } else {
+    std::lock_guard<std::mutex> lock(free_occ_mu<MODE>());
+    free_occ<MODE>().emplace_back(key, *per_sm);
+  }
+  return LV_OK;
+}
+
+lv_status ensure_bound(lv_ctx *ctx, int64_t n) {
+  if (n <= ctx->bound_cap) return LV_OK;
+  LV_CUDA(cudaDeviceSynchronize());
+  if (ctx->d_bound) cudaFree(ctx->d_bound);
+  ctx->d_bound = nullptr;
+  ctx->bound_cap = 0;
+  const int64_t cap = std::max<int64_t>(n, 1 << 16);
+  if (cudaMalloc(&ctx->d_bound, cap * sizeof(int64_t)) != cudaSuccess) {
+    ctx->d_bound = nullptr;
+    return LV_ENOMEM;
+  }
+  ctx->bound_cap = cap;
+  return LV_OK;
+}
+
+// Bounds and tile kernel for the given batches.  Without a context, `bound`
+// has room for the tiles' bounds (bound_cap 32-bit entries).
+template <int MODE>
+lv_status run_tiles_mode(lv_ctx *ctx, int sms, TileArgs &a, void *bound, int64_t bound_cap, cudaStream_t stream) {
+  const size_t smem = sizeof(TSmem) + ((MODE & M_TEN) ? sizeof(TenSmem) : 0);
+  int per_sm = 0;
+  lv_status st = tiles_occupancy<MODE>(ctx, smem, &per_sm);
+  if (st != LV_OK) return st;
+  const int64_t ctas = (int64_t)sms * per_sm;
+  const TilePlan plan = plan_tiles(a.n_batch, a.n_req, ctas * kTWarps);
+  if (ctx) {
+    st = ensure_bound(ctx, plan.n_tiles + 1);
+    if (st != LV_OK) return st;
+    bound = ctx->d_bound;
+  } else if (plan.n_tiles + 1 > bound_cap) {
+    return LV_EINVAL;
+  }
+  const bool narrow = a.n_batch < (1ll << 32);
+  a.bound = narrow ? nullptr : static_cast<int64_t *>(bound);
+  a.bound32 = narrow ? static_cast<uint32_t *>(bound) : nullptr;
+  a.n_tiles = plan.n_tiles;
+  const int64_t blocks = std::min<int64_t>((a.n_batch + 1 + 255) / 256, (int64_t)sms * 16);
+  if (narrow)
+    k_tile_bounds<uint32_t><<<(unsigned)blocks, 256, 0, stream>>>(a.off, a.n_batch, a.n_req, plan.n_tiles, plan.magic,
+                                                                  static_cast<uint32_t *>(bound), a.status);
+  else
+    k_tile_bounds<int64_t><<<(unsigned)blocks, 256, 0, stream>>>(a.off, a.n_batch, a.n_req, plan.n_tiles, plan.magic,
+                                                                 static_cast<int64_t *>(bound), a.status);
+  LV_CUDA(cudaGetLastError());
+  cudaEvent_t stop = nullptr;
+  if (ctx) {
+    st = timing_begin(ctx, LV_TIME_TILES, stream, &stop);
+    if (st != LV_OK) return st;
+  }
+  k_tiles<MODE><<<(unsigned)std::min<int64_t>(plan.n_tiles, ctas), kTThreads, smem, stream>>>(a);
+  LV_CUDA(cudaGetLastError());
+  return ctx ? timing_end(stop, stream) : LV_OK;
+}
+
+lv_status run_tiles(lv_ctx *ctx, TileArgs &a, int mode, cudaStream_t stream) {
+  if (a.n_batch == 0) return LV_OK;
+  const int sms = ctx->sms;
   switch (mode) {
-    case M_ATTR: return launch_warps_mode<M_ATTR>(ctx, sms, a, stream, g);
-    case M_ATTR | M_FIX: return launch_warps_mode<M_ATTR | M_FIX>(ctx, sms, a, stream, g);
-    case M_ATTR | M_TEN: return launch_warps_mode<M_ATTR | M_TEN>(ctx, sms, a, stream, g);
-    case M_ATTR | M_TEN | M_FIX: return launch_warps_mode<M_ATTR | M_TEN | M_FIX>(ctx, sms, a, stream, g);
-    case M_ATTR | M_F32: return launch_warps_mode<M_ATTR | M_F32>(ctx, sms, a, stream, g);
-    case M_ATTR | M_TEN | M_F32: return launch_warps_mode<M_ATTR | M_TEN | M_F32>(ctx, sms, a, stream, g);
-    case M_FEAT: return launch_warps_mode<M_FEAT>(ctx, sms, a, stream, g);
-    case M_FEAT | M_FIT: return launch_warps_mode<M_FEAT | M_FIT>(ctx, sms, a, stream, g);
+    case M_ATTR: return run_tiles_mode<M_ATTR>(ctx, sms, a, nullptr, 0, stream);
+    case M_ATTR | M_FIX: return run_tiles_mode<M_ATTR | M_FIX>(ctx, sms, a, nullptr, 0, stream);
+    case M_ATTR | M_TEN: return run_tiles_mode<M_ATTR | M_TEN>(ctx, sms, a, nullptr, 0, stream);
+    case M_ATTR | M_TEN | M_FIX: return run_tiles_mode<M_ATTR | M_TEN | M_FIX>(ctx, sms, a, nullptr, 0, stream);
+    case M_ATTR | M_F32: return run_tiles_mode<M_ATTR | M_F32>(ctx, sms, a, nullptr, 0, stream);
+    case M_ATTR | M_TEN | M_F32: return run_tiles_mode<M_ATTR | M_TEN | M_F32>(ctx, sms, a, nullptr, 0, stream);
+    case M_FEAT: return run_tiles_mode<M_FEAT>(ctx, sms, a, nullptr, 0, stream);
     default: return LV_EINVAL;
   }
 }
@@ -539,7 +647,7 @@ lv_status fit_pass(lv_ctx *ctx, const lv_batches *b, const double *y, int32_t n_
   a.fit.n_y = n_y;
   a.fit.partial = partial;
   ctx->last_grid = 0;
-  st = run_tiles(ctx, a, M_FEAT | M_FIT, stream);
+  st = run_fit_tiles(ctx, a, stream);
   if (st != LV_OK) return st;
   const int n_cta = (int)ctx->last_grid;
   k_fit_reduce<<<n_ent, kFitRedThreads, 0, stream>>>(partial, n_cta, n_ent, totals);
@@ -714,6 +822,7 @@ void lv_ctx_destroy(lv_ctx *ctx) {
   cudaDeviceSynchronize();
   if (ctx->d_status) cudaFree(ctx->d_status);
   if (ctx->d_tiles) cudaFree(ctx->d_tiles);
+  if (ctx->d_bound) cudaFree(ctx->d_bound);
   if (ctx->d_ctr) cudaFree(ctx->d_ctr);
   if (ctx->d_jumbo) cudaFree(ctx->d_jumbo);
   if (ctx->d_ktab) cudaFree(ctx->d_ktab);
@@ -1218,15 +1327,13 @@ lv_status lv_whatif_admit(lv_ctx *ctx, const lv_model *model, const lv_batches *
 
 namespace {
 
-constexpr int64_t kNoAllocMaxTiles = 1 << 16;  // => n_batch + n_req <= 65,536 * kDW
-constexpr size_t kNoAllocPartBytes = sizeof(TilePart) * (size_t)(kNoAllocMaxTiles + 1);
-constexpr size_t kNoAllocTabOffset = (kNoAllocPartBytes + 255) & ~(size_t)255;
-constexpr size_t kNoAllocCtrOffset = (kNoAllocTabOffset + sizeof(KEntry) * 4 * (kKTableN + 1) + 255) & ~(size_t)255;
-constexpr size_t kNoAllocJumboOffset = kNoAllocCtrOffset + 256;
-constexpr int64_t kNoAllocJumboCap = kNoAllocMaxTiles * kDW / (kJumbo + 1) + 1;
-constexpr size_t kNoAllocBytes = kNoAllocJumboOffset + sizeof(int64_t) * (size_t)kNoAllocJumboCap;
-// the size stated in include/llmvisor.h ("about 2.6 MB")
-static_assert(kNoAllocBytes > 2500000 && kNoAllocBytes < 2700000, "no-alloc scratch size as documented");
+constexpr int64_t kNoAllocMaxUnits = 65536 * 1024;  // n_batch + n_req
+// most tiles: every unit an empty batch, and a partial round of 32 warps on each of 256 SMs
+constexpr int64_t kNoAllocBounds = kTW * kNoAllocMaxUnits / kTDMax + 32 * 256 + 2;
+constexpr size_t kNoAllocTabOffset = (sizeof(uint32_t) * (size_t)kNoAllocBounds + 255) & ~(size_t)255;
+constexpr size_t kNoAllocBytes = kNoAllocTabOffset + sizeof(KEntry) * 4 * (kKTableN + 1);
+// the size stated in include/llmvisor.h ("about 3.4 MB")
+static_assert(kNoAllocBytes > 3300000 && kNoAllocBytes < 3400000, "no-alloc scratch size as documented");
 
 }  // namespace
 
@@ -1268,8 +1375,7 @@ extern "C" lv_status lv_attribute_noalloc(const lv_model *model, const lv_batche
   if (T && !aligned(T, 8)) return LV_EINVAL;
   if (share && !aligned(share, 8)) return LV_EINVAL;
   if (status && !aligned(status, 4)) return LV_EINVAL;
-  const int64_t n_tiles = (b->n_batch + b->n_req + kDW - 1) / kDW;
-  if (n_tiles > kNoAllocMaxTiles) return LV_EINVAL;
+  if (b->n_batch > kNoAllocMaxUnits || b->n_req > kNoAllocMaxUnits - b->n_batch) return LV_EINVAL;
   int dev = 0;
   LV_CUDA(cudaGetDevice(&dev));
   void *scratch = nullptr;
@@ -1311,20 +1417,7 @@ extern "C" lv_status lv_attribute_noalloc(const lv_model *model, const lv_batche
   a.share = share;
   a.status = status;
   a.mp = mp;
-  a.n_tiles = n_tiles;
-  a.D = kDW;
-  unsigned char *base = static_cast<unsigned char *>(scratch);
-  TilePart *part = reinterpret_cast<TilePart *>(base);
-  a.part = part;
-  a.ctr = reinterpret_cast<unsigned long long *>(base + kNoAllocCtrOffset);
-  a.jumbo_n = a.ctr + 1;
-  a.jumbo = reinterpret_cast<int64_t *>(base + kNoAllocJumboOffset);
-  a.jumbo_cap = kNoAllocJumboCap;
-  LV_CUDA(cudaMemsetAsync(a.ctr, 0, 2 * sizeof(unsigned long long), stream));
-  const int64_t pblocks = std::min<int64_t>((b->n_batch + 1 + 255) / 256, (int64_t)sms * 16);
-  k_partition<<<(unsigned)pblocks, 256, 0, stream>>>(a.off, a.n_batch, a.n_req, a.n_tiles, kDW, part, status);
-  LV_CUDA(cudaGetLastError());
-  int64_t ctas = 0;
-  return mp.fixed ? launch_warps_mode<M_ATTR | M_FIX>(nullptr, sms, a, stream, &ctas)
-                  : launch_warps_mode<M_ATTR>(nullptr, sms, a, stream, &ctas);
+  static_assert(kNoAllocMaxUnits < (1ll << 32), "32-bit tile bounds");
+  return mp.fixed ? run_tiles_mode<M_ATTR | M_FIX>(nullptr, sms, a, scratch, kNoAllocBounds, stream)
+                  : run_tiles_mode<M_ATTR>(nullptr, sms, a, scratch, kNoAllocBounds, stream);
 }

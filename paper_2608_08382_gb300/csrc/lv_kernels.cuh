@@ -166,6 +166,8 @@ struct TileArgs {
   const int64_t *off;
   int64_t n_req, n_batch;
   const TilePart *part;  // [n_tiles + 1]
+  const int64_t *bound;    // [n_tiles + 1] first batch of each tile (k_tiles), or null:
+  const uint32_t *bound32;  // the same in 32 bits (fewer than 2^32 batches)
   int64_t n_tiles;
   int64_t D;             // merge positions per tile
   double *T, *share;

@@ -1,0 +1,949 @@
+// Tile kernel of the attribution and feature passes (sm_103a).
+//
+// Work decomposition.  Batch b starts at merge position kTW * b + off[b];
+// k_tile_bounds cuts the positions every D and tile t owns the batches whose
+// start falls in window t (whole batches, nothing shared with neighbours).
+// Warps take tiles round-robin and work alone: no block-wide barrier is taken
+// while tiles are processed, so one warp's memory latency is hidden by the
+// other warps' arithmetic.  A warp takes its tile in three steps:
+//   1. lane j sums requests 8j .. 8j+7 of each 256, a warp scan turns the sums
+//      into prefixes (exact integers) in shared memory;
+//   2. one lane per batch takes its batch's sums as a difference of two
+//      prefixes, then the segment, the per-request constant and T; non-empty
+//      batches leave a record and a head bit at their first request;
+//   3. one lane per four consecutive requests finds their record from the head
+//      bits, attributes them and adds them to the tenants; what is off the
+//      common path is listed and worked off 32 at a time.
+// So a request costs about the same instructions whatever the batch sizes, and
+// no lane idles on a batch's remainder.  The requests are read twice, the
+// second time from L1 or L2 (24 tiles of kTDMax positions per SM; with 1,024
+// positions and the next tile prefetched the L2 no longer held them and the
+// DRAM reads doubled).  A batch that reaches past a tile's kTCap requests is
+// walked by its warp alone, or, above kTAlone requests, by the whole CTA after
+// its tiles (a warp alone on a batch of 4,096 set the time of a small input).
+// All sums are exact integers, so results do not depend on the schedule.
+//
+// What bounds it: instruction issue and the integer pipe (about 200 warp
+// instructions per 32 requests at 60 % issue with 24 warps per SM), not HBM.
+// Against a kernel that walked one batch per warp (fp64 shares, 16 tenants,
+// one call, GB300): 9.75e6 requests in batches of 1 to 64, 238 us before and
+// 127 us after; 9.75e7, 1,750 and 999; 6.5e5, 113 and 31; 1.36e8 in batches of
+// 16 to 256, 1,132 and 1,000; 2.6e7 in Pareto batches, 780 and 722.
+#pragma once
+
+#include "lv_warp.cuh"
+
+namespace lv {
+
+constexpr int kTThreads = 768;             // threads of a CTA, one CTA per SM (one tenant table)
+constexpr int kTWarps = kTThreads / 32;
+constexpr int kTW = 8;                     // merge positions a batch takes besides its requests
+constexpr int kTDMax = 768;                // merge positions per tile, at most
+constexpr int kTDMin = 128;
+constexpr int kTCap = 1024;                // requests of a tile, at most
+constexpr int kTNb = kTDMax / kTW;         // batches of a tile, at most
+constexpr int kTRec = kTDMax / (kTW + 1) + 5;     // non-empty ones, and room to read past the last
+constexpr int kTBlocks = kTCap / 256 + 1;         // blocks of 256 requests, one more for a bound at the end
+constexpr int kTWords = kTCap / 32 + 1;
+constexpr int kTList = 31 + 128;           // deferred requests at most: a rest and one step's
+constexpr int64_t kTAlone = 512;           // requests a warp walks alone
+constexpr int kTBigs = 64;                 // larger batches a CTA keeps for later
+constexpr int kTabN = 4096;                // batch sizes of the K table
+constexpr uint32_t kTSmall = 1u << 23;     // p and c of a tile on the common path are below this
+static_assert(kTCap % 256 == 0 && kTDMax + 3 < kTCap, "only a tile's last batch can reach past its requests");
+static_assert(kTCap <= kTabN, "a tile's batches are in the K table");
+
+// A batch's record: its share constant K + A1 + A3 (three words) and the
+// biased exponent of word 1's unit << 20; A2 (two words), n << 4 | fast << 3 |
+// slow << 2 | segment, and the fourth word of the constant (used off the fast
+// path).  fp32 variant: K, a1, a2, a3 as floats in k.
+struct TileRec {
+  uint4 k, a;
+};
+
+// One warp's tile.  pre: per 8 requests {S1, S2, S3 + prefills << 55} of the
+// requests before them in their 256; tot: each 256's totals.
+struct WarpTile {
+  alignas(16) uint4 pre[kTBlocks * 32];
+  alignas(16) uint4 tot[kTBlocks];
+  alignas(16) TileRec rec[kTRec];
+  uint32_t bits[kTWords];  // head bits: a batch starts at this request
+  uint16_t rank[kTWords];  // heads before word w
+  uint32_t list[kTList];   // deferred requests: index | record << 16
+};
+
+struct TSmem {
+  WarpTile tile[kTWarps];
+  alignas(16) SegS seg[4];
+  alignas(16) SegFix fx[4];
+  float cf[4][5];                     // coefficients as float (fp32 variant)
+  alignas(16) Sums red[kTWarps];
+  alignas(16) int64_t big[kTBigs];    // batches left for the whole CTA
+  int n_big;
+};
+
+// ---------------------------------------------------------------- bounds
+
+// x / D for 0 <= x < 2^44 and 2 <= D < 2^12, with magic = floor((2^64 - 1) / D) + 1.
+__device__ __forceinline__ int64_t div_magic(int64_t x, uint64_t magic) {
+  return (int64_t)__umul64hi((uint64_t)x, magic);
+}
+
+// part[t] = the first batch whose start position kTW * b + off[b] is at least
+// t * D, for t in [0, n_tiles); part[n_tiles] = n_batch.  Batch b writes the t
+// in (f(b-1) / D, f(b) / D], so every entry is written once.  Checks the
+// offsets.  HBM-bound: 8 B per batch; the divisions are multiplications (two
+// 64-bit divisions per batch made it compute-bound: 51 us on 1e7 batches).
+template <class V>
+__global__ void k_tile_bounds(const int64_t *__restrict__ off, int64_t n_batch, int64_t n_req, int64_t n_tiles,
+                              uint64_t magic, V *__restrict__ part, int *status) {
+  int bad = 0;
+  for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b <= n_batch;
+       b += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t raw = __ldg(off + b);
+    int64_t tmin = 0;
+    if (b == 0) {
+      if (raw != 0) bad = 1;
+    } else {
+      const int64_t rp = __ldg(off + b - 1);
+      if (rp > raw) bad = 1;
+      tmin = div_magic(kTW * (b - 1) + clampi(rp, 0, n_req), magic) + 1;
+    }
+    int64_t tmax = div_magic(kTW * b + clampi(raw, 0, n_req), magic);
+    if (b == n_batch) {
+      if (raw != n_req) bad = 1;
+      tmax = n_tiles;
+    }
+    if (tmax > n_tiles) tmax = n_tiles;
+    for (int64_t t = tmin; t <= tmax; ++t) part[t] = (V)b;
+  }
+  if (bad) flag(status, kStatusData);
+}
+
+__device__ __forceinline__ int64_t tile_bound(const TileArgs &a, int64_t t) {
+  return a.bound32 ? (int64_t)a.bound32[t] : a.bound[t];
+}
+
+// ---------------------------------------------------------------- loads
+
+struct Quad {
+  int4 p, c, x;  // x: phases (step 1) or tenants (step 3)
+};
+
+// A tile's request arrays from its first staged request (16-byte aligned);
+// lim: requests from there to the end of the arrays.
+struct TileSrc {
+  const int32_t *p, *c, *ph, *u;
+  int lim;
+};
+
+// The quad that holds the end of the arrays, or none of them: zero past it.
+__device__ __noinline__ Quad quad_tail(const int32_t *p, const int32_t *c, const int32_t *x, int e, int lim) {
+  int v[3][4];
+  const int32_t *src[3] = {p, c, x};
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[a][k] = src[a] && e + k < lim ? src[a][e + k] : 0;
+  return Quad{make_int4(v[0][0], v[0][1], v[0][2], v[0][3]), make_int4(v[1][0], v[1][1], v[1][2], v[1][3]),
+              make_int4(v[2][0], v[2][1], v[2][2], v[2][3])};
+}
+
+// Four requests from index e (a multiple of 4).
+template <bool X>
+__device__ __forceinline__ Quad load_quad(const int32_t *p, const int32_t *c, const int32_t *x, int e, int lim) {
+  Quad q;
+  if (e + 4 <= lim) {
+    q.p = *reinterpret_cast<const int4 *>(p + e);
+    q.c = *reinterpret_cast<const int4 *>(c + e);
+    q.x = X ? *reinterpret_cast<const int4 *>(x + e) : make_int4(0, 0, 0, 0);
+  } else {
+    q = quad_tail(p, c, X ? x : nullptr, e, lim);
+  }
+  return q;
+}
+
+// ---------------------------------------------------------------- step 1: prefixes
+
+struct Req8 {
+  Quad q[2];
+};
+
+__device__ __forceinline__ Req8 load_req8(const TileSrc &t, int e) {
+  Req8 r;
+  r.q[0] = load_quad<true>(t.p, t.c, t.ph, e, t.lim);
+  r.q[1] = load_quad<true>(t.p, t.c, t.ph, e + 4, t.lim);
+  return r;
+}
+
+// Sums of 8 requests whose p and c are below kTSmall: S1, S2, S3 + prefills << 55.
+struct TSum {
+  uint32_t s1, s2;
+  uint64_t s3;
+};
+
+// The first `take` of 8 requests.
+__device__ __forceinline__ TSum sum_req8(const Req8 &r, int take) {
+  TSum s{0u, 0u, 0ull};
+  uint32_t f = 0;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const Quad &v = r.q[h];
+    const int32_t p[4] = {v.p.x, v.p.y, v.p.z, v.p.w}, c[4] = {v.c.x, v.c.y, v.c.z, v.c.w},
+                  q[4] = {v.x.x, v.x.y, v.x.z, v.x.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const bool in = 4 * h + k < take;
+      const uint32_t pk = in ? (uint32_t)p[k] : 0u;
+      s.s1 += pk;
+      s.s2 += in ? (uint32_t)c[k] : 0u;
+      s.s3 += (uint64_t)pk * pk;
+      f += in ? (uint32_t)q[k] : 0u;
+    }
+  }
+  s.s3 += (uint64_t)f << 55;
+  return s;
+}
+
+// Prefixes of the tile's requests; true when some p or c is too large for
+// them (or negative) or some phase is not 0 or 1.
+__device__ __forceinline__ bool tile_prefix(WarpTile &wt, const TileSrc &src, int cnt, int lane) {
+  uint32_t big = 0;
+  int e = 8 * lane;
+  Req8 nx = load_req8(src, e);
+#pragma unroll 1
+  for (int k = 0; k * 256 <= cnt; ++k) {
+    const Req8 r = nx;
+    e += 256;
+    if (k * 256 + 256 <= cnt) nx = load_req8(src, e);
+    const Quad &x = r.q[0], &y = r.q[1];
+    const uint32_t op = (uint32_t)(x.p.x | x.p.y | x.p.z | x.p.w | y.p.x | y.p.y | y.p.z | y.p.w | x.c.x | x.c.y |
+                                   x.c.z | x.c.w | y.c.x | y.c.y | y.c.z | y.c.w);
+    const uint32_t of = (uint32_t)(x.x.x | x.x.y | x.x.z | x.x.w | y.x.x | y.x.y | y.x.z | y.x.w);
+    big |= (op & ~(kTSmall - 1u)) | (of & ~1u);
+    TSum s = sum_req8(r, 8);
+    const TSum o = s;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t x1 = __shfl_up_sync(kFull, s.s1, d), x2 = __shfl_up_sync(kFull, s.s2, d);
+      const uint64_t x3 = __shfl_up_sync(kFull, s.s3, d);
+      if (lane >= d) {
+        s.s1 += x1;
+        s.s2 += x2;
+        s.s3 += x3;
+      }
+    }
+    if (lane == 31) wt.tot[k] = make_uint4(s.s1, s.s2, (uint32_t)s.s3, (uint32_t)(s.s3 >> 32));
+    s.s3 -= o.s3;
+    wt.pre[32 * k + lane] = make_uint4(s.s1 - o.s1, s.s2 - o.s2, (uint32_t)s.s3, (uint32_t)(s.s3 >> 32));
+  }
+  return __any_sync(kFull, big != 0u);
+}
+
+// Sums of the requests before index x of its 256.
+__device__ __forceinline__ TSum prefix_at(const WarpTile &wt, const TileSrc &src, int x) {
+  const uint4 v = wt.pre[x >> 3];
+  TSum r{v.x, v.y, (uint64_t)v.z | ((uint64_t)v.w << 32)};
+  if (x & 7) {
+    const TSum s = sum_req8(load_req8(src, x & ~7), x & 7);
+    r.s1 += s.s1;
+    r.s2 += s.s2;
+    r.s3 += s.s3;
+  }
+  return r;
+}
+
+// ---------------------------------------------------------------- step 2: batches
+
+// Share constants of a batch of n requests in segment s; kTab: n is within the
+// K table (every staged batch).
+template <int MODE, bool kTab>
+__device__ __forceinline__ TileRec tile_record(const TileArgs &a, const TSmem &ts, int s, int64_t n) {
+  TileRec r;
+  if (MODE & M_F32) {
+    const float *k = ts.cf[s];
+    const float fn = (float)n;
+    r.k = make_uint4(__float_as_uint(__fadd_rn(__fdiv_rn(k[0], fn), __fmul_rn(k[4], fn))), __float_as_uint(k[1]),
+                     __float_as_uint(k[2]), __float_as_uint(k[3]));
+    r.a = make_uint4(0u, 0u, 0u, 0u);
+    return r;
+  }
+  bool slow = false;
+  const SegS &sg = ts.seg[s];
+  i128 kf;
+  if ((MODE & M_FIX) && kTab) {
+    kf = a.mp.ktab[s * (kTabN + 1) + (int)n].kf;
+    slow = kf.hi == kKSlowHi;
+  } else {
+    kf = batch_const_w<MODE>(a, nullptr, s, n, &slow);
+  }
+  const i128 k = (MODE & M_FIX) ? add128(kf, sg.A13) : kf;
+  // fast: 2^64 <= constant < 2^95 (then the share, below 2^95 more, is in [2^64, 2^96)) and A2 < 2^64
+  const bool fast = (MODE & M_FIX) && !slow && sg.a2_narrow && k.hi != 0 && k.hi < (1ull << 31);
+  r.k = make_uint4((uint32_t)k.lo, (uint32_t)(k.lo >> 32), (uint32_t)k.hi, (uint32_t)(sg.E + 32) << 20);
+  r.a = make_uint4((uint32_t)sg.A2.lo, (uint32_t)(sg.A2.lo >> 32),
+                   ((uint32_t)n << 4) | (fast ? 8u : 0u) | (slow ? 4u : 0u) | (uint32_t)s, (uint32_t)(k.hi >> 32));
+  return r;
+}
+
+// v shifted so that its leading bit (in v2, not zero) is bit 95, rounded to
+// nearest even by the hardware's 64-bit integer conversion (the rest is ORed
+// into the last of the top 64 bits), in units of 2^(E + 64): ebase = (E + 32)
+// << 20.  The conversion's unit is otherwise idle; rounding by integer
+// instructions takes some 15 more.
+__device__ __forceinline__ double round_top(uint32_t v0, uint32_t v1, uint32_t v2, uint32_t ebase) {
+  const int s = __clz((int)v2);
+  const uint32_t t2 = __funnelshift_l(v1, v2, s), t0 = v0 << s;
+  const uint32_t t1 = __funnelshift_l(v0, v1, s) | min(t0, 1u);
+  const double x = __ull2double_rn(((uint64_t)t2 << 32) | t1);
+  return __hiloint2double(__double2hiint(x) + (int)(ebase - ((uint32_t)s << 20)), __double2loint(x));
+}
+
+// Eq. 1 exactly in fixed point, one rounding, for sums below 2^32 and a
+// segment whose coefficients are in [0, 2^92) (t32): 96 x 32-bit products,
+// whose sum stays below 2^127.  The general evaluation, which gives the same
+// value, otherwise (kept out of line).
+__device__ __forceinline__ double tile_eq1(const TileArgs &a, const TSmem &ts, int s, const BatchAgg &g) {
+  const SegFix &f = ts.fx[s];
+  const uint64_t wide = ((uint64_t)g.s1 | (uint64_t)g.s2 | (uint64_t)g.s3 | ((uint64_t)g.n << 16)) >> 32;
+  if (ts.seg[s].pad && wide == 0) {
+    uint32_t w0 = (uint32_t)f.B.lo, w1 = (uint32_t)(f.B.lo >> 32), w2 = (uint32_t)f.B.hi, w3 = 0u;
+    const uint32_t x[4] = {(uint32_t)g.s1, (uint32_t)g.s2, (uint32_t)g.s3, (uint32_t)g.n * (uint32_t)g.n};
+    const i128 *A[4] = {&f.A1, &f.A2, &f.A3, &f.A4};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint32_t a0 = (uint32_t)A[i]->lo, a1 = (uint32_t)(A[i]->lo >> 32), a2 = (uint32_t)A[i]->hi;
+      asm("mad.lo.cc.u32 %0, %4, %7, %0;\n\t"
+          "madc.hi.cc.u32 %1, %4, %7, %1;\n\t"
+          "madc.lo.cc.u32 %2, %6, %7, %2;\n\t"
+          "madc.hi.u32 %3, %6, %7, %3;\n\t"
+          "mad.lo.cc.u32 %1, %5, %7, %1;\n\t"
+          "madc.hi.cc.u32 %2, %5, %7, %2;\n\t"
+          "addc.u32 %3, %3, 0;"
+          : "+r"(w0), "+r"(w1), "+r"(w2), "+r"(w3)
+          : "r"(a0), "r"(a1), "r"(a2), "r"(x[i]));
+    }
+    if (w3 == 0u && w2 != 0u && g.n > 0) return round_top(w0, w1, w2, (uint32_t)(f.E + 32) << 20);
+  }
+  return eq1_fix(a.mp, s, g);
+}
+
+// A batch's outputs.
+template <int MODE>
+__device__ __forceinline__ void tile_emit(const TileArgs &a, const TSmem &ts, int64_t b, const BatchAgg &g, int s) {
+  if ((MODE & M_ATTR) && (MODE & M_F32)) {
+    if (a.T32) {
+      const float *k = ts.cf[s];
+      float T = __fmaf_rn(k[1], (float)g.s1, k[0]);
+      T = __fmaf_rn(k[2], (float)g.s2, T);
+      T = __fmaf_rn(k[3], (float)g.s3, T);
+      T = __fmaf_rn(k[4], (float)(g.n * g.n), T);
+      a.T32[b] = g.n > 0 ? T : 0.0f;
+    }
+  } else if ((MODE & M_ATTR) && (MODE & M_FIX)) {
+    if (a.T) a.T[b] = tile_eq1(a, ts, s, g);
+  } else {
+    emit_batch<MODE>(a, b, g, s, nullptr);
+  }
+}
+
+// ---------------------------------------------------------------- step 3: requests
+
+// Hot tenants (ids below H) in shared memory.  The sum of a tenant's q = share
+// * 2^72, modulo 2^128, is four 32-bit words.  Words 0 and 1 have kTCopies
+// copies, to one of which a lane always adds, so that one tenant's many
+// requests do not all serialise in one bank; words 2 and 3, which few
+// additions reach, have one.
+constexpr int kTCopies = 2;
+struct TenSmem {
+  // after the tenants' words, one per lane where lanes with nothing to add do so
+  uint32_t w0[kHotMax * kTCopies + 32], w1[kHotMax * kTCopies + 32];
+  uint32_t w2[kHotMax], w3[kHotMax];
+};
+constexpr uint32_t kTPlane = sizeof(uint32_t) * (kHotMax * kTCopies + 32);  // bytes from a word 0 to its word 1
+
+struct TenTab {
+  uint32_t w, base;  // shared-memory byte addresses: the lane's copy of tenant 0's word 0, and the table
+  uint32_t H;
+};
+
+// Shared-memory atomic add at a byte address (address space stated, so that it
+// compiles to the shared-memory instruction wherever the table comes from).
+__device__ __forceinline__ uint32_t atom_shared(uint32_t addr, uint32_t v) {
+  uint32_t o;
+  asm volatile("atom.shared.add.u32 %0, [%1], %2;" : "=r"(o) : "r"(addr), "r"(v));
+  return o;
+}
+
+// x + y and its carry.
+__device__ __forceinline__ uint32_t carry_of(uint32_t x, uint32_t y) {
+  uint32_t c;
+  asm("{\n .reg .u32 t;\n add.cc.u32 t, %1, %2;\n addc.u32 %0, 0, 0;\n}" : "=r"(c) : "r"(x), "r"(y));
+  return c;
+}
+
+// q = (h1:h0) 2^64 + (hi:lo), modulo 2^128, to tenant u < H.  Each word's
+// atomic returns its old value, so the lane whose addition wraps a word
+// carries into the next: the sum stays exact under any interleaving.
+__device__ __forceinline__ void ten_carry(const TenTab tt, uint32_t u, uint32_t h0, uint32_t h1) {
+  if (h0 | h1) {
+    const uint32_t a = tt.base + (uint32_t)offsetof(TenSmem, w2) + 4u * u;
+    h1 += carry_of(atom_shared(a, h0), h0);
+    if (h1) atom_shared(a + 4u * kHotMax, h1);
+  }
+}
+__device__ __forceinline__ void ten_add(const TenTab tt, uint32_t u, uint32_t lo, uint32_t hi, uint32_t h0,
+                                        uint32_t h1) {
+  const uint32_t w = tt.w + 4u * kTCopies * u;
+  const uint32_t c0 = carry_of(atom_shared(w, lo), lo), a1 = hi + c0;
+  const uint32_t c1 = carry_of(atom_shared(w + kTPlane, a1), a1) + (a1 < c0 ? 1u : 0u);
+  h0 += c1;
+  h1 += h0 < c1 ? 1u : 0u;
+  ten_carry(tt, u, h0, h1);
+}
+
+// Tenant contributions of a lane's four positive shares (d: their doubles'
+// words) in the common case, a valid tenant and a share below 2^-9 s (then q <
+// 2^63); go[k] is cleared otherwise.  q is the hardware's conversion of d 2^72
+// to a 64-bit integer, which rounds to nearest even.  The four low words'
+// atomics are issued together, then the four high words', so that a lane waits
+// for two of them and not for eight; lanes with nothing to add use a word of
+// their own, so there is no branch.
+__device__ __forceinline__ void ten_add4(const TileArgs &a, const TenTab tt, bool *go, const uint32_t *u,
+                                         const uint32_t *dlo, const uint32_t *dhi, int lane) {
+  uint32_t w[4], lo[4], hi[4], c1[4];
+  bool cold = false;
+  const uint32_t sink = tt.base + 4u * (kHotMax * kTCopies + lane);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    go[k] = go[k] && dhi[k] < ((1023u - 9u) << 20) && u[k] < (uint32_t)a.n_tenants;
+    const bool hot = go[k] && u[k] < tt.H;
+    const long long q = __double2ll_rn(__hiloint2double((int)(dhi[k] - ((uint32_t)kTenLsb << 20)), (int)dlo[k]));
+    lo[k] = (uint32_t)q;
+    hi[k] = (uint32_t)(q >> 32);
+    w[k] = tt.w + 4u * kTCopies * u[k];
+    w[k] = hot ? w[k] : sink;
+    cold |= go[k] && !hot;
+  }
+  if (cold) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (go[k] && u[k] >= tt.H) {
+        unsigned long long *pw = a.ten_pend + 4 * (int64_t)u[k];
+        atomicAdd(pw, (unsigned long long)lo[k]);
+        atomicAdd(pw + 1, (unsigned long long)hi[k]);
+      }
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) c1[k] = atom_shared(w[k], lo[k]);
+#pragma unroll
+  for (int k = 0; k < 4; ++k)  // hi <= 2^31: no wrap
+    asm("{\n .reg .u32 t;\n add.cc.u32 t, %1, %2;\n addc.u32 %0, %0, 0;\n}" : "+r"(hi[k]) : "r"(c1[k]), "r"(lo[k]));
+#pragma unroll
+  for (int k = 0; k < 4; ++k) c1[k] = atom_shared(w[k] + kTPlane, hi[k]);
+  uint32_t any = 0;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    c1[k] = carry_of(c1[k], hi[k]);
+    any |= c1[k];
+  }
+  if (any) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (c1[k] && go[k] && u[k] < tt.H) ten_carry(tt, u[k], 1u, 0u);
+  }
+}
+
+// Any positive share with q of at most three words and a valid tenant.
+__device__ __forceinline__ bool tile_tenant(const TileArgs &a, const TenTab tt, uint32_t u, uint32_t dlo,
+                                            uint32_t dhi) {
+  const uint32_t mh = (dhi & 0xfffffu) | 0x100000u;
+  const int sh = (int)(dhi >> 20) - (1075 + kTenLsb);
+  if ((unsigned)sh > 42u || u >= (uint32_t)a.n_tenants) return false;
+  const bool lowp = sh < 32;
+  const int t = lowp ? sh : sh - 32;
+  const uint32_t x0 = dlo << t, x1 = __funnelshift_l(dlo, mh, t), x2 = t ? mh >> (32 - t) : 0u;
+  const uint32_t q0 = lowp ? x0 : 0u, q1 = lowp ? x1 : x0, q2 = lowp ? x2 : x1;
+  if (u < tt.H) {
+    ten_add(tt, u, q0, q1, q2, 0u);
+    return true;
+  }
+  unsigned long long *pw = a.ten_pend + 4 * (int64_t)u;
+  if (q0) atomicAdd(pw, (unsigned long long)q0);
+  if (q1) atomicAdd(pw + 1, (unsigned long long)q1);
+  if (q2) atomicAdd(pw + 2, (unsigned long long)q2);
+  return true;
+}
+
+// The general tenant add (any sign and magnitude).
+__device__ __forceinline__ void tile_tenant_any(const TileArgs &a, const TenTab tt, int32_t u, const Rounded &r,
+                                                int *bad) {
+  if (u < 0 || u >= a.n_tenants) {
+    *bad = 1;
+    u = u < 0 ? 0 : a.n_tenants - 1;
+  }
+  const i128 q = share_to_tenant_fix(r, bad);
+  if ((q.lo | q.hi) == 0) return;
+  if (u < a.H)
+    ten_add(tt, (uint32_t)u, (uint32_t)q.lo, (uint32_t)(q.lo >> 32), (uint32_t)q.hi, (uint32_t)(q.hi >> 32));
+  else
+    pend_add(a.ten_pend, u, q);
+}
+
+// The general path of one request.  Out of line: the fast path leaves it the
+// rare ones (fp64 mode, values out of range).
+template <int MODE>
+__device__ __noinline__ void tile_slow(const TileArgs &a, const TenTab tt, const TSmem &ts, const TileRec &rec,
+                                       int64_t n, int64_t i, int32_t p, int32_t c, int32_t u) {
+  const int s = (int)(rec.a.z & 3u);
+  const bool slow = (rec.a.z & 4u) != 0u;
+  const SegS &sg = ts.seg[s];
+  i128 kf = mk128((uint64_t)rec.k.x | ((uint64_t)rec.k.y << 32), (uint64_t)rec.k.z | ((uint64_t)rec.a.w << 32));
+  if (MODE & M_FIX) kf = add128(kf, neg128(sg.A13));
+  p = max(p, 0);
+  c = max(c, 0);
+  const Rounded r = (MODE & M_FIX) && !slow && p <= kPMaxFix
+                        ? share_fix(sg, kf, (uint32_t)p, (uint32_t)c)
+                        : share_slow(a.mp, s, (MODE & M_FIX) != 0, kf, p, c, n);
+  if (a.share) __stcs(a.share + i, r.d);
+  if (MODE & M_TEN) {
+    int bad = 0;
+    tile_tenant_any(a, tt, u, r, &bad);
+    if (bad) flag(a.status, kStatusData);
+  }
+}
+
+// Constant + A2 c on the fast path: below 2^96, no carry leaves word 2.
+__device__ __forceinline__ double tile_value(const TileRec &r, uint32_t k0, uint32_t k1, uint32_t k2, int32_t c) {
+  uint32_t v0, v1, v2;
+  asm("mad.lo.cc.u32 %0, %3, %5, %6;\n\t"
+      "madc.hi.cc.u32 %1, %3, %5, %7;\n\t"
+      "addc.u32 %2, %8, 0;\n\t"
+      "mad.lo.cc.u32 %1, %4, %5, %1;\n\t"
+      "madc.hi.u32 %2, %4, %5, %2;"
+      : "=&r"(v0), "=&r"(v1), "=&r"(v2)
+      : "r"(r.a.x), "r"(r.a.y), "r"((uint32_t)c), "r"(k0), "r"(k1), "r"(k2));
+  return round_top(v0, v1, v2, r.k.w);
+}
+
+// A request's exact share on the fast path, rounded to nearest even; false
+// where the path does not apply.  The constant is K + A1 + A3 for p = 1; a
+// prefill adds (p - 1)(A1 + A3 (p + 1)).  With p_narrow (A1 < 2^95, A3 < 2^64)
+// and p <= 2^24 that is below 2^120, so the 128-bit sum is exact; it must be
+// below 2^95.
+__device__ __forceinline__ bool tile_share(const SegS *segs, const TileRec &r, int32_t p, int32_t c, double *d) {
+  uint32_t k0 = r.k.x, k1 = r.k.y, k2 = r.k.z;
+  bool ok = (r.a.z & 8u) != 0u;
+  if (p != 1) {
+    const SegS &sg = segs[r.a.z & 3u];
+    ok = ok && p > 1 && p <= kPMaxFix && sg.p_narrow;
+    const i128 g = add128(sg.A1, mul_u64_u32(sg.A3.lo, (uint32_t)p + 1u));
+    const i128 b = add128(mk128((uint64_t)k0 | ((uint64_t)k1 << 32), (uint64_t)k2), mul128_u32(g, (uint32_t)p - 1u));
+    k0 = (uint32_t)b.lo;
+    k1 = (uint32_t)(b.lo >> 32);
+    k2 = (uint32_t)b.hi;
+    ok = ok && b.hi < (1ull << 31);
+  }
+  *d = tile_value(r, k0, k1, k2, max(c, 0));
+  return ok;
+}
+
+__device__ __forceinline__ void store4(double *p, const double *d) {
+  asm volatile("st.global.cs.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(d[0]), "d"(d[1]), "d"(d[2]), "d"(d[3])
+               : "memory");
+}
+
+// One request through the fast path where it applies, else the general one.
+template <int MODE>
+__device__ __forceinline__ bool tile_one(const TileArgs &a, const TenTab tt, const TSmem &ts, const TileRec &rec,
+                                         int64_t n, int64_t i, int32_t p, int32_t c, int32_t u, double *d) {
+  bool ok = (MODE & M_FIX) && tile_share(ts.seg, rec, p, c, d);
+  if (MODE & M_TEN)
+    ok = ok && tile_tenant(a, tt, (uint32_t)u, (uint32_t)__double2loint(*d), (uint32_t)__double2hiint(*d));
+  if (!ok) tile_slow<MODE>(a, tt, ts, rec, n, i, p, c, u);
+  return ok;
+}
+
+// One request of the fp32 variant.
+template <int MODE>
+__device__ __forceinline__ float tile_one_f32(const TileArgs &a, const TenTab tt, const TileRec &rec, int32_t p,
+                                              int32_t c, int32_t u, int *bad) {
+  const Share32 q{__uint_as_float(rec.k.x), __uint_as_float(rec.k.y), __uint_as_float(rec.k.z),
+                  __uint_as_float(rec.k.w)};
+  const float s = share_f32(q, p, c);
+  if (MODE & M_TEN) {
+    // a positive normal float's double: the same significand, the exponent rebiased
+    const uint32_t f = __float_as_uint(s);
+    const bool normal = f >= 0x00800000u && f < 0x7f800000u;
+    if (!normal || !tile_tenant(a, tt, (uint32_t)u, f << 29, (f >> 3) + ((1023u - 127u) << 20)))
+      tile_tenant_any(a, tt, u, decompose((double)s), bad);
+  }
+  return s;
+}
+
+// The last min(n, 32) deferred requests of the tile, one per lane: prefills,
+// tenants and values off the common path, with every lane busy.  Returns how
+// many are left.
+template <int MODE>
+__device__ __noinline__ int tile_flush(const TileArgs &a, const TenTab tt, const TSmem &ts, const WarpTile &wt,
+                                       int64_t rbase, int n, int lane) {
+  const int left = max(n - 32, 0);
+  __syncwarp();
+  if (left + lane < n) {
+    const uint32_t v = wt.list[left + lane];
+    const TileRec rec = wt.rec[v >> 16];
+    const int64_t i = rbase + (v & 0xffffu);
+    const int32_t p = a.p[i], c = a.c[i], u = (MODE & M_TEN) ? a.ten[i] : 0;
+    if (MODE & M_F32) {
+      int bad = 0;
+      const float f = tile_one_f32<MODE>(a, tt, rec, p, c, u, &bad);
+      if (a.share32) __stcs(a.share32 + i, f);
+      if (bad) flag(a.status, kStatusData);
+    } else {
+      double d;
+      if (tile_one<MODE>(a, tt, ts, rec, (int64_t)(rec.a.z >> 4), i, p, c, u, &d) && a.share) __stcs(a.share + i, d);
+    }
+  }
+  __syncwarp();
+  return left;
+}
+
+// The tile's shares, four consecutive requests per lane and step.  The loop
+// takes decode requests (p = 1; fp32 variant: any) of the batch that the
+// lane's first one belongs to, on the common path, without a
+// branch; the rest goes to the warp's list, which is worked off 32 at
+// a time.  vec: the share array allows 32-byte (fp32: 16-byte) stores.
+template <int MODE>
+__device__ __forceinline__ void tile_shares(const TileArgs &a, const TenTab tt, const TSmem &ts, WarpTile &wt,
+                                            const TileSrc &src, int64_t rbase, int first, int cnt, bool vec,
+                                            int lane) {
+  constexpr bool kTen = (MODE & M_TEN) != 0, kF32 = (MODE & M_F32) != 0;
+  int nl = 0;
+  Quad nx = load_quad<kTen>(src.p, src.c, src.u, 4 * lane, src.lim);
+#pragma unroll 1
+  for (int b = 0; b < cnt; b += 128) {
+    const int e = b + 4 * lane;
+    const Quad v = nx;
+    if (b + 128 < cnt) nx = load_quad<kTen>(src.p, src.c, src.u, e + 128, src.lim);
+    const int32_t p[4] = {v.p.x, v.p.y, v.p.z, v.p.w}, c[4] = {v.c.x, v.c.y, v.c.z, v.c.w};
+    const uint32_t u[4] = {(uint32_t)v.x.x, (uint32_t)v.x.y, (uint32_t)v.x.z, (uint32_t)v.x.w};
+    // the quad's requests that are the tile's, and those before the next head
+    const int hi = min(max(cnt - e, 0), 4), lo = max(first - e, 0);
+    const uint32_t vm = ((1u << hi) - 1u) & (15u << lo);
+    const uint32_t word = wt.bits[b / 32 + (lane >> 3)];
+    const int sh = e & 31;
+    const uint32_t hb = (word >> sh) & 14u;
+    const uint32_t run = vm & ((hb & (0u - hb)) - 1u);  // no head: all four
+    // record of the first request; -1 before the tile's first batch
+    const int r0 = min((int)wt.rank[b / 32 + (lane >> 3)] + __popc(word & ((2u << sh) - 1u)), kTRec - 4) - 1;
+    const TileRec rec = wt.rec[max(r0, 0)];
+    const int32_t pe = (rec.a.z & 8u) ? 1 : -1;
+    bool go[4];
+    uint32_t dlo[4], dhi[4];
+    float f[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      go[k] = ((run >> k) & 1u) != 0u && r0 >= 0;
+      if (kF32) {
+        const Share32 q{__uint_as_float(rec.k.x), __uint_as_float(rec.k.y), __uint_as_float(rec.k.z),
+                        __uint_as_float(rec.k.w)};
+        f[k] = share_f32(q, p[k], c[k]);
+        // a positive normal float's double: the same significand, the exponent rebiased
+        const uint32_t x = __float_as_uint(f[k]);
+        dlo[k] = x << 29;
+        dhi[k] = (x >> 3) + ((1023u - 127u) << 20);
+        if (kTen) go[k] = go[k] && x - 0x00800000u < 0x7f000000u;
+      } else {
+        go[k] = go[k] && (MODE & M_FIX) && p[k] == pe;
+        const double d = tile_value(rec, rec.k.x, rec.k.y, rec.k.z, c[k]);
+        dlo[k] = (uint32_t)__double2loint(d);
+        dhi[k] = (uint32_t)__double2hiint(d);
+      }
+    }
+    if (kTen) ten_add4(a, tt, go, u, dlo, dhi, lane);
+    uint32_t dm = vm;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) dm &= go[k] ? ~(1u << k) : ~0u;
+    const int64_t i0 = rbase + e;
+    if (kF32 && a.share32) {
+      if (vec && (go[0] && go[1] && go[2] && go[3])) {
+        __stcs(reinterpret_cast<float4 *>(a.share32 + i0), make_float4(f[0], f[1], f[2], f[3]));
+      } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (go[k]) __stcs(a.share32 + i0 + k, f[k]);
+      }
+    }
+    if (!kF32 && a.share) {
+      double d[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) d[k] = __hiloint2double((int)dhi[k], (int)dlo[k]);
+      if (vec && (go[0] && go[1] && go[2] && go[3])) {
+        store4(a.share + i0, d);
+      } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (go[k]) __stcs(a.share + i0 + k, d[k]);
+      }
+    }
+    if (__any_sync(kFull, dm != 0u)) {
+      const uint32_t lt = (1u << lane) - 1u;
+      int at = nl;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const uint32_t bm = __ballot_sync(kFull, (dm >> k) & 1u);
+        at += __popc(bm & lt);
+        nl += __popc(bm);
+      }
+      for (uint32_t m = dm; m; m &= m - 1u) {
+        const int k = __ffs(m) - 1;
+        const int rk = max(r0 + __popc(hb & ((2u << k) - 1u)), 0);
+        wt.list[at++] = (uint32_t)(e + k) | ((uint32_t)rk << 16);
+      }
+      while (nl >= 32) nl = tile_flush<MODE>(a, tt, ts, wt, rbase, nl, lane);
+    }
+  }
+  if (nl > 0) tile_flush<MODE>(a, tt, ts, wt, rbase, nl, lane);
+}
+
+// One batch walked by `kThreads` threads (a warp, or the CTA) from global
+// memory: sums, then a strided share pass.
+template <int MODE, int kThreads>
+__device__ __noinline__ void walk_batch(const TileArgs &a, const TenTab tt, TSmem &ts, int64_t b, int64_t r0,
+                                        int64_t n) {
+  const int tid = kThreads == 32 ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
+  int bad = 0;
+  Sums acc{0, 0, 0, 0};
+  for (int64_t i = tid; i < n; i += 4 * kThreads) {
+    int32_t p[4], c[4], f[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int64_t j = i + k * kThreads;
+      p[k] = j < n ? a.p[r0 + j] : 0;
+      c[k] = j < n ? a.c[r0 + j] : 0;
+      f[k] = j < n ? a.ph[r0 + j] : 0;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      check_req(p[k], c[k], f[k], &bad);
+      acc.s1 += p[k];
+      acc.s2 += c[k];
+      acc.s3 += (int64_t)p[k] * p[k];
+      acc.ph |= f[k];
+    }
+  }
+  acc = warp_sum(acc);
+  if (kThreads > 32) {
+    if ((threadIdx.x & 31) == 0) ts.red[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    acc = Sums{0, 0, 0, 0};
+#pragma unroll
+    for (int w = 0; w < kTWarps; ++w) acc = add_sums(acc, ts.red[w]);
+    __syncthreads();  // ts.red is rewritten for the next batch
+  }
+  const BatchAgg g{acc.s1, acc.s2, acc.s3, n, acc.ph > 0};
+  const int s = segment_of(a.mp, g);
+  if (tid == 0) tile_emit<MODE>(a, ts, b, g, s);
+  if ((MODE & M_ATTR) && n > 0) {
+    const TileRec rec = tile_record<MODE, false>(a, ts, s, n);
+    for (int64_t i = tid; i < n; i += kThreads) {
+      const int64_t q = r0 + i;
+      const int32_t p = a.p[q], c = a.c[q], u = (MODE & M_TEN) ? a.ten[q] : 0;
+      if (MODE & M_F32) {
+        const float f = tile_one_f32<MODE>(a, tt, rec, max(p, 0), max(c, 0), u, &bad);
+        if (a.share32) __stcs(a.share32 + q, f);
+      } else {
+        double d;
+        if (tile_one<MODE>(a, tt, ts, rec, n, q, p, c, u, &d) && a.share) __stcs(a.share + q, d);
+      }
+    }
+  }
+  if (bad) flag(a.status, kStatusData);
+}
+
+// ---------------------------------------------------------------- kernel
+
+template <int MODE>
+__global__ void __launch_bounds__(kTThreads, 1) k_tiles(const TileArgs a) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  TSmem &ts = *reinterpret_cast<TSmem *>(smem_raw);
+  constexpr bool kTen = (MODE & M_TEN) != 0;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  int bad = 0;
+
+  TenSmem &ten = *reinterpret_cast<TenSmem *>(smem_raw + sizeof(TSmem));
+  TenTab tt{};
+  if (kTen) {
+    tt.H = (uint32_t)a.H;
+    tt.base = smem_u32(&ten);
+    tt.w = smem_u32(ten.w0) + 4u * (lane & (kTCopies - 1));
+    uint32_t *z = reinterpret_cast<uint32_t *>(&ten);
+    for (int i = tid; i < (int)(sizeof(TenSmem) / 4); i += kTThreads) z[i] = 0;
+  }
+  if (MODE & M_ATTR) {
+    init_segs<MODE>(a, ts.seg);
+    if (tid < 4) {
+      const SegFix &f = a.mp.fx[tid];
+      ts.fx[tid] = f;
+      ts.seg[tid].pad = f.t_narrow && ((f.B.hi | f.A1.hi | f.A2.hi | f.A3.hi | f.A4.hi) < (1ull << 28));
+    }
+    if ((MODE & M_F32) && tid < 20) ts.cf[tid / 5][tid % 5] = __double2float_rn(a.mp.coef[tid / 5][tid % 5]);
+  }
+  if (tid == 0) ts.n_big = 0;
+  __syncthreads();
+
+  WarpTile &wt = ts.tile[wid];
+  const bool vec = (MODE & M_F32) ? ((uintptr_t)a.share32 & 15) == 0 : ((uintptr_t)a.share & 31) == 0;
+  // tile t's batches [b0, b1) and requests [r0, r1) are fetched while the tile
+  // before it is worked on
+  const int64_t stride = (int64_t)gridDim.x * kTWarps;
+  int64_t t = (int64_t)wid * gridDim.x + blockIdx.x;
+  int64_t b0 = 0, b1 = 0, r0 = 0, r1 = 0;
+  if (t < a.n_tiles) {
+    b0 = clampi(tile_bound(a, t), 0, a.n_batch);
+    b1 = clampi(tile_bound(a, t + 1), b0, a.n_batch);
+    r0 = clampi(a.off[b0], 0, a.n_req);
+    r1 = clampi(a.off[b1], r0, a.n_req);
+  }
+  while (t < a.n_tiles) {
+    const int64_t tn = t + stride;
+    int64_t n0 = 0, n1 = 0;
+    if (tn < a.n_tiles) {
+      n0 = tile_bound(a, tn);
+      n1 = tile_bound(a, tn + 1);
+    }
+    if (b1 - b0 > kTNb) {
+      b1 = b0 + kTNb;  // invalid offsets
+      bad = 1;
+    }
+    const int nb = (int)(b1 - b0);
+    const int64_t rbase = r0 & ~(int64_t)3;
+    int64_t off0 = lane <= nb ? a.off[b0 + lane] : 0;  // the first round's offsets
+    if (r1 - rbase > kTCap) {
+      // the last batch reaches too far: the tile's requests end at its start
+      r1 = nb > 0 ? clampi(a.off[b1 - 1], r0, a.n_req) : r0;
+      if (r1 - rbase > kTCap) r1 = rbase + kTCap;  // invalid offsets
+    }
+    const int cnt = (int)(r1 - rbase), first = (int)(r0 - rbase);
+    const TileSrc src{a.p + rbase, a.c + rbase, a.ph + rbase, kTen ? a.ten + rbase : nullptr,
+                      (int)(a.n_req - rbase < 0x40000000 ? a.n_req - rbase : 0x40000000)};
+
+    // 1. prefixes
+    if (MODE & M_ATTR) {
+      for (int i = lane; i < kTWords; i += 32) {
+        wt.bits[i] = 0;
+        if (i == 0) wt.rank[0] = 0;
+      }
+    }
+    const bool wide = tile_prefix(wt, src, cnt, lane);
+    __syncwarp();
+    n0 = clampi(n0, 0, a.n_batch);
+    n1 = clampi(n1, n0, a.n_batch);
+    int64_t nr0 = a.off[n0], nr1 = a.off[n1];
+
+    // 2. batches
+    int before = 0;  // non-empty batches of earlier rounds
+    bool direct = false;
+#pragma unroll 1
+    for (int i0 = 0; i0 < nb; i0 += 31) {
+      // lane 31 holds the bound after lane 30's batch
+      const int i = i0 + lane;
+      const int64_t o0 = i0 == 0 ? off0 : i <= nb ? a.off[b0 + i] : 0;
+      const int64_t o1 = __shfl_down_sync(kFull, o0, 1);
+      const bool act = lane < 31 && i < nb;
+      // staged: both bounds among the tile's requests, in order
+      const uint64_t d0 = (uint64_t)(o0 - rbase);
+      const int x = d0 <= (uint64_t)cnt ? (int)d0 : -1;
+      const int x1 = __shfl_down_sync(kFull, x, 1);
+      const bool staged = act && x >= 0 && x1 >= x && !wide;
+      TSum lo{0u, 0u, 0ull};
+      if (i <= nb && x >= 0) lo = prefix_at(wt, src, x);
+      const TSum hi{__shfl_down_sync(kFull, lo.s1, 1), __shfl_down_sync(kFull, lo.s2, 1),
+                    __shfl_down_sync(kFull, lo.s3, 1)};
+      const int n = staged ? x1 - x : 0;
+      const uint32_t ne = __ballot_sync(kFull, n > 0);
+      if (staged) {
+        constexpr uint64_t kM55 = (1ull << 55) - 1ull;
+        int64_t s1 = (int64_t)hi.s1 - lo.s1, s2 = (int64_t)hi.s2 - lo.s2;
+        int64_t s3 = (int64_t)(hi.s3 & kM55) - (int64_t)(lo.s3 & kM55);
+        int f = (int)(hi.s3 >> 55) - (int)(lo.s3 >> 55);
+        for (int k = x >> 8; k < (x1 >> 8); ++k) {
+          const uint4 v = wt.tot[k];
+          const uint64_t v3 = (uint64_t)v.z | ((uint64_t)v.w << 32);
+          s1 += v.x;
+          s2 += v.y;
+          s3 += (int64_t)(v3 & kM55);
+          f += (int)(v3 >> 55);
+        }
+        const BatchAgg g{s1, s2, s3, n, f > 0};
+        const int sg = segment_of(a.mp, g);
+        const int rank = before + __popc(ne & ((1u << lane) - 1u));
+        if ((MODE & M_ATTR) && n > 0 && rank < kTRec) {
+          wt.rec[rank] = tile_record<MODE, true>(a, ts, sg, n);
+          atomicOr(&wt.bits[x >> 5], 1u << (x & 31));
+          for (int w = (x >> 5) + 1; w <= (x1 >> 5); ++w) wt.rank[w] = (uint16_t)(rank + 1);
+        }
+        tile_emit<MODE>(a, ts, b0 + i, g, sg);
+      }
+      before += __popc(ne);
+      direct |= __any_sync(kFull, act && !staged);
+    }
+    __syncwarp();
+    nr0 = clampi(nr0, 0, a.n_req);
+    nr1 = clampi(nr1, nr0, a.n_req);
+
+    // 3. requests
+    if ((MODE & M_ATTR) && !wide && (kTen || a.share || a.share32))
+      tile_shares<MODE>(a, tt, ts, wt, src, rbase, first, cnt, vec, lane);
+    if (direct) {
+      // the last batch; every batch of a wide tile
+      for (int i = 0; i < nb; ++i) {
+        const int64_t o0 = a.off[b0 + i], o1 = a.off[b0 + i + 1];
+        const uint64_t d0 = (uint64_t)(o0 - rbase), d1 = (uint64_t)(o1 - rbase);
+        if (d0 <= d1 && d1 <= (uint64_t)cnt && !wide) continue;
+        const int64_t c0 = clampi(o0, 0, a.n_req), c1 = clampi(o1, c0, a.n_req);
+        if (c0 != o0 || c1 != o1) bad = 1;
+        int slot = kTBigs;
+        if (c1 - c0 > kTAlone) {
+          if (lane == 0) slot = atomicAdd(&ts.n_big, 1);
+          slot = __shfl_sync(kFull, slot, 0);
+        }
+        if (slot < kTBigs) {
+          if (lane == 0) ts.big[slot] = b0 + i;
+        } else {
+          walk_batch<MODE, 32>(a, tt, ts, b0 + i, c0, c1 - c0);
+        }
+      }
+    }
+    __syncwarp();
+    t = tn;
+    b0 = n0;
+    b1 = n1;
+    r0 = nr0;
+    r1 = nr1;
+  }
+
+  if (bad) flag(a.status, kStatusData);
+  __syncthreads();
+  const int nbig = min(ts.n_big, kTBigs);
+  for (int k = 0; k < nbig; ++k) {
+    const int64_t b = ts.big[k];
+    const int64_t c0 = clampi(a.off[b], 0, a.n_req), c1 = clampi(a.off[b + 1], c0, a.n_req);
+    walk_batch<MODE, kTThreads>(a, tt, ts, b, c0, c1 - c0);
+  }
+  if (kTen) {
+    __syncthreads();
+    for (int u = tid; u < a.H; u += kTThreads) {
+      i128 v = mk128(0ull, (uint64_t)ten.w2[u] | ((uint64_t)ten.w3[u] << 32));
+#pragma unroll
+      for (int r = 0; r < kTCopies; ++r) {
+        const int i = u * kTCopies + r;
+        v = add128(v, mk128((uint64_t)ten.w0[i] | ((uint64_t)ten.w1[i] << 32), 0ull));
+      }
+      if (v.lo | v.hi) pend_add(a.ten_pend, u, v);
+    }
+  }
+}
+
+}  // namespace lv
