@@ -49,7 +49,8 @@ sys.path.insert(0, ROOT)
 METRIC = "attributed requests/sec on 1 GB300; achieved HBM GB/s vs ~8 TB/s peak"
 KERNEL_SOURCES = ["paper_2608_08382_gb300/csrc/lv_kernels.cuh", "paper_2608_08382_gb300/csrc/lv_fixed.cuh",
                   "paper_2608_08382_gb300/csrc/lv_api.cu", "paper_2608_08382_gb300/csrc/lv_fit.cuh",
-                  "paper_2608_08382_gb300/csrc/lv_whatif.cuh", "paper_2608_08382_gb300/csrc/lv_warp.cuh",
+                  "paper_2608_08382_gb300/csrc/lv_whatif.cuh", "paper_2608_08382_gb300/csrc/lv_step.cuh",
+                  "paper_2608_08382_gb300/csrc/lv_tile.cuh",
                   "paper_2608_08382_gb300/csrc/lv_metrics.cuh"]
 
 
@@ -295,8 +296,8 @@ def _setup_attr(lv, ctx, w, stream, f32=False):
 
     return dict(step=step, e2e_step=e2e_step, units=w.n_req, unit="requests/s", metric=METRIC,
                 h2d=h2d,
-                d2h=(4 if f32 else 8) * (w.n_req + w.n_batch) + 8 * w.n_tenants, launches_per_step=5,
-                kernel="k_warps", time_mask=lv.LV_TIME_TILES,
+                d2h=(4 if f32 else 8) * (w.n_req + w.n_batch) + 8 * w.n_tenants, launches_per_step=4,
+                kernel="k_tiles", time_mask=lv.LV_TIME_TILES,
                 bytes_per_launch=(20.0 if f32 else 24.0) * w.n_req + (12.0 if f32 else 16.0) * w.n_batch,
                 bytes_rule=("20 B/request (p, c, phase, tenant read; fp32 share written) + 12 B/batch (offset read; "
                             "fp32 T written)" if f32 else
@@ -438,7 +439,7 @@ def _setup_fit(lv, ctx, w, stream):
 
     return dict(step=step, e2e_step=e2e_step, units=w.n_req, unit="requests/s", metric=METRIC_FIT,
                 h2d=sum(int(t.numel() * t.element_size()) for t in hp.values()) + int(hY.numel() * 8),
-                d2h=72 * 4 * 2 + 4, launches_per_step=5, kernel="k_warps", time_mask=lv.LV_TIME_TILES,
+                d2h=72 * 4 * 2 + 4, launches_per_step=5, kernel="k_tiles", time_mask=lv.LV_TIME_TILES,
                 bytes_per_launch=12.0 * w.n_req + 8.0 * (w.n_batch + 1) + 16.0 * w.n_batch,
                 bytes_rule="12 B/request (p, c, phase read) + 8 B/batch offset + 2 x 8 B/batch latencies read",
                 config={"n_batch": w.n_batch, "n_req": w.n_req, "n_y": 2, "seed": w.seed,
@@ -598,8 +599,7 @@ def run_ours(args, world, rank, local):
     achieved = s["bytes_per_launch"] / (kavg_ms / 1e3) / 1e9
     peak, peak_kind = measured_peaks()
     traffic = ncu_traffic(s["kernel"], args.workload)
-    timed = s.get("timed") or ("k_warps + k_jumbo, one event pair per launch pair" if s["kernel"] == "k_warps"
-                               else s["kernel"])
+    timed = s.get("timed") or s["kernel"]
     config = {"workload": desc, **s["config"], "parallelism": f"replicas{world}"}
     config.setdefault("l2", "inputs far larger than the 129 MB L2, no flush")
     line = {

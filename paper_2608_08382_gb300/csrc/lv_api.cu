@@ -15,8 +15,8 @@
 #include "lv_fit.cuh"
 #include "lv_kernels.cuh"
 #include "lv_metrics.cuh"
+#include "lv_step.cuh"
 #include "lv_tile.cuh"
-#include "lv_warp.cuh"
 #include "lv_whatif.cuh"
 
 using namespace lv;
@@ -26,13 +26,8 @@ struct lv_ctx {
   int sms = 0;
   int arith = LV_ARITH_AUTO;
   int *d_status = nullptr;
-  TilePart *d_tiles = nullptr;
-  int64_t tiles_cap = 0;
   int64_t *d_bound = nullptr;  // first batch of each tile (k_tiles)
   int64_t bound_cap = 0;
-  unsigned long long *d_ctr = nullptr;  // [0] warp tiles handed out, [1] jumbo batches queued
-  int64_t *d_jumbo = nullptr;
-  int64_t jumbo_cap = 0;
   KEntry *d_ktab = nullptr;
   int ktab_nk = 0;
   bool ktab_valid = false;
@@ -43,8 +38,7 @@ struct lv_ctx {
   cudaStream_t ktab_stream = nullptr;
   void *d_fit = nullptr;      // fit partials + solve output
   size_t fit_cap = 0;
-  int64_t last_grid = 0;      // CTAs of the most recent tile-kernel launch
-  std::vector<std::pair<uint64_t, int>> occ;  // (mode << 32 | dynamic smem) -> k_warps CTAs per SM
+  std::vector<std::pair<uint64_t, int>> occ;  // (mode << 32 | dynamic smem) -> k_tiles CTAs per SM
   void *d_wi = nullptr;       // what-if per-candidate / per-pending tables
   size_t wi_cap = 0;
   void *d_acc = nullptr;      // accuracy metrics: relative-error bits, partials, histograms
@@ -182,20 +176,6 @@ lv_status check_batches(const lv_batches *b, bool need_tenant) {
   return LV_OK;
 }
 
-lv_status ensure_tiles(lv_ctx *ctx, int64_t n) {
-  if (n <= ctx->tiles_cap) return LV_OK;
-  LV_CUDA(cudaDeviceSynchronize());
-  if (ctx->d_tiles) cudaFree(ctx->d_tiles);
-  ctx->d_tiles = nullptr;
-  int64_t cap = std::max<int64_t>(n, 1 << 16);
-  if (cudaMalloc(&ctx->d_tiles, cap * sizeof(TilePart)) != cudaSuccess) {
-    ctx->tiles_cap = 0;
-    return LV_ENOMEM;
-  }
-  ctx->tiles_cap = cap;
-  return LV_OK;
-}
-
 // Builds (or reuses) the per-model parameters and K table on `stream`.
 // Event record and wait that stay valid while `stream` is being captured into a
 // CUDA graph: the graph then records (waits for) the event itself at every
@@ -286,17 +266,7 @@ lv_status timing_end(cudaEvent_t stop, cudaStream_t stream) {
   return LV_OK;
 }
 
-// Dynamic shared memory of k_warps for a tenant table of H entries and n_y fit vectors.
-template <int MODE>
-size_t warps_smem(int H, int n_y) {
-  return sizeof(WSmem) + ((MODE & M_TEN) ? ten_bytes(H) : 0) +
-         ((MODE & M_FIT) ? (size_t)kWarps * 4 * fit_entries(n_y) * sizeof(FitAcc) : 0) +
-         ((MODE & M_ATTR) ? (size_t)kWarps * sizeof(DeferList) : 0);
-}
-
-constexpr int kJumboCtasPerSm = 2;
-
-// Occupancy of k_warps<MODE> for launches without a context, by (mode << 32 |
+// Occupancy of k_tiles<MODE> for launches without a context, by (mode << 32 |
 // dynamic shared memory); the kernel attributes are process-wide as well.
 template <int MODE>
 std::vector<std::pair<uint64_t, int>> &free_occ() {
@@ -307,113 +277,6 @@ template <int MODE>
 std::mutex &free_occ_mu() {
   static std::mutex m;
   return m;
-}
-
-// Upper bound on the CTAs of one k_warps + k_jumbo pair (rows of fit partials).
-int64_t max_tile_ctas(int sms) { return (int64_t)sms * (2048 / kWThreads + kJumboCtasPerSm); }
-
-// k_warps then k_jumbo for the partitioned batches in `a` (a.part, a.ctr,
-// a.jumbo* set, counters zeroed on `stream`).  *ctas receives the number of
-// CTAs launched (fit partial rows).  ctx may be null (no timing).
-template <int MODE>
-lv_status launch_warps_mode(lv_ctx *ctx, int sms, TileArgs &a, cudaStream_t stream, int64_t *ctas) {
-  *ctas = 0;
-  const size_t smem = warps_smem<MODE>(a.H, a.fit.n_y);
-  const size_t jsmem = sizeof(JSmem) + ((MODE & M_TEN) ? ten_bytes(a.H) : 0);
-  const uint64_t key = ((uint64_t)MODE << 32) | smem;
-  int per_sm = 0;
-  if (ctx) {
-    for (const auto &e : ctx->occ)
-      if (e.first == key) per_sm = e.second;
-  } else {
-    // context-free callers (lv_attribute_noalloc): a process-wide cache per mode
-    std::lock_guard<std::mutex> lock(free_occ_mu<MODE>());
-    for (const auto &e : free_occ<MODE>())
-      if (e.first == key) per_sm = e.second;
-  }
-  if (per_sm == 0) {
-    // kernel attributes and occupancy: once per (context, mode, shared-memory size)
-    LV_CUDA(cudaFuncSetAttribute(k_warps<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)warps_smem<MODE>(kHotMax, kFitMaxY)));
-    LV_CUDA(cudaFuncSetAttribute(k_jumbo<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(sizeof(JSmem) + ten_bytes(kHotMax))));
-    LV_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_warps<MODE>, kWThreads, smem));
-    if (per_sm < 1) per_sm = 1;
-    if (ctx) {
-      ctx->occ.emplace_back(key, per_sm);
-    } else {
-      std::lock_guard<std::mutex> lock(free_occ_mu<MODE>());
-      free_occ<MODE>().emplace_back(key, per_sm);
-    }
-  }
-  const int64_t grid = std::min<int64_t>(a.n_tiles, (int64_t)sms * per_sm);
-  if (grid <= 0) return LV_OK;
-  // k_jumbo: at most one CTA per batch that can exceed kJumbo requests (none
-  // for small inputs, e.g. a single serving step of a few hundred requests)
-  const int64_t jgrid = std::min<int64_t>((int64_t)sms * kJumboCtasPerSm, a.n_req / (kJumbo + 1));
-  cudaEvent_t stop = nullptr;
-  if (ctx) {
-    lv_status st = timing_begin(ctx, LV_TIME_TILES, stream, &stop);
-    if (st != LV_OK) return st;
-  }
-  k_warps<MODE><<<(unsigned)grid, kWThreads, smem, stream>>>(a);
-  LV_CUDA(cudaGetLastError());
-  if (jgrid > 0) {
-    k_jumbo<MODE><<<(unsigned)jgrid, kJBlock, jsmem, stream>>>(a, (int)grid);
-    LV_CUDA(cudaGetLastError());
-  }
-  *ctas = grid + jgrid;
-  return ctx ? timing_end(stop, stream) : LV_OK;
-}
-
-lv_status ensure_sched(lv_ctx *ctx, int64_t jumbo_cap) {
-  if (!ctx->d_ctr && cudaMalloc(&ctx->d_ctr, 2 * sizeof(unsigned long long)) != cudaSuccess) {
-    ctx->d_ctr = nullptr;
-    return LV_ENOMEM;
-  }
-  if (jumbo_cap <= ctx->jumbo_cap) return LV_OK;
-  LV_CUDA(cudaDeviceSynchronize());
-  if (ctx->d_jumbo) cudaFree(ctx->d_jumbo);
-  ctx->d_jumbo = nullptr;
-  ctx->jumbo_cap = 0;
-  const int64_t cap = std::max<int64_t>(jumbo_cap, 1 << 12);
-  if (cudaMalloc(&ctx->d_jumbo, sizeof(int64_t) * cap) != cudaSuccess) return LV_ENOMEM;
-  ctx->jumbo_cap = cap;
-  return LV_OK;
-}
-
-// Most batches of more than kJumbo requests that valid offsets allow.
-int64_t jumbo_bound(int64_t n_req) { return n_req / (kJumbo + 1) + 1; }
-
-// Partition + warp and jumbo kernels for the given batches.
-lv_status run_fit_tiles(lv_ctx *ctx, TileArgs &a, cudaStream_t stream) {
-  ctx->last_grid = 0;
-  const int64_t units = a.n_batch + a.n_req;
-  // larger tiles fill the per-lane batch groups better and cost fewer tile
-  // starts; keep at least six tiles per resident warp for the dynamic
-  // schedule's tail (4 kDW measured 3 % faster than 2 kDW on the fit workload)
-  const int64_t warps = (int64_t)ctx->sms * (2048 / kWThreads) * kWarps;
-  a.D = units / (4 * kDW) >= 6 * warps ? 4 * kDW : units / (2 * kDW) >= 6 * warps ? 2 * kDW : kDW;
-  a.n_tiles = (units + a.D - 1) / a.D;
-  if (a.n_batch == 0) return LV_OK;
-  lv_status st = ensure_tiles(ctx, a.n_tiles + 1);
-  if (st != LV_OK) return st;
-  st = ensure_sched(ctx, jumbo_bound(a.n_req));
-  if (st != LV_OK) return st;
-  a.part = ctx->d_tiles;
-  a.ctr = ctx->d_ctr;
-  a.jumbo_n = ctx->d_ctr + 1;
-  a.jumbo = ctx->d_jumbo;
-  a.jumbo_cap = ctx->jumbo_cap;
-  LV_CUDA(cudaMemsetAsync(ctx->d_ctr, 0, 2 * sizeof(unsigned long long), stream));
-  const int64_t nthreads = a.n_batch + 1;
-  const int64_t pblocks = std::min<int64_t>((nthreads + 255) / 256, (int64_t)ctx->sms * 16);
-  k_partition<<<(unsigned)pblocks, 256, 0, stream>>>(a.off, a.n_batch, a.n_req, a.n_tiles, a.D, ctx->d_tiles,
-                                                     ctx->d_status);
-  LV_CUDA(cudaGetLastError());
-  int64_t *g = &ctx->last_grid;
-  const int sms = ctx->sms;
-  return launch_warps_mode<M_FEAT | M_FIT>(ctx, sms, a, stream, g);
 }
 
 // Tiles of the batches: D merge positions each, so that the warps' rounds of
@@ -438,7 +301,7 @@ TilePlan plan_tiles(int64_t n_batch, int64_t n_req, int64_t warps) {
 // without one, process; shared-memory size).
 template <int MODE>
 lv_status tiles_occupancy(lv_ctx *ctx, size_t smem, int *per_sm) {
-  const uint64_t key = ((uint64_t)(MODE | 1 << 16) << 32) | smem;
+  const uint64_t key = ((uint64_t)MODE << 32) | smem;
   *per_sm = 0;
   if (ctx) {
     for (const auto &e : ctx->occ)
@@ -527,6 +390,7 @@ lv_status run_tiles(lv_ctx *ctx, TileArgs &a, int mode, cudaStream_t stream) {
     case M_ATTR | M_F32: return run_tiles_mode<M_ATTR | M_F32>(ctx, sms, a, nullptr, 0, stream);
     case M_ATTR | M_TEN | M_F32: return run_tiles_mode<M_ATTR | M_TEN | M_F32>(ctx, sms, a, nullptr, 0, stream);
     case M_FEAT: return run_tiles_mode<M_FEAT>(ctx, sms, a, nullptr, 0, stream);
+    case M_FIT: return run_tiles_mode<M_FIT>(ctx, sms, a, nullptr, 0, stream);
     default: return LV_EINVAL;
   }
 }
@@ -614,12 +478,15 @@ lv_status fit_pass(lv_ctx *ctx, const lv_batches *b, const double *y, int32_t n_
   lv_status st = check_batches(b, false);
   if (st != LV_OK) return st;
   if (b->n_batch > 0 && (!y || !aligned(y, 8))) return LV_EINVAL;
-  // scratch: per-CTA partials (at most 2048 / kBlock CTAs per SM), totals, solve output
+  // scratch: per-CTA partials, totals, solve output, each batch's sums and segment
   const int NE = fit_entries(n_y), n_ent = 4 * NE;
-  const int64_t max_cta = max_tile_ctas(ctx->sms);
-  const size_t o_tot = ((size_t)max_cta * n_ent * sizeof(FitAcc) + 255) & ~(size_t)255;
+  const int rows = std::max(1, 2 * ctx->sms / (1 + n_y));  // two CTAs per SM over the kinds of entry
+  const size_t nb = (size_t)b->n_batch;
+  const size_t o_tot = ((size_t)rows * n_ent * sizeof(FitAcc) + 255) & ~(size_t)255;
   const size_t o_out = (o_tot + (size_t)n_ent * sizeof(FitAcc) + 255) & ~(size_t)255;
-  const size_t need = o_out + sizeof(FitOut) * 4 * kFitMaxY;
+  const size_t o_feat = (o_out + sizeof(FitOut) * 4 * kFitMaxY + 255) & ~(size_t)255;
+  const size_t o_seg = o_feat + 4 * sizeof(int64_t) * nb;
+  const size_t need = o_seg + nb;
   if (need > ctx->fit_cap) {
     LV_CUDA(cudaDeviceSynchronize());
     if (ctx->d_fit) cudaFree(ctx->d_fit);
@@ -632,6 +499,8 @@ lv_status fit_pass(lv_ctx *ctx, const lv_batches *b, const double *y, int32_t n_
   FitAcc *partial = reinterpret_cast<FitAcc *>(base);
   FitAcc *totals = reinterpret_cast<FitAcc *>(base + o_tot);
   FitOut *out = reinterpret_cast<FitOut *>(base + o_out);
+  int64_t *feat = reinterpret_cast<int64_t *>(base + o_feat);
+  uint8_t *seg = base + o_seg;
 
   TileArgs a{};
   a.p = b->p;
@@ -643,14 +512,14 @@ lv_status fit_pass(lv_ctx *ctx, const lv_batches *b, const double *y, int32_t n_
   a.status = ctx->d_status;
   a.mp.split[0] = split[0];
   a.mp.split[1] = split[1];
-  a.fit.y = y;
-  a.fit.n_y = n_y;
-  a.fit.partial = partial;
-  ctx->last_grid = 0;
-  st = run_fit_tiles(ctx, a, stream);
+  a.bfeat = feat;
+  a.bseg = seg;
+  st = run_tiles(ctx, a, M_FIT, stream);
   if (st != LV_OK) return st;
-  const int n_cta = (int)ctx->last_grid;
-  k_fit_reduce<<<n_ent, kFitRedThreads, 0, stream>>>(partial, n_cta, n_ent, totals);
+  k_fit_gram<<<dim3((unsigned)rows, 1 + n_y), kGramThreads, 0, stream>>>(feat, seg, b->n_batch, y, n_y, partial,
+                                                                         ctx->d_status);
+  LV_CUDA(cudaGetLastError());
+  k_fit_reduce<<<n_ent, kFitRedThreads, 0, stream>>>(partial, rows, n_ent, totals);
   LV_CUDA(cudaGetLastError());
   *totals_out = totals;
   *out_out = out;
@@ -821,10 +690,7 @@ void lv_ctx_destroy(lv_ctx *ctx) {
   if (!ctx) return;
   cudaDeviceSynchronize();
   if (ctx->d_status) cudaFree(ctx->d_status);
-  if (ctx->d_tiles) cudaFree(ctx->d_tiles);
   if (ctx->d_bound) cudaFree(ctx->d_bound);
-  if (ctx->d_ctr) cudaFree(ctx->d_ctr);
-  if (ctx->d_jumbo) cudaFree(ctx->d_jumbo);
   if (ctx->d_ktab) cudaFree(ctx->d_ktab);
   if (ctx->d_fit) cudaFree(ctx->d_fit);
   if (ctx->d_wi) cudaFree(ctx->d_wi);

@@ -9,17 +9,199 @@
 //     product is below 2^96);
 //   - X^T y in 256-bit fixed point with y rounded to a multiple of 2^-100 s
 //     (exact for any latency whose lowest bit is at least 2^-100 s).
-// The tile kernel computes the batch sums anyway; in fit mode each of the
-// (group, entry) accumulators is owned by one thread of the CTA, which adds the
-// contributions of the tile's batches of its group in registers.  CTA partials
-// are reduced exactly (integer adds) and each group's small system is solved in
-// double-double (about 106-bit) arithmetic after power-of-two column scaling,
-// by Cholesky, with singular and under-determined groups reported.
+// The tile kernel writes each batch's sums and segment, and k_fit_gram adds the
+// products with one lane per batch.  CTA partials are reduced exactly (integer
+// adds) and each group's small system is solved in double-double (about
+// 106-bit) arithmetic after power-of-two column scaling, with singular and
+// under-determined groups reported.
 #pragma once
 
 #include "lv_kernels.cuh"
 
 namespace lv {
+
+// ---------------------------------------------------------------- products
+
+// One row of blocks (blockIdx.y) per kind of entry: 0 the Gram matrix and the
+// flag, 1 + k the latency vector k's X^T y and y'y.  For each group a warp
+// collects the batches of that group in a queue and works them off 32 at a
+// time, one batch per lane, its accumulators in registers (exact integers: the
+// Gram's in 128 bits, X^T y modulo 2^192, y'y in 256).  Entry order
+// in `partial`: 15 Gram pairs (a <= b, row order), 5 X^T y per y, one y'y per
+// y, one flag (some batch has S1 != S3).
+// Bound by the integer multiplies, some 160 lane instructions a batch for the
+// Gram and 230 per latency vector.  With one entry per lane and all lanes on
+// one batch, inside the kernel over the requests, the same sums took
+// about 0.35 of 0.96 ms on 2e6 batches with two vectors.
+constexpr int kGramThreads = 256;
+constexpr int kGramWarps = kGramThreads / 32;
+constexpr int kGramMax = 16;  // entries of one row of blocks, at most
+
+template <int W>
+__device__ __forceinline__ void add_words(uint64_t *v, const uint64_t *o) {
+  uint64_t c = 0;
+#pragma unroll
+  for (int w = 0; w < W; ++w) {
+    const uint64_t t = v[w] + c, s = t + o[w];
+    c = (t < c ? 1ull : 0ull) + (s < t ? 1ull : 0ull);
+    v[w] = s;
+  }
+}
+
+// Sum over the warp of a W-word integer (modulo 2^(64 W)), into dst (lane 0),
+// sign-extended to four words when `sign`.
+template <int W>
+__device__ __forceinline__ void warp_words(uint64_t *v, FitAcc *dst, bool sign, int lane) {
+#pragma unroll
+  for (int d = 16; d; d >>= 1) {
+    uint64_t o[W];
+#pragma unroll
+    for (int w = 0; w < W; ++w) o[w] = __shfl_xor_sync(0xffffffffu, v[w], d);
+    add_words<W>(v, o);
+  }
+  if (lane == 0) {
+    const uint64_t fill = sign && (int64_t)v[W - 1] < 0 ? ~0ull : 0ull;
+#pragma unroll
+    for (int w = 0; w < 4; ++w) dst->w[w] = w < W ? v[w] : fill;
+  }
+}
+
+struct GramAcc {
+  uint64_t lin[5][2];   // n, S1, S2, S3, n^2
+  uint64_t sq[10][2];   // S1 S1, S1 S2, S1 S3, S1 n^2, S2 S2, ...
+  bool flag;
+};
+
+struct FitYAcc {
+  uint64_t xy[5][3];
+  uint64_t yy[4];
+};
+
+__device__ __forceinline__ void gram_add(GramAcc &g, const uint64_t *x) {
+#pragma unroll
+  for (int i = 0; i < 5; ++i) {
+    g.lin[i][0] += x[i];
+    g.lin[i][1] += g.lin[i][0] < x[i] ? 1ull : 0ull;
+  }
+  int e = 0;
+#pragma unroll
+  for (int i = 1; i < 5; ++i)
+#pragma unroll
+    for (int j = i; j < 5; ++j, ++e) {
+      const uint64_t p[2] = {x[i] * x[j], __umul64hi(x[i], x[j])};
+      add_words<2>(g.sq[e], p);
+    }
+  g.flag |= x[1] != x[3];
+}
+
+__device__ __forceinline__ void fit_y_add(FitYAcc &g, const uint64_t *x, i128 Y) {
+  const uint64_t neg = is_neg128(Y) ? ~0ull : 0ull;
+#pragma unroll
+  for (int i = 0; i < 5; ++i) {
+    // x Y modulo 2^192: x times Y's two words as unsigned, less x 2^128 for a negative Y
+    uint64_t p[3] = {x[i] * Y.lo, __umul64hi(x[i], Y.lo), __umul64hi(x[i], Y.hi) - (x[i] & neg)};
+    const uint64_t m = x[i] * Y.hi;
+    p[1] += m;
+    p[2] += p[1] < m ? 1ull : 0ull;
+    add_words<3>(g.xy[i], p);
+  }
+  // y'y: Y^2 (below 2^250) shifted right by 64 bits
+  if (neg) Y = neg128(Y);
+  const uint64_t l = Y.lo, h = Y.hi;
+  uint64_t w[4] = {__umul64hi(l, l), h * h, __umul64hi(h, h), 0ull};
+  const uint64_t hl[4] = {h * l, __umul64hi(h, l), 0ull, 0ull};
+  add_words<3>(w, hl);
+  add_words<3>(w, hl);
+  add_words<4>(g.yy, w);
+}
+
+__global__ void __launch_bounds__(kGramThreads, 2)
+    k_fit_gram(const int64_t *__restrict__ feat, const uint8_t *__restrict__ seg, int64_t nb,
+               const double *__restrict__ y, int n_y, FitAcc *__restrict__ partial, int *status) {
+  __shared__ int64_t queue[kGramWarps][64];
+  __shared__ FitAcc part[kGramWarps][kGramMax];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int k = (int)blockIdx.y - 1;  // latency vector, -1: the Gram matrix
+  const int NE = fit_entries(n_y);
+  const int64_t stride = (int64_t)gridDim.x * kGramThreads;
+  int64_t *q = queue[wid];
+  int bad = 0;
+#pragma unroll 1
+  for (int g = 0; g < 4; ++g) {
+    GramAcc ga{};
+    FitYAcc ya{};
+    int qn = 0;
+    for (int64_t i0 = blockIdx.x * (int64_t)kGramThreads + wid * 32; i0 < nb || qn > 0; i0 += stride) {
+      const bool rest = i0 >= nb;  // no batches left: work off the queue
+      if (!rest) {
+        const int64_t i = i0 + lane;
+        const bool in = i < nb && seg[i] == g;
+        const uint32_t m = __ballot_sync(0xffffffffu, in);
+        if (in) q[qn + __popc(m & ((1u << lane) - 1u))] = i;
+        qn += __popc(m);
+        __syncwarp();
+      }
+      if (qn < 32 && !rest) continue;
+      const int take = qn < 32 ? qn : 32;
+      const int64_t b = lane < take ? q[qn - take + lane] : -1;
+      qn -= take;
+      __syncwarp();
+      uint64_t x[5] = {0ull, 0ull, 0ull, 0ull, 0ull};
+      if (b >= 0) {
+        const uint64_t n = (uint64_t)feat[3 * nb + b];
+        x[0] = 1;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) x[1 + c] = (uint64_t)feat[c * nb + b];
+        x[4] = n * n;
+        if ((x[1] | x[2] | x[3] | x[4]) >= (uint64_t)kFitFeatMax || n >= (1ull << 24)) {
+          flag(status, kStatusOverflow);
+          x[0] = x[1] = x[2] = x[3] = x[4] = 0;
+        }
+      }
+      if (k < 0) {
+        gram_add(ga, x);
+      } else {
+        bool ovf = false;
+        const i128 Y = x[0] ? double_to_fix(y[k * nb + b], kFitYLsb, &ovf) : mk128(0, 0);
+        if (ovf) bad = 1;
+        fit_y_add(ya, x, Y);
+      }
+    }
+    FitAcc *pw = part[wid];
+    int ne;
+    if (k < 0) {
+      ne = 16;
+#pragma unroll
+      for (int i = 0; i < 5; ++i) warp_words<2>(ga.lin[i], pw + i, false, lane);
+#pragma unroll
+      for (int e = 0; e < 10; ++e) warp_words<2>(ga.sq[e], pw + 5 + e, false, lane);
+      const bool any = __any_sync(0xffffffffu, ga.flag);
+      if (lane == 0) pw[15] = FitAcc{{any ? 1ull : 0ull, 0ull, 0ull, 0ull}};
+    } else {
+      ne = 6;
+#pragma unroll
+      for (int i = 0; i < 5; ++i) warp_words<3>(ya.xy[i], pw + i, true, lane);
+      warp_words<4>(ya.yy, pw + 5, false, lane);
+    }
+    __syncthreads();
+    if ((int)threadIdx.x < ne) {
+      const int e = threadIdx.x;
+      const bool is_flag = k < 0 && e == 15;
+      FitAcc s{{0ull, 0ull, 0ull, 0ull}};
+      for (int w = 0; w < kGramWarps; ++w) {
+        const FitAcc &v = part[w][e];
+        if (is_flag)
+          s.w[0] |= v.w[0];
+        else
+          acc_add256(s.w, v.w[0], v.w[1], v.w[2], v.w[3]);
+      }
+      const int at = k < 0 ? (is_flag ? NE - 1 : e) : e < 5 ? 15 + 5 * k + e : 15 + 5 * n_y + k;
+      partial[(int64_t)blockIdx.x * (4 * NE) + g * NE + at] = s;
+    }
+    __syncthreads();
+  }
+  if (bad) flag(status, kStatusData);
+}
 
 // ---------------------------------------------------------------- reduction across CTAs
 

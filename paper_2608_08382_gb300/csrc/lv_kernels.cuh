@@ -1,7 +1,7 @@
 // Device code shared by the LLMVisor kernels (sm_103a): model parameters, the
-// merge-path partition, exact fixed-point evaluation of Eq. 1 and of the
-// per-request shares, exact tenant accumulation, and the small kernels around
-// them.  The request-streaming kernels themselves are in lv_warp.cuh.
+// exact fixed-point evaluation of Eq. 1 and of the per-request shares, exact
+// tenant accumulation, and the small kernels around them.  The kernel over the
+// requests of many batches is in lv_tile.cuh, the one-step kernel in lv_step.cuh.
 #pragma once
 
 #include <cstddef>
@@ -13,7 +13,6 @@ namespace lv {
 
 constexpr int kBlock = 256;                        // threads per CTA of the small kernels
 constexpr int kHotMax = 512;                       // tenants kept in shared memory per CTA
-constexpr int kNK = 256;                           // per-batch constants cached in shared memory for n <= kNK
 constexpr int64_t kPMaxFix = 1ll << 24;            // p beyond this uses the fp64 share path
 constexpr int kTenLsb = -72;                       // tenant totals: shares rounded to 2^-72 s, summed exactly
 
@@ -66,12 +65,6 @@ struct FitAcc {
   uint64_t w[4];  // 256-bit two's complement (Gram: low 128 bits; flag: w[0])
 };
 
-struct FitArgs {
-  const double *y;  // [n_y][n_batch]
-  int n_y;
-  FitAcc *partial;  // [gridDim.x][4 * fit_entries(n_y)]
-};
-
 __device__ __forceinline__ void acc_add256(uint64_t *w, uint64_t a0, uint64_t a1, uint64_t a2, uint64_t a3) {
   uint64_t s = w[0] + a0;
   uint64_t c = s < a0 ? 1ull : 0ull;
@@ -94,95 +87,21 @@ __device__ __forceinline__ i128 y_fixed(double y, bool *ovf) {
   return double_to_fix(y, kFitYLsb, ovf);
 }
 
-// One batch into the owner's accumulator.  x[0..4] = 1, S1, S2, S3, n^2.
-__device__ __forceinline__ void fit_owner_add(FitAcc &acc, int e, int n_y, const int64_t x[5], const double *yv,
-                                              int64_t nb, int64_t gb, bool s1_ne_s3, int *bad) {
-  if (e < 15) {
-    // Gram pair (a, b), a <= b, in row order
-    int a = 0, r = e;
-    while (r >= 5 - a) {
-      r -= 5 - a;
-      ++a;
-    }
-    const int b = a + r;
-    const uint64_t u = (uint64_t)x[a], v = (uint64_t)x[b];
-    acc_add256(acc.w, u * v, __umul64hi(u, v), 0, 0);
-  } else if (e < 15 + 5 * n_y) {
-    const int col = (e - 15) % 5, k = (e - 15) / 5;
-    bool ovf = false;
-    const i128 Y = y_fixed(yv[k * nb + gb], &ovf);
-    if (ovf) *bad = 1;
-    const bool neg = is_neg128(Y);
-    const i128 M = neg ? neg128(Y) : Y;
-    const uint64_t xv = (uint64_t)x[col];
-    // |Y| * x as 192 bits
-    const uint64_t p0 = M.lo * xv, p1 = __umul64hi(M.lo, xv);
-    const uint64_t q0 = M.hi * xv, q1 = __umul64hi(M.hi, xv);
-    uint64_t w0 = p0, w1 = p1 + q0, w2 = q1 + (w1 < p1 ? 1ull : 0ull), w3 = 0;
-    if (neg) {
-      w0 = ~w0;
-      w1 = ~w1;
-      w2 = ~w2;
-      w3 = ~w3;
-      w0 += 1;
-      if (w0 == 0) {
-        w1 += 1;
-        if (w1 == 0) {
-          w2 += 1;
-          if (w2 == 0) w3 += 1;
-        }
-      }
-    }
-    acc_add256(acc.w, w0, w1, w2, w3);
-  } else if (e < 15 + 6 * n_y) {
-    // y'y: Y^2 (below 2^250) shifted right by 64 bits; a sum of integers, so
-    // order independent, with an error below n * 2^-136 s^2
-    const int k = e - 15 - 5 * n_y;
-    bool ovf = false;
-    i128 Y = y_fixed(yv[k * nb + gb], &ovf);
-    if (ovf) *bad = 1;
-    if (is_neg128(Y)) Y = neg128(Y);
-    const uint64_t l = Y.lo, h = Y.hi;
-    const uint64_t ll1 = __umul64hi(l, l), hl0 = h * l, hl1 = __umul64hi(h, l);
-    const uint64_t hh0 = h * h, hh1 = __umul64hi(h, h);
-    // words 1..3 of l*l + 2^64 * 2*h*l + 2^128 * h*h (word 0 is dropped)
-    uint64_t w[4] = {ll1, hh0, hh1, 0};
-    acc_add256(w, hl0, hl1, 0, 0);
-    acc_add256(w, hl0, hl1, 0, 0);
-    acc_add256(acc.w, w[0], w[1], w[2], 0);
-  } else {
-    if (s1_ne_s3) acc.w[0] |= 1ull;
-  }
-}
-
-// First batch of a tile and its first request.
-struct TilePart {
-  int64_t b;
-  int64_t r;
-};
-
 struct TileArgs {
   const int32_t *p, *c, *ph, *ten;
   const int64_t *off;
   int64_t n_req, n_batch;
-  const TilePart *part;  // [n_tiles + 1]
   const int64_t *bound;    // [n_tiles + 1] first batch of each tile (k_tiles), or null:
   const uint32_t *bound32;  // the same in 32 bits (fewer than 2^32 batches)
   int64_t n_tiles;
-  int64_t D;             // merge positions per tile
   double *T, *share;
   float *T32, *share32;  // fp32 variant (M_F32): T and shares as float, or null
-  int64_t *bfeat;   // [5][n_batch] or null
-  uint8_t *bseg;    // [n_batch] or null
+  int64_t *bfeat;   // [5][n_batch] or null; M_FIT: [4][n_batch] S1, S2, S3, n
+  uint8_t *bseg;    // [n_batch] or null; M_FIT: 255 for an empty batch
   unsigned long long *ten_pend;  // [n_tenants][4] 32-bit limbs in 64-bit words, or null
   int32_t n_tenants, H;
   int *status;
   ModelP mp;
-  FitArgs fit;
-  unsigned long long *ctr;      // warp tiles handed out so far (zeroed before the launch)
-  unsigned long long *jumbo_n;  // batches queued for k_jumbo (zeroed before the launch)
-  int64_t *jumbo;               // [jumbo_cap] queued batch indices
-  int64_t jumbo_cap;
 };
 
 __device__ __forceinline__ void flag(int *status, int bit) {
@@ -191,44 +110,6 @@ __device__ __forceinline__ void flag(int *status, int bit) {
 
 __device__ __forceinline__ int64_t clampi(int64_t v, int64_t lo, int64_t hi) {
   return v < lo ? lo : (v > hi ? hi : v);
-}
-
-// ---------------------------------------------------------------- merge-path partition
-
-// part[k] = {b, off[b]} for the first batch b with b + off[b] >= k*D, for
-// k in [0, n_tiles); part[n_tiles] = {n_batch, n_req}.  Batch b writes the k in
-// (f(b-1)/D, f(b)/D], so every entry is written once by a coalesced pass.
-__global__ void k_partition(const int64_t *__restrict__ off, int64_t n_batch, int64_t n_req, int64_t n_tiles,
-                            int64_t D, TilePart *__restrict__ part, int *status) {
-  int bad = 0;
-  for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b <= n_batch;
-       b += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t raw = __ldg(off + b);
-    const int64_t ob = clampi(raw, 0, n_req);
-    int64_t kmin;
-    if (b == 0) {
-      if (raw != 0) bad = 1;
-      kmin = 0;
-    } else {
-      const int64_t rp = __ldg(off + b - 1);
-      if (rp > raw) bad = 1;
-      kmin = (b - 1 + clampi(rp, 0, n_req)) / D + 1;
-    }
-    int64_t kmax = (b + ob) / D;
-    if (b == n_batch) {
-      if (raw != n_req) bad = 1;
-      kmax = n_tiles;
-    }
-    if (kmin < 0) kmin = 0;
-    if (kmax > n_tiles) kmax = n_tiles;
-    for (int64_t k = kmin; k <= kmax; ++k) {
-      TilePart tp;
-      tp.b = b;
-      tp.r = ob;
-      part[k] = tp;
-    }
-  }
-  if (bad) flag(status, kStatusData);
 }
 
 // ---------------------------------------------------------------- batch sums
@@ -310,33 +191,11 @@ __device__ __forceinline__ bool eq1_fast(const SegFix &f, const BatchAgg &g, dou
   return true;
 }
 
-// Eq. 1 in single precision (the fp32 variant): coefficients rounded to float,
-// the sums converted, four fused multiply-adds.
-__device__ __forceinline__ float eq1_f32(const double *k, const BatchAgg &g) {
-  if (g.n == 0) return 0.0f;
-  float T = __double2float_rn(k[0]);
-  T = __fmaf_rn(__double2float_rn(k[1]), (float)g.s1, T);
-  T = __fmaf_rn(__double2float_rn(k[2]), (float)g.s2, T);
-  T = __fmaf_rn(__double2float_rn(k[3]), (float)g.s3, T);
-  T = __fmaf_rn(__double2float_rn(k[4]), (float)(g.n * g.n), T);
-  return T;
-}
-
-// Single-precision share coefficients of a segment and batch size n:
-// {K = fl(beta/n) + fl(a4 n), a1, a2, a3}.
+// Single-precision share coefficients of a batch: {K = fl(beta/n) + fl(a4 n),
+// a1, a2, a3}.
 struct Share32 {
   float K, a1, a2, a3;
 };
-
-__device__ __forceinline__ Share32 share32_const(const double *k, int64_t n) {
-  const float fn = (float)n;
-  Share32 r;
-  r.K = n > 0 ? __fadd_rn(__fdiv_rn(__double2float_rn(k[0]), fn), __fmul_rn(__double2float_rn(k[4]), fn)) : 0.0f;
-  r.a1 = __double2float_rn(k[1]);
-  r.a2 = __double2float_rn(k[2]);
-  r.a3 = __double2float_rn(k[3]);
-  return r;
-}
 
 // K + p (a1 + a3 p) + a2 c in fused multiply-adds.
 __device__ __forceinline__ float share_f32(const Share32 &q, int32_t p, int32_t c) {
@@ -521,7 +380,7 @@ enum : int {
   M_TEN = 4,     // accumulate tenant totals (with M_ATTR)
   M_FEAT = 8,    // write batch features / segment codes only
   M_FIX = 16,    // fixed-point arithmetic (else fp64)
-  M_FIT = 32,    // accumulate the least-squares statistics (with M_FEAT's reduction)
+  M_FIT = 32,    // write the batch sums of the least-squares statistics (instead of M_FEAT's outputs)
   M_F32 = 64,    // single-precision T and shares (into a.T32 / a.share32), with M_ATTR
 };
 
@@ -536,8 +395,7 @@ struct SegS {
   int pad;
 };
 
-// fx: the segments' fixed-point parameters (a shared-memory copy in k_warps,
-// where the lanes of a warp take different segments).
+// fx: the segments' fixed-point parameters.
 template <int MODE>
 __device__ __forceinline__ void emit_batch(const TileArgs &a, int64_t gb, const BatchAgg &g, int s, const SegFix *fx) {
   if (MODE & M_FEAT) {
@@ -550,7 +408,6 @@ __device__ __forceinline__ void emit_batch(const TileArgs &a, int64_t gb, const 
     }
     if (a.bseg) a.bseg[gb] = (uint8_t)s;
   }
-  if ((MODE & M_ATTR) && (MODE & M_F32) && a.T32) a.T32[gb] = eq1_f32(a.mp.coef[s], g);
   if ((MODE & M_ATTR) && !(MODE & M_F32) && a.T) {
     double T;
     if (!(MODE & M_FIX))

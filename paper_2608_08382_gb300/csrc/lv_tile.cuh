@@ -31,7 +31,7 @@
 // 16 to 256, 1,132 and 1,000; 2.6e7 in Pareto batches, 780 and 722.
 #pragma once
 
-#include "lv_warp.cuh"
+#include "lv_step.cuh"
 
 namespace lv {
 
@@ -275,7 +275,7 @@ __device__ __forceinline__ TileRec tile_record(const TileArgs &a, const TSmem &t
     kf = a.mp.ktab[s * (kTabN + 1) + (int)n].kf;
     slow = kf.hi == kKSlowHi;
   } else {
-    kf = batch_const_w<MODE>(a, nullptr, s, n, &slow);
+    kf = batch_const_w<MODE>(a, s, n, &slow);
   }
   const i128 k = (MODE & M_FIX) ? add128(kf, sg.A13) : kf;
   // fast: 2^64 <= constant < 2^95 (then the share, below 2^95 more, is in [2^64, 2^96)) and A2 < 2^64
@@ -342,6 +342,12 @@ __device__ __forceinline__ void tile_emit(const TileArgs &a, const TSmem &ts, in
     }
   } else if ((MODE & M_ATTR) && (MODE & M_FIX)) {
     if (a.T) a.T[b] = tile_eq1(a, ts, s, g);
+  } else if (MODE & M_FIT) {
+    a.bfeat[b] = g.s1;
+    a.bfeat[a.n_batch + b] = g.s2;
+    a.bfeat[2 * a.n_batch + b] = g.s3;
+    a.bfeat[3 * a.n_batch + b] = g.n;
+    a.bseg[b] = g.n > 0 ? (uint8_t)s : (uint8_t)255;
   } else {
     emit_batch<MODE>(a, b, g, s, nullptr);
   }
@@ -619,6 +625,17 @@ __device__ __forceinline__ void tile_shares(const TileArgs &a, const TenTab tt, 
                                             const TileSrc &src, int64_t rbase, int first, int cnt, bool vec,
                                             int lane) {
   constexpr bool kTen = (MODE & M_TEN) != 0, kF32 = (MODE & M_F32) != 0;
+  if (!(MODE & (M_FIX | M_F32))) {
+    // fp64 mode has no common path: one request per lane, in order
+    for (int e = lane; e < cnt; e += 32) {
+      if (e < first) continue;
+      const uint32_t word = wt.bits[e >> 5];
+      const int r = min((int)wt.rank[e >> 5] + __popc(word & ((2u << (e & 31)) - 1u)), kTRec) - 1;
+      const TileRec &rec = wt.rec[max(r, 0)];
+      tile_slow<MODE>(a, tt, ts, rec, (int64_t)(rec.a.z >> 4), rbase + e, src.p[e], src.c[e], kTen ? src.u[e] : 0);
+    }
+    return;
+  }
   int nl = 0;
   Quad nx = load_quad<kTen>(src.p, src.c, src.u, 4 * lane, src.lim);
 #pragma unroll 1

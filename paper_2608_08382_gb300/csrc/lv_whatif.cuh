@@ -16,7 +16,7 @@
 #pragma once
 
 #include "lv_kernels.cuh"
-#include "lv_warp.cuh"
+#include "lv_step.cuh"
 
 namespace lv {
 
