@@ -1000,7 +1000,7 @@ lv_status lv_fit(lv_ctx *ctx, const lv_batches *b, const double *y, int32_t n_y,
   FitOut *out = nullptr;
   lv_status st = fit_pass(ctx, b, y, n_y, inout[0].split, stream, &totals, &out);
   if (st != LV_OK) return st;
-  k_fit_solve<<<4 * kFitMaxY, 32, 0, stream>>>(totals, n_y, out);
+  k_fit_solve<<<4 * kFitMaxY, 64, 0, stream>>>(totals, n_y, out);
   LV_CUDA(cudaGetLastError());
   FitOut h[4 * kFitMaxY];
   LV_CUDA(cudaMemcpyAsync(h, out, sizeof(FitOut) * 4 * (size_t)n_y, cudaMemcpyDeviceToHost, stream));

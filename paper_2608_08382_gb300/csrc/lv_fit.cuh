@@ -29,13 +29,16 @@ namespace lv {
 // Gram's in 128 bits, X^T y modulo 2^192, y'y in 256).  Entry order
 // in `partial`: 15 Gram pairs (a <= b, row order), 5 X^T y per y, one y'y per
 // y, one flag (some batch has S1 != S3).
-// Bound by the integer multiplies, some 160 lane instructions a batch for the
-// Gram and 230 per latency vector.  With one entry per lane and all lanes on
-// one batch, inside the kernel over the requests, the same sums took
-// about 0.35 of 0.96 ms on 2e6 batches with two vectors.
+// Bound by instruction issue and latency (some 160 lane instructions a batch
+// for the Gram, 230 per latency vector; 16 warps per SM at 128 registers): 2e6
+// batches with two vectors take 150 us; 245 with one row of 32 segments looked
+// at per turn and nothing loaded ahead.  With one entry per lane and all lanes
+// on one batch, inside the kernel over the requests, the same sums took about
+// 0.35 of 0.96 ms.
 constexpr int kGramThreads = 256;
 constexpr int kGramWarps = kGramThreads / 32;
 constexpr int kGramMax = 16;  // entries of one row of blocks, at most
+constexpr int kGramScan = 8;  // rows of 32 batches looked at together
 
 template <int W>
 __device__ __forceinline__ void add_words(uint64_t *v, const uint64_t *o) {
@@ -70,6 +73,12 @@ struct GramAcc {
   uint64_t lin[5][2];   // n, S1, S2, S3, n^2
   uint64_t sq[10][2];   // S1 S1, S1 S2, S1 S3, S1 n^2, S2 S2, ...
   bool flag;
+};
+
+// A batch as loaded (n = 0: none).
+struct GramRaw {
+  int64_t s1, s2, s3, n;
+  double y;
 };
 
 struct FitYAcc {
@@ -115,61 +124,90 @@ __device__ __forceinline__ void fit_y_add(FitYAcc &g, const uint64_t *x, i128 Y)
   add_words<4>(g.yy, w);
 }
 
-__global__ void __launch_bounds__(kGramThreads, 2)
-    k_fit_gram(const int64_t *__restrict__ feat, const uint8_t *__restrict__ seg, int64_t nb,
-               const double *__restrict__ y, int n_y, FitAcc *__restrict__ partial, int *status) {
-  __shared__ int64_t queue[kGramWarps][64];
-  __shared__ FitAcc part[kGramWarps][kGramMax];
+struct GramSmem {
+  int64_t queue[kGramWarps][32 * (kGramScan + 1)];
+  FitAcc part[kGramWarps][kGramMax];
+};
+
+// kGram: the Gram matrix and the flag, else the latency vector k.
+template <bool kGram>
+__device__ __forceinline__ void fit_rows(GramSmem &sm, const int64_t *__restrict__ feat,
+                                         const uint8_t *__restrict__ seg, int64_t nb, const double *__restrict__ y,
+                                         int n_y, int k, FitAcc *__restrict__ partial, int *status) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int k = (int)blockIdx.y - 1;  // latency vector, -1: the Gram matrix
   const int NE = fit_entries(n_y);
-  const int64_t stride = (int64_t)gridDim.x * kGramThreads;
-  int64_t *q = queue[wid];
+  const int64_t stride = (int64_t)gridDim.x * kGramWarps * kGramScan * 32;
+  int64_t *q = sm.queue[wid];
   int bad = 0;
+  const double *yk = y + (int64_t)k * nb;
+  int s[kGramScan];
+  auto scan = [&](int64_t i0) {  // segments of kGramScan rows of 32 batches, their loads in flight together
+#pragma unroll
+    for (int r = 0; r < kGramScan; ++r) {
+      const int64_t i = i0 + 32 * r + lane;
+      s[r] = i < nb ? seg[i] : 255;
+    }
+  };
 #pragma unroll 1
   for (int g = 0; g < 4; ++g) {
     GramAcc ga{};
     FitYAcc ya{};
-    int qn = 0;
-    for (int64_t i0 = blockIdx.x * (int64_t)kGramThreads + wid * 32; i0 < nb || qn > 0; i0 += stride) {
-      const bool rest = i0 >= nb;  // no batches left: work off the queue
-      if (!rest) {
-        const int64_t i = i0 + lane;
-        const bool in = i < nb && seg[i] == g;
-        const uint32_t m = __ballot_sync(0xffffffffu, in);
-        if (in) q[qn + __popc(m & ((1u << lane) - 1u))] = i;
-        qn += __popc(m);
-        __syncwarp();
+    GramRaw cur{0, 0, 0, 0, 0.0};
+    auto add = [&]() {
+      uint64_t x[5] = {cur.n > 0 ? 1ull : 0ull, (uint64_t)cur.s1, (uint64_t)cur.s2, (uint64_t)cur.s3,
+                       (uint64_t)cur.n * (uint64_t)cur.n};
+      if ((x[1] | x[2] | x[3] | x[4]) >= (uint64_t)kFitFeatMax || (uint64_t)cur.n >= (1ull << 24)) {
+        flag(status, kStatusOverflow);
+        x[0] = x[1] = x[2] = x[3] = x[4] = 0;
       }
-      if (qn < 32 && !rest) continue;
-      const int take = qn < 32 ? qn : 32;
-      const int64_t b = lane < take ? q[qn - take + lane] : -1;
-      qn -= take;
-      __syncwarp();
-      uint64_t x[5] = {0ull, 0ull, 0ull, 0ull, 0ull};
-      if (b >= 0) {
-        const uint64_t n = (uint64_t)feat[3 * nb + b];
-        x[0] = 1;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) x[1 + c] = (uint64_t)feat[c * nb + b];
-        x[4] = n * n;
-        if ((x[1] | x[2] | x[3] | x[4]) >= (uint64_t)kFitFeatMax || n >= (1ull << 24)) {
-          flag(status, kStatusOverflow);
-          x[0] = x[1] = x[2] = x[3] = x[4] = 0;
-        }
-      }
-      if (k < 0) {
+      if (kGram) {
         gram_add(ga, x);
       } else {
         bool ovf = false;
-        const i128 Y = x[0] ? double_to_fix(y[k * nb + b], kFitYLsb, &ovf) : mk128(0, 0);
+        const i128 Y = x[0] ? double_to_fix(cur.y, kFitYLsb, &ovf) : mk128(0, 0);
         if (ovf) bad = 1;
         fit_y_add(ya, x, Y);
       }
+    };
+    int qn = 0;
+    int64_t i0 = ((int64_t)blockIdx.x * kGramWarps + wid) * kGramScan * 32;
+    scan(i0);
+    while (i0 < nb || qn > 0) {
+      const bool rest = i0 >= nb;  // no batches left: work off the queue
+      if (!rest) {
+#pragma unroll
+        for (int r = 0; r < kGramScan; ++r) {
+          const uint32_t m = __ballot_sync(0xffffffffu, s[r] == g);
+          if (s[r] == g) q[qn + __popc(m & ((1u << lane) - 1u))] = i0 + 32 * r + lane;
+          qn += __popc(m);
+        }
+        i0 += stride;
+        scan(i0);  // for the next turn
+        __syncwarp();
+      }
+#pragma unroll 1
+      while (qn >= 32 || (rest && qn > 0)) {
+        // the next 32 batches' values are loaded while the ones before them are added
+        const int take = qn < 32 ? qn : 32;
+        GramRaw nx{0, 0, 0, 0, 0.0};
+        if (lane < take) {
+          const int64_t b = q[qn - take + lane];
+          nx.s1 = feat[b];
+          nx.s2 = feat[nb + b];
+          nx.s3 = feat[2 * nb + b];
+          nx.n = feat[3 * nb + b];
+          if (!kGram) nx.y = yk[b];
+        }
+        qn -= take;
+        add();
+        cur = nx;
+      }
+      __syncwarp();  // the queue's slots are written again
     }
-    FitAcc *pw = part[wid];
+    add();
+    FitAcc *pw = sm.part[wid];
     int ne;
-    if (k < 0) {
+    if (kGram) {
       ne = 16;
 #pragma unroll
       for (int i = 0; i < 5; ++i) warp_words<2>(ga.lin[i], pw + i, false, lane);
@@ -186,21 +224,31 @@ __global__ void __launch_bounds__(kGramThreads, 2)
     __syncthreads();
     if ((int)threadIdx.x < ne) {
       const int e = threadIdx.x;
-      const bool is_flag = k < 0 && e == 15;
+      const bool is_flag = kGram && e == 15;
       FitAcc s{{0ull, 0ull, 0ull, 0ull}};
       for (int w = 0; w < kGramWarps; ++w) {
-        const FitAcc &v = part[w][e];
+        const FitAcc &v = sm.part[w][e];
         if (is_flag)
           s.w[0] |= v.w[0];
         else
           acc_add256(s.w, v.w[0], v.w[1], v.w[2], v.w[3]);
       }
-      const int at = k < 0 ? (is_flag ? NE - 1 : e) : e < 5 ? 15 + 5 * k + e : 15 + 5 * n_y + k;
+      const int at = kGram ? (is_flag ? NE - 1 : e) : e < 5 ? 15 + 5 * k + e : 15 + 5 * n_y + k;
       partial[(int64_t)blockIdx.x * (4 * NE) + g * NE + at] = s;
     }
     __syncthreads();
   }
   if (bad) flag(status, kStatusData);
+}
+
+__global__ void __launch_bounds__(kGramThreads, 2)
+    k_fit_gram(const int64_t *__restrict__ feat, const uint8_t *__restrict__ seg, int64_t nb,
+               const double *__restrict__ y, int n_y, FitAcc *__restrict__ partial, int *status) {
+  __shared__ GramSmem sm;
+  if (blockIdx.y == 0)
+    fit_rows<true>(sm, feat, seg, nb, y, n_y, 0, partial, status);
+  else
+    fit_rows<false>(sm, feat, seg, nb, y, n_y, (int)blockIdx.y - 1, partial, status);
 }
 
 // ---------------------------------------------------------------- reduction across CTAs
@@ -288,7 +336,17 @@ __device__ __forceinline__ dd dd_div(dd x, dd y) {
   return dd_add(q, dd{q3, 0.0});
 }
 
-__device__ __forceinline__ dd dd_scale(dd x, int e) { return dd{ldexp(x.hi, e), ldexp(x.lo, e)}; }
+// x 2^e for results in the normal range (-1022 <= e <= 1023).
+__device__ __forceinline__ double scale2(double x, int e) { return __dmul_rn(x, __hiloint2double((e + 1023) << 20, 0)); }
+__device__ __forceinline__ dd dd_scale(dd x, int e) { return dd{scale2(x.hi, e), scale2(x.lo, e)}; }
+
+// 1 / d for d.hi > 0: the double reciprocal and one Newton step, whose
+// correction needs only a double.
+__device__ __forceinline__ dd dd_inv(dd d) {
+  const double r = __drcp_rn(d.hi);
+  const double e = __fma_rn(-d.lo, r, __fma_rn(-d.hi, r, 1.0));
+  return quick_two_sum(r, __dmul_rn(r, e));
+}
 
 // Signed 256-bit integer (w, two's complement) times 2^E as double-double.
 // The leading 123 bits form a window whose value is below 2^123, so its
@@ -296,26 +354,27 @@ __device__ __forceinline__ dd dd_scale(dd x, int e) { return dd{ldexp(x.hi, e), 
 // overflow; hi is that rounding and lo the correctly rounded exact remainder.
 // Bits below the window are dropped (relative 2^-122).
 __device__ __forceinline__ dd int256_to_dd(const uint64_t *w, int E) {
-  uint64_t v[4] = {w[0], w[1], w[2], w[3]};
-  const bool neg = (int64_t)v[3] < 0;
+  uint64_t v0 = w[0], v1 = w[1], v2 = w[2], v3 = w[3];
+  const bool neg = (int64_t)v3 < 0;
   if (neg) {
-    for (int i = 0; i < 4; ++i) v[i] = ~v[i];
-    for (int i = 0; i < 4; ++i) {
-      if (++v[i] != 0) break;
-    }
+    v0 = ~v0 + 1ull;
+    v1 = ~v1 + (v0 == 0 ? 1ull : 0ull);
+    v2 = ~v2 + ((v0 | v1) == 0 ? 1ull : 0ull);
+    v3 = ~v3 + ((v0 | v1 | v2) == 0 ? 1ull : 0ull);
   }
-  int top = 3;
-  while (top > 0 && v[top] == 0) --top;
-  if (v[top] == 0) return dd{0.0, 0.0};
-  const int L = 64 * top + 63 - __clzll((long long)v[top]);  // leading bit
+  const int top = v3 ? 3 : v2 ? 2 : v1 ? 1 : 0;
+  const uint64_t vt = v3 ? v3 : v2 ? v2 : v1 ? v1 : v0;
+  if (vt == 0) return dd{0.0, 0.0};
+  const int L = 64 * top + 63 - __clzll((long long)vt);  // leading bit
   i128 win;
   int Ew = E;
   if (L <= 122) {
-    win = mk128(v[0], v[1]);
+    win = mk128(v0, v1);
   } else {
     const int sh = L - 122;  // right shift that puts the leading bit on bit 122
     const int q = sh >> 6, rb = sh & 63;
-    const uint64_t a0 = v[q], a1 = q + 1 < 4 ? v[q + 1] : 0, a2 = q + 2 < 4 ? v[q + 2] : 0;
+    const uint64_t a0 = q == 0 ? v0 : q == 1 ? v1 : v2, a1 = q == 0 ? v1 : q == 1 ? v2 : v3,
+                   a2 = q == 0 ? v2 : q == 1 ? v3 : 0ull;
     win.lo = rb ? (a0 >> rb) | (a1 << (64 - rb)) : a0;
     win.hi = rb ? (a1 >> rb) | (a2 << (64 - rb)) : a1;
     Ew = E + sh;
@@ -352,21 +411,23 @@ __device__ __forceinline__ void gram_ab(int e, int &a, int &b) {
 
 __device__ __forceinline__ dd dd_sub(dd x, dd y) { return dd_add(x, dd_neg(y)); }
 
-// One warp per (y vector k, group g), block k * 4 + g: builds, scales and
+// One block per (y vector k, group g), block k * 4 + g: builds, scales and
 // solves the normal equations from the exact totals.  Lanes convert the 21
-// totals at once; the Cholesky factorisation goes column by column, the pivot
-// on one lane and the rest of the column on the lanes of its rows; the
-// substitutions run on lane 0; the residual sum of squares adds its 30 terms
-// on 30 lanes.  A dropped a3 column becomes a unit row and column with a zero
-// right-hand side (its coefficient solves to 0).  Each pivot is inverted once
-// in double-double and the eliminations multiply.  Loops stay rolled: the
-// kernel runs once per fit, so its code is fetched cold.
-__global__ void __launch_bounds__(32) k_fit_solve(const FitAcc *__restrict__ totals, int n_y, FitOut *__restrict__ out) {
-  __shared__ dd G[15], R[5], L[15], rs[5], inv[5], zz[5];
-  __shared__ dd YY;
+// totals at once.  The elimination (L D L^T, right-looking, the right-hand side
+// as a sixth row) takes one column at a time: every lane inverts the pivot, and
+// each of the remaining entries is updated on its own lane, so a column costs
+// one inverse, two products and one sum of dependent double-double arithmetic;
+// the back substitution and the residual sum go side by side the same way,
+// while the second warp forms the total sum of squares.  A dropped a3 column
+// becomes a unit row and column with a zero right-hand side (its coefficient
+// solves to 0).  Bound by the latency of that chain (one warp, 22 us;
+// with a left-looking Cholesky factorisation, one lane on the pivot, 79).  Loops
+// stay rolled: the kernel runs once per fit, so its code is fetched cold.
+__global__ void __launch_bounds__(64) k_fit_solve(const FitAcc *__restrict__ totals, int n_y, FitOut *__restrict__ out) {
+  __shared__ dd G[15], R[5], A[15], B[5], inv[5];
+  __shared__ dd YY, SST;
   __shared__ double cf[5];
-  __shared__ int sc[5], sing;
-  const int lane = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31;
   const int k = blockIdx.x / 4, g = blockIdx.x % 4;
   if (k >= n_y) return;
   const int NE = fit_entries(n_y);
@@ -382,81 +443,78 @@ __global__ void __launch_bounds__(32) k_fit_solve(const FitAcc *__restrict__ tot
   if (drop3) o.dropped = 1 << 3;
   if (n < (drop3 ? 4 : 5)) {
     o.status = LV_ENODATA;
-    if (lane == 0) out[k * 4 + g] = o;
+    if (tid == 0) out[k * 4 + g] = o;
     return;
   }
   // exact totals as double-double, one per lane
-  if (lane < 15)
-    G[lane] = int256_to_dd(T[lane].w, 0);
-  else if (lane < 20)
-    R[lane - 15] = int256_to_dd(T[15 + k * 5 + (lane - 15)].w, kFitYLsb);
-  else if (lane == 20)
-    YY = int256_to_dd(T[15 + 5 * n_y + k].w, kFitYYLsb);
-  if (lane == 0) sing = 0;
-  __syncwarp();
+  if (tid < 21) {
+    const int e = tid < 15 ? tid : tid < 20 ? 15 + k * 5 + (tid - 15) : 15 + 5 * n_y + k;
+    const dd v = int256_to_dd(T[e].w, tid < 15 ? 0 : tid < 20 ? kFitYLsb : kFitYYLsb);
+    if (tid < 15)
+      G[tid] = v;
+    else if (tid < 20)
+      R[tid - 15] = v;
+    else
+      YY = v;
+  }
+  __syncthreads();
+  if (tid >= 32) {
+    if (lane == 0) SST = dd_sub(YY, dd_mul(dd_mul(R[0], R[0]), dd_inv(dd{(double)n, 0.0})));
+    __syncthreads();
+    return;
+  }
   if (drop3 && lane < 5) G[gram_idx(lane, 3)] = dd{lane == 3 ? 1.0 : 0.0, 0.0};
   if (drop3 && lane == 5) R[3] = dd{0.0, 0.0};
   __syncwarp();
-  // power-of-two column scaling: scaled diagonal near 1
-  if (lane < 5) {
-    int ex;
-    frexp(G[gram_idx(lane, lane)].hi, &ex);
-    sc[lane] = -(ex / 2);
-  }
+  // power-of-two column scaling: scaled diagonal near 1; lane e < 15 holds
+  // entry (a, b), a <= b, lane 15 + b the right-hand side of row b
+  int a = 5, b = lane - 15;
+  if (lane < 15) gram_ab(lane, a, b);
+  const bool mine = lane < 20;
+  auto scale_of = [&](int c) {
+    const int ex = (int)((__double_as_longlong(G[gram_idx(c, c)].hi) >> 52) & 0x7ff) - 1022;  // as frexp gives it
+    return -(ex / 2);
+  };
+  dd v{0.0, 0.0};
+  if (mine) v = lane < 15 ? dd_scale(G[lane], scale_of(a) + scale_of(b)) : dd_scale(R[b], scale_of(b));
+  if (lane < 15) A[lane] = v;
+  if (mine && lane >= 15) B[b] = v;
   __syncwarp();
-  if (lane < 15) {
-    int a, b;
-    gram_ab(lane, a, b);
-    L[lane] = dd_scale(G[lane], sc[a] + sc[b]);
-  } else if (lane < 20) {
-    rs[lane - 15] = dd_scale(R[lane - 15], sc[lane - 15]);
-  }
-  __syncwarp();
-  // Cholesky G = L L^T (lower triangle in L, indexed symmetrically)
+  bool sing = false;
   for (int j = 0; j < 5; ++j) {
-    if (lane == j) {
-      dd d = L[gram_idx(j, j)];
-      for (int m = 0; m < j; ++m) d = dd_sub(d, dd_mul(L[gram_idx(j, m)], L[gram_idx(j, m)]));
-      if (!(d.hi > 1e-24)) {
-        sing = 1;
-      } else {
-        // square root in double-double: s0 = sqrt(d.hi) and one Newton step, whose
-        // correction needs only a double factor 1/(2 s0); the inverse by one
-        // Newton step from the double reciprocal r0 = 1/s0
-        const double s0 = sqrt(d.hi), r0 = 1.0 / s0;
-        const dd s0sq = dd_mul(dd{s0, 0.0}, dd{s0, 0.0});
-        const dd s = dd_add(dd{s0, 0.0}, dd_mul(dd_sub(d, s0sq), dd{0.5 * r0, 0.0}));
-        L[gram_idx(j, j)] = s;
-        const dd e = dd_sub(dd{1.0, 0.0}, dd_mul(s, dd{r0, 0.0}));
-        inv[j] = dd_add(dd{r0, 0.0}, dd_mul(dd{r0, 0.0}, e));
-      }
+    const dd d = A[gram_idx(j, j)];
+    if (!(d.hi > 1e-24)) {
+      sing = true;
+      break;
+    }
+    const dd r = dd_inv(d);
+    if (lane == 0) inv[j] = r;
+    // entry (a, b) of the rest: less l_aj A_bj, l_aj = A_aj / d; a right-hand side: less l_bj B_j
+    if (mine && b > j && (lane >= 15 || a > j)) {
+      const dd x = lane < 15 ? A[gram_idx(a, j)] : B[j];
+      v = dd_sub(v, dd_mul(dd_mul(x, r), A[gram_idx(b, j)]));
     }
     __syncwarp();
-    if (sing) {
-      o.status = LV_ESINGULAR;
-      if (lane == 0) out[k * 4 + g] = o;
-      return;
-    }
-    if (lane > j && lane < 5) {
-      dd v = L[gram_idx(lane, j)];
-      for (int m = 0; m < j; ++m) v = dd_sub(v, dd_mul(L[gram_idx(lane, m)], L[gram_idx(j, m)]));
-      L[gram_idx(lane, j)] = dd_mul(v, inv[j]);
-    }
+    if (lane < 15)
+      A[lane] = v;
+    else if (mine)
+      B[b] = v;
     __syncwarp();
   }
-  if (lane == 0) {
-    for (int i = 0; i < 5; ++i) {
-      dd v = rs[i];
-      for (int m = 0; m < i; ++m) v = dd_sub(v, dd_mul(L[gram_idx(i, m)], zz[m]));
-      zz[i] = dd_mul(v, inv[i]);
-    }
-    for (int i = 4; i >= 0; --i) {
-      dd v = zz[i];
-      for (int m = i + 1; m < 5; ++m) v = dd_sub(v, dd_mul(L[gram_idx(m, i)], zz[m]));
-      zz[i] = dd_mul(v, inv[i]);  // the solution overwrites z, highest index first
-      cf[i] = (drop3 && i == 3) ? 0.0 : ldexp(zz[i].hi + zz[i].lo, sc[i]);
-    }
+  if (sing) {
+    o.status = LV_ESINGULAR;
+    if (lane == 0) out[k * 4 + g] = o;
+    __syncthreads();
+    return;
   }
+  // L^T x = D^-1 b, highest index first: lane i holds x_i
+  dd x{0.0, 0.0};
+  if (lane < 5) x = dd_mul(B[lane], inv[lane]);
+  for (int m = 4; m > 0; --m) {
+    const dd xm{__shfl_sync(0xffffffffu, x.hi, m), __shfl_sync(0xffffffffu, x.lo, m)};
+    if (lane < m) x = dd_sub(x, dd_mul(dd_mul(A[gram_idx(lane, m)], inv[lane]), xm));
+  }
+  if (lane < 5) cf[lane] = (drop3 && lane == 3) ? 0.0 : scale2(x.hi + x.lo, scale_of(lane));
   __syncwarp();
   for (int i = 0; i < 5; ++i) o.coef[i] = cf[i];
   // residuals of the rounded coefficients: SSR = y'y - 2 c'X'y + c'Gc (unscaled),
@@ -468,15 +526,13 @@ __global__ void __launch_bounds__(32) k_fit_solve(const FitAcc *__restrict__ tot
   } else if (lane < 30) {
     term = dd_neg(dd_scale(dd_mul(dd{cf[lane - 25], 0.0}, R[lane - 25]), 1));
   }
-#pragma unroll
   for (int d = 16; d; d >>= 1)
     term = dd_add(term, dd{__shfl_xor_sync(0xffffffffu, term.hi, d), __shfl_xor_sync(0xffffffffu, term.lo, d)});
+  __syncthreads();  // SST
   if (lane == 0) {
-    const dd sy = R[0];
     const dd ssr = dd_add(YY, term);
-    const dd sst = dd_sub(YY, dd_div(dd_mul(sy, sy), dd{(double)n, 0.0}));
     o.ssr = ssr.hi + ssr.lo;
-    const double sstv = sst.hi + sst.lo;
+    const double sstv = SST.hi + SST.lo;
     o.r2 = sstv != 0.0 ? 1.0 - o.ssr / sstv : __longlong_as_double(0x7ff8000000000000ll);
     o.status = LV_OK;
     out[k * 4 + g] = o;
