@@ -502,7 +502,7 @@ def _setup_whatif(lv, ctx, q, stream, admit=False):
     per_pair = 17 if admit else 16
     return dict(step=step, e2e_step=e2e_step, units=npairs, unit="pairs/s",
                 metric=METRIC_ADMIT if admit else METRIC_WHATIF,
-                h2d=h2d, d2h=per_pair * npairs, launches_per_step=6, kernel="k_wi_pairs",
+                h2d=h2d, d2h=per_pair * npairs, launches_per_step=2, kernel="k_wi_pairs",
                 time_mask=lv.LV_TIME_PAIRS, bytes_per_launch=float(per_pair) * npairs,
                 bytes_rule=(f"{per_pair} B/pair written (T_new, share_new" + (", admit" if admit else "") +
                             "); candidate and pending tables are cache-resident"),

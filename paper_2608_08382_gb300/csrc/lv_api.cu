@@ -554,12 +554,11 @@ lv_status whatif_run(lv_ctx *ctx, const lv_model *model, const lv_batches *cand,
   ModelP mp;
   st = prepare_model(ctx, model, stream, &mp);
   if (st != LV_OK) return st;
-  // scratch: candidate sums, segment codes, candidate and pending tables
-  const size_t o_feat = 0;
+  // scratch: the candidate table and, for the tile pass, candidate sums and segment codes
+  const bool by_block = nc <= (int64_t)kWiDirectPerSm * ctx->sms;
+  const size_t o_feat = (sizeof(CandP) * (size_t)nc + 255) & ~(size_t)255;
   const size_t o_seg = o_feat + sizeof(int64_t) * 5 * (size_t)nc;
-  const size_t o_cand = (o_seg + (size_t)nc + 255) & ~(size_t)255;
-  const size_t o_pend = (o_cand + sizeof(CandP) * (size_t)nc + 255) & ~(size_t)255;
-  const size_t need = o_pend + sizeof(PendP) * (size_t)np;
+  const size_t need = by_block ? o_feat : o_seg + (size_t)nc;
   if (need > ctx->wi_cap) {
     LV_CUDA(cudaDeviceSynchronize());
     if (ctx->d_wi) cudaFree(ctx->d_wi);
@@ -569,38 +568,47 @@ lv_status whatif_run(lv_ctx *ctx, const lv_model *model, const lv_batches *cand,
     ctx->wi_cap = need;
   }
   unsigned char *base = static_cast<unsigned char *>(ctx->d_wi);
-  int64_t *bfeat = reinterpret_cast<int64_t *>(base + o_feat);
-  uint8_t *bseg = base + o_seg;
-  CandP *candp = reinterpret_cast<CandP *>(base + o_cand);
-  PendP *pendp = reinterpret_cast<PendP *>(base + o_pend);
-
-  TileArgs a{};
-  a.p = cand->p;
-  a.c = cand->c;
-  a.ph = cand->phase;
-  a.off = cand->offsets;
-  a.n_req = cand->n_req;
-  a.n_batch = nc;
-  a.bfeat = bfeat;
-  a.bseg = bseg;
-  a.status = ctx->d_status;
-  a.mp = mp;
-  st = run_tiles(ctx, a, M_FEAT, stream);
-  if (st != LV_OK) return st;
-  k_wi_cand<<<(unsigned)((nc + 127) / 128), 128, 0, stream>>>(mp, bfeat, bseg, nc, candp);
-  LV_CUDA(cudaGetLastError());
-  k_wi_pend<<<(unsigned)((np + 127) / 128), 128, 0, stream>>>(mp, p_new, c_new, phase_new, np, pendp, adm,
-                                                              ctx->d_status);
-  LV_CUDA(cudaGetLastError());
-  const int64_t gx = (nc + kWiCols - 1) / kWiCols;
-  const int64_t rows_per_launch = (int64_t)65535 * kWiRows;
+  CandP *candp = reinterpret_cast<CandP *>(base);
+  cudaEvent_t stop;
+  if (by_block) {
+    st = timing_begin(ctx, LV_TIME_TILES, stream, &stop);
+    if (st != LV_OK) return st;
+    k_wi_cand_direct<<<(unsigned)nc, kWiCandThreads, 0, stream>>>(mp, cand->p, cand->c, cand->phase, cand->offsets,
+                                                                  cand->n_req, nc, candp, ctx->d_status);
+    LV_CUDA(cudaGetLastError());
+    st = timing_end(stop, stream);
+    if (st != LV_OK) return st;
+  } else {
+    TileArgs a{};
+    a.p = cand->p;
+    a.c = cand->c;
+    a.ph = cand->phase;
+    a.off = cand->offsets;
+    a.n_req = cand->n_req;
+    a.n_batch = nc;
+    a.bfeat = reinterpret_cast<int64_t *>(base + o_feat);
+    a.bseg = base + o_seg;
+    a.status = ctx->d_status;
+    a.mp = mp;
+    st = run_tiles(ctx, a, M_FEAT, stream);
+    if (st != LV_OK) return st;
+    k_wi_cand<<<(unsigned)((nc + 127) / 128), 128, 0, stream>>>(mp, a.bfeat, a.bseg, nc, candp);
+    LV_CUDA(cudaGetLastError());
+  }
+  // columns and rows of a block: as many columns as there are candidates for,
+  // and fewer rows while the blocks would not give every SM eight
+  const int lc = nc > 64 ? 7 : nc > 32 ? 6 : 5;
+  const int64_t gx = (nc + (1 << lc) - 1) >> lc;
+  int rpb = kWiRows;
+  while (rpb > (kWiThreads >> lc) && rpb > 4 && gx * ((np + rpb - 1) / rpb) < 8 * (int64_t)ctx->sms) rpb /= 2;
+  const int64_t rows_per_launch = (int64_t)65535 * rpb;
   for (int64_t j = 0; j < np; j += rows_per_launch) {
     const int64_t rows = std::min<int64_t>(rows_per_launch, np - j);
-    const dim3 grid((unsigned)gx, (unsigned)((rows + kWiRows - 1) / kWiRows));
-    cudaEvent_t stop;
+    const dim3 grid((unsigned)gx, (unsigned)((rows + rpb - 1) / rpb));
     st = timing_begin(ctx, LV_TIME_PAIRS, stream, &stop);
     if (st != LV_OK) return st;
-    k_wi_pairs<<<grid, kWiCols, 0, stream>>>(mp, candp, pendp, nc, np, j, T_new, share_new, adm.slo, adm.admit);
+    k_wi_pairs<<<grid, kWiThreads, 0, stream>>>(mp, candp, nc, p_new, c_new, phase_new, np, j, lc, rpb, adm, T_new,
+                                                share_new, ctx->d_status);
     LV_CUDA(cudaGetLastError());
     st = timing_end(stop, stream);
     if (st != LV_OK) return st;

@@ -9,14 +9,16 @@
 //        =            U_b[s]                            +         V_j[s]
 //     t_j = [fl(beta/(n+1)) + fl(a4 (n+1))]             +         V_j[s]
 //        =            W_b[s]                            +         V_j[s]
-// U, W and V are exact 128-bit fixed-point values, precomputed for all four
-// segments, so every pair costs a segment select, two exact additions and two
-// roundings.  In fp64 mode (or outside the exact range) a pair is evaluated
-// left to right in double like any other batch.
+// U, W and V are exact 128-bit fixed-point values, formed for all four segments
+// once per candidate (U, W) and once per block of pairs and row (V), so every
+// pair costs a segment select, two exact additions and two roundings.  In fp64
+// mode (or outside the exact range) a pair is evaluated left to right in double
+// like any other batch.
 #pragma once
 
 #include "lv_kernels.cuh"
 #include "lv_step.cuh"
+#include "lv_tile.cuh"
 
 namespace lv {
 
@@ -28,11 +30,24 @@ struct CandP {
   int32_t slow;  // 1: evaluate pairs of this candidate in fp64
 };
 
+// A pending request in a block of pairs.
 struct PendP {
   i128 V[4];
   int32_t p, c, phase, slow;
   double Lu, Bu;  // admission: the request's tenant's running total and budget
+  int64_t Bk;     // order_key of the budget, below every sum's where it is NaN
 };
+
+// Order of doubles as signed integers (not NaN; -0 below +0).
+__device__ __forceinline__ int64_t order_key(double x) {
+  const int64_t b = (int64_t)__double_as_longlong(x);
+  return b ^ ((b >> 63) & INT64_MAX);
+}
+// The key of a bound that x <= bound is tested against: -0 taken as +0, NaN
+// below everything.
+__device__ __forceinline__ int64_t bound_key(double x) {
+  return x != x ? INT64_MIN : order_key(__dadd_rn(x, 0.0));
+}
 
 // Admission inputs (null: plain what-if).  A pair (j, b) is admissible when
 // L[u_j] + share_new[j][b] <= budget[u_j] (one fp64 addition) and
@@ -45,7 +60,91 @@ struct AdmitArgs {
   uint8_t *admit;  // [n_pending][n_cand]
 };
 
-// Per candidate: U_b[s], W_b[s] for every segment, from the batch sums.
+// U_b[s] (half 0) or W_b[s] (half 1) of a candidate; *slow where the exact
+// range does not hold it.
+__device__ __forceinline__ i128 cand_const(const ModelP &mp, int s, int half, int64_t s1, int64_t s2, int64_t s3,
+                                           int64_t n, bool *slow) {
+  const int64_t n1 = n + 1;
+  if (half) return batch_k(mp, s, n1, slow).kf;
+  const SegFix &f = mp.fx[s];
+  const uint64_t F4 = (uint64_t)n1 * (uint64_t)n1;
+  if ((uint64_t)s1 > f.lim[0] || (uint64_t)s2 > f.lim[1] || (uint64_t)s3 > f.lim[2] || F4 > f.lim[3] ||
+      n1 > 0x7fffffffll) {
+    *slow = true;
+    return mk128(0, 0);
+  }
+  i128 U = f.B;
+  U = add128(U, mul128_u64(f.A1, (uint64_t)s1));
+  U = add128(U, mul128_u64(f.A2, (uint64_t)s2));
+  U = add128(U, mul128_u64(f.A3, (uint64_t)s3));
+  return add128(U, mul128_u64(f.A4, F4));
+}
+
+// Candidates straight from their requests, one block each: block sums, then
+// one thread per constant.  One launch in place of the tile bounds, the tile
+// pass and k_wi_cand: a planning call's few hundred to few thousand candidates
+// are bound by the chain of launches and of dependent loads (1,024
+// candidates of 144 requests: 29 us for that chain).  With more than
+// kWiDirectPerSm candidates per SM the tile pass, which packs small
+// batches, is as fast and takes over.
+constexpr int kWiCandThreads = 128;
+constexpr int kWiDirectPerSm = 16;
+__global__ void __launch_bounds__(kWiCandThreads) k_wi_cand_direct(ModelP mp, const int32_t *__restrict__ p,
+                                                                  const int32_t *__restrict__ c,
+                                                                  const int32_t *__restrict__ ph,
+                                                                  const int64_t *__restrict__ off, int64_t n_req,
+                                                                  int64_t nc, CandP *__restrict__ out, int *status) {
+  __shared__ Sums red[kWiCandThreads / 32];
+  const int64_t b = blockIdx.x;
+  const int tid = threadIdx.x;
+  int bad = 0;
+  const int64_t o0 = off[b], o1 = off[b + 1];
+  const int64_t r0 = clampi(o0, 0, n_req), r1 = clampi(o1, r0, n_req);
+  if (r0 != o0 || r1 != o1 || (b == 0 && o0 != 0) || (b == nc - 1 && o1 != n_req)) bad = 1;
+  Sums acc{0, 0, 0, 0};
+  for (int64_t i = r0 + tid; i < r1; i += 4 * kWiCandThreads) {
+    int32_t pv[4], cv[4], fv[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int64_t j = i + k * kWiCandThreads;
+      pv[k] = j < r1 ? p[j] : 0;
+      cv[k] = j < r1 ? c[j] : 0;
+      fv[k] = j < r1 ? ph[j] : 0;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      check_req(pv[k], cv[k], fv[k], &bad);
+      acc.s1 += pv[k];
+      acc.s2 += cv[k];
+      acc.s3 += (int64_t)pv[k] * pv[k];
+      acc.ph |= fv[k];
+    }
+  }
+  acc = warp_sum(acc);
+  if ((tid & 31) == 0) red[tid >> 5] = acc;
+  if (bad) flag(status, kStatusData);
+  __syncthreads();
+  if (tid >= 32) return;
+  acc = red[0];
+#pragma unroll
+  for (int w = 1; w < kWiCandThreads / 32; ++w) acc = add_sums(acc, red[w]);
+  bool slow = !mp.fixed;
+  if (tid < 8 && mp.fixed) {
+    const i128 v = cand_const(mp, tid & 3, tid >> 2, acc.s1, acc.s2, acc.s3, r1 - r0, &slow);
+    (tid < 4 ? out[b].U : out[b].W)[tid & 3] = v;
+  }
+  slow = __any_sync(kFull, slow);
+  if (tid == 0) {
+    out[b].s1 = acc.s1;
+    out[b].s2 = acc.s2;
+    out[b].s3 = acc.s3;
+    out[b].n = r1 - r0;
+    out[b].prefill = acc.ph > 0 ? 1 : 0;
+    out[b].slow = slow ? 1 : 0;
+  }
+}
+
+// The same from batch sums and segment codes (the tile pass).
 __global__ void k_wi_cand(ModelP mp, const int64_t *__restrict__ bfeat, const uint8_t *__restrict__ bseg,
                           int64_t nc, CandP *__restrict__ out) {
   const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -56,84 +155,22 @@ __global__ void k_wi_cand(ModelP mp, const int64_t *__restrict__ bfeat, const ui
   cp.s3 = bfeat[2 * nc + b];
   cp.n = bfeat[3 * nc + b];
   cp.prefill = (bseg[b] >> 1) & 1;
-  cp.slow = mp.fixed ? 0 : 1;
-  const int64_t n1 = cp.n + 1;
-  const uint64_t F4 = (uint64_t)n1 * (uint64_t)n1;
+  bool slow = !mp.fixed;
 #pragma unroll
   for (int s = 0; s < 4; ++s) {
-    cp.U[s] = mk128(0, 0);
-    cp.W[s] = mk128(0, 0);
-    if (!mp.fixed) continue;
-    const SegFix &f = mp.fx[s];
-    if ((uint64_t)cp.s1 > f.lim[0] || (uint64_t)cp.s2 > f.lim[1] || (uint64_t)cp.s3 > f.lim[2] || F4 > f.lim[3] ||
-        n1 > 0x7fffffffll) {
-      cp.slow = 1;
-      continue;
-    }
-    i128 U = f.B;
-    U = add128(U, mul128_u64(f.A1, (uint64_t)cp.s1));
-    U = add128(U, mul128_u64(f.A2, (uint64_t)cp.s2));
-    U = add128(U, mul128_u64(f.A3, (uint64_t)cp.s3));
-    U = add128(U, mul128_u64(f.A4, F4));
-    cp.U[s] = U;
-    bool slow = false;
-    cp.W[s] = batch_k(mp, s, n1, &slow).kf;
-    if (slow) cp.slow = 1;
+    cp.U[s] = mp.fixed ? cand_const(mp, s, 0, cp.s1, cp.s2, cp.s3, cp.n, &slow) : mk128(0, 0);
+    cp.W[s] = mp.fixed ? cand_const(mp, s, 1, cp.s1, cp.s2, cp.s3, cp.n, &slow) : mk128(0, 0);
   }
+  cp.slow = slow ? 1 : 0;
   out[b] = cp;
-}
-
-// Per pending request: V_j[s] = a1 p + a2 c + a3 p^2 for every segment.
-// With admission, also the request's tenant's total and budget (a tenant id
-// out of range records a data error and makes every pair of the request
-// inadmissible: NaN compares false).
-__global__ void k_wi_pend(ModelP mp, const int32_t *__restrict__ p_new, const int32_t *__restrict__ c_new,
-                          const int32_t *__restrict__ ph_new, int64_t np, PendP *__restrict__ out, AdmitArgs adm,
-                          int *status) {
-  const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (j >= np) return;
-  int32_t p = p_new[j], c = c_new[j], ph = ph_new[j];
-  int bad = 0;
-  check_req(p, c, ph, &bad);
-  PendP q;
-  q.p = p;
-  q.c = c;
-  q.phase = ph;
-  q.slow = (!mp.fixed || p > kPMaxFix) ? 1 : 0;
-  q.Lu = q.Bu = 0.0;
-  if (adm.admit) {
-    const int32_t u = adm.tenant[j];
-    if (u < 0 || u >= adm.n_tenants) {
-      bad = 1;
-      q.Lu = __longlong_as_double(0x7ff8000000000000ll);
-    } else {
-      q.Lu = adm.L[u];
-      q.Bu = adm.budget[u];
-    }
-  }
-  if (bad) flag(status, kStatusData);
-#pragma unroll
-  for (int s = 0; s < 4; ++s) {
-    q.V[s] = mk128(0, 0);
-    if (q.slow) continue;
-    const SegFix &f = mp.fx[s];
-    const i128 r = add128(f.A1, mul128_u32(f.A3, (uint32_t)p));
-    i128 V = mul128_u32(r, (uint32_t)p);
-    V = add128(V, f.a2_narrow ? mul_u64_u32(f.A2.lo, (uint32_t)c) : mul128_u32(f.A2, (uint32_t)c));
-    q.V[s] = V;
-  }
-  out[j] = q;
 }
 
 // V * 2^E rounded to double: the leading-word rounding for the common
 // magnitude 2^64 <= V < 2^96, the general rounding otherwise.
 __device__ __forceinline__ double round_fix(i128 V, int E) {
   const uint32_t v3 = (uint32_t)(V.hi >> 32), v2 = (uint32_t)V.hi;
-  if (v3 == 0u && v2 != 0u) {
-    uint64_t m;
-    int ex2;
-    return round96((uint32_t)V.lo, (uint32_t)(V.lo >> 32), v2, E, m, ex2);
-  }
+  if (v3 == 0u && v2 != 0u)
+    return round_top((uint32_t)V.lo, (uint32_t)(V.lo >> 32), v2, (uint32_t)(E + 32) << 20);
   return fix_to_double(V, E).d;
 }
 
@@ -147,70 +184,118 @@ __device__ __noinline__ void wi_pair_slow(const ModelP &mp, int s, int64_t s1, i
   *share = share_fp64(mp.coef[s], e.q, e.a4n, p, c);
 }
 
-constexpr int kWiCols = 128;  // candidates per block (one per thread)
-constexpr int kWiRows = 32;   // pending requests per block
+constexpr int kWiThreads = 128;  // threads per block
+constexpr int kWiRows = 32;      // pending requests per block, at most
 
-// Pair grid: block (bx, by) covers candidates [bx*kWiCols, +kWiCols) and pending
-// rows [j0 + by*kWiRows, +kWiRows); consecutive threads write consecutive
+// Pair grid: block (bx, by) covers candidates [bx * C, + C), C = 2^lc, and
+// pending rows [j_base + by * rows, + rows); thread t takes candidate t mod C
+// and every (128 / C)-th row.  Consecutive threads write consecutive
 // candidates of a row, so the row-major [pending][candidate] outputs are
-// coalesced.
-__global__ void __launch_bounds__(kWiCols) k_wi_pairs(ModelP mp, const CandP *__restrict__ cand,
-                                                       const PendP *__restrict__ pend, int64_t nc, int64_t np,
-                                                       int64_t j_base, double *__restrict__ T_new,
-                                                       double *__restrict__ share_new, double slo,
-                                                       uint8_t *__restrict__ admit) {
-  static_assert(kWiRows <= kWiCols, "one pending row per thread at most");
+// coalesced.  The host picks C and rows so that few candidates or few rows
+// still fill the chip (500 x 24 pairs: 15 us with 128 columns and 32 rows, 5.7
+// so).  The block's rows get their V here, one thread per row and segment; a
+// candidate's U and W of the segment in use stay in registers (they change with
+// the row only where the merged batch crosses the split or turns prefill), so a
+// pair reads one V from shared memory.  Bound by the stores: 16-17 B a pair
+// (4.2e6 pairs, 67 MB: 21.5 us, 24.4 with U and W read per pair).
+__global__ void __launch_bounds__(kWiThreads) k_wi_pairs(ModelP mp, const CandP *__restrict__ cand, int64_t nc,
+                                                         const int32_t *__restrict__ p_new,
+                                                         const int32_t *__restrict__ c_new,
+                                                         const int32_t *__restrict__ ph_new, int64_t np,
+                                                         int64_t j_base, int lc, int rows_per_block, AdmitArgs adm,
+                                                         double *__restrict__ T_new, double *__restrict__ share_new,
+                                                         int *status) {
   __shared__ PendP sp[kWiRows];
   __shared__ int sE[4];
-  const int64_t b = blockIdx.x * (int64_t)kWiCols + threadIdx.x;
-  const int64_t j0 = j_base + blockIdx.y * (int64_t)kWiRows;
-  const int rows = (int)(np - j0 < kWiRows ? np - j0 : kWiRows);
+  const int tid = threadIdx.x;
+  const int64_t j0 = j_base + blockIdx.y * (int64_t)rows_per_block;
+  const int rows = (int)(np - j0 < rows_per_block ? np - j0 : rows_per_block);
   int rslow = 0;
-  if (threadIdx.x < rows) {
-    sp[threadIdx.x] = pend[j0 + threadIdx.x];
-    rslow = sp[threadIdx.x].slow;
+  for (int i = tid; i < 4 * rows; i += kWiThreads) {
+    const int r = i >> 2, s = i & 3;
+    const int64_t j = j0 + r;
+    int32_t p = p_new[j], c = c_new[j], ph = ph_new[j];
+    int bad = 0;
+    check_req(p, c, ph, &bad);
+    const int slow = (!mp.fixed || p > kPMaxFix) ? 1 : 0;
+    rslow |= slow;
+    i128 V = mk128(0, 0);
+    if (!slow) {
+      const SegFix &f = mp.fx[s];
+      V = mul128_u32(add128(f.A1, mul128_u32(f.A3, (uint32_t)p)), (uint32_t)p);
+      V = add128(V, a2_times(f, (uint32_t)c));
+    }
+    sp[r].V[s] = V;
+    if (s == 0) {
+      sp[r].p = p;
+      sp[r].c = c;
+      sp[r].phase = ph;
+      sp[r].slow = slow;
+      if (adm.admit) {
+        // a tenant id out of range makes every pair of the request inadmissible: NaN compares false
+        const int32_t u = adm.tenant[j];
+        const bool in = u >= 0 && u < adm.n_tenants;
+        if (!in) bad = 1;
+        sp[r].Lu = in ? adm.L[u] : __longlong_as_double(0x7ff8000000000000ll);
+        sp[r].Bu = in ? adm.budget[u] : 0.0;
+        sp[r].Bk = bound_key(sp[r].Bu);
+      }
+      if (bad) flag(status, kStatusData);
+    }
   }
-  if (threadIdx.x < 4) sE[threadIdx.x] = mp.fx[threadIdx.x].E;
+  if (tid < 4) sE[tid] = mp.fx[tid].E;
   rslow = __syncthreads_or(rslow);
+  const int64_t b = ((int64_t)blockIdx.x << lc) + (tid & ((1 << lc) - 1));
   if (b >= nc) return;
   const CandP *cb = cand + b;
-  const int64_t s1 = cb->s1, s2 = cb->s2, s3 = cb->s3, n1 = cb->n + 1;
-  const int prefill = cb->prefill, cslow = cb->slow;
-  const int64_t sp0 = mp.split[0], sp1 = mp.split[1];
-  if (!cslow && !rslow && rows == kWiRows) {
-    // every pair of the block exact: no out-of-line call, rows unrolled for
-    // independent loads and roundings in flight
+  const int64_t s1 = cb->s1, sp0 = mp.split[0], sp1 = mp.split[1];
+  const int prefill = cb->prefill, step = kWiThreads >> lc;
+  int64_t o = (j0 + (tid >> lc)) * nc + b;
+  const int64_t ostep = step * nc;
+  if (!cb->slow && !rslow) {
+    // every pair of the block exact: no out-of-line call
+    int cur = -1, E = 0;
+    const int64_t slo_key = bound_key(adm.slo);
+    i128 U = mk128(0, 0), W = mk128(0, 0);
 #pragma unroll 4
-    for (int r = 0; r < kWiRows; ++r) {
-      const int32_t p = sp[r].p;
+    for (int r = tid >> lc; r < rows; r += step, o += ostep) {
       const int phase = (prefill | sp[r].phase) ? 1 : 0;
-      const int s = phase * 2 + ((s1 + p >= (phase ? sp1 : sp0)) ? 1 : 0);
+      const int s = phase * 2 + ((s1 + sp[r].p >= (phase ? sp1 : sp0)) ? 1 : 0);
+      if (s != cur) {
+        cur = s;
+        U = cb->U[s];
+        W = cb->W[s];
+        E = sE[s];
+      }
       const i128 V = sp[r].V[s];
-      const double T = round_fix(add128(cb->U[s], V), sE[s]);
-      const double sh = round_fix(add128(cb->W[s], V), sE[s]);
-      const int64_t o = (j0 + r) * nc + b;
+      const double T = round_fix(add128(U, V), E);
+      const double sh = round_fix(add128(W, V), E);
       if (T_new) __stcs(T_new + o, T);
       if (share_new) __stcs(share_new + o, sh);
-      if (admit) admit[o] = (__dadd_rn(sp[r].Lu, sh) <= sp[r].Bu && T <= slo) ? 1 : 0;
+      // comparisons as integers: with two fp64 ones per pair as well as the
+      // addition, the fp64 pipe took longer than the stores (4.2e6 pairs: 52
+      // us a call).  A NaN sum has the largest key.
+      if (adm.admit)
+        adm.admit[o] = (order_key(__dadd_rn(sp[r].Lu, sh)) <= sp[r].Bk && order_key(T) <= slo_key) ? 1 : 0;
     }
     return;
   }
-  for (int r = 0; r < rows; ++r) {
+  const int64_t s2 = cb->s2, s3 = cb->s3, n1 = cb->n + 1;
+  for (int r = tid >> lc; r < rows; r += step, o += ostep) {
     const int32_t p = sp[r].p, c = sp[r].c;
     const int phase = (prefill | sp[r].phase) ? 1 : 0;
     const int s = phase * 2 + ((s1 + p >= (phase ? sp1 : sp0)) ? 1 : 0);
     double T, sh;
-    if (cslow | sp[r].slow) {
+    if (cb->slow | sp[r].slow) {
       wi_pair_slow(mp, s, s1 + p, s2 + c, s3 + (int64_t)p * p, n1, p, c, &T, &sh);
     } else {
       const i128 V = sp[r].V[s];
       T = round_fix(add128(cb->U[s], V), sE[s]);
       sh = round_fix(add128(cb->W[s], V), sE[s]);
     }
-    const int64_t o = (j0 + r) * nc + b;
     if (T_new) __stcs(T_new + o, T);
     if (share_new) __stcs(share_new + o, sh);
-    if (admit) admit[o] = (__dadd_rn(sp[r].Lu, sh) <= sp[r].Bu && T <= slo) ? 1 : 0;
+    if (adm.admit) adm.admit[o] = (__dadd_rn(sp[r].Lu, sh) <= sp[r].Bu && T <= adm.slo) ? 1 : 0;
   }
 }
 
