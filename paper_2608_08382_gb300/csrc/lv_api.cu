@@ -43,6 +43,7 @@ struct lv_ctx {
   size_t wi_cap = 0;
   void *d_acc = nullptr;      // accuracy metrics: relative-error bits, partials, histograms
   size_t acc_cap = 0;
+  bool ten_attr = false;      // k_tenant_acc's shared-memory limit is set
   int acc_occ = 0;            // CTAs per SM of the accuracy kernel (0: not yet queried)
   double *h_acc = nullptr;    // accuracy results: pinned host memory the kernel writes (mapped)
   double *hd_acc = nullptr;   // its device address
@@ -313,7 +314,7 @@ lv_status tiles_occupancy(lv_ctx *ctx, size_t smem, int *per_sm) {
   }
   if (*per_sm) return LV_OK;
   LV_CUDA(cudaFuncSetAttribute(k_tiles<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)(sizeof(TSmem) + ((MODE & M_TEN) ? sizeof(TenSmem) : 0))));
+                               (int)(sizeof(TSmem) + ((MODE & M_TEN) ? ten_table_bytes(kHotMax) : 0))));
   LV_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_tiles<MODE>, kTThreads, smem));
   if (*per_sm < 1) *per_sm = 1;
   if (ctx) {
@@ -344,7 +345,7 @@ lv_status ensure_bound(lv_ctx *ctx, int64_t n) {
 // has room for the tiles' bounds (bound_cap 32-bit entries).
 template <int MODE>
 lv_status run_tiles_mode(lv_ctx *ctx, int sms, TileArgs &a, void *bound, int64_t bound_cap, cudaStream_t stream) {
-  const size_t smem = sizeof(TSmem) + ((MODE & M_TEN) ? sizeof(TenSmem) : 0);
+  const size_t smem = sizeof(TSmem) + ((MODE & M_TEN) ? ten_table_bytes(kHotMax) : 0);
   int per_sm = 0;
   lv_status st = tiles_occupancy<MODE>(ctx, smem, &per_sm);
   if (st != LV_OK) return st;
@@ -950,17 +951,18 @@ lv_status lv_tenant_accumulate(lv_ctx *ctx, lv_tenant_acc *acc, const double *sh
   if (n_req > 0 && (!share || !tenant || !aligned(share, 8) || !aligned(tenant, 4))) return LV_EINVAL;
   cudaStream_t stream = (cudaStream_t)stream_;
   if (n_req > 0) {
-    const int H = std::min<int32_t>(acc->n_tenants, kHotMax);
-    const size_t smem = ten_bytes(H);
-    static bool configured = false;
-    if (!configured) {
+    // a CTA's table costs about 350 global additions per hot tenant over all
+    // CTAs; a share of a cold tenant two
+    const bool all = acc->n_tenants <= kAccHotMax && n_req >= 256 * (int64_t)acc->n_tenants;
+    const int H = all ? acc->n_tenants : std::min<int32_t>(acc->n_tenants, kHotMax);
+    if (!ctx->ten_attr) {
       LV_CUDA(cudaFuncSetAttribute(k_tenant_acc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)ten_bytes(kHotMax)));
-      configured = true;
+                                   (int)ten_table_bytes(kAccHotMax)));
+      ctx->ten_attr = true;
     }
-    const int64_t blocks = std::min<int64_t>((n_req + kBlock - 1) / kBlock, (int64_t)ctx->sms * 4);
-    k_tenant_acc<<<(unsigned)blocks, kBlock, smem, stream>>>(share, tenant, n_req, acc->d_pend, acc->n_tenants, H,
-                                                              ctx->d_status);
+    const int64_t blocks = std::min<int64_t>((n_req + 4 * kAccThreads - 1) / (4 * kAccThreads), (int64_t)ctx->sms);
+    k_tenant_acc<<<(unsigned)blocks, kAccThreads, ten_table_bytes(H), stream>>>(
+        share, tenant, n_req, acc->d_pend, acc->n_tenants, H, ctx->d_status);
     LV_CUDA(cudaGetLastError());
   }
   return fold_tenants(ctx, acc, stream);

@@ -162,6 +162,53 @@ __device__ __noinline__ double eq1_fix(const ModelP &mp, int s, const BatchAgg &
   return fix_to_double(V, f.E).d;
 }
 
+// v shifted so that its leading bit (in v2, not zero) is bit 95, rounded to
+// nearest even by the hardware's 64-bit integer conversion (the rest is ORed
+// into the last of the top 64 bits), in units of 2^(E + 64): ebase = (E + 32)
+// << 20.  The conversion's unit is otherwise idle; rounding by integer
+// instructions takes some 15 more.
+__device__ __forceinline__ double round_top(uint32_t v0, uint32_t v1, uint32_t v2, uint32_t ebase) {
+  const int s = __clz((int)v2);
+  const uint32_t t2 = __funnelshift_l(v1, v2, s), t0 = v0 << s;
+  const uint32_t t1 = __funnelshift_l(v0, v1, s) | min(t0, 1u);
+  const double x = __ull2double_rn(((uint64_t)t2 << 32) | t1);
+  return __hiloint2double(__double2hiint(x) + (int)(ebase - ((uint32_t)s << 20)), __double2loint(x));
+}
+
+// Whether eq1_exact's short products apply to a segment: B, A1..A4 all in [0, 2^92).
+__device__ __forceinline__ bool seg_t32(const SegFix &f) {
+  return f.t_narrow && ((f.B.hi | f.A1.hi | f.A2.hi | f.A3.hi | f.A4.hi) < (1ull << 28));
+}
+
+// Eq. 1 exactly in fixed point, one rounding: for sums below 2^32 and a
+// segment of seg_t32, 96 x 32-bit products, whose sum stays below 2^127; the
+// general evaluation, which gives the same value, otherwise (kept out of line).
+// f: segment s's parameters (a shared-memory copy where lanes take different
+// segments).
+__device__ __forceinline__ double eq1_exact(const ModelP &mp, const SegFix &f, bool t32, int s, const BatchAgg &g) {
+  const uint64_t wide = ((uint64_t)g.s1 | (uint64_t)g.s2 | (uint64_t)g.s3 | ((uint64_t)g.n << 16)) >> 32;
+  if (t32 && wide == 0) {
+    uint32_t w0 = (uint32_t)f.B.lo, w1 = (uint32_t)(f.B.lo >> 32), w2 = (uint32_t)f.B.hi, w3 = 0u;
+    const uint32_t x[4] = {(uint32_t)g.s1, (uint32_t)g.s2, (uint32_t)g.s3, (uint32_t)g.n * (uint32_t)g.n};
+    const i128 *A[4] = {&f.A1, &f.A2, &f.A3, &f.A4};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint32_t a0 = (uint32_t)A[i]->lo, a1 = (uint32_t)(A[i]->lo >> 32), a2 = (uint32_t)A[i]->hi;
+      asm("mad.lo.cc.u32 %0, %4, %7, %0;\n\t"
+          "madc.hi.cc.u32 %1, %4, %7, %1;\n\t"
+          "madc.lo.cc.u32 %2, %6, %7, %2;\n\t"
+          "madc.hi.u32 %3, %6, %7, %3;\n\t"
+          "mad.lo.cc.u32 %1, %5, %7, %1;\n\t"
+          "madc.hi.cc.u32 %2, %5, %7, %2;\n\t"
+          "addc.u32 %3, %3, 0;"
+          : "+r"(w0), "+r"(w1), "+r"(w2), "+r"(w3)
+          : "r"(a0), "r"(a1), "r"(a2), "r"(x[i]));
+    }
+    if (w3 == 0u && w2 != 0u && g.n > 0) return round_top(w0, w1, w2, (uint32_t)(f.E + 32) << 20);
+  }
+  return eq1_fix(mp, s, g);
+}
+
 // Eq. 1 in fixed point for the common case: every coefficient in [0, 2^96)
 // (t_narrow), each product A_k S_k below 2^96 and the sum in [2^64, 2^96);
 // 64x64-bit products with the coefficients' high words folded in, and the
@@ -392,7 +439,7 @@ struct SegS {
   int E;
   int a2_narrow;
   int p_narrow;  // 1: 0 <= A1 < 2^95 and 0 <= A3 < 2^64 (prefill constant in 128 bits)
-  int pad;
+  int t32;       // seg_t32
 };
 
 // fx: the segments' fixed-point parameters.
@@ -481,32 +528,6 @@ __global__ void k_tenant_totals(const i128 *__restrict__ state, double *__restri
   const int u = blockIdx.x * blockDim.x + threadIdx.x;
   if (u >= n_tenants) return;
   L[u] = fix_to_double(state[u], kTenLsb).d;
-}
-
-// Standalone pass 1 over given shares: grid-stride, hot tenants in shared memory.
-__global__ void __launch_bounds__(kBlock) k_tenant_acc(const double *__restrict__ share,
-                                                        const int32_t *__restrict__ ten, int64_t n,
-                                                        unsigned long long *pend, int32_t n_tenants, int32_t H,
-                                                        int *status) {
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  uint32_t *tt = reinterpret_cast<uint32_t *>(smem_raw);
-  for (int i = threadIdx.x; i < 4 * ten_plane(H); i += kBlock) tt[i] = 0;
-  __syncthreads();
-  int bad = 0;
-  TileArgs a{};
-  a.n_tenants = n_tenants;
-  a.H = H;
-  a.ten_pend = pend;
-  const int64_t stride = (int64_t)gridDim.x * kBlock;
-  for (int64_t i = blockIdx.x * (int64_t)kBlock + threadIdx.x; i < n; i += stride) {
-    tenant_add(a, tt, __ldcs(ten + i), decompose(__ldcs(share + i)), &bad);
-  }
-  if (bad) flag(status, kStatusData);
-  __syncthreads();
-  for (int u = threadIdx.x; u < H; u += kBlock) {
-    const i128 v = hot_value(tt, H, u);
-    if (v.lo | v.hi) pend_add(pend, u, v);
-  }
 }
 
 // ---------------------------------------------------------------- small kernels

@@ -149,7 +149,7 @@ __device__ __forceinline__ void init_segs(const TileArgs &a, SegS *seg) {
     g.E = f.E;
     g.a2_narrow = f.a2_narrow;
     g.p_narrow = ((uint64_t)f.A1.hi < (1ull << 31) && f.A3.hi == 0) ? 1 : 0;
-    g.pad = 0;
+    g.t32 = seg_t32(f);
     seg[threadIdx.x] = g;
   }
 }

@@ -32,6 +32,7 @@
 #pragma once
 
 #include "lv_step.cuh"
+#include "lv_tenant.cuh"
 
 namespace lv {
 
@@ -286,48 +287,6 @@ __device__ __forceinline__ TileRec tile_record(const TileArgs &a, const TSmem &t
   return r;
 }
 
-// v shifted so that its leading bit (in v2, not zero) is bit 95, rounded to
-// nearest even by the hardware's 64-bit integer conversion (the rest is ORed
-// into the last of the top 64 bits), in units of 2^(E + 64): ebase = (E + 32)
-// << 20.  The conversion's unit is otherwise idle; rounding by integer
-// instructions takes some 15 more.
-__device__ __forceinline__ double round_top(uint32_t v0, uint32_t v1, uint32_t v2, uint32_t ebase) {
-  const int s = __clz((int)v2);
-  const uint32_t t2 = __funnelshift_l(v1, v2, s), t0 = v0 << s;
-  const uint32_t t1 = __funnelshift_l(v0, v1, s) | min(t0, 1u);
-  const double x = __ull2double_rn(((uint64_t)t2 << 32) | t1);
-  return __hiloint2double(__double2hiint(x) + (int)(ebase - ((uint32_t)s << 20)), __double2loint(x));
-}
-
-// Eq. 1 exactly in fixed point, one rounding, for sums below 2^32 and a
-// segment whose coefficients are in [0, 2^92) (t32): 96 x 32-bit products,
-// whose sum stays below 2^127.  The general evaluation, which gives the same
-// value, otherwise (kept out of line).
-__device__ __forceinline__ double tile_eq1(const TileArgs &a, const TSmem &ts, int s, const BatchAgg &g) {
-  const SegFix &f = ts.fx[s];
-  const uint64_t wide = ((uint64_t)g.s1 | (uint64_t)g.s2 | (uint64_t)g.s3 | ((uint64_t)g.n << 16)) >> 32;
-  if (ts.seg[s].pad && wide == 0) {
-    uint32_t w0 = (uint32_t)f.B.lo, w1 = (uint32_t)(f.B.lo >> 32), w2 = (uint32_t)f.B.hi, w3 = 0u;
-    const uint32_t x[4] = {(uint32_t)g.s1, (uint32_t)g.s2, (uint32_t)g.s3, (uint32_t)g.n * (uint32_t)g.n};
-    const i128 *A[4] = {&f.A1, &f.A2, &f.A3, &f.A4};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const uint32_t a0 = (uint32_t)A[i]->lo, a1 = (uint32_t)(A[i]->lo >> 32), a2 = (uint32_t)A[i]->hi;
-      asm("mad.lo.cc.u32 %0, %4, %7, %0;\n\t"
-          "madc.hi.cc.u32 %1, %4, %7, %1;\n\t"
-          "madc.lo.cc.u32 %2, %6, %7, %2;\n\t"
-          "madc.hi.u32 %3, %6, %7, %3;\n\t"
-          "mad.lo.cc.u32 %1, %5, %7, %1;\n\t"
-          "madc.hi.cc.u32 %2, %5, %7, %2;\n\t"
-          "addc.u32 %3, %3, 0;"
-          : "+r"(w0), "+r"(w1), "+r"(w2), "+r"(w3)
-          : "r"(a0), "r"(a1), "r"(a2), "r"(x[i]));
-    }
-    if (w3 == 0u && w2 != 0u && g.n > 0) return round_top(w0, w1, w2, (uint32_t)(f.E + 32) << 20);
-  }
-  return eq1_fix(a.mp, s, g);
-}
-
 // A batch's outputs.
 template <int MODE>
 __device__ __forceinline__ void tile_emit(const TileArgs &a, const TSmem &ts, int64_t b, const BatchAgg &g, int s) {
@@ -341,7 +300,7 @@ __device__ __forceinline__ void tile_emit(const TileArgs &a, const TSmem &ts, in
       a.T32[b] = g.n > 0 ? T : 0.0f;
     }
   } else if ((MODE & M_ATTR) && (MODE & M_FIX)) {
-    if (a.T) a.T[b] = tile_eq1(a, ts, s, g);
+    if (a.T) a.T[b] = eq1_exact(a.mp, ts.fx[s], ts.seg[s].t32, s, g);
   } else if (MODE & M_FIT) {
     a.bfeat[b] = g.s1;
     a.bfeat[a.n_batch + b] = g.s2;
@@ -355,153 +314,17 @@ __device__ __forceinline__ void tile_emit(const TileArgs &a, const TSmem &ts, in
 
 // ---------------------------------------------------------------- step 3: requests
 
-// Hot tenants (ids below H) in shared memory.  The sum of a tenant's q = share
-// * 2^72, modulo 2^128, is four 32-bit words.  Words 0 and 1 have kTCopies
-// copies, to one of which a lane always adds, so that one tenant's many
-// requests do not all serialise in one bank; words 2 and 3, which few
-// additions reach, have one.
-constexpr int kTCopies = 2;
-struct TenSmem {
-  // after the tenants' words, one per lane where lanes with nothing to add do so
-  uint32_t w0[kHotMax * kTCopies + 32], w1[kHotMax * kTCopies + 32];
-  uint32_t w2[kHotMax], w3[kHotMax];
-};
-constexpr uint32_t kTPlane = sizeof(uint32_t) * (kHotMax * kTCopies + 32);  // bytes from a word 0 to its word 1
-
-struct TenTab {
-  uint32_t w, base;  // shared-memory byte addresses: the lane's copy of tenant 0's word 0, and the table
-  uint32_t H;
-};
-
-// Shared-memory atomic add at a byte address (address space stated, so that it
-// compiles to the shared-memory instruction wherever the table comes from).
-__device__ __forceinline__ uint32_t atom_shared(uint32_t addr, uint32_t v) {
-  uint32_t o;
-  asm volatile("atom.shared.add.u32 %0, [%1], %2;" : "=r"(o) : "r"(addr), "r"(v));
-  return o;
-}
-
-// x + y and its carry.
-__device__ __forceinline__ uint32_t carry_of(uint32_t x, uint32_t y) {
-  uint32_t c;
-  asm("{\n .reg .u32 t;\n add.cc.u32 t, %1, %2;\n addc.u32 %0, 0, 0;\n}" : "=r"(c) : "r"(x), "r"(y));
-  return c;
-}
-
-// q = (h1:h0) 2^64 + (hi:lo), modulo 2^128, to tenant u < H.  Each word's
-// atomic returns its old value, so the lane whose addition wraps a word
-// carries into the next: the sum stays exact under any interleaving.
-__device__ __forceinline__ void ten_carry(const TenTab tt, uint32_t u, uint32_t h0, uint32_t h1) {
-  if (h0 | h1) {
-    const uint32_t a = tt.base + (uint32_t)offsetof(TenSmem, w2) + 4u * u;
-    h1 += carry_of(atom_shared(a, h0), h0);
-    if (h1) atom_shared(a + 4u * kHotMax, h1);
-  }
-}
-__device__ __forceinline__ void ten_add(const TenTab tt, uint32_t u, uint32_t lo, uint32_t hi, uint32_t h0,
-                                        uint32_t h1) {
-  const uint32_t w = tt.w + 4u * kTCopies * u;
-  const uint32_t c0 = carry_of(atom_shared(w, lo), lo), a1 = hi + c0;
-  const uint32_t c1 = carry_of(atom_shared(w + kTPlane, a1), a1) + (a1 < c0 ? 1u : 0u);
-  h0 += c1;
-  h1 += h0 < c1 ? 1u : 0u;
-  ten_carry(tt, u, h0, h1);
-}
-
-// Tenant contributions of a lane's four positive shares (d: their doubles'
-// words) in the common case, a valid tenant and a share below 2^-9 s (then q <
-// 2^63); go[k] is cleared otherwise.  q is the hardware's conversion of d 2^72
-// to a 64-bit integer, which rounds to nearest even.  The four low words'
-// atomics are issued together, then the four high words', so that a lane waits
-// for two of them and not for eight; lanes with nothing to add use a word of
-// their own, so there is no branch.
-__device__ __forceinline__ void ten_add4(const TileArgs &a, const TenTab tt, bool *go, const uint32_t *u,
-                                         const uint32_t *dlo, const uint32_t *dhi, int lane) {
-  uint32_t w[4], lo[4], hi[4], c1[4];
-  bool cold = false;
-  const uint32_t sink = tt.base + 4u * (kHotMax * kTCopies + lane);
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    go[k] = go[k] && dhi[k] < ((1023u - 9u) << 20) && u[k] < (uint32_t)a.n_tenants;
-    const bool hot = go[k] && u[k] < tt.H;
-    const long long q = __double2ll_rn(__hiloint2double((int)(dhi[k] - ((uint32_t)kTenLsb << 20)), (int)dlo[k]));
-    lo[k] = (uint32_t)q;
-    hi[k] = (uint32_t)(q >> 32);
-    w[k] = tt.w + 4u * kTCopies * u[k];
-    w[k] = hot ? w[k] : sink;
-    cold |= go[k] && !hot;
-  }
-  if (cold) {
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      if (go[k] && u[k] >= tt.H) {
-        unsigned long long *pw = a.ten_pend + 4 * (int64_t)u[k];
-        atomicAdd(pw, (unsigned long long)lo[k]);
-        atomicAdd(pw + 1, (unsigned long long)hi[k]);
-      }
-    }
-  }
-#pragma unroll
-  for (int k = 0; k < 4; ++k) c1[k] = atom_shared(w[k], lo[k]);
-#pragma unroll
-  for (int k = 0; k < 4; ++k)  // hi <= 2^31: no wrap
-    asm("{\n .reg .u32 t;\n add.cc.u32 t, %1, %2;\n addc.u32 %0, %0, 0;\n}" : "+r"(hi[k]) : "r"(c1[k]), "r"(lo[k]));
-#pragma unroll
-  for (int k = 0; k < 4; ++k) c1[k] = atom_shared(w[k] + kTPlane, hi[k]);
-  uint32_t any = 0;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    c1[k] = carry_of(c1[k], hi[k]);
-    any |= c1[k];
-  }
-  if (any) {
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-      if (c1[k] && go[k] && u[k] < tt.H) ten_carry(tt, u[k], 1u, 0u);
-  }
-}
-
-// Any positive share with q of at most three words and a valid tenant.
-__device__ __forceinline__ bool tile_tenant(const TileArgs &a, const TenTab tt, uint32_t u, uint32_t dlo,
-                                            uint32_t dhi) {
-  const uint32_t mh = (dhi & 0xfffffu) | 0x100000u;
-  const int sh = (int)(dhi >> 20) - (1075 + kTenLsb);
-  if ((unsigned)sh > 42u || u >= (uint32_t)a.n_tenants) return false;
-  const bool lowp = sh < 32;
-  const int t = lowp ? sh : sh - 32;
-  const uint32_t x0 = dlo << t, x1 = __funnelshift_l(dlo, mh, t), x2 = t ? mh >> (32 - t) : 0u;
-  const uint32_t q0 = lowp ? x0 : 0u, q1 = lowp ? x1 : x0, q2 = lowp ? x2 : x1;
-  if (u < tt.H) {
-    ten_add(tt, u, q0, q1, q2, 0u);
-    return true;
-  }
-  unsigned long long *pw = a.ten_pend + 4 * (int64_t)u;
-  if (q0) atomicAdd(pw, (unsigned long long)q0);
-  if (q1) atomicAdd(pw + 1, (unsigned long long)q1);
-  if (q2) atomicAdd(pw + 2, (unsigned long long)q2);
-  return true;
-}
-
-// The general tenant add (any sign and magnitude).
-__device__ __forceinline__ void tile_tenant_any(const TileArgs &a, const TenTab tt, int32_t u, const Rounded &r,
-                                                int *bad) {
-  if (u < 0 || u >= a.n_tenants) {
-    *bad = 1;
-    u = u < 0 ? 0 : a.n_tenants - 1;
-  }
-  const i128 q = share_to_tenant_fix(r, bad);
-  if ((q.lo | q.hi) == 0) return;
-  if (u < a.H)
-    ten_add(tt, (uint32_t)u, (uint32_t)q.lo, (uint32_t)(q.lo >> 32), (uint32_t)q.hi, (uint32_t)(q.hi >> 32));
-  else
-    pend_add(a.ten_pend, u, q);
+// The CTA's tenant table, which follows TSmem (formed again in the functions
+// kept out of line, so that the loops hold it in fewer registers).
+__device__ __forceinline__ TenTab tile_table(const TileArgs &a, const TSmem &ts) {
+  return ten_table(reinterpret_cast<const uint32_t *>(&ts + 1), kHotMax, a.H, a.n_tenants, a.ten_pend);
 }
 
 // The general path of one request.  Out of line: the fast path leaves it the
 // rare ones (fp64 mode, values out of range).
 template <int MODE>
-__device__ __noinline__ void tile_slow(const TileArgs &a, const TenTab tt, const TSmem &ts, const TileRec &rec,
-                                       int64_t n, int64_t i, int32_t p, int32_t c, int32_t u) {
+__device__ __noinline__ void tile_slow(const TileArgs &a, const TSmem &ts, const TileRec &rec, int64_t n, int64_t i,
+                                       int32_t p, int32_t c, int32_t u) {
   const int s = (int)(rec.a.z & 3u);
   const bool slow = (rec.a.z & 4u) != 0u;
   const SegS &sg = ts.seg[s];
@@ -515,7 +338,7 @@ __device__ __noinline__ void tile_slow(const TileArgs &a, const TenTab tt, const
   if (a.share) __stcs(a.share + i, r.d);
   if (MODE & M_TEN) {
     int bad = 0;
-    tile_tenant_any(a, tt, u, r, &bad);
+    tenant_add_any(tile_table(a, ts), u, r, &bad);
     if (bad) flag(a.status, kStatusData);
   }
 }
@@ -562,18 +385,18 @@ __device__ __forceinline__ void store4(double *p, const double *d) {
 
 // One request through the fast path where it applies, else the general one.
 template <int MODE>
-__device__ __forceinline__ bool tile_one(const TileArgs &a, const TenTab tt, const TSmem &ts, const TileRec &rec,
+__device__ __forceinline__ bool tile_one(const TileArgs &a, const TenTab &tt, const TSmem &ts, const TileRec &rec,
                                          int64_t n, int64_t i, int32_t p, int32_t c, int32_t u, double *d) {
   bool ok = (MODE & M_FIX) && tile_share(ts.seg, rec, p, c, d);
   if (MODE & M_TEN)
-    ok = ok && tile_tenant(a, tt, (uint32_t)u, (uint32_t)__double2loint(*d), (uint32_t)__double2hiint(*d));
-  if (!ok) tile_slow<MODE>(a, tt, ts, rec, n, i, p, c, u);
+    ok = ok && tenant_add_pos(tt, (uint32_t)u, (uint32_t)__double2loint(*d), (uint32_t)__double2hiint(*d));
+  if (!ok) tile_slow<MODE>(a, ts, rec, n, i, p, c, u);
   return ok;
 }
 
 // One request of the fp32 variant.
 template <int MODE>
-__device__ __forceinline__ float tile_one_f32(const TileArgs &a, const TenTab tt, const TileRec &rec, int32_t p,
+__device__ __forceinline__ float tile_one_f32(const TileArgs &a, const TenTab &tt, const TileRec &rec, int32_t p,
                                               int32_t c, int32_t u, int *bad) {
   const Share32 q{__uint_as_float(rec.k.x), __uint_as_float(rec.k.y), __uint_as_float(rec.k.z),
                   __uint_as_float(rec.k.w)};
@@ -582,8 +405,8 @@ __device__ __forceinline__ float tile_one_f32(const TileArgs &a, const TenTab tt
     // a positive normal float's double: the same significand, the exponent rebiased
     const uint32_t f = __float_as_uint(s);
     const bool normal = f >= 0x00800000u && f < 0x7f800000u;
-    if (!normal || !tile_tenant(a, tt, (uint32_t)u, f << 29, (f >> 3) + ((1023u - 127u) << 20)))
-      tile_tenant_any(a, tt, u, decompose((double)s), bad);
+    if (!normal || !tenant_add_pos(tt, (uint32_t)u, f << 29, (f >> 3) + ((1023u - 127u) << 20)))
+      tenant_add_any(tt, u, decompose((double)s), bad);
   }
   return s;
 }
@@ -592,8 +415,9 @@ __device__ __forceinline__ float tile_one_f32(const TileArgs &a, const TenTab tt
 // tenants and values off the common path, with every lane busy.  Returns how
 // many are left.
 template <int MODE>
-__device__ __noinline__ int tile_flush(const TileArgs &a, const TenTab tt, const TSmem &ts, const WarpTile &wt,
-                                       int64_t rbase, int n, int lane) {
+__device__ __noinline__ int tile_flush(const TileArgs &a, const TSmem &ts, const WarpTile &wt, int64_t rbase, int n,
+                                       int lane) {
+  const TenTab tt = tile_table(a, ts);
   const int left = max(n - 32, 0);
   __syncwarp();
   if (left + lane < n) {
@@ -621,7 +445,7 @@ __device__ __noinline__ int tile_flush(const TileArgs &a, const TenTab tt, const
 // branch; the rest goes to the warp's list, which is worked off 32 at
 // a time.  vec: the share array allows 32-byte (fp32: 16-byte) stores.
 template <int MODE>
-__device__ __forceinline__ void tile_shares(const TileArgs &a, const TenTab tt, const TSmem &ts, WarpTile &wt,
+__device__ __forceinline__ void tile_shares(const TileArgs &a, const TenTab &tt, const TSmem &ts, WarpTile &wt,
                                             const TileSrc &src, int64_t rbase, int first, int cnt, bool vec,
                                             int lane) {
   constexpr bool kTen = (MODE & M_TEN) != 0, kF32 = (MODE & M_F32) != 0;
@@ -632,7 +456,7 @@ __device__ __forceinline__ void tile_shares(const TileArgs &a, const TenTab tt, 
       const uint32_t word = wt.bits[e >> 5];
       const int r = min((int)wt.rank[e >> 5] + __popc(word & ((2u << (e & 31)) - 1u)), kTRec) - 1;
       const TileRec &rec = wt.rec[max(r, 0)];
-      tile_slow<MODE>(a, tt, ts, rec, (int64_t)(rec.a.z >> 4), rbase + e, src.p[e], src.c[e], kTen ? src.u[e] : 0);
+      tile_slow<MODE>(a, ts, rec, (int64_t)(rec.a.z >> 4), rbase + e, src.p[e], src.c[e], kTen ? src.u[e] : 0);
     }
     return;
   }
@@ -678,7 +502,7 @@ __device__ __forceinline__ void tile_shares(const TileArgs &a, const TenTab tt, 
         dhi[k] = (uint32_t)__double2hiint(d);
       }
     }
-    if (kTen) ten_add4(a, tt, go, u, dlo, dhi, lane);
+    if (kTen) ten_add4(tt, go, u, dlo, dhi);
     uint32_t dm = vm;
 #pragma unroll
     for (int k = 0; k < 4; ++k) dm &= go[k] ? ~(1u << k) : ~0u;
@@ -718,17 +542,17 @@ __device__ __forceinline__ void tile_shares(const TileArgs &a, const TenTab tt, 
         const int rk = max(r0 + __popc(hb & ((2u << k) - 1u)), 0);
         wt.list[at++] = (uint32_t)(e + k) | ((uint32_t)rk << 16);
       }
-      while (nl >= 32) nl = tile_flush<MODE>(a, tt, ts, wt, rbase, nl, lane);
+      while (nl >= 32) nl = tile_flush<MODE>(a, ts, wt, rbase, nl, lane);
     }
   }
-  if (nl > 0) tile_flush<MODE>(a, tt, ts, wt, rbase, nl, lane);
+  if (nl > 0) tile_flush<MODE>(a, ts, wt, rbase, nl, lane);
 }
 
 // One batch walked by `kThreads` threads (a warp, or the CTA) from global
 // memory: sums, then a strided share pass.
 template <int MODE, int kThreads>
-__device__ __noinline__ void walk_batch(const TileArgs &a, const TenTab tt, TSmem &ts, int64_t b, int64_t r0,
-                                        int64_t n) {
+__device__ __noinline__ void walk_batch(const TileArgs &a, TSmem &ts, int64_t b, int64_t r0, int64_t n) {
+  const TenTab tt = tile_table(a, ts);
   const int tid = kThreads == 32 ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
   int bad = 0;
   Sums acc{0, 0, 0, 0};
@@ -789,22 +613,15 @@ __global__ void __launch_bounds__(kTThreads, 1) k_tiles(const TileArgs a) {
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   int bad = 0;
 
-  TenSmem &ten = *reinterpret_cast<TenSmem *>(smem_raw + sizeof(TSmem));
+  uint32_t *tw = reinterpret_cast<uint32_t *>(smem_raw + sizeof(TSmem));
   TenTab tt{};
   if (kTen) {
-    tt.H = (uint32_t)a.H;
-    tt.base = smem_u32(&ten);
-    tt.w = smem_u32(ten.w0) + 4u * (lane & (kTCopies - 1));
-    uint32_t *z = reinterpret_cast<uint32_t *>(&ten);
-    for (int i = tid; i < (int)(sizeof(TenSmem) / 4); i += kTThreads) z[i] = 0;
+    tt = tile_table(a, ts);
+    for (int i = tid; i < (int)(ten_table_bytes(kHotMax) / 4); i += kTThreads) tw[i] = 0;
   }
   if (MODE & M_ATTR) {
     init_segs<MODE>(a, ts.seg);
-    if (tid < 4) {
-      const SegFix &f = a.mp.fx[tid];
-      ts.fx[tid] = f;
-      ts.seg[tid].pad = f.t_narrow && ((f.B.hi | f.A1.hi | f.A2.hi | f.A3.hi | f.A4.hi) < (1ull << 28));
-    }
+    if (tid < 4) ts.fx[tid] = a.mp.fx[tid];
     if ((MODE & M_F32) && tid < 20) ts.cf[tid / 5][tid % 5] = __double2float_rn(a.mp.coef[tid / 5][tid % 5]);
   }
   if (tid == 0) ts.n_big = 0;
@@ -929,7 +746,7 @@ __global__ void __launch_bounds__(kTThreads, 1) k_tiles(const TileArgs a) {
         if (slot < kTBigs) {
           if (lane == 0) ts.big[slot] = b0 + i;
         } else {
-          walk_batch<MODE, 32>(a, tt, ts, b0 + i, c0, c1 - c0);
+          walk_batch<MODE, 32>(a, ts, b0 + i, c0, c1 - c0);
         }
       }
     }
@@ -947,19 +764,11 @@ __global__ void __launch_bounds__(kTThreads, 1) k_tiles(const TileArgs a) {
   for (int k = 0; k < nbig; ++k) {
     const int64_t b = ts.big[k];
     const int64_t c0 = clampi(a.off[b], 0, a.n_req), c1 = clampi(a.off[b + 1], c0, a.n_req);
-    walk_batch<MODE, kTThreads>(a, tt, ts, b, c0, c1 - c0);
+    walk_batch<MODE, kTThreads>(a, ts, b, c0, c1 - c0);
   }
   if (kTen) {
     __syncthreads();
-    for (int u = tid; u < a.H; u += kTThreads) {
-      i128 v = mk128(0ull, (uint64_t)ten.w2[u] | ((uint64_t)ten.w3[u] << 32));
-#pragma unroll
-      for (int r = 0; r < kTCopies; ++r) {
-        const int i = u * kTCopies + r;
-        v = add128(v, mk128((uint64_t)ten.w0[i] | ((uint64_t)ten.w1[i] << 32), 0ull));
-      }
-      if (v.lo | v.hi) pend_add(a.ten_pend, u, v);
-    }
+    ten_table_flush(tw, kHotMax, a.H, a.ten_pend, tid, kTThreads);
   }
 }
 
