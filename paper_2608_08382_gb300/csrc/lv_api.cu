@@ -765,9 +765,9 @@ lv_status lv_features(lv_ctx *ctx, const lv_arch *arch, const lv_model *model, c
     st = lv_arch_constants(arch, phi, &W);
     if (st != LV_OK) return st;
     if (b->n_req > 0) {
-      const int64_t blocks = std::min<int64_t>((b->n_req + 255) / 256, (int64_t)ctx->sms * 8);
-      k_req_features<<<(unsigned)blocks, 256, 0, stream>>>(b->p, b->c, b->n_req, phi[0], phi[1], phi[2], req_feat,
-                                                           ctx->d_status);
+      const int64_t per = 256 * kReqRows;  // n_req <= 2^40: at most 2^30 blocks
+      k_req_features<<<(unsigned)((b->n_req + per - 1) / per), 256, 0, stream>>>(
+          b->p, b->c, b->n_req, phi[0], phi[1], phi[2], req_feat, ctx->d_status);
       LV_CUDA(cudaGetLastError());
     }
   }
