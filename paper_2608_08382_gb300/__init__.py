@@ -132,16 +132,23 @@ def _check(status, where):
 
 
 def _ptr(t):
-    if t is None:
-        return None
-    return ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+_torch = None  # set once torch's CUDA state exists
 
 
 def _stream(stream):
+    """The stream's handle; None is torch's current stream.  A serving step's call is bound by its
+    host side, so the current stream is taken as a bare handle, without a torch.cuda.Stream object."""
+    global _torch
     if stream is None:
-        import torch
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
+        if _torch is None:
+            import torch
+            torch.cuda.current_stream()
+            _torch = torch
+        return _torch._C._cuda_getCurrentRawStream(_torch._C._cuda_getDevice())
+    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
 # ------------------------------------------------------------------ structs
@@ -181,14 +188,9 @@ class Batches:
     n_tenants: int = 0
 
     def struct(self) -> lv_batches:
-        b = lv_batches()
-        b.p, b.c, b.phase = _ptr(self.p), _ptr(self.c), _ptr(self.phase)
-        b.tenant = _ptr(self.tenant)
-        b.offsets = _ptr(self.offsets)
-        b.n_req = int(self.p.numel())
-        b.n_batch = int(self.offsets.numel()) - 1
-        b.n_tenants = int(self.n_tenants)
-        return b
+        p, off = self.p, self.offsets
+        return lv_batches(p.data_ptr(), _ptr(self.c), _ptr(self.phase), _ptr(self.tenant), off.data_ptr(), p.numel(),
+                          off.numel() - 1, int(self.n_tenants), 0)
 
     @property
     def n_req(self):

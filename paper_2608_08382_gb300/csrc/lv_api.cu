@@ -32,6 +32,10 @@ struct lv_ctx {
   int ktab_nk = 0;
   bool ktab_valid = false;
   lv_model ktab_model{};
+  bool mp_valid = false;  // parameters of the previous call's model
+  int mp_arith = 0;
+  lv_model mp_model{};
+  ModelP mp{};
   int ktab_fixed = -1;
   cudaEvent_t ev_built = nullptr;
   cudaEvent_t ev_used = nullptr;
@@ -73,15 +77,12 @@ bool aligned(const void *p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p
 
 int lsb_exp(double x) {
   // x = M * 2^e with M odd; returns e.  x != 0, finite.
-  int e;
-  const double f = std::frexp(std::fabs(x), &e);  // x = f * 2^e, 0.5 <= f < 1
-  uint64_t M = (uint64_t)std::ldexp(f, 53);
-  int ex = e - 53;
-  while ((M & 1ull) == 0) {
-    M >>= 1;
-    ++ex;
-  }
-  return ex;
+  uint64_t b;
+  std::memcpy(&b, &x, 8);
+  const int be = (int)((b >> 52) & 0x7ff);
+  uint64_t M = b & ((1ull << 52) - 1);
+  if (be) M |= 1ull << 52;
+  return (be ? be - 1075 : -1074) + __builtin_ctzll(M);
 }
 
 int msb_exp(double x) {
@@ -198,7 +199,7 @@ lv_status wait_event(cudaStream_t stream, cudaEvent_t ev) {
 }
 
 // Per-model launch parameters, formed on the host (no K table).
-void model_params(const lv_ctx *ctx, const lv_model *m, ModelP *mp) {
+void form_params(const lv_model *m, int arith, ModelP *mp) {
   std::memset(mp, 0, sizeof(*mp));
   for (int s = 0; s < 4; ++s) {
     const lv_coef &k = m->seg[s >> 1][s & 1];
@@ -212,7 +213,19 @@ void model_params(const lv_ctx *ctx, const lv_model *m, ModelP *mp) {
   mp->split[1] = m->split[1];
   mp->nk = kKTableN;
   mp->fixed = 0;
-  if (ctx->arith == LV_ARITH_AUTO) mp->fixed = derive_fixed(m, kKTableN, mp) ? 1 : 0;
+  if (arith == LV_ARITH_AUTO) mp->fixed = derive_fixed(m, kKTableN, mp) ? 1 : 0;
+}
+
+// The context's copy where the model and the arithmetic have the same values
+// as in its previous call (a program's model changes rarely).
+void model_params(lv_ctx *ctx, const lv_model *m, ModelP *mp) {
+  if (!ctx->mp_valid || ctx->mp_arith != ctx->arith || std::memcmp(&ctx->mp_model, m, sizeof(lv_model)) != 0) {
+    form_params(m, ctx->arith, &ctx->mp);
+    ctx->mp_model = *m;
+    ctx->mp_arith = ctx->arith;
+    ctx->mp_valid = true;
+  }
+  *mp = ctx->mp;
 }
 
 lv_status prepare_model(lv_ctx *ctx, const lv_model *m, cudaStream_t stream, ModelP *mp) {
@@ -1263,19 +1276,7 @@ extern "C" lv_status lv_attribute_noalloc(const lv_model *model, const lv_batche
   if (b->n_batch == 0 || (!T && !share)) return LV_OK;
 
   ModelP mp;
-  std::memset(&mp, 0, sizeof(mp));
-  for (int s = 0; s < 4; ++s) {
-    const lv_coef &k = model->seg[s >> 1][s & 1];
-    mp.coef[s][0] = k.beta;
-    mp.coef[s][1] = k.a1;
-    mp.coef[s][2] = k.a2;
-    mp.coef[s][3] = k.a3;
-    mp.coef[s][4] = k.a4;
-  }
-  mp.split[0] = model->split[0];
-  mp.split[1] = model->split[1];
-  mp.nk = kKTableN;
-  mp.fixed = derive_fixed(model, kKTableN, &mp) ? 1 : 0;
+  form_params(model, LV_ARITH_AUTO, &mp);
   KEntry *ktab = reinterpret_cast<KEntry *>(static_cast<unsigned char *>(scratch) + kNoAllocTabOffset);
   mp.ktab = ktab;
   const int nk = 4 * (kKTableN + 1);
