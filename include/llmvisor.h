@@ -334,7 +334,7 @@ lv_status lv_whatif_admit(lv_ctx *ctx, const lv_model *model, const lv_batches *
  * Computes exactly what lv_attribute computes for T and share (no tenant
  * accumulation), with default arithmetic, using instead of an lv_ctx a fixed
  * scratch area that lives in the library image as a static device array
- * (about 3.4 MB on every GPU that loads the library, held until the process
+ * (about 2.3 MB on every GPU that loads the library, held until the process
  * exits).  It calls no cudaMalloc, cudaFree or other allocating routine.
  *  - Limit: n_batch + n_req must not exceed 67,108,864; larger inputs return
  *    LV_EINVAL before anything is launched.

@@ -1221,8 +1221,8 @@ constexpr int64_t kNoAllocMaxUnits = 65536 * 1024;  // n_batch + n_req
 constexpr int64_t kNoAllocBounds = kTW * kNoAllocMaxUnits / kTDMax + 32 * 256 + 2;
 constexpr size_t kNoAllocTabOffset = (sizeof(uint32_t) * (size_t)kNoAllocBounds + 255) & ~(size_t)255;
 constexpr size_t kNoAllocBytes = kNoAllocTabOffset + sizeof(KEntry) * 4 * (kKTableN + 1);
-// the size stated in include/llmvisor.h ("about 3.4 MB")
-static_assert(kNoAllocBytes > 3300000 && kNoAllocBytes < 3400000, "no-alloc scratch size as documented");
+// the size stated in include/llmvisor.h ("about 2.3 MB")
+static_assert(kNoAllocBytes > 2250000 && kNoAllocBytes < 2350000, "no-alloc scratch size as documented");
 
 }  // namespace
 

@@ -147,7 +147,7 @@ __device__ __forceinline__ double eq1_fp64(const double *k, const BatchAgg &g) {
 
 // Eq. 1 exactly in fixed point, one rounding; falls back to fp64 outside the
 // exact range.  Once per batch, so kept out of line.
-__device__ __noinline__ double eq1_fix(const ModelP &mp, int s, const BatchAgg &g) {
+__device__ __noinline__ double eq1_fix(const ModelP &mp, int s, BatchAgg g) {
   if (g.n == 0) return 0.0;
   const SegFix &f = mp.fx[s];
   const uint64_t F4 = (uint64_t)g.n * (uint64_t)g.n;
@@ -190,10 +190,10 @@ __device__ __forceinline__ double eq1_exact(const ModelP &mp, const SegFix &f, b
   if (t32 && wide == 0) {
     uint32_t w0 = (uint32_t)f.B.lo, w1 = (uint32_t)(f.B.lo >> 32), w2 = (uint32_t)f.B.hi, w3 = 0u;
     const uint32_t x[4] = {(uint32_t)g.s1, (uint32_t)g.s2, (uint32_t)g.s3, (uint32_t)g.n * (uint32_t)g.n};
-    const i128 *A[4] = {&f.A1, &f.A2, &f.A3, &f.A4};
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const uint32_t a0 = (uint32_t)A[i]->lo, a1 = (uint32_t)(A[i]->lo >> 32), a2 = (uint32_t)A[i]->hi;
+      const i128 A = i == 0 ? f.A1 : i == 1 ? f.A2 : i == 2 ? f.A3 : f.A4;
+      const uint32_t a0 = (uint32_t)A.lo, a1 = (uint32_t)(A.lo >> 32), a2 = (uint32_t)A.hi;
       asm("mad.lo.cc.u32 %0, %4, %7, %0;\n\t"
           "madc.hi.cc.u32 %1, %4, %7, %1;\n\t"
           "madc.lo.cc.u32 %2, %6, %7, %2;\n\t"

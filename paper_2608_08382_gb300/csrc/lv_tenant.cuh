@@ -85,9 +85,10 @@ __device__ __forceinline__ void ten_add(const TenTab &tt, uint32_t u, uint32_t l
 }
 
 // Tenant contributions of a lane's four positive normal shares (d: their
-// doubles' words) in the common case, a valid tenant and a share below 2^-9 s
-// (then q < 2^63); go[k] is cleared otherwise.  q is the hardware's conversion
-// of d 2^72 to a 64-bit integer, which rounds to nearest even.  The four low
+// doubles' words) in the common case, a valid tenant and a share in [2^-20, 2^-8)
+// s (then q is whole and below 2^64); go[k] is cleared otherwise.  (Shifts, and
+// not the hardware's conversion to a 64-bit integer: that runs at 1/64 rate,
+// and the shares' rounding needs one already.)  The four low
 // words' atomics are issued together, then the four high words', so that a lane
 // waits for two of them and not for eight; lanes with nothing to add use a word
 // of their own, so there is no branch.
@@ -97,11 +98,11 @@ __device__ __forceinline__ void ten_add4(const TenTab &tt, bool *go, const uint3
   bool cold = false;
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    go[k] = go[k] && dhi[k] < ((1023u - 9u) << 20) && u[k] < tt.n;
+    const uint32_t sh = (dhi[k] >> 20) - (uint32_t)(1075 + kTenLsb);
+    lo[k] = dlo[k] << (sh & 31u);
+    hi[k] = __funnelshift_l(dlo[k], (dhi[k] & 0xfffffu) | 0x100000u, sh);
+    go[k] = go[k] && sh <= 11u && hi[k] != 0xffffffffu && u[k] < tt.n;
     const bool hot = go[k] && u[k] < tt.H;
-    const long long q = __double2ll_rn(__hiloint2double((int)(dhi[k] - ((uint32_t)kTenLsb << 20)), (int)dlo[k]));
-    lo[k] = (uint32_t)q;
-    hi[k] = (uint32_t)(q >> 32);
     w[k] = tt.w + 8u * u[k];
     w[k] = hot ? w[k] : tt.sink;
     cold |= go[k] && !hot;
@@ -119,7 +120,7 @@ __device__ __forceinline__ void ten_add4(const TenTab &tt, bool *go, const uint3
 #pragma unroll
   for (int k = 0; k < 4; ++k) c1[k] = atom_shared(w[k], lo[k]);
 #pragma unroll
-  for (int k = 0; k < 4; ++k)  // hi <= 2^31: no wrap
+  for (int k = 0; k < 4; ++k)  // no wrap
     asm("{\n .reg .u32 t;\n add.cc.u32 t, %1, %2;\n addc.u32 %0, %0, 0;\n}" : "+r"(hi[k]) : "r"(c1[k]), "r"(lo[k]));
 #pragma unroll
   for (int k = 0; k < 4; ++k) c1[k] = atom_shared(w[k] + tt.plane, hi[k]);

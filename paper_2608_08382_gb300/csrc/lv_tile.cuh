@@ -16,19 +16,25 @@
 //      common path is listed and worked off 32 at a time.
 // So a request costs about the same instructions whatever the batch sizes, and
 // no lane idles on a batch's remainder.  The requests are read twice, the
-// second time from L1 or L2 (24 tiles of kTDMax positions per SM; with 1,024
-// positions and the next tile prefetched the L2 no longer held them and the
-// DRAM reads doubled).  A batch that reaches past a tile's kTCap requests is
-// walked by its warp alone, or, above kTAlone requests, by the whole CTA after
-// its tiles (a warp alone on a batch of 4,096 set the time of a small input).
-// All sums are exact integers, so results do not depend on the schedule.
+// second time from L1 or L2.  A batch that reaches past a tile's kTCap requests
+// is walked by its warp alone, or, above kTAlone requests, by the whole CTA
+// after its tiles (a warp alone on a batch of 4,096 set the time of a small
+// input).  All sums are exact integers, so results do not depend on the
+// schedule.
 //
-// What bounds it: instruction issue and the integer pipe (about 200 warp
-// instructions per 32 requests at 60 % issue with 24 warps per SM), not HBM.
-// Against a kernel that walked one batch per warp (fp64 shares, 16 tenants,
-// one call, GB300): 9.75e6 requests in batches of 1 to 64, 238 us before and
-// 127 us after; 9.75e7, 1,750 and 999; 6.5e5, 113 and 31; 1.36e8 in batches of
-// 16 to 256, 1,132 and 1,000; 2.6e7 in Pareto batches, 780 and 722.
+// What bounds it: instruction issue and the integer pipe (about 170 warp
+// instructions per 32 requests), not HBM.  The shape follows from that: 20 warps
+// per SM with 96 registers each spill little (24 warps of 80 took 9 % longer,
+// 32 of 64 a third), and the largest tile whose shared memory (182 KB) leaves the
+// L1 60 KB (tiles of 1,376 positions leave it 28 KB and took 15 % longer, tiles
+// of 768 8 %, from their fixed cost).  The loop of step 3 is kept free of calls
+// and small enough for the instruction cache (unrolled twice it took a third
+// longer).
+// Against a kernel that walked one batch per warp (one call, GB300): 1.36e8
+// requests in batches of 16 to 256, fp64 shares, 256 tenants, 1,130 us before
+// and 880 now; 3.25e7 in batches of 1 to 64, 16 tenants, 583 and 301; 6.5e5, 113
+// and 30; 2.6e7 in Pareto batches, 65,536 tenants, 816 and 575; fp32, 4.1e7 in
+// batches of 16 to 256, 323 and 244.
 #pragma once
 
 #include "lv_step.cuh"
@@ -36,17 +42,17 @@
 
 namespace lv {
 
-constexpr int kTThreads = 768;             // threads of a CTA, one CTA per SM (one tenant table)
+constexpr int kTThreads = 640;             // threads of a CTA, one CTA per SM (one tenant table)
 constexpr int kTWarps = kTThreads / 32;
 constexpr int kTW = 8;                     // merge positions a batch takes besides its requests
-constexpr int kTDMax = 768;                // merge positions per tile, at most
+constexpr int kTDMax = 1248;               // merge positions per tile, at most
 constexpr int kTDMin = 128;
-constexpr int kTCap = 1024;                // requests of a tile, at most
+constexpr int kTCap = 1536;                // requests of a tile, at most
 constexpr int kTNb = kTDMax / kTW;         // batches of a tile, at most
 constexpr int kTRec = kTDMax / (kTW + 1) + 5;     // non-empty ones, and room to read past the last
 constexpr int kTBlocks = kTCap / 256 + 1;         // blocks of 256 requests, one more for a bound at the end
 constexpr int kTWords = kTCap / 32 + 1;
-constexpr int kTList = 31 + 128;           // deferred requests at most: a rest and one step's
+constexpr int kTDense = 40;                // batches of fewer requests on average: a record per request in step 3
 constexpr int64_t kTAlone = 512;           // requests a warp walks alone
 constexpr int kTBigs = 64;                 // larger batches a CTA keeps for later
 constexpr int kTabN = 4096;                // batch sizes of the K table
@@ -65,12 +71,14 @@ struct TileRec {
 // One warp's tile.  pre: per 8 requests {S1, S2, S3 + prefills << 55} of the
 // requests before them in their 256; tot: each 256's totals.
 struct WarpTile {
-  alignas(16) uint4 pre[kTBlocks * 32];
+  union {
+    alignas(16) uint4 pre[kTBlocks * 32];
+    uint16_t list[kTCap];  // step 3: requests off the common path
+  };
   alignas(16) uint4 tot[kTBlocks];
   alignas(16) TileRec rec[kTRec];
   uint32_t bits[kTWords];  // head bits: a batch starts at this request
   uint16_t rank[kTWords];  // heads before word w
-  uint32_t list[kTList];   // deferred requests: index | record << 16
 };
 
 struct TSmem {
@@ -138,19 +146,8 @@ struct TileSrc {
   int lim;
 };
 
-// The quad that holds the end of the arrays, or none of them: zero past it.
-__device__ __noinline__ Quad quad_tail(const int32_t *p, const int32_t *c, const int32_t *x, int e, int lim) {
-  int v[3][4];
-  const int32_t *src[3] = {p, c, x};
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int k = 0; k < 4; ++k) v[a][k] = src[a] && e + k < lim ? src[a][e + k] : 0;
-  return Quad{make_int4(v[0][0], v[0][1], v[0][2], v[0][3]), make_int4(v[1][0], v[1][1], v[1][2], v[1][3]),
-              make_int4(v[2][0], v[2][1], v[2][2], v[2][3])};
-}
-
-// Four requests from index e (a multiple of 4).
+// Four requests from index e (a multiple of 4).  Past the end of the arrays: the
+// last request again, which no sum or share of the tile takes.
 template <bool X>
 __device__ __forceinline__ Quad load_quad(const int32_t *p, const int32_t *c, const int32_t *x, int e, int lim) {
   Quad q;
@@ -159,7 +156,13 @@ __device__ __forceinline__ Quad load_quad(const int32_t *p, const int32_t *c, co
     q.c = *reinterpret_cast<const int4 *>(c + e);
     q.x = X ? *reinterpret_cast<const int4 *>(x + e) : make_int4(0, 0, 0, 0);
   } else {
-    q = quad_tail(p, c, X ? x : nullptr, e, lim);
+    q.p = q.c = q.x = make_int4(0, 0, 0, 0);
+    if (e < lim) {
+      const int i1 = min(e + 1, lim - 1), i2 = min(e + 2, lim - 1);
+      q.p = make_int4(p[e], p[i1], p[i2], p[i2]);
+      q.c = make_int4(c[e], c[i1], c[i2], c[i2]);
+      if (X) q.x = make_int4(x[e], x[i1], x[i2], x[i2]);
+    }
   }
   return q;
 }
@@ -411,40 +414,44 @@ __device__ __forceinline__ float tile_one_f32(const TileArgs &a, const TenTab &t
   return s;
 }
 
-// The last min(n, 32) deferred requests of the tile, one per lane: prefills,
-// tenants and values off the common path, with every lane busy.  Returns how
-// many are left.
+// The record of the request at index e; before the tile's first batch, the first.
+__device__ __forceinline__ int tile_rank(const WarpTile &wt, int e) {
+  const int r = (int)wt.rank[e >> 5] + __popc(wt.bits[e >> 5] & ((2u << (e & 31)) - 1u));
+  return max(min(r, kTRec) - 1, 0);
+}
+
+// The tile's n listed requests, one per lane: prefills, tenants and values off
+// the common path, with every lane busy.
 template <int MODE>
-__device__ __noinline__ int tile_flush(const TileArgs &a, const TSmem &ts, const WarpTile &wt, int64_t rbase, int n,
-                                       int lane) {
-  const TenTab tt = tile_table(a, ts);
-  const int left = max(n - 32, 0);
+__device__ __forceinline__ void tile_rest(const TileArgs &a, const TenTab &tt, const TSmem &ts, const WarpTile &wt,
+                                          const TileSrc &src, int64_t rbase, int n, int lane) {
   __syncwarp();
-  if (left + lane < n) {
-    const uint32_t v = wt.list[left + lane];
-    const TileRec rec = wt.rec[v >> 16];
-    const int64_t i = rbase + (v & 0xffffu);
-    const int32_t p = a.p[i], c = a.c[i], u = (MODE & M_TEN) ? a.ten[i] : 0;
+  int bad = 0;
+#pragma unroll 1
+  for (int k = lane; k < n; k += 32) {
+    const int e = wt.list[k];
+    const TileRec &rec = wt.rec[tile_rank(wt, e)];
+    const int32_t p = src.p[e], c = src.c[e], u = (MODE & M_TEN) ? src.u[e] : 0;
     if (MODE & M_F32) {
-      int bad = 0;
       const float f = tile_one_f32<MODE>(a, tt, rec, p, c, u, &bad);
-      if (a.share32) __stcs(a.share32 + i, f);
-      if (bad) flag(a.status, kStatusData);
+      if (a.share32) __stcs(a.share32 + rbase + e, f);
     } else {
       double d;
-      if (tile_one<MODE>(a, tt, ts, rec, (int64_t)(rec.a.z >> 4), i, p, c, u, &d) && a.share) __stcs(a.share + i, d);
+      if (tile_one<MODE>(a, tt, ts, rec, (int64_t)(rec.a.z >> 4), rbase + e, p, c, u, &d) && a.share)
+        __stcs(a.share + rbase + e, d);
     }
   }
-  __syncwarp();
-  return left;
+  if (bad) flag(a.status, kStatusData);
 }
 
 // The tile's shares, four consecutive requests per lane and step.  The loop
-// takes decode requests (p = 1; fp32 variant: any) of the batch that the
-// lane's first one belongs to, on the common path, without a
-// branch; the rest goes to the warp's list, which is worked off 32 at
-// a time.  vec: the share array allows 32-byte (fp32: 16-byte) stores.
-template <int MODE>
+// takes decode requests (p = 1; fp32 variant: any) on the common path, without a
+// branch or a call; the rest goes to the warp's list, worked off after it.
+// kPer: a record per request (tiles of small batches); otherwise the lane's
+// four share the first one's record, and what lies past a batch's start among
+// them goes to the list.  vec: the share array allows 32-byte (fp32: 16-byte)
+// stores.
+template <int MODE, bool kPer>
 __device__ __forceinline__ void tile_shares(const TileArgs &a, const TenTab &tt, const TSmem &ts, WarpTile &wt,
                                             const TileSrc &src, int64_t rbase, int first, int cnt, bool vec,
                                             int lane) {
@@ -453,9 +460,7 @@ __device__ __forceinline__ void tile_shares(const TileArgs &a, const TenTab &tt,
     // fp64 mode has no common path: one request per lane, in order
     for (int e = lane; e < cnt; e += 32) {
       if (e < first) continue;
-      const uint32_t word = wt.bits[e >> 5];
-      const int r = min((int)wt.rank[e >> 5] + __popc(word & ((2u << (e & 31)) - 1u)), kTRec) - 1;
-      const TileRec &rec = wt.rec[max(r, 0)];
+      const TileRec &rec = wt.rec[tile_rank(wt, e)];
       tile_slow<MODE>(a, ts, rec, (int64_t)(rec.a.z >> 4), rbase + e, src.p[e], src.c[e], kTen ? src.u[e] : 0);
     }
     return;
@@ -475,17 +480,17 @@ __device__ __forceinline__ void tile_shares(const TileArgs &a, const TenTab &tt,
     const uint32_t word = wt.bits[b / 32 + (lane >> 3)];
     const int sh = e & 31;
     const uint32_t hb = (word >> sh) & 14u;
-    const uint32_t run = vm & ((hb & (0u - hb)) - 1u);  // no head: all four
+    const uint32_t run = kPer ? vm : vm & ((hb & (0u - hb)) - 1u);  // no head: all four
     // record of the first request; -1 before the tile's first batch
     const int r0 = min((int)wt.rank[b / 32 + (lane >> 3)] + __popc(word & ((2u << sh) - 1u)), kTRec - 4) - 1;
-    const TileRec rec = wt.rec[max(r0, 0)];
-    const int32_t pe = (rec.a.z & 8u) ? 1 : -1;
+    TileRec rec = wt.rec[max(r0, 0)];
     bool go[4];
     uint32_t dlo[4], dhi[4];
     float f[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      go[k] = ((run >> k) & 1u) != 0u && r0 >= 0;
+      if (kPer && k > 0) rec = wt.rec[max(r0 + __popc(hb & ((2u << k) - 1u)), 0)];
+      go[k] = ((run >> k) & 1u) != 0u && (kPer || r0 >= 0);
       if (kF32) {
         const Share32 q{__uint_as_float(rec.k.x), __uint_as_float(rec.k.y), __uint_as_float(rec.k.z),
                         __uint_as_float(rec.k.w)};
@@ -496,7 +501,7 @@ __device__ __forceinline__ void tile_shares(const TileArgs &a, const TenTab &tt,
         dhi[k] = (x >> 3) + ((1023u - 127u) << 20);
         if (kTen) go[k] = go[k] && x - 0x00800000u < 0x7f000000u;
       } else {
-        go[k] = go[k] && (MODE & M_FIX) && p[k] == pe;
+        go[k] = go[k] && (MODE & M_FIX) && (rec.a.z & 8u) && p[k] == 1;
         const double d = tile_value(rec, rec.k.x, rec.k.y, rec.k.z, c[k]);
         dlo[k] = (uint32_t)__double2loint(d);
         dhi[k] = (uint32_t)__double2hiint(d);
@@ -537,15 +542,12 @@ __device__ __forceinline__ void tile_shares(const TileArgs &a, const TenTab &tt,
         at += __popc(bm & lt);
         nl += __popc(bm);
       }
-      for (uint32_t m = dm; m; m &= m - 1u) {
-        const int k = __ffs(m) - 1;
-        const int rk = max(r0 + __popc(hb & ((2u << k) - 1u)), 0);
-        wt.list[at++] = (uint32_t)(e + k) | ((uint32_t)rk << 16);
-      }
-      while (nl >= 32) nl = tile_flush<MODE>(a, ts, wt, rbase, nl, lane);
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if ((dm >> k) & 1u) wt.list[at++] = (uint16_t)(e + k);
     }
   }
-  if (nl > 0) tile_flush<MODE>(a, ts, wt, rbase, nl, lane);
+  if (nl > 0) tile_rest<MODE>(a, tt, ts, wt, src, rbase, nl, lane);
 }
 
 // One batch walked by `kThreads` threads (a warp, or the CTA) from global
@@ -729,7 +731,12 @@ __global__ void __launch_bounds__(kTThreads, 1) k_tiles(const TileArgs a) {
 
     // 3. requests
     if ((MODE & M_ATTR) && !wide && (kTen || a.share || a.share32))
-      tile_shares<MODE>(a, tt, ts, wt, src, rbase, first, cnt, vec, lane);
+{
+      if (!(MODE & (M_FIX | M_F32)) || before * kTDense <= cnt)
+        tile_shares<MODE, false>(a, tt, ts, wt, src, rbase, first, cnt, vec, lane);
+      else
+        tile_shares<MODE, true>(a, tt, ts, wt, src, rbase, first, cnt, vec, lane);
+    }
     if (direct) {
       // the last batch; every batch of a wide tile
       for (int i = 0; i < nb; ++i) {

@@ -24,8 +24,8 @@ def _check(lv, ctx, w, acc=True):
     base._check_parity(w, T, share, L)
 
 
-@pytest.mark.parametrize("lo,hi,n", [(0, 2, 6000), (1, 8, 3000), (250, 262, 400), (500, 520, 300), (760, 776, 200),
-                                     (1016, 1032, 150), (513, 5000, 200)])
+@pytest.mark.parametrize("lo,hi,n", [(0, 2, 6000), (1, 8, 3000), (30, 50, 900), (250, 262, 400), (284, 292, 300),
+                                     (500, 520, 300), (1240, 1256, 200), (1528, 1544, 150), (513, 5000, 200)])
 @pytest.mark.parametrize("cut", [0, 1, 3])
 def test_sizes_around_the_tile(lv, ctx, lo, hi, n, cut):
     """Sizes lo..hi, the last batch cut so that the arrays end 0, 1 or 3 requests into a quad."""
