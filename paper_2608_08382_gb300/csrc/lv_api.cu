@@ -61,7 +61,9 @@ struct lv_tenant_acc {
   lv_ctx *ctx = nullptr;
   int32_t n_tenants = 0;
   unsigned long long *d_pend = nullptr;  // [n][4]
-  i128 *d_state = nullptr;               // [n]
+  i128 *d_state = nullptr;               // [n], after d_pend in one allocation
+  unsigned *d_ticket = nullptr;          // after it: CTAs done with a fold
+  size_t bytes = 0;                      // of the allocation
 };
 
 namespace {
@@ -298,6 +300,8 @@ std::mutex &free_occ_mu() {
 struct TilePlan {
   int64_t n_tiles;
   uint64_t magic;
+  int64_t D;
+  bool search;  // at most one tile per warp: the warps find the bounds
 };
 
 TilePlan plan_tiles(int64_t n_batch, int64_t n_req, int64_t warps) {
@@ -308,6 +312,8 @@ TilePlan plan_tiles(int64_t n_batch, int64_t n_req, int64_t warps) {
   TilePlan p;
   p.n_tiles = (units + D - 1) / D;
   p.magic = UINT64_MAX / (uint64_t)D + 1;
+  p.D = D;
+  p.search = rounds == 1;
   return p;
 }
 
@@ -364,25 +370,29 @@ lv_status run_tiles_mode(lv_ctx *ctx, int sms, TileArgs &a, void *bound, int64_t
   if (st != LV_OK) return st;
   const int64_t ctas = (int64_t)sms * per_sm;
   const TilePlan plan = plan_tiles(a.n_batch, a.n_req, ctas * kTWarps);
-  if (ctx) {
-    st = ensure_bound(ctx, plan.n_tiles + 1);
-    if (st != LV_OK) return st;
-    bound = ctx->d_bound;
-  } else if (plan.n_tiles + 1 > bound_cap) {
-    return LV_EINVAL;
-  }
-  const bool narrow = a.n_batch < (1ll << 32);
-  a.bound = narrow ? nullptr : static_cast<int64_t *>(bound);
-  a.bound32 = narrow ? static_cast<uint32_t *>(bound) : nullptr;
   a.n_tiles = plan.n_tiles;
-  const int64_t blocks = std::min<int64_t>((a.n_batch + 1 + 255) / 256, (int64_t)sms * 16);
-  if (narrow)
-    k_tile_bounds<uint32_t><<<(unsigned)blocks, 256, 0, stream>>>(a.off, a.n_batch, a.n_req, plan.n_tiles, plan.magic,
-                                                                  static_cast<uint32_t *>(bound), a.status);
-  else
-    k_tile_bounds<int64_t><<<(unsigned)blocks, 256, 0, stream>>>(a.off, a.n_batch, a.n_req, plan.n_tiles, plan.magic,
-                                                                 static_cast<int64_t *>(bound), a.status);
-  LV_CUDA(cudaGetLastError());
+  a.D = plan.search ? plan.D : 0;
+  if (!plan.search) {
+    if (ctx) {
+      st = ensure_bound(ctx, plan.n_tiles + 1);
+      if (st != LV_OK) return st;
+      bound = ctx->d_bound;
+    } else if (plan.n_tiles + 1 > bound_cap) {
+      return LV_EINVAL;
+    }
+    const int64_t blocks = std::min<int64_t>((a.n_batch + 1 + 255) / 256, (int64_t)sms * 16);
+    if (a.n_batch < (1ll << 32)) {
+      a.bound32 = static_cast<uint32_t *>(bound);
+      k_tile_bounds<uint32_t><<<(unsigned)blocks, 256, 0, stream>>>(a.off, a.n_batch, a.n_req, plan.n_tiles,
+                                                                    plan.magic, static_cast<uint32_t *>(bound),
+                                                                    a.status);
+    } else {
+      a.bound = static_cast<int64_t *>(bound);
+      k_tile_bounds<int64_t><<<(unsigned)blocks, 256, 0, stream>>>(a.off, a.n_batch, a.n_req, plan.n_tiles, plan.magic,
+                                                                   static_cast<int64_t *>(bound), a.status);
+    }
+    LV_CUDA(cudaGetLastError());
+  }
   cudaEvent_t stop = nullptr;
   if (ctx) {
     st = timing_begin(ctx, LV_TIME_TILES, stream, &stop);
@@ -477,11 +487,28 @@ bool step_sized(const lv_batches *b) {
   return b->n_req <= kSmallMaxReq && b->n_batch <= kSmallMaxBatch && b->n_batch > 0;
 }
 
+// Whether a kernel that adds to the accumulator folds it as well.
+bool folds_inline(const lv_tenant_acc *acc) { return acc && acc->n_tenants <= kFoldInline; }
+
 lv_status fold_tenants(lv_ctx *ctx, lv_tenant_acc *acc, cudaStream_t stream) {
   const int n = acc->n_tenants;
   k_tenant_fold<<<(n + 255) / 256, 256, 0, stream>>>(acc->d_pend, acc->d_state, n, ctx->d_status);
   LV_CUDA(cudaGetLastError());
   return LV_OK;
+}
+
+// The tile pass of an attribution, its fold, and the event after the last use
+// of the K table.
+lv_status run_attr(lv_ctx *ctx, TileArgs &a, int mode, lv_tenant_acc *acc, cudaStream_t stream) {
+  if (folds_inline(acc) && a.n_batch > 0) {
+    a.ten_state = acc->d_state;
+    a.ten_ticket = acc->d_ticket;
+  }
+  lv_status st = run_tiles(ctx, a, mode, stream);
+  if (st != LV_OK) return st;
+  st = record_event(ctx->ev_used, stream);
+  if (st != LV_OK) return st;
+  return acc && !a.ten_state ? fold_tenants(ctx, acc, stream) : LV_OK;
 }
 
 // The exact pass of lv_fit and lv_fit_vtc: per-CTA partials of the fit
@@ -848,12 +875,7 @@ lv_status lv_attribute(lv_ctx *ctx, const lv_model *model, const lv_batches *b, 
   st = prepare_model(ctx, model, stream, &mp);
   if (st != LV_OK) return st;
   TileArgs a = attr_args(ctx, b, T, share, acc, mp, &mode);
-  st = run_tiles(ctx, a, mode, stream);
-  if (st != LV_OK) return st;
-  st = record_event(ctx->ev_used, stream);
-  if (st != LV_OK) return st;
-  if (acc) return fold_tenants(ctx, acc, stream);
-  return LV_OK;
+  return run_attr(ctx, a, mode, acc, stream);
 }
 
 lv_status lv_attribute_step(lv_ctx *ctx, const lv_model *model, const lv_batches *b, double *T, double *share,
@@ -912,12 +934,7 @@ lv_status lv_attribute_f32(lv_ctx *ctx, const lv_model *model, const lv_batches 
     a.n_tenants = acc->n_tenants;
     a.H = std::min<int32_t>(acc->n_tenants, kHotMax);
   }
-  st = run_tiles(ctx, a, mode, stream);
-  if (st != LV_OK) return st;
-  st = record_event(ctx->ev_used, stream);
-  if (st != LV_OK) return st;
-  if (acc) return fold_tenants(ctx, acc, stream);
-  return LV_OK;
+  return run_attr(ctx, a, mode, acc, stream);
 }
 
 lv_status lv_tenant_acc_create(lv_ctx *ctx, int32_t n_tenants, lv_tenant_acc **out) {
@@ -927,14 +944,16 @@ lv_status lv_tenant_acc_create(lv_ctx *ctx, int32_t n_tenants, lv_tenant_acc **o
   if (!acc) return LV_ENOMEM;
   acc->ctx = ctx;
   acc->n_tenants = n_tenants;
-  if (cudaMalloc(&acc->d_pend, sizeof(unsigned long long) * 4 * (size_t)n_tenants) != cudaSuccess ||
-      cudaMalloc(&acc->d_state, sizeof(i128) * (size_t)n_tenants) != cudaSuccess) {
+  const size_t pend = sizeof(unsigned long long) * 4 * (size_t)n_tenants, state = sizeof(i128) * (size_t)n_tenants;
+  acc->bytes = pend + state + 16;
+  if (cudaMalloc(&acc->d_pend, acc->bytes) != cudaSuccess) {
+    acc->d_pend = nullptr;
     lv_tenant_acc_destroy(acc);
     return LV_ENOMEM;
   }
-  if (cudaMemset(acc->d_pend, 0, sizeof(unsigned long long) * 4 * (size_t)n_tenants) != cudaSuccess ||
-      cudaMemset(acc->d_state, 0, sizeof(i128) * (size_t)n_tenants) != cudaSuccess ||
-      cudaDeviceSynchronize() != cudaSuccess) {
+  acc->d_state = reinterpret_cast<i128 *>(reinterpret_cast<unsigned char *>(acc->d_pend) + pend);
+  acc->d_ticket = reinterpret_cast<unsigned *>(reinterpret_cast<unsigned char *>(acc->d_pend) + pend + state);
+  if (cudaMemset(acc->d_pend, 0, acc->bytes) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) {
     lv_tenant_acc_destroy(acc);
     return LV_ECUDA;
   }
@@ -946,15 +965,12 @@ void lv_tenant_acc_destroy(lv_tenant_acc *acc) {
   if (!acc) return;
   cudaDeviceSynchronize();
   if (acc->d_pend) cudaFree(acc->d_pend);
-  if (acc->d_state) cudaFree(acc->d_state);
   delete acc;
 }
 
 lv_status lv_tenant_acc_reset(lv_tenant_acc *acc, void *stream) {
   if (!acc) return LV_EINVAL;
-  LV_CUDA(cudaMemsetAsync(acc->d_pend, 0, sizeof(unsigned long long) * 4 * (size_t)acc->n_tenants,
-                          (cudaStream_t)stream));
-  LV_CUDA(cudaMemsetAsync(acc->d_state, 0, sizeof(i128) * (size_t)acc->n_tenants, (cudaStream_t)stream));
+  LV_CUDA(cudaMemsetAsync(acc->d_pend, 0, acc->bytes, (cudaStream_t)stream));
   return LV_OK;
 }
 
@@ -975,10 +991,11 @@ lv_status lv_tenant_accumulate(lv_ctx *ctx, lv_tenant_acc *acc, const double *sh
     }
     const int64_t blocks = std::min<int64_t>((n_req + 4 * kAccThreads - 1) / (4 * kAccThreads), (int64_t)ctx->sms);
     k_tenant_acc<<<(unsigned)blocks, kAccThreads, ten_table_bytes(H), stream>>>(
-        share, tenant, n_req, acc->d_pend, acc->n_tenants, H, ctx->d_status);
+        share, tenant, n_req, acc->d_pend, acc->n_tenants, H, ctx->d_status,
+        folds_inline(acc) ? acc->d_state : nullptr, acc->d_ticket);
     LV_CUDA(cudaGetLastError());
   }
-  return fold_tenants(ctx, acc, stream);
+  return n_req > 0 && folds_inline(acc) ? LV_OK : fold_tenants(ctx, acc, stream);
 }
 
 lv_status lv_tenant_totals(lv_ctx *ctx, lv_tenant_acc *acc, double *L, void *stream_) {

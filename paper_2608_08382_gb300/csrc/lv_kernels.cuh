@@ -94,11 +94,14 @@ struct TileArgs {
   const int64_t *bound;    // [n_tiles + 1] first batch of each tile (k_tiles), or null:
   const uint32_t *bound32;  // the same in 32 bits (fewer than 2^32 batches)
   int64_t n_tiles;
+  int64_t D;             // merge positions per tile where the warps find their bounds themselves, or 0
   double *T, *share;
   float *T32, *share32;  // fp32 variant (M_F32): T and shares as float, or null
   int64_t *bfeat;   // [5][n_batch] or null; M_FIT: [4][n_batch] S1, S2, S3, n
   uint8_t *bseg;    // [n_batch] or null; M_FIT: 255 for an empty batch
   unsigned long long *ten_pend;  // [n_tenants][4] 32-bit limbs in 64-bit words, or null
+  i128 *ten_state;               // the tenants' exact state where the kernel folds it, or null
+  unsigned *ten_ticket;          // CTAs done (zero between launches)
   int32_t n_tenants, H;
   int *status;
   ModelP mp;
@@ -505,23 +508,27 @@ __device__ __noinline__ Rounded share_slow(const ModelP &mp, int s, bool fixed, 
 
 // state[u] += pending limbs of u; pending limbs cleared.  Deterministic: pure
 // integer arithmetic on exact sums.
-__global__ void k_tenant_fold(unsigned long long *__restrict__ pend, i128 *__restrict__ state, int32_t n_tenants,
-                              int *status) {
-  const int u = blockIdx.x * blockDim.x + threadIdx.x;
-  if (u >= n_tenants) return;
+__device__ __forceinline__ void fold_tenant(unsigned long long *pend, i128 *state, int u, int *status) {
   unsigned long long *w = pend + 4 * (int64_t)u;
-  const long long w0 = (long long)w[0], w1 = (long long)w[1], w2 = (long long)w[2], w3 = (long long)w[3];
-  if ((w0 | w1 | w2 | w3) == 0) return;
-  i128 v = mk128((uint64_t)w0, (uint64_t)(w0 >> 63));
-  v = add128(v, shl128((uint64_t)w1, (uint64_t)(w1 >> 63), 32));
-  v = add128(v, mk128(0, (uint64_t)w2));
-  v = add128(v, mk128(0, (uint64_t)w3 << 32));
+  const longlong2 *p = reinterpret_cast<const longlong2 *>(w);
+  const longlong2 a = __ldcg(p), b = __ldcg(p + 1);
+  if ((a.x | a.y | b.x | b.y) == 0) return;
+  i128 v = mk128((uint64_t)a.x, (uint64_t)(a.x >> 63));
+  v = add128(v, shl128((uint64_t)a.y, (uint64_t)(a.y >> 63), 32));
+  v = add128(v, mk128(0, (uint64_t)b.x));
+  v = add128(v, mk128(0, (uint64_t)b.y << 32));
   const i128 old = state[u];
   const i128 nw = add128(old, v);
   // overflow of the signed 128-bit total (|total| >= 2^127 * 2^-72 s = 2^55 s)
   if (is_neg128(old) == is_neg128(v) && is_neg128(nw) != is_neg128(old)) flag(status, kStatusData);
   state[u] = nw;
   w[0] = w[1] = w[2] = w[3] = 0;
+}
+
+__global__ void k_tenant_fold(unsigned long long *__restrict__ pend, i128 *__restrict__ state, int32_t n_tenants,
+                              int *status) {
+  const int u = blockIdx.x * blockDim.x + threadIdx.x;
+  if (u < n_tenants) fold_tenant(pend, state, u, status);
 }
 
 __global__ void k_tenant_totals(const i128 *__restrict__ state, double *__restrict__ L, int32_t n_tenants) {

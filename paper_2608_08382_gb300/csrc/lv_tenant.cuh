@@ -50,6 +50,23 @@ __device__ __forceinline__ void ten_table_flush(const uint32_t *smem, int cap, i
   }
 }
 
+// The fold by the last CTA to finish (every CTA calls this once its additions
+// to the pending counters are issued): for few tenants one CTA's pass over them
+// costs less than a launch of k_tenant_fold (3 us and the gap before it).
+constexpr int kFoldInline = 2048;
+__device__ __forceinline__ void ten_fold_last(unsigned long long *pend, i128 *state, unsigned *ticket, int n,
+                                              int *status, int tid, int threads) {
+  __shared__ bool last;
+  __threadfence();  // this thread's additions before the CTA's ticket
+  __syncthreads();
+  if (tid == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  for (int u = tid; u < n; u += threads) fold_tenant(pend, state, u, status);
+  if (tid == 0) *ticket = 0u;
+}
+
 // Shared-memory atomic add at a byte address (address space stated, so that it
 // compiles to the shared-memory instruction wherever the table comes from).
 __device__ __forceinline__ uint32_t atom_shared(uint32_t addr, uint32_t v) {
@@ -191,7 +208,7 @@ constexpr int kAccThreads = 1024;
 constexpr int kAccHotMax = 8192;
 __global__ void __launch_bounds__(kAccThreads, 1)
     k_tenant_acc(const double *__restrict__ share, const int32_t *__restrict__ ten, int64_t n,
-                 unsigned long long *pend, int32_t n_tenants, int32_t H, int *status) {
+                 unsigned long long *pend, int32_t n_tenants, int32_t H, int *status, i128 *state, unsigned *ticket) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   uint32_t *tw = reinterpret_cast<uint32_t *>(smem_raw);
   const TenTab tt = ten_table(tw, H, H, n_tenants, pend);
@@ -221,6 +238,7 @@ __global__ void __launch_bounds__(kAccThreads, 1)
   }
   __syncthreads();
   ten_table_flush(tw, H, H, pend, threadIdx.x, kAccThreads);
+  if (state) ten_fold_last(pend, state, ticket, n_tenants, status, threadIdx.x, kAccThreads);
 }
 
 }  // namespace lv

@@ -133,6 +133,31 @@ __device__ __forceinline__ int64_t tile_bound(const TileArgs &a, int64_t t) {
   return a.bound32 ? (int64_t)a.bound32[t] : a.bound[t];
 }
 
+// The bounds of tile t by a warp's own search, for inputs of at most one tile
+// per warp: 16 offsets are looked at per round and bound, so 20,000 batches
+// take four rounds of one load each, less than k_tile_bounds and the gap after
+// it.  (Lanes 0..15 look for bound t, the others for t + 1.)
+__device__ __forceinline__ void tile_search(const TileArgs &a, int64_t t, int lane, int64_t *b0, int64_t *b1) {
+  const int half = lane >> 4, l = lane & 15;
+  const int64_t target = (t + half) * a.D;
+  int64_t lo = 0, hi = a.n_batch;  // the bound is in [lo, hi]; tile n_tiles ends at n_batch
+  if (t + half >= a.n_tiles) lo = hi;
+  while (__any_sync(kFull, lo < hi)) {
+    const int64_t m = lo + (((hi - lo) * l) >> 4);
+    const bool at = lo >= hi || kTW * m + clampi(a.off[m], 0, a.n_req) >= target;
+    const uint32_t bal = (__ballot_sync(kFull, at) >> (16 * half)) & 0xffffu;
+    const int c = bal ? __ffs(bal) - 1 : 16;  // the first c probes lie before the bound
+    const int64_t before = __shfl_sync(kFull, m, 16 * half + max(c - 1, 0)),
+                  after = __shfl_sync(kFull, m, 16 * half + min(c, 15));
+    if (lo < hi) {
+      if (c < 16) hi = after;
+      lo = c > 0 ? before + 1 : hi;
+    }
+  }
+  *b0 = __shfl_sync(kFull, lo, 0);
+  *b1 = __shfl_sync(kFull, lo, 16);
+}
+
 // ---------------------------------------------------------------- loads
 
 struct Quad {
@@ -636,9 +661,22 @@ __global__ void __launch_bounds__(kTThreads, 1) k_tiles(const TileArgs a) {
   const int64_t stride = (int64_t)gridDim.x * kTWarps;
   int64_t t = (int64_t)wid * gridDim.x + blockIdx.x;
   int64_t b0 = 0, b1 = 0, r0 = 0, r1 = 0;
+  if (a.D) {
+    // k_tile_bounds' checks of the offsets
+    const int64_t threads = (int64_t)gridDim.x * kTThreads;
+    for (int64_t i = blockIdx.x * (int64_t)kTThreads + tid; i < a.n_batch; i += threads)
+      if (a.off[i] > a.off[i + 1]) bad = 1;
+    if (blockIdx.x == 0 && tid == 0 && (a.off[0] != 0 || a.off[a.n_batch] != a.n_req)) bad = 1;
+  }
   if (t < a.n_tiles) {
-    b0 = clampi(tile_bound(a, t), 0, a.n_batch);
-    b1 = clampi(tile_bound(a, t + 1), b0, a.n_batch);
+    if (a.D) {
+      tile_search(a, t, lane, &b0, &b1);
+    } else {
+      b0 = tile_bound(a, t);
+      b1 = tile_bound(a, t + 1);
+    }
+    b0 = clampi(b0, 0, a.n_batch);
+    b1 = clampi(b1, b0, a.n_batch);
     r0 = clampi(a.off[b0], 0, a.n_req);
     r1 = clampi(a.off[b1], r0, a.n_req);
   }
@@ -776,6 +814,7 @@ __global__ void __launch_bounds__(kTThreads, 1) k_tiles(const TileArgs a) {
   if (kTen) {
     __syncthreads();
     ten_table_flush(tw, kHotMax, a.H, a.ten_pend, tid, kTThreads);
+    if (a.ten_state) ten_fold_last(a.ten_pend, a.ten_state, a.ten_ticket, a.n_tenants, a.status, tid, kTThreads);
   }
 }
 
