@@ -102,13 +102,15 @@ __device__ __forceinline__ void ten_add(const TenTab &tt, uint32_t u, uint32_t l
 }
 
 // Tenant contributions of a lane's four positive normal shares (d: their
-// doubles' words) in the common case, a valid tenant and a share in [2^-20, 2^-8)
-// s (then q is whole and below 2^64); go[k] is cleared otherwise.  (Shifts, and
+// doubles' words) in the common case, a valid tenant and a share in [2^-20, 2^-8 (1 -
+// 2^-21)) s (then q is whole and below 2^64 - 2^32, so a carry into its high
+// word does not wrap); go[k] is cleared otherwise.  (Shifts, and
 // not the hardware's conversion to a 64-bit integer: that runs at 1/64 rate,
 // and the shares' rounding needs one already.)  The four low
 // words' atomics are issued together, then the four high words', so that a lane
 // waits for two of them and not for eight; lanes with nothing to add use a word
 // of their own, so there is no branch.
+constexpr uint32_t kShareLo = (uint32_t)(1075 + kTenLsb) << 20, kShareHi = kShareLo + (12u << 20) - 1u;
 __device__ __forceinline__ void ten_add4(const TenTab &tt, bool *go, const uint32_t *u, const uint32_t *dlo,
                                          const uint32_t *dhi) {
   uint32_t w[4], lo[4], hi[4], c1[4];
@@ -118,7 +120,7 @@ __device__ __forceinline__ void ten_add4(const TenTab &tt, bool *go, const uint3
     const uint32_t sh = (dhi[k] >> 20) - (uint32_t)(1075 + kTenLsb);
     lo[k] = dlo[k] << (sh & 31u);
     hi[k] = __funnelshift_l(dlo[k], (dhi[k] & 0xfffffu) | 0x100000u, sh);
-    go[k] = go[k] && sh <= 11u && hi[k] != 0xffffffffu && u[k] < tt.n;
+    go[k] = go[k] && dhi[k] - kShareLo < kShareHi - kShareLo && u[k] < tt.n;
     const bool hot = go[k] && u[k] < tt.H;
     w[k] = tt.w + 8u * u[k];
     w[k] = hot ? w[k] : tt.sink;

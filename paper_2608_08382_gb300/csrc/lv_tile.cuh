@@ -79,6 +79,7 @@ struct WarpTile {
   alignas(16) TileRec rec[kTRec];
   uint32_t bits[kTWords];  // head bits: a batch starts at this request
   uint16_t rank[kTWords];  // heads before word w
+  uint32_t n_list;         // entries of list
 };
 
 struct TSmem {
@@ -490,7 +491,6 @@ __device__ __forceinline__ void tile_shares(const TileArgs &a, const TenTab &tt,
     }
     return;
   }
-  int nl = 0;
   Quad nx = load_quad<kTen>(src.p, src.c, src.u, 4 * lane, src.lim);
 #pragma unroll 1
   for (int b = 0; b < cnt; b += 128) {
@@ -558,20 +558,16 @@ __device__ __forceinline__ void tile_shares(const TileArgs &a, const TenTab &tt,
           if (go[k]) __stcs(a.share + i0 + k, d[k]);
       }
     }
-    if (__any_sync(kFull, dm != 0u)) {
-      const uint32_t lt = (1u << lane) - 1u;
-      int at = nl;
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const uint32_t bm = __ballot_sync(kFull, (dm >> k) & 1u);
-        at += __popc(bm & lt);
-        nl += __popc(bm);
-      }
+    if (dm) {
+      // slots by a shared-memory add: few lanes come here, and the list's order is free
+      uint32_t at = atomicAdd(&wt.n_list, (uint32_t)__popc(dm));
 #pragma unroll
       for (int k = 0; k < 4; ++k)
         if ((dm >> k) & 1u) wt.list[at++] = (uint16_t)(e + k);
     }
   }
+  __syncwarp();
+  const int nl = (int)wt.n_list;
   if (nl > 0) tile_rest<MODE>(a, tt, ts, wt, src, rbase, nl, lane);
 }
 
@@ -707,7 +703,10 @@ __global__ void __launch_bounds__(kTThreads, 1) k_tiles(const TileArgs a) {
     if (MODE & M_ATTR) {
       for (int i = lane; i < kTWords; i += 32) {
         wt.bits[i] = 0;
-        if (i == 0) wt.rank[0] = 0;
+        if (i == 0) {
+          wt.rank[0] = 0;
+          wt.n_list = 0;
+        }
       }
     }
     const bool wide = tile_prefix(wt, src, cnt, lane);
