@@ -29,51 +29,96 @@ namespace lv {
 // Gram's in 128 bits, X^T y modulo 2^192, y'y in 256).  Entry order
 // in `partial`: 15 Gram pairs (a <= b, row order), 5 X^T y per y, one y'y per
 // y, one flag (some batch has S1 != S3).
-// Bound by instruction issue and latency (some 160 lane instructions a batch
-// for the Gram, 230 per latency vector; 16 warps per SM at 128 registers): 2e6
-// batches with two vectors take 150 us; 245 with one row of 32 segments looked
-// at per turn and nothing loaded ahead.  With one entry per lane and all lanes
-// on one batch, inside the kernel over the requests, the same sums took about
-// 0.35 of 0.96 ms.
+// Bound by instruction issue (16 warps per SM at 128 registers; the products
+// are carry-chained 32-bit multiply-adds, a quarter fewer instructions than
+// 64-bit ones): 2e6 batches with two vectors take 117 us; 150 with 64-bit
+// products, 245 with, besides, one row of 32 segments looked at per turn and
+// nothing loaded ahead.  With one entry per lane and all lanes on one batch,
+// inside the kernel over the requests, the same sums took about 0.35 of 0.96 ms.
 constexpr int kGramThreads = 256;
 constexpr int kGramWarps = kGramThreads / 32;
 constexpr int kGramMax = 16;  // entries of one row of blocks, at most
 constexpr int kGramScan = 8;  // rows of 32 batches looked at together
 
+// v += o for W 32-bit words (modulo 2^(32 W)).
 template <int W>
-__device__ __forceinline__ void add_words(uint64_t *v, const uint64_t *o) {
+__device__ __forceinline__ void add_words(uint32_t *v, const uint32_t *o) {
   uint64_t c = 0;
 #pragma unroll
   for (int w = 0; w < W; ++w) {
-    const uint64_t t = v[w] + c, s = t + o[w];
-    c = (t < c ? 1ull : 0ull) + (s < t ? 1ull : 0ull);
-    v[w] = s;
+    c += (uint64_t)v[w] + o[w];
+    v[w] = (uint32_t)c;
+    c >>= 32;
   }
 }
 
-// Sum over the warp of a W-word integer (modulo 2^(64 W)), into dst (lane 0),
-// sign-extended to four words when `sign`.
+// Sum over the warp of a W-word integer (modulo 2^(32 W)), into dst (lane 0),
+// sign-extended when `sign`.
 template <int W>
-__device__ __forceinline__ void warp_words(uint64_t *v, FitAcc *dst, bool sign, int lane) {
+__device__ __forceinline__ void warp_words(uint32_t *v, FitAcc *dst, bool sign, int lane) {
 #pragma unroll
   for (int d = 16; d; d >>= 1) {
-    uint64_t o[W];
+    uint32_t o[W];
 #pragma unroll
     for (int w = 0; w < W; ++w) o[w] = __shfl_xor_sync(0xffffffffu, v[w], d);
     add_words<W>(v, o);
   }
   if (lane == 0) {
-    const uint64_t fill = sign && (int64_t)v[W - 1] < 0 ? ~0ull : 0ull;
+    const uint32_t fill = sign && (int32_t)v[W - 1] < 0 ? ~0u : 0u;
 #pragma unroll
-    for (int w = 0; w < 4; ++w) dst->w[w] = w < W ? v[w] : fill;
+    for (int w = 0; w < 4; ++w)
+      dst->w[w] = (uint64_t)(2 * w < W ? v[2 * w < W ? 2 * w : 0] : fill) |
+                  (uint64_t)(2 * w + 1 < W ? v[2 * w + 1 < W ? 2 * w + 1 : 0] : fill) << 32;
   }
 }
 
-struct GramAcc {
-  uint64_t lin[5][2];   // n, S1, S2, S3, n^2
-  uint64_t sq[10][2];   // S1 S1, S1 S2, S1 S3, S1 n^2, S2 S2, ...
-  bool flag;
+// A feature below 2^48 in two words.
+struct Feat48 {
+  uint32_t l, h;
 };
+
+// a (4 words) += x y for x, y below 2^48.
+__device__ __forceinline__ void mac48(uint32_t *a, Feat48 x, Feat48 y) {
+  const uint64_t m = (uint64_t)x.l * y.h + (uint64_t)x.h * y.l;  // below 2^49
+  asm("mad.lo.cc.u32 %0, %4, %5, %0;\n\t"
+      "madc.hi.cc.u32 %1, %4, %5, %1;\n\t"
+      "addc.cc.u32 %2, %2, 0;\n\t"
+      "addc.u32 %3, %3, 0;\n\t"
+      "add.cc.u32 %1, %1, %6;\n\t"
+      "addc.cc.u32 %2, %2, %7;\n\t"
+      "addc.u32 %3, %3, 0;"
+      : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3])
+      : "r"(x.l), "r"(y.l), "r"((uint32_t)m), "r"((uint32_t)(m >> 32) + x.h * y.h));
+}
+
+// a (6 words) += x Y modulo 2^192 for x below 2^48 and Y of four words, two's
+// complement (neg: all ones where it is negative): Y as unsigned, less x 2^128.
+__device__ __forceinline__ void mac48x128(uint32_t *a, Feat48 x, const uint32_t *Y, uint32_t neg) {
+  asm("mad.lo.cc.u32 %0, %6, %8, %0;\n\t"
+      "madc.hi.cc.u32 %1, %6, %8, %1;\n\t"
+      "madc.lo.cc.u32 %2, %6, %10, %2;\n\t"
+      "madc.hi.cc.u32 %3, %6, %10, %3;\n\t"
+      "addc.cc.u32 %4, %4, 0;\n\t"
+      "addc.u32 %5, %5, 0;\n\t"
+      "mad.lo.cc.u32 %1, %6, %9, %1;\n\t"
+      "madc.hi.cc.u32 %2, %6, %9, %2;\n\t"
+      "madc.lo.cc.u32 %3, %6, %11, %3;\n\t"
+      "madc.hi.cc.u32 %4, %6, %11, %4;\n\t"
+      "addc.u32 %5, %5, 0;\n\t"
+      "mad.lo.cc.u32 %1, %7, %8, %1;\n\t"
+      "madc.hi.cc.u32 %2, %7, %8, %2;\n\t"
+      "madc.lo.cc.u32 %3, %7, %10, %3;\n\t"
+      "madc.hi.cc.u32 %4, %7, %10, %4;\n\t"
+      "addc.u32 %5, %5, 0;\n\t"
+      "mad.lo.cc.u32 %2, %7, %9, %2;\n\t"
+      "madc.hi.cc.u32 %3, %7, %9, %3;\n\t"
+      "madc.lo.cc.u32 %4, %7, %11, %4;\n\t"
+      "madc.hi.u32 %5, %7, %11, %5;\n\t"
+      "sub.cc.u32 %4, %4, %12;\n\t"
+      "subc.u32 %5, %5, %13;"
+      : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(a[4]), "+r"(a[5])
+      : "r"(x.l), "r"(x.h), "r"(Y[0]), "r"(Y[1]), "r"(Y[2]), "r"(Y[3]), "r"(x.l & neg), "r"(x.h & neg));
+}
 
 // A batch as loaded (n = 0: none).
 struct GramRaw {
@@ -81,47 +126,47 @@ struct GramRaw {
   double y;
 };
 
-struct FitYAcc {
-  uint64_t xy[5][3];
-  uint64_t yy[4];
+struct GramAcc {
+  uint32_t lin[5][3];  // n, S1, S2, S3, n^2 (below 2^96: fewer than 2^48 batches)
+  uint32_t sq[10][4];  // S1 S1, S1 S2, S1 S3, S1 n^2, S2 S2, ...
+  bool flag;
 };
 
-__device__ __forceinline__ void gram_add(GramAcc &g, const uint64_t *x) {
+struct FitYAcc {
+  uint32_t xy[5][6];
+  uint32_t yy[8];
+};
+
+__device__ __forceinline__ void gram_add(GramAcc &g, const Feat48 *x) {
 #pragma unroll
   for (int i = 0; i < 5; ++i) {
-    g.lin[i][0] += x[i];
-    g.lin[i][1] += g.lin[i][0] < x[i] ? 1ull : 0ull;
+    const uint32_t o[3] = {x[i].l, x[i].h, 0u};
+    add_words<3>(g.lin[i], o);
   }
   int e = 0;
 #pragma unroll
   for (int i = 1; i < 5; ++i)
 #pragma unroll
-    for (int j = i; j < 5; ++j, ++e) {
-      const uint64_t p[2] = {x[i] * x[j], __umul64hi(x[i], x[j])};
-      add_words<2>(g.sq[e], p);
-    }
-  g.flag |= x[1] != x[3];
+    for (int j = i; j < 5; ++j, ++e) mac48(g.sq[e], x[i], x[j]);
+  g.flag |= x[1].l != x[3].l || x[1].h != x[3].h;
 }
 
-__device__ __forceinline__ void fit_y_add(FitYAcc &g, const uint64_t *x, i128 Y) {
-  const uint64_t neg = is_neg128(Y) ? ~0ull : 0ull;
+__device__ __forceinline__ void fit_y_add(FitYAcc &g, const Feat48 *x, i128 Y) {
+  uint32_t y[4] = {(uint32_t)Y.lo, (uint32_t)(Y.lo >> 32), (uint32_t)Y.hi, (uint32_t)(Y.hi >> 32)};
+  const uint32_t neg = is_neg128(Y) ? ~0u : 0u;
+  const uint32_t one[6] = {y[0], y[1], y[2], y[3], neg, neg};  // the column of ones (Y = 0 where there is no batch)
+  add_words<6>(g.xy[0], one);
 #pragma unroll
-  for (int i = 0; i < 5; ++i) {
-    // x Y modulo 2^192: x times Y's two words as unsigned, less x 2^128 for a negative Y
-    uint64_t p[3] = {x[i] * Y.lo, __umul64hi(x[i], Y.lo), __umul64hi(x[i], Y.hi) - (x[i] & neg)};
-    const uint64_t m = x[i] * Y.hi;
-    p[1] += m;
-    p[2] += p[1] < m ? 1ull : 0ull;
-    add_words<3>(g.xy[i], p);
-  }
+  for (int i = 1; i < 5; ++i) mac48x128(g.xy[i], x[i], y, neg);
   // y'y: Y^2 (below 2^250) shifted right by 64 bits
   if (neg) Y = neg128(Y);
   const uint64_t l = Y.lo, h = Y.hi;
   uint64_t w[4] = {__umul64hi(l, l), h * h, __umul64hi(h, h), 0ull};
-  const uint64_t hl[4] = {h * l, __umul64hi(h, l), 0ull, 0ull};
-  add_words<3>(w, hl);
-  add_words<3>(w, hl);
-  add_words<4>(g.yy, w);
+  const uint64_t h0 = h * l, h1 = __umul64hi(h, l);
+  acc_add256(w, h0 << 1, (h1 << 1) | (h0 >> 63), h1 >> 63, 0ull);
+  const uint32_t o[8] = {(uint32_t)w[0], (uint32_t)(w[0] >> 32), (uint32_t)w[1], (uint32_t)(w[1] >> 32),
+                         (uint32_t)w[2], (uint32_t)(w[2] >> 32), 0u, 0u};
+  add_words<8>(g.yy, o);
 }
 
 struct GramSmem {
@@ -154,17 +199,18 @@ __device__ __forceinline__ void fit_rows(GramSmem &sm, const int64_t *__restrict
     FitYAcc ya{};
     GramRaw cur{0, 0, 0, 0, 0.0};
     auto add = [&]() {
-      uint64_t x[5] = {cur.n > 0 ? 1ull : 0ull, (uint64_t)cur.s1, (uint64_t)cur.s2, (uint64_t)cur.s3,
-                       (uint64_t)cur.n * (uint64_t)cur.n};
-      if ((x[1] | x[2] | x[3] | x[4]) >= (uint64_t)kFitFeatMax || (uint64_t)cur.n >= (1ull << 24)) {
-        flag(status, kStatusOverflow);
-        x[0] = x[1] = x[2] = x[3] = x[4] = 0;
-      }
+      const uint64_t v[5] = {cur.n > 0 ? 1ull : 0ull, (uint64_t)cur.s1, (uint64_t)cur.s2, (uint64_t)cur.s3,
+                             (uint64_t)cur.n * (uint64_t)cur.n};
+      const bool ok = (v[1] | v[2] | v[3] | v[4]) < (uint64_t)kFitFeatMax && (uint64_t)cur.n < (1ull << 24);
+      if (!ok) flag(status, kStatusOverflow);
+      Feat48 x[5];
+#pragma unroll
+      for (int c = 0; c < 5; ++c) x[c] = Feat48{ok ? (uint32_t)v[c] : 0u, ok ? (uint32_t)(v[c] >> 32) : 0u};
       if (kGram) {
         gram_add(ga, x);
       } else {
         bool ovf = false;
-        const i128 Y = x[0] ? double_to_fix(cur.y, kFitYLsb, &ovf) : mk128(0, 0);
+        const i128 Y = x[0].l ? double_to_fix(cur.y, kFitYLsb, &ovf) : mk128(0, 0);
         if (ovf) bad = 1;
         fit_y_add(ya, x, Y);
       }
@@ -210,16 +256,16 @@ __device__ __forceinline__ void fit_rows(GramSmem &sm, const int64_t *__restrict
     if (kGram) {
       ne = 16;
 #pragma unroll
-      for (int i = 0; i < 5; ++i) warp_words<2>(ga.lin[i], pw + i, false, lane);
+      for (int i = 0; i < 5; ++i) warp_words<3>(ga.lin[i], pw + i, false, lane);
 #pragma unroll
-      for (int e = 0; e < 10; ++e) warp_words<2>(ga.sq[e], pw + 5 + e, false, lane);
+      for (int e = 0; e < 10; ++e) warp_words<4>(ga.sq[e], pw + 5 + e, false, lane);
       const bool any = __any_sync(0xffffffffu, ga.flag);
       if (lane == 0) pw[15] = FitAcc{{any ? 1ull : 0ull, 0ull, 0ull, 0ull}};
     } else {
       ne = 6;
 #pragma unroll
-      for (int i = 0; i < 5; ++i) warp_words<3>(ya.xy[i], pw + i, true, lane);
-      warp_words<4>(ya.yy, pw + 5, false, lane);
+      for (int i = 0; i < 5; ++i) warp_words<6>(ya.xy[i], pw + i, true, lane);
+      warp_words<8>(ya.yy, pw + 5, false, lane);
     }
     __syncthreads();
     if ((int)threadIdx.x < ne) {
