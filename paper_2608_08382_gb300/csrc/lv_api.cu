@@ -258,6 +258,24 @@ lv_status prepare_model(lv_ctx *ctx, const lv_model *m, cudaStream_t stream, Mod
   return LV_OK;
 }
 
+// Launches a kernel that may start while the one before it in the stream runs
+// (it calls wait_previous itself).
+template <class... P, class... A>
+lv_status launch_after(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t stream, A... args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  LV_CUDA(cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...));
+  return LV_OK;
+}
+
 // Event pair around a measured launch (when timing is on; not while the stream
 // is being captured into a graph).
 lv_status timing_begin(lv_ctx *ctx, int kind, cudaStream_t stream, cudaEvent_t *stop) {
@@ -398,8 +416,14 @@ lv_status run_tiles_mode(lv_ctx *ctx, int sms, TileArgs &a, void *bound, int64_t
     st = timing_begin(ctx, LV_TIME_TILES, stream, &stop);
     if (st != LV_OK) return st;
   }
-  k_tiles<MODE><<<(unsigned)std::min<int64_t>(plan.n_tiles, ctas), kTThreads, smem, stream>>>(a);
-  LV_CUDA(cudaGetLastError());
+  const unsigned grid = (unsigned)std::min<int64_t>(plan.n_tiles, ctas);
+  if (plan.search) {
+    k_tiles<MODE><<<grid, kTThreads, smem, stream>>>(a);
+    LV_CUDA(cudaGetLastError());
+  } else {
+    st = launch_after(k_tiles<MODE>, grid, kTThreads, smem, stream, a);
+    if (st != LV_OK) return st;
+  }
   return ctx ? timing_end(stop, stream) : LV_OK;
 }
 
@@ -557,11 +581,11 @@ lv_status fit_pass(lv_ctx *ctx, const lv_batches *b, const double *y, int32_t n_
   a.bseg = seg;
   st = run_tiles(ctx, a, M_FIT, stream);
   if (st != LV_OK) return st;
-  k_fit_gram<<<dim3((unsigned)rows, 1 + n_y), kGramThreads, 0, stream>>>(feat, seg, b->n_batch, y, n_y, partial,
-                                                                         ctx->d_status);
-  LV_CUDA(cudaGetLastError());
-  k_fit_reduce<<<n_ent, kFitRedThreads, 0, stream>>>(partial, rows, n_ent, totals);
-  LV_CUDA(cudaGetLastError());
+  st = launch_after(k_fit_gram, dim3((unsigned)rows, 1 + n_y), kGramThreads, 0, stream, feat, seg, b->n_batch, y, n_y,
+                    partial, ctx->d_status);
+  if (st != LV_OK) return st;
+  st = launch_after(k_fit_reduce, n_ent, kFitRedThreads, 0, stream, partial, rows, n_ent, totals);
+  if (st != LV_OK) return st;
   *totals_out = totals;
   *out_out = out;
   return LV_OK;
@@ -648,9 +672,9 @@ lv_status whatif_run(lv_ctx *ctx, const lv_model *model, const lv_batches *cand,
     const dim3 grid((unsigned)gx, (unsigned)((rows + rpb - 1) / rpb));
     st = timing_begin(ctx, LV_TIME_PAIRS, stream, &stop);
     if (st != LV_OK) return st;
-    k_wi_pairs<<<grid, kWiThreads, 0, stream>>>(mp, candp, nc, p_new, c_new, phase_new, np, j, lc, rpb, adm, T_new,
-                                                share_new, ctx->d_status);
-    LV_CUDA(cudaGetLastError());
+    st = launch_after(k_wi_pairs, grid, kWiThreads, 0, stream, mp, candp, nc, p_new, c_new, phase_new, np, j, lc, rpb,
+                      adm, T_new, share_new, ctx->d_status);
+    if (st != LV_OK) return st;
     st = timing_end(stop, stream);
     if (st != LV_OK) return st;
   }
@@ -1001,9 +1025,7 @@ lv_status lv_tenant_accumulate(lv_ctx *ctx, lv_tenant_acc *acc, const double *sh
 lv_status lv_tenant_totals(lv_ctx *ctx, lv_tenant_acc *acc, double *L, void *stream_) {
   if (!ctx || !acc || acc->ctx != ctx || !L || !aligned(L, 8)) return LV_EINVAL;
   const int n = acc->n_tenants;
-  k_tenant_totals<<<(n + 255) / 256, 256, 0, (cudaStream_t)stream_>>>(acc->d_state, L, n);
-  LV_CUDA(cudaGetLastError());
-  return LV_OK;
+  return launch_after(k_tenant_totals, (unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream_, acc->d_state, L, n);
 }
 
 int64_t lv_tenant_acc_state_bytes(const lv_tenant_acc *acc) {
@@ -1040,8 +1062,8 @@ lv_status lv_fit(lv_ctx *ctx, const lv_batches *b, const double *y, int32_t n_y,
   FitOut *out = nullptr;
   lv_status st = fit_pass(ctx, b, y, n_y, inout[0].split, stream, &totals, &out);
   if (st != LV_OK) return st;
-  k_fit_solve<<<4 * kFitMaxY, 64, 0, stream>>>(totals, n_y, out);
-  LV_CUDA(cudaGetLastError());
+  st = launch_after(k_fit_solve, 4 * kFitMaxY, 64, 0, stream, totals, n_y, out);
+  if (st != LV_OK) return st;
   FitOut h[4 * kFitMaxY];
   LV_CUDA(cudaMemcpyAsync(h, out, sizeof(FitOut) * 4 * (size_t)n_y, cudaMemcpyDeviceToHost, stream));
   st = fit_status(ctx, stream);

@@ -176,8 +176,7 @@ struct GramSmem {
 
 // kGram: the Gram matrix and the flag, else the latency vector k.
 template <bool kGram>
-__device__ __forceinline__ void fit_rows(GramSmem &sm, const int64_t *__restrict__ feat,
-                                         const uint8_t *__restrict__ seg, int64_t nb, const double *__restrict__ y,
+__device__ __forceinline__ void fit_rows(GramSmem &sm, const int64_t *feat, const uint8_t *seg, int64_t nb, const double *__restrict__ y,
                                          int n_y, int k, FitAcc *__restrict__ partial, int *status) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int NE = fit_entries(n_y);
@@ -288,9 +287,11 @@ __device__ __forceinline__ void fit_rows(GramSmem &sm, const int64_t *__restrict
 }
 
 __global__ void __launch_bounds__(kGramThreads, 2)
-    k_fit_gram(const int64_t *__restrict__ feat, const uint8_t *__restrict__ seg, int64_t nb,
-               const double *__restrict__ y, int n_y, FitAcc *__restrict__ partial, int *status) {
+    k_fit_gram(const int64_t *feat, const uint8_t *seg, int64_t nb, const double *__restrict__ y, int n_y,
+               FitAcc *__restrict__ partial, int *status) {
   __shared__ GramSmem sm;
+  let_next();
+  wait_previous();
   if (blockIdx.y == 0)
     fit_rows<true>(sm, feat, seg, nb, y, n_y, 0, partial, status);
   else
@@ -304,8 +305,10 @@ __global__ void __launch_bounds__(kGramThreads, 2)
 // associative, so the exact result does not depend on the order; the flag
 // entries are ORed.
 constexpr int kFitRedThreads = 256;
-__global__ void __launch_bounds__(kFitRedThreads) k_fit_reduce(const FitAcc *__restrict__ partial, int n_cta,
-                                                               int n_ent, FitAcc *__restrict__ totals) {
+__global__ void __launch_bounds__(kFitRedThreads) k_fit_reduce(const FitAcc *partial, int n_cta, int n_ent,
+                                                               FitAcc *__restrict__ totals) {
+  let_next();
+  wait_previous();
   __shared__ FitAcc red[kFitRedThreads];
   const int ge = blockIdx.x;
   const bool is_flag = ge % (n_ent / 4) == n_ent / 4 - 1;
@@ -469,7 +472,8 @@ __device__ __forceinline__ dd dd_sub(dd x, dd y) { return dd_add(x, dd_neg(y)); 
 // solves to 0).  Bound by the latency of that chain (one warp, 22 us;
 // with a left-looking Cholesky factorisation, one lane on the pivot, 79).  Loops
 // stay rolled: the kernel runs once per fit, so its code is fetched cold.
-__global__ void __launch_bounds__(64) k_fit_solve(const FitAcc *__restrict__ totals, int n_y, FitOut *__restrict__ out) {
+__global__ void __launch_bounds__(64) k_fit_solve(const FitAcc *totals, int n_y, FitOut *__restrict__ out) {
+  wait_previous();
   __shared__ dd G[15], R[5], A[15], B[5], inv[5];
   __shared__ dd YY, SST;
   __shared__ double cf[5];

@@ -102,14 +102,12 @@ __device__ __forceinline__ void ten_add(const TenTab &tt, uint32_t u, uint32_t l
 }
 
 // Tenant contributions of a lane's four positive normal shares (d: their
-// doubles' words) in the common case, a valid tenant and a share in [2^-20, 2^-8 (1 -
-// 2^-21)) s (then q is whole and below 2^64 - 2^32, so a carry into its high
-// word does not wrap); go[k] is cleared otherwise.  (Shifts, and
-// not the hardware's conversion to a 64-bit integer: that runs at 1/64 rate,
-// and the shares' rounding needs one already.)  The four low
-// words' atomics are issued together, then the four high words', so that a lane
-// waits for two of them and not for eight; lanes with nothing to add use a word
-// of their own, so there is no branch.
+// doubles' words) in the common case, a valid tenant and a share in [2^-20, 2^-8
+// (1 - 2^-21)) s (then q is whole and below 2^64 - 2^32, so a carry into its
+// high word does not wrap); go[k] is cleared otherwise.  The four low words'
+// atomics are issued together, then the four high words', so that a lane waits
+// for two of them and not for eight; lanes with nothing to add use a word of
+// their own, so there is no branch.
 constexpr uint32_t kShareLo = (uint32_t)(1075 + kTenLsb) << 20, kShareHi = kShareLo + (12u << 20) - 1u;
 __device__ __forceinline__ void ten_add4(const TenTab &tt, bool *go, const uint32_t *u, const uint32_t *dlo,
                                          const uint32_t *dhi) {

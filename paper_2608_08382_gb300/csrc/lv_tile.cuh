@@ -107,6 +107,7 @@ __device__ __forceinline__ int64_t div_magic(int64_t x, uint64_t magic) {
 template <class V>
 __global__ void k_tile_bounds(const int64_t *__restrict__ off, int64_t n_batch, int64_t n_req, int64_t n_tiles,
                               uint64_t magic, V *__restrict__ part, int *status) {
+  let_next();
   int bad = 0;
   for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b <= n_batch;
        b += (int64_t)gridDim.x * blockDim.x) {
@@ -649,6 +650,7 @@ __global__ void __launch_bounds__(kTThreads, 1) k_tiles(const TileArgs a) {
   }
   if (tid == 0) ts.n_big = 0;
   __syncthreads();
+  wait_previous();
 
   WarpTile &wt = ts.tile[wid];
   const bool vec = (MODE & M_F32) ? ((uintptr_t)a.share32 & 15) == 0 : ((uintptr_t)a.share & 31) == 0;

@@ -32,6 +32,7 @@ struct CandP {
 
 // A pending request in a block of pairs.
 struct PendP {
+  uint4 V3[4];  // V's low three words
   i128 V[4];
   int32_t p, c, phase, slow;
   double Lu, Bu;  // admission: the request's tenant's running total and budget
@@ -94,6 +95,7 @@ __global__ void __launch_bounds__(kWiCandThreads) k_wi_cand_direct(ModelP mp, co
                                                                   const int32_t *__restrict__ ph,
                                                                   const int64_t *__restrict__ off, int64_t n_req,
                                                                   int64_t nc, CandP *__restrict__ out, int *status) {
+  let_next();
   __shared__ Sums red[kWiCandThreads / 32];
   const int64_t b = blockIdx.x;
   const int tid = threadIdx.x;
@@ -174,6 +176,15 @@ __device__ __forceinline__ double round_fix(i128 V, int E) {
   return fix_to_double(V, E).d;
 }
 
+// x + V, both below 2^95 and x at least 2^64, rounded (ebase as round_top's).
+__device__ __forceinline__ double sum_round(const uint32_t *x, const uint4 &V, uint32_t ebase) {
+  uint32_t v0, v1, v2;
+  asm("add.cc.u32 %0, %3, %6;\n\taddc.cc.u32 %1, %4, %7;\n\taddc.u32 %2, %5, %8;"
+      : "=r"(v0), "=r"(v1), "=r"(v2)
+      : "r"(x[0]), "r"(x[1]), "r"(x[2]), "r"(V.x), "r"(V.y), "r"(V.z));
+  return round_top(v0, v1, v2, ebase);
+}
+
 // Left-to-right fp64 evaluation of one pair (fp64 mode, or outside the exact range).
 __device__ __noinline__ void wi_pair_slow(const ModelP &mp, int s, int64_t s1, int64_t s2, int64_t s3, int64_t n1,
                                           int32_t p, int32_t c, double *T, double *share) {
@@ -198,7 +209,7 @@ constexpr int kWiRows = 32;      // pending requests per block, at most
 // the row only where the merged batch crosses the split or turns prefill), so a
 // pair reads one V from shared memory.  Bound by the stores: 16-17 B a pair
 // (4.2e6 pairs, 67 MB: 21.5 us, 24.4 with U and W read per pair).
-__global__ void __launch_bounds__(kWiThreads) k_wi_pairs(ModelP mp, const CandP *__restrict__ cand, int64_t nc,
+__global__ void __launch_bounds__(kWiThreads) k_wi_pairs(ModelP mp, const CandP *cand, int64_t nc,
                                                          const int32_t *__restrict__ p_new,
                                                          const int32_t *__restrict__ c_new,
                                                          const int32_t *__restrict__ ph_new, int64_t np,
@@ -226,6 +237,8 @@ __global__ void __launch_bounds__(kWiThreads) k_wi_pairs(ModelP mp, const CandP 
       V = add128(V, a2_times(f, (uint32_t)c));
     }
     sp[r].V[s] = V;
+    sp[r].V3[s] = make_uint4((uint32_t)V.lo, (uint32_t)(V.lo >> 32), (uint32_t)V.hi, 0u);
+    rslow |= V.hi >= (1ull << 31) ? 1 : 0;
     if (s == 0) {
       sp[r].p = p;
       sp[r].c = c;
@@ -245,6 +258,7 @@ __global__ void __launch_bounds__(kWiThreads) k_wi_pairs(ModelP mp, const CandP 
   }
   if (tid < 4) sE[tid] = mp.fx[tid].E;
   rslow = __syncthreads_or(rslow);
+  wait_previous();  // the candidates' kernel: the rows above do not need it
   const int64_t b = ((int64_t)blockIdx.x << lc) + (tid & ((1 << lc) - 1));
   if (b >= nc) return;
   const CandP *cb = cand + b;
@@ -253,30 +267,49 @@ __global__ void __launch_bounds__(kWiThreads) k_wi_pairs(ModelP mp, const CandP 
   int64_t o = (j0 + (tid >> lc)) * nc + b;
   const int64_t ostep = step * nc;
   if (!cb->slow && !rslow) {
-    // every pair of the block exact: no out-of-line call
-    int cur = -1, E = 0;
+    // every V of the block below 2^95 and p at most 2^24: with U and W in
+    // [2^64, 2^95), three words hold the sums and one rounding form does
+    const int32_t thr0 = (int32_t)clampi(sp0 - s1, INT32_MIN, INT32_MAX),
+                  thr1 = (int32_t)clampi(sp1 - s1, INT32_MIN, INT32_MAX);
     const int64_t slo_key = bound_key(adm.slo);
-    i128 U = mk128(0, 0), W = mk128(0, 0);
+    double *Tp = T_new ? T_new + o : nullptr, *Sp = share_new ? share_new + o : nullptr;
+    uint8_t *Ap = adm.admit ? adm.admit + o : nullptr;
+    int cur = -1;
+    uint32_t u[3] = {0u, 0u, 0u}, w[3] = {0u, 0u, 0u}, eb = 0u;
+    bool narrow = false;
 #pragma unroll 4
-    for (int r = tid >> lc; r < rows; r += step, o += ostep) {
-      const int phase = (prefill | sp[r].phase) ? 1 : 0;
-      const int s = phase * 2 + ((s1 + sp[r].p >= (phase ? sp1 : sp0)) ? 1 : 0);
+    for (int r = tid >> lc; r < rows; r += step) {
+      const int phase = prefill | sp[r].phase;
+      const int s = phase * 2 + (sp[r].p >= (phase ? thr1 : thr0) ? 1 : 0);
       if (s != cur) {
         cur = s;
-        U = cb->U[s];
-        W = cb->W[s];
-        E = sE[s];
+        const i128 U = cb->U[s], W = cb->W[s];
+        u[0] = (uint32_t)U.lo, u[1] = (uint32_t)(U.lo >> 32), u[2] = (uint32_t)U.hi;
+        w[0] = (uint32_t)W.lo, w[1] = (uint32_t)(W.lo >> 32), w[2] = (uint32_t)W.hi;
+        eb = (uint32_t)(sE[s] + 32) << 20;
+        narrow = U.hi - 1ull < (1ull << 31) - 1ull && W.hi - 1ull < (1ull << 31) - 1ull;
       }
-      const i128 V = sp[r].V[s];
-      const double T = round_fix(add128(U, V), E);
-      const double sh = round_fix(add128(W, V), E);
-      if (T_new) __stcs(T_new + o, T);
-      if (share_new) __stcs(share_new + o, sh);
+      const uint4 V = sp[r].V3[s];
+      double T = sum_round(u, V, eb), sh = sum_round(w, V, eb);
+      if (!narrow) {
+        T = round_fix(add128(cb->U[s], sp[r].V[s]), sE[s]);
+        sh = round_fix(add128(cb->W[s], sp[r].V[s]), sE[s]);
+      }
+      if (Tp) {
+        __stcs(Tp, T);
+        Tp += ostep;
+      }
+      if (Sp) {
+        __stcs(Sp, sh);
+        Sp += ostep;
+      }
       // comparisons as integers: with two fp64 ones per pair as well as the
       // addition, the fp64 pipe took longer than the stores (4.2e6 pairs: 52
-      // us a call).  A NaN sum has the largest key.
-      if (adm.admit)
-        adm.admit[o] = (order_key(__dadd_rn(sp[r].Lu, sh)) <= sp[r].Bk && order_key(T) <= slo_key) ? 1 : 0;
+      // us a call, 34 so).  A NaN sum has the largest key.
+      if (Ap) {
+        *Ap = (order_key(__dadd_rn(sp[r].Lu, sh)) <= sp[r].Bk && order_key(T) <= slo_key) ? 1 : 0;
+        Ap += ostep;
+      }
     }
     return;
   }
