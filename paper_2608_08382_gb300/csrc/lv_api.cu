@@ -1157,7 +1157,12 @@ lv_status lv_accuracy(lv_ctx *ctx, const double *y, const double *T, int64_t n, 
   static_assert(o_hist2 + 4 * kAccTargets * kSelBins <= o_rel, "accuracy scratch head");
   const size_t rel_bytes = ((size_t)n * sizeof(uint64_t) + 255) & ~(size_t)255;
   const size_t o_sorted = o_rel + rel_bytes, o_bucket = o_sorted + rel_bytes;
-  const size_t o_segs = o_bucket + sizeof(uint64_t) * kAccTargets * kSelBins * kAccBucket;
+  // buckets that hold a second-digit bin of the usual distributions: a bin that
+  // outgrows its bucket is ranked from every block's segment by one block,
+  // which took 0.3 of 0.54 ms on 8e6 samples with 64 places
+  int lb = kAccBucketLo;
+  while (lb < kAccBucketHi && ((int64_t)1 << lb) * 32768 < n) ++lb;
+  const size_t o_segs = o_bucket + (sizeof(uint64_t) * kAccTargets * kSelBins << lb);
   const size_t o_part = o_segs + ((sizeof(uint64_t) * 2 * kAccTargets * (size_t)blocks + 255) & ~(size_t)255);
   const size_t need = o_part + sizeof(uint64_t) * kAccPartW * (size_t)blocks;
   if (need > ctx->acc_cap) {
@@ -1177,6 +1182,7 @@ lv_status lv_accuracy(lv_ctx *ctx, const double *y, const double *T, int64_t n, 
   a.relbits = reinterpret_cast<uint64_t *>(base + o_rel);
   a.cand = reinterpret_cast<uint64_t *>(base + o_sorted);
   a.bucket = reinterpret_cast<uint64_t *>(base + o_bucket);
+  a.lb = lb;
   a.segs = reinterpret_cast<uint64_t *>(base + o_segs);
   a.part = reinterpret_cast<uint64_t *>(base + o_part);
   a.res = ctx->hd_acc;

@@ -40,6 +40,10 @@
 //           first samples in a bucket; the block of each target then picks its
 //           second digit and ranks the bin's samples (from the bucket, or the
 //           blocks' segments when the bin outgrew it).
+// On 2e6 samples the call takes 79 us (93 with an emulated 64-bit reciprocal in
+// the division), 240 us on 8e6 (558 before the buckets grew with the count):
+// the instructions of the exact pass, then the barriers, about 23 us at
+// any size; the 32 MB of 2e6 samples take 5 us at the copy rate.
 #pragma once
 
 #include <cstdint>
@@ -56,7 +60,7 @@ constexpr int kAccWords = 14;   // the exact sums of one block
 constexpr int kSelBits = 11;    // radix digit
 constexpr int kSelBins = 1 << kSelBits;
 constexpr int kAccStage = 8192;  // a block's rel values kept in shared memory when its range fits
-constexpr int kAccBucket = 64;   // samples kept per second-digit bin
+constexpr int kAccBucketLo = 6, kAccBucketHi = 10;  // lg of the samples kept per second-digit bin
 constexpr int kAccGrid = 78;  // wide grid: S = kAccGrid - Emax puts every |v 2^S| below 2^79
 // Range of Emax for the exact path: within it the definition's own fp64
 // arithmetic (squared deviations, their products in r2_corr) neither overflows
@@ -81,7 +85,8 @@ struct AccArgs {
   uint64_t *relbits;          // n rel bit patterns (all ones: not a sample)
   uint64_t *cand;             // each block's samples sorted by first digit within its range, n patterns
   uint64_t *segs;             // per block and first-digit slot: offset and length of its segment
-  uint64_t *bucket;           // kAccTargets * kSelBins buckets of kAccBucket patterns
+  uint64_t *bucket;           // kAccTargets * kSelBins buckets of 2^lb patterns
+  int lb;
   uint64_t *part;             // kAccPartW words per block
   double *res;                // results (host memory, mapped): 8 sums, 3 patterns, error word
   int *err;                   // the barrier's error word (device memory)
@@ -183,43 +188,29 @@ __device__ __forceinline__ float rcp_approx(float x) {
 }
 
 // floor(Ma 2^54 / B) for 2^52 <= Ma, B < 2^53 (so the quotient lies in
-// [2^53, 2^55)), and whether the remainder is non-zero.  Through a 64-bit
-// reciprocal V ~ 2^116 / B: a single-precision reciprocal of B's top 24 bits
-// (relative error about 2^-21) refined by two Newton-Raphson steps
-// V += V (2^116 - B V) / 2^116, each squaring the error, to within a few units
-// of 2^116 / B; then the quotient estimate Ma V / 2^62, which lies at most one
-// below the true quotient, settled on the exact remainder Ma 2^54 - Q B
-// (below 2^64 in magnitude, so formed modulo 2^64).  The products run on the
-// multiply-add pipe.
+// [2^53, 2^55)), and whether the remainder is non-zero.  Long division in
+// three digits of 18 bits, each from single-precision arithmetic on the leading
+// bits and settled by an exact remainder: with Bt = B >> 29 and v = R >> 22, the
+// digit floor(R 2^18 / B) is about v 2^11 / Bt.  The truncations, the reciprocal
+// (one ulp) and the roundings err by less than 2^-21.1; the reciprocal is taken
+// 2^-20 low, so that a digit is never too large and at most 1.7 too small:
+// every remainder R 2^18 - q B lies in [0, 1.7 B) (formed modulo 2^64), v fits 32
+// bits, and one subtraction settles the last.  (With a 64-bit reciprocal
+// refined by two Newton steps, whose products are emulated 64-bit ones, about
+// 70 instructions more.)
 __device__ __forceinline__ uint64_t acc_div54(uint64_t Ma, uint64_t B, bool &rem_nz) {
-  // B >> 29 lies in [2^23, 2^24): its float is exponent 150 and the low 23 bits
-  const uint32_t fb = __float_as_uint(rcp_approx(__uint_as_float((150u << 23) | ((uint32_t)(B >> 29) & 0x7FFFFFu))));
-  const int sh = (int)(fb >> 23) - 63;  // the reciprocal lies in (2^-24, 2^-23]: 40 or 41
-  const uint64_t mf = (uint64_t)((fb & 0x7FFFFFu) | 0x800000u);
-  uint64_t V = sh >= 41 ? ~0ull : mf << sh;  // 2^-23 exactly would give 2^64
-  {
-    const __int128 E = (__int128)(((u128)1 << 116) - (u128)B * V);  // |E| < 2^96
-    const int64_t Ep = (int64_t)(E >> 52);
-    const uint64_t c = __umul64hi(V, (uint64_t)(Ep < 0 ? -Ep : Ep));
-    V = Ep < 0 ? V - c : V + c;
-  }
-  {
-    const __int128 E = (__int128)(((u128)1 << 116) - (u128)B * V);  // |E| < 2^75
-    const int64_t Ep = (int64_t)(E >> 12);
-    const uint64_t c = __umul64hi(V, (uint64_t)(Ep < 0 ? -Ep : Ep)) >> 40;
-    V = Ep < 0 ? V - c : V + c;
-  }
-  uint64_t Q = (__umul64hi(Ma, V) << 2) | ((Ma * V) >> 62);
-  uint64_t R = (Ma << 54) - Q * B;
-  if ((int64_t)R < 0) {  // not reached when the bounds above hold
-    R += B;
-    --Q;
+  // Bt lies in [2^23, 2^24): its float is exponent 150 and the low 23 bits
+  const float bt = __uint_as_float((150u << 23) | ((uint32_t)(B >> 29) & 0x7FFFFFu));
+  const float k = rcp_approx(bt) * (2048.0f * (1.0f - 0x1p-20f));
+  const uint32_t b0 = (uint32_t)B, b1 = (uint32_t)(B >> 32);
+  uint64_t R = Ma, Q = 0;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const uint32_t q = __float2uint_rz(__fmul_rn(__uint2float_rn((uint32_t)(R >> 22)), k));
+    R = (R << 18) - ((uint64_t)q * b0 + ((uint64_t)(q * b1) << 32));
+    Q = (Q << 18) + q;
   }
   if (R >= B) {
-    R -= B;
-    ++Q;
-  }
-  if (R >= B) {  // not reached when the bounds above hold
     R -= B;
     ++Q;
   }
@@ -298,17 +289,15 @@ __device__ __forceinline__ uint64_t acc_rel_bits64(uint64_t d, uint64_t My, int 
 }
 
 __device__ __forceinline__ void add128w(uint64_t *a, u128 x) {
-  const u128 s = (((u128)a[1] << 64) | a[0]) + x;
-  a[0] = (uint64_t)s;
-  a[1] = (uint64_t)(s >> 64);
+  asm("add.cc.u64 %0, %0, %2;\n\taddc.u64 %1, %1, %3;"
+      : "+l"(a[0]), "+l"(a[1])
+      : "l"((uint64_t)x), "l"((uint64_t)(x >> 64)));
 }
 
 __device__ __forceinline__ void add192w(uint64_t *a, uint64_t w0, uint64_t w1, uint64_t w2) {
-  u128 s = (u128)a[0] + w0;
-  a[0] = (uint64_t)s;
-  s = (u128)a[1] + w1 + (uint64_t)(s >> 64);
-  a[1] = (uint64_t)s;
-  a[2] += w2 + (uint64_t)(s >> 64);
+  asm("add.cc.u64 %0, %0, %3;\n\taddc.cc.u64 %1, %1, %4;\n\taddc.u64 %2, %2, %5;"
+      : "+l"(a[0]), "+l"(a[1]), "+l"(a[2])
+      : "l"(w0), "l"(w1), "l"(w2));
 }
 
 // a += X^2 for X < 2^81 (a: 192 bits).
@@ -321,7 +310,10 @@ __device__ __forceinline__ void add_sq(uint64_t *a, u128 X) {
 
 // a += x^2 for x < 2^64 (a: 192 bits).
 __device__ __forceinline__ void add_sq64(uint64_t *a, uint64_t x) {
-  add192w(a, x * x, __umul64hi(x, x), 0ull);
+  const uint32_t l = (uint32_t)x, h = (uint32_t)(x >> 32);
+  const uint64_t c = (uint64_t)l * h;  // x^2 = l^2 + c 2^33 + h^2 2^64
+  add192w(a, (uint64_t)l * l, (uint64_t)h * h, 0ull);
+  add192w(a, c << 33, c >> 31, 0ull);
 }
 
 // The exact sums: [0] count, [1..2] sum Y, [3..4] sum T (two's complement),
@@ -1148,7 +1140,7 @@ __global__ void __launch_bounds__(kAccBlock) k_acc(AccArgs a) {
 
   // ---- second digit: each block histograms the next 11 bits of its samples
   // in the targets' first-digit bins (its sorted segments), keeping each
-  // bin's first kAccBucket samples in a bucket and publishing where its
+  // bin's first 2^lb samples in a bucket and publishing where its
   // segments lie
   {
     const int lo2 = L.shift - kSelBits;
@@ -1156,11 +1148,11 @@ __global__ void __launch_bounds__(kAccBlock) k_acc(AccArgs a) {
       if (L.slot[t] != t || L.pf[t] == ~0ull) continue;  // the same in every block
       const int b = L.bin[t];
       unsigned int *h2 = a.hist2 + t * kSelBins;
-      uint64_t *bk = a.bucket + (int64_t)t * kSelBins * kAccBucket;
+      uint64_t *bk = a.bucket + ((int64_t)t * kSelBins << a.lb);
       acc_for_segment(sorted + lo + bof1[b], (int)bh1[b], [&](uint64_t v) {
         const int d = (int)((v >> lo2) & (uint64_t)(kSelBins - 1));
         const unsigned int p = atomicAdd(h2 + d, 1u);
-        if (p < kAccBucket) bk[d * kAccBucket + p] = v;  // the bin's first samples, kept for the finish
+        if (p < (1u << a.lb)) bk[(d << a.lb) + p] = v;  // the bin's first samples, kept for the finish
       });
       if (tid == 0) {
         a.segs[2 * (blockIdx.x * kAccTargets + t)] = (uint64_t)(lo + bof1[b]);
@@ -1192,9 +1184,9 @@ __global__ void __launch_bounds__(kAccBlock) k_acc(AccArgs a) {
       }
       __syncthreads();
       const int cur = L.shift - kSelBits;
-      if (F.cnt[t] <= kAccBucket)
-        r = acc_finish(a.bucket + ((int64_t)s * kSelBins + (int64_t)(F.pf[t] & (kSelBins - 1))) * kAccBucket,
-                       F.cnt[t], F.pf[t], cur, F.rk[t], F.cnt[t], sh);
+      if (F.cnt[t] <= (1 << a.lb))
+        r = acc_finish(a.bucket + (((int64_t)s * kSelBins + (int64_t)(F.pf[t] & (kSelBins - 1))) << a.lb), F.cnt[t],
+                       F.pf[t], cur, F.rk[t], F.cnt[t], sh);
       else
         r = acc_finish_segs(a.segs, sorted, nb, s, F.pf[t], cur, F.rk[t], F.cnt[t], sh);
     }
