@@ -322,11 +322,11 @@ struct TilePlan {
   bool search;  // at most one tile per warp: the warps find the bounds
 };
 
-TilePlan plan_tiles(int64_t n_batch, int64_t n_req, int64_t warps) {
+TilePlan plan_tiles(int64_t n_batch, int64_t n_req, int64_t warps, int64_t d_max) {
   const int64_t units = kTW * n_batch + n_req;
-  const int64_t rounds = (units + warps * kTDMax - 1) / (warps * kTDMax);
+  const int64_t rounds = (units + warps * d_max - 1) / (warps * d_max);
   int64_t D = (units + warps * rounds - 1) / (warps * rounds);
-  D = std::min<int64_t>(kTDMax, std::max<int64_t>(kTDMin, (D + 7) & ~(int64_t)7));
+  D = std::min<int64_t>(d_max, std::max<int64_t>(kTDMin, (D + 7) & ~(int64_t)7));
   TilePlan p;
   p.n_tiles = (units + D - 1) / D;
   p.magic = UINT64_MAX / (uint64_t)D + 1;
@@ -351,7 +351,7 @@ lv_status tiles_occupancy(lv_ctx *ctx, size_t smem, int *per_sm) {
   }
   if (*per_sm) return LV_OK;
   LV_CUDA(cudaFuncSetAttribute(k_tiles<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)(sizeof(TSmem) + ((MODE & M_TEN) ? ten_table_bytes(kHotMax) : 0))));
+                               (int)(sizeof(TSmem<MODE>) + ((MODE & M_TEN) ? ten_table_bytes(kHotMax) : 0))));
   LV_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_tiles<MODE>, kTThreads, smem));
   if (*per_sm < 1) *per_sm = 1;
   if (ctx) {
@@ -382,12 +382,12 @@ lv_status ensure_bound(lv_ctx *ctx, int64_t n) {
 // has room for the tiles' bounds (bound_cap 32-bit entries).
 template <int MODE>
 lv_status run_tiles_mode(lv_ctx *ctx, int sms, TileArgs &a, void *bound, int64_t bound_cap, cudaStream_t stream) {
-  const size_t smem = sizeof(TSmem) + ((MODE & M_TEN) ? ten_table_bytes(kHotMax) : 0);
+  const size_t smem = sizeof(TSmem<MODE>) + ((MODE & M_TEN) ? ten_table_bytes(kHotMax) : 0);
   int per_sm = 0;
   lv_status st = tiles_occupancy<MODE>(ctx, smem, &per_sm);
   if (st != LV_OK) return st;
   const int64_t ctas = (int64_t)sms * per_sm;
-  const TilePlan plan = plan_tiles(a.n_batch, a.n_req, ctas * kTWarps);
+  const TilePlan plan = plan_tiles(a.n_batch, a.n_req, ctas * kTWarps, Geo<MODE>::kD);
   a.n_tiles = plan.n_tiles;
   a.D = plan.search ? plan.D : 0;
   if (!plan.search) {
@@ -1263,7 +1263,7 @@ namespace {
 
 constexpr int64_t kNoAllocMaxUnits = 65536 * 1024;  // n_batch + n_req
 // most tiles: every unit an empty batch, and a partial round of 32 warps on each of 256 SMs
-constexpr int64_t kNoAllocBounds = kTW * kNoAllocMaxUnits / kTDMax + 32 * 256 + 2;
+constexpr int64_t kNoAllocBounds = kTW * kNoAllocMaxUnits / Geo<M_ATTR>::kD + 32 * 256 + 2;
 constexpr size_t kNoAllocTabOffset = (sizeof(uint32_t) * (size_t)kNoAllocBounds + 255) & ~(size_t)255;
 constexpr size_t kNoAllocBytes = kNoAllocTabOffset + sizeof(KEntry) * 4 * (kKTableN + 1);
 // the size stated in include/llmvisor.h ("about 2.3 MB")

@@ -16,7 +16,7 @@
 //      common path is listed and worked off 32 at a time.
 // So a request costs about the same instructions whatever the batch sizes, and
 // no lane idles on a batch's remainder.  The requests are read twice, the
-// second time from L1 or L2.  A batch that reaches past a tile's kTCap requests
+// second time from L1 or L2.  A batch that reaches past a tile's requests
 // is walked by its warp alone, or, above kTAlone requests, by the whole CTA
 // after its tiles (a warp alone on a batch of 4,096 set the time of a small
 // input).  All sums are exact integers, so results do not depend on the
@@ -45,20 +45,29 @@ namespace lv {
 constexpr int kTThreads = 640;             // threads of a CTA, one CTA per SM (one tenant table)
 constexpr int kTWarps = kTThreads / 32;
 constexpr int kTW = 8;                     // merge positions a batch takes besides its requests
-constexpr int kTDMax = 1248;               // merge positions per tile, at most
 constexpr int kTDMin = 128;
-constexpr int kTCap = 1536;                // requests of a tile, at most
-constexpr int kTNb = kTDMax / kTW;         // batches of a tile, at most
-constexpr int kTRec = kTDMax / (kTW + 1) + 5;     // non-empty ones, and room to read past the last
-constexpr int kTBlocks = kTCap / 256 + 1;         // blocks of 256 requests, one more for a bound at the end
-constexpr int kTWords = kTCap / 32 + 1;
 constexpr int kTDense = 40;                // batches of fewer requests on average: a record per request in step 3
 constexpr int64_t kTAlone = 512;           // requests a warp walks alone
 constexpr int kTBigs = 64;                 // larger batches a CTA keeps for later
 constexpr int kTabN = 4096;                // batch sizes of the K table
 constexpr uint32_t kTSmall = 1u << 23;     // p and c of a tile on the common path are below this
-static_assert(kTCap % 256 == 0 && kTDMax + 3 < kTCap, "only a tile's last batch can reach past its requests");
-static_assert(kTCap <= kTabN, "a tile's batches are in the K table");
+
+// A tile's size.  The passes that write only batch features keep no records, so
+// their tiles can be twice as large and leave the L1 more.  2.57e8 requests take
+// 508 us (6.1 TB/s); a whole fit 766 us, 780 with the other passes' shape, 764
+// with 3,256 positions, 802 with 4,064, 788 with 24 warps, 792 with 16.
+template <int MODE>
+struct Geo {
+  static constexpr bool kAttr = (MODE & M_ATTR) != 0;
+  static constexpr int kD = kAttr ? 1248 : 2496;           // merge positions, at most
+  static constexpr int kCap = kAttr ? 1536 : 2560;         // requests, at most
+  static constexpr int kNb = kD / kTW;                     // batches, at most
+  static constexpr int kRec = kAttr ? kD / (kTW + 1) + 5 : 1;  // non-empty ones, and room to read past the last
+  static constexpr int kBlocks = kCap / 256 + 1;           // blocks of 256 requests, one more for a bound at the end
+  static constexpr int kWords = kAttr ? kCap / 32 + 1 : 1;
+  static_assert(kCap % 256 == 0 && kD + 3 < kCap, "only a tile's last batch can reach past its requests");
+  static_assert(!kAttr || kCap <= kTabN, "a tile's batches are in the K table");
+};
 
 // A batch's record: its share constant K + A1 + A3 (three words) and the
 // biased exponent of word 1's unit << 20; A2 (two words), n << 4 | fast << 3 |
@@ -70,20 +79,23 @@ struct TileRec {
 
 // One warp's tile.  pre: per 8 requests {S1, S2, S3 + prefills << 55} of the
 // requests before them in their 256; tot: each 256's totals.
+template <int MODE>
 struct WarpTile {
+  using G = Geo<MODE>;
   union {
-    alignas(16) uint4 pre[kTBlocks * 32];
-    uint16_t list[kTCap];  // step 3: requests off the common path
+    alignas(16) uint4 pre[G::kBlocks * 32];
+    uint16_t list[G::kCap];  // step 3: requests off the common path
   };
-  alignas(16) uint4 tot[kTBlocks];
-  alignas(16) TileRec rec[kTRec];
-  uint32_t bits[kTWords];  // head bits: a batch starts at this request
-  uint16_t rank[kTWords];  // heads before word w
+  alignas(16) uint4 tot[G::kBlocks];
+  alignas(16) TileRec rec[G::kRec];
+  uint32_t bits[G::kWords];  // head bits: a batch starts at this request
+  uint16_t rank[G::kWords];  // heads before word w
   uint32_t n_list;         // entries of list
 };
 
+template <int MODE>
 struct TSmem {
-  WarpTile tile[kTWarps];
+  WarpTile<MODE> tile[kTWarps];
   alignas(16) SegS seg[4];
   alignas(16) SegFix fx[4];
   float cf[4][5];                     // coefficients as float (fp32 variant)
@@ -238,7 +250,8 @@ __device__ __forceinline__ TSum sum_req8(const Req8 &r, int take) {
 
 // Prefixes of the tile's requests; true when some p or c is too large for
 // them (or negative) or some phase is not 0 or 1.
-__device__ __forceinline__ bool tile_prefix(WarpTile &wt, const TileSrc &src, int cnt, int lane) {
+template <int MODE>
+__device__ __forceinline__ bool tile_prefix(WarpTile<MODE> &wt, const TileSrc &src, int cnt, int lane) {
   uint32_t big = 0;
   int e = 8 * lane;
   Req8 nx = load_req8(src, e);
@@ -272,7 +285,8 @@ __device__ __forceinline__ bool tile_prefix(WarpTile &wt, const TileSrc &src, in
 }
 
 // Sums of the requests before index x of its 256.
-__device__ __forceinline__ TSum prefix_at(const WarpTile &wt, const TileSrc &src, int x) {
+template <int MODE>
+__device__ __forceinline__ TSum prefix_at(const WarpTile<MODE> &wt, const TileSrc &src, int x) {
   const uint4 v = wt.pre[x >> 3];
   TSum r{v.x, v.y, (uint64_t)v.z | ((uint64_t)v.w << 32)};
   if (x & 7) {
@@ -289,7 +303,7 @@ __device__ __forceinline__ TSum prefix_at(const WarpTile &wt, const TileSrc &src
 // Share constants of a batch of n requests in segment s; kTab: n is within the
 // K table (every staged batch).
 template <int MODE, bool kTab>
-__device__ __forceinline__ TileRec tile_record(const TileArgs &a, const TSmem &ts, int s, int64_t n) {
+__device__ __forceinline__ TileRec tile_record(const TileArgs &a, const TSmem<MODE> &ts, int s, int64_t n) {
   TileRec r;
   if (MODE & M_F32) {
     const float *k = ts.cf[s];
@@ -319,7 +333,7 @@ __device__ __forceinline__ TileRec tile_record(const TileArgs &a, const TSmem &t
 
 // A batch's outputs.
 template <int MODE>
-__device__ __forceinline__ void tile_emit(const TileArgs &a, const TSmem &ts, int64_t b, const BatchAgg &g, int s) {
+__device__ __forceinline__ void tile_emit(const TileArgs &a, const TSmem<MODE> &ts, int64_t b, const BatchAgg &g, int s) {
   if ((MODE & M_ATTR) && (MODE & M_F32)) {
     if (a.T32) {
       const float *k = ts.cf[s];
@@ -346,14 +360,15 @@ __device__ __forceinline__ void tile_emit(const TileArgs &a, const TSmem &ts, in
 
 // The CTA's tenant table, which follows TSmem (formed again in the functions
 // kept out of line, so that the loops hold it in fewer registers).
-__device__ __forceinline__ TenTab tile_table(const TileArgs &a, const TSmem &ts) {
+template <int MODE>
+__device__ __forceinline__ TenTab tile_table(const TileArgs &a, const TSmem<MODE> &ts) {
   return ten_table(reinterpret_cast<const uint32_t *>(&ts + 1), kHotMax, a.H, a.n_tenants, a.ten_pend);
 }
 
 // The general path of one request.  Out of line: the fast path leaves it the
 // rare ones (fp64 mode, values out of range).
 template <int MODE>
-__device__ __noinline__ void tile_slow(const TileArgs &a, const TSmem &ts, const TileRec &rec, int64_t n, int64_t i,
+__device__ __noinline__ void tile_slow(const TileArgs &a, const TSmem<MODE> &ts, const TileRec &rec, int64_t n, int64_t i,
                                        int32_t p, int32_t c, int32_t u) {
   const int s = (int)(rec.a.z & 3u);
   const bool slow = (rec.a.z & 4u) != 0u;
@@ -415,7 +430,7 @@ __device__ __forceinline__ void store4(double *p, const double *d) {
 
 // One request through the fast path where it applies, else the general one.
 template <int MODE>
-__device__ __forceinline__ bool tile_one(const TileArgs &a, const TenTab &tt, const TSmem &ts, const TileRec &rec,
+__device__ __forceinline__ bool tile_one(const TileArgs &a, const TenTab &tt, const TSmem<MODE> &ts, const TileRec &rec,
                                          int64_t n, int64_t i, int32_t p, int32_t c, int32_t u, double *d) {
   bool ok = (MODE & M_FIX) && tile_share(ts.seg, rec, p, c, d);
   if (MODE & M_TEN)
@@ -442,15 +457,16 @@ __device__ __forceinline__ float tile_one_f32(const TileArgs &a, const TenTab &t
 }
 
 // The record of the request at index e; before the tile's first batch, the first.
-__device__ __forceinline__ int tile_rank(const WarpTile &wt, int e) {
+template <int MODE>
+__device__ __forceinline__ int tile_rank(const WarpTile<MODE> &wt, int e) {
   const int r = (int)wt.rank[e >> 5] + __popc(wt.bits[e >> 5] & ((2u << (e & 31)) - 1u));
-  return max(min(r, kTRec) - 1, 0);
+  return max(min(r, Geo<MODE>::kRec) - 1, 0);
 }
 
 // The tile's n listed requests, one per lane: prefills, tenants and values off
 // the common path, with every lane busy.
 template <int MODE>
-__device__ __forceinline__ void tile_rest(const TileArgs &a, const TenTab &tt, const TSmem &ts, const WarpTile &wt,
+__device__ __forceinline__ void tile_rest(const TileArgs &a, const TenTab &tt, const TSmem<MODE> &ts, const WarpTile<MODE> &wt,
                                           const TileSrc &src, int64_t rbase, int n, int lane) {
   __syncwarp();
   int bad = 0;
@@ -479,7 +495,7 @@ __device__ __forceinline__ void tile_rest(const TileArgs &a, const TenTab &tt, c
 // them goes to the list.  vec: the share array allows 32-byte (fp32: 16-byte)
 // stores.
 template <int MODE, bool kPer>
-__device__ __forceinline__ void tile_shares(const TileArgs &a, const TenTab &tt, const TSmem &ts, WarpTile &wt,
+__device__ __forceinline__ void tile_shares(const TileArgs &a, const TenTab &tt, const TSmem<MODE> &ts, WarpTile<MODE> &wt,
                                             const TileSrc &src, int64_t rbase, int first, int cnt, bool vec,
                                             int lane) {
   constexpr bool kTen = (MODE & M_TEN) != 0, kF32 = (MODE & M_F32) != 0;
@@ -508,7 +524,7 @@ __device__ __forceinline__ void tile_shares(const TileArgs &a, const TenTab &tt,
     const uint32_t hb = (word >> sh) & 14u;
     const uint32_t run = kPer ? vm : vm & ((hb & (0u - hb)) - 1u);  // no head: all four
     // record of the first request; -1 before the tile's first batch
-    const int r0 = min((int)wt.rank[b / 32 + (lane >> 3)] + __popc(word & ((2u << sh) - 1u)), kTRec - 4) - 1;
+    const int r0 = min((int)wt.rank[b / 32 + (lane >> 3)] + __popc(word & ((2u << sh) - 1u)), Geo<MODE>::kRec - 4) - 1;
     TileRec rec = wt.rec[max(r0, 0)];
     bool go[4];
     uint32_t dlo[4], dhi[4];
@@ -575,7 +591,7 @@ __device__ __forceinline__ void tile_shares(const TileArgs &a, const TenTab &tt,
 // One batch walked by `kThreads` threads (a warp, or the CTA) from global
 // memory: sums, then a strided share pass.
 template <int MODE, int kThreads>
-__device__ __noinline__ void walk_batch(const TileArgs &a, TSmem &ts, int64_t b, int64_t r0, int64_t n) {
+__device__ __noinline__ void walk_batch(const TileArgs &a, TSmem<MODE> &ts, int64_t b, int64_t r0, int64_t n) {
   const TenTab tt = tile_table(a, ts);
   const int tid = kThreads == 32 ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
   int bad = 0;
@@ -632,12 +648,12 @@ __device__ __noinline__ void walk_batch(const TileArgs &a, TSmem &ts, int64_t b,
 template <int MODE>
 __global__ void __launch_bounds__(kTThreads, 1) k_tiles(const TileArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  TSmem &ts = *reinterpret_cast<TSmem *>(smem_raw);
+  TSmem<MODE> &ts = *reinterpret_cast<TSmem<MODE> *>(smem_raw);
   constexpr bool kTen = (MODE & M_TEN) != 0;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   int bad = 0;
 
-  uint32_t *tw = reinterpret_cast<uint32_t *>(smem_raw + sizeof(TSmem));
+  uint32_t *tw = reinterpret_cast<uint32_t *>(smem_raw + sizeof(TSmem<MODE>));
   TenTab tt{};
   if (kTen) {
     tt = tile_table(a, ts);
@@ -652,7 +668,7 @@ __global__ void __launch_bounds__(kTThreads, 1) k_tiles(const TileArgs a) {
   __syncthreads();
   wait_previous();
 
-  WarpTile &wt = ts.tile[wid];
+  WarpTile<MODE> &wt = ts.tile[wid];
   const bool vec = (MODE & M_F32) ? ((uintptr_t)a.share32 & 15) == 0 : ((uintptr_t)a.share & 31) == 0;
   // tile t's batches [b0, b1) and requests [r0, r1) are fetched while the tile
   // before it is worked on
@@ -685,17 +701,17 @@ __global__ void __launch_bounds__(kTThreads, 1) k_tiles(const TileArgs a) {
       n0 = tile_bound(a, tn);
       n1 = tile_bound(a, tn + 1);
     }
-    if (b1 - b0 > kTNb) {
-      b1 = b0 + kTNb;  // invalid offsets
+    if (b1 - b0 > Geo<MODE>::kNb) {
+      b1 = b0 + Geo<MODE>::kNb;  // invalid offsets
       bad = 1;
     }
     const int nb = (int)(b1 - b0);
     const int64_t rbase = r0 & ~(int64_t)3;
     int64_t off0 = lane <= nb ? a.off[b0 + lane] : 0;  // the first round's offsets
-    if (r1 - rbase > kTCap) {
+    if (r1 - rbase > Geo<MODE>::kCap) {
       // the last batch reaches too far: the tile's requests end at its start
       r1 = nb > 0 ? clampi(a.off[b1 - 1], r0, a.n_req) : r0;
-      if (r1 - rbase > kTCap) r1 = rbase + kTCap;  // invalid offsets
+      if (r1 - rbase > Geo<MODE>::kCap) r1 = rbase + Geo<MODE>::kCap;  // invalid offsets
     }
     const int cnt = (int)(r1 - rbase), first = (int)(r0 - rbase);
     const TileSrc src{a.p + rbase, a.c + rbase, a.ph + rbase, kTen ? a.ten + rbase : nullptr,
@@ -703,7 +719,7 @@ __global__ void __launch_bounds__(kTThreads, 1) k_tiles(const TileArgs a) {
 
     // 1. prefixes
     if (MODE & M_ATTR) {
-      for (int i = lane; i < kTWords; i += 32) {
+      for (int i = lane; i < Geo<MODE>::kWords; i += 32) {
         wt.bits[i] = 0;
         if (i == 0) {
           wt.rank[0] = 0;
@@ -754,7 +770,7 @@ __global__ void __launch_bounds__(kTThreads, 1) k_tiles(const TileArgs a) {
         const BatchAgg g{s1, s2, s3, n, f > 0};
         const int sg = segment_of(a.mp, g);
         const int rank = before + __popc(ne & ((1u << lane) - 1u));
-        if ((MODE & M_ATTR) && n > 0 && rank < kTRec) {
+        if ((MODE & M_ATTR) && n > 0 && rank < Geo<MODE>::kRec) {
           wt.rec[rank] = tile_record<MODE, true>(a, ts, sg, n);
           atomicOr(&wt.bits[x >> 5], 1u << (x & 31));
           for (int w = (x >> 5) + 1; w <= (x1 >> 5); ++w) wt.rank[w] = (uint16_t)(rank + 1);
@@ -769,8 +785,7 @@ __global__ void __launch_bounds__(kTThreads, 1) k_tiles(const TileArgs a) {
     nr1 = clampi(nr1, nr0, a.n_req);
 
     // 3. requests
-    if ((MODE & M_ATTR) && !wide && (kTen || a.share || a.share32))
-{
+    if ((MODE & M_ATTR) && !wide && (kTen || a.share || a.share32)) {
       if (!(MODE & (M_FIX | M_F32)) || before * kTDense <= cnt)
         tile_shares<MODE, false>(a, tt, ts, wt, src, rbase, first, cnt, vec, lane);
       else

@@ -76,3 +76,27 @@ def test_features_match_attribution_sums(lv, ctx):
     assert ctx.status() == lv.LV_OK
     feat, seg = oracle.batch_features(w.offsets, w.p, w.c, w.phase, w.split)
     assert np.array_equal(bf.cpu().numpy(), feat) and np.array_equal(bs.cpu().numpy(), seg)
+
+
+@pytest.mark.parametrize("lo,hi,n,cut", [(0, 1, 1_200_000, 1), (1, 40, 300_000, 0), (2470, 2500, 4000, 3),
+                                         (2548, 2566, 3500, 1), (3000, 6000, 60, 0)])
+def test_feature_sizes_around_the_tile(lv, ctx, lo, hi, n, cut):
+    """The feature pass has tiles of its own: exact sums at the edges of their positions and
+    requests (inputs of more than 7.6e6 positions, so that the tiles have their full size)."""
+    import torch
+    rng = np.random.default_rng(100 * hi + cut)
+    sizes = rng.integers(lo, hi + 1, n)
+    sizes[-1] = 8
+    sizes[-1] += (cut - int(sizes.sum())) % 4
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    m = int(off[-1])
+    ph = (rng.random(m) < 0.002).astype(np.int32)
+    p, c = np.where(ph == 1, rng.integers(1, 8192, m), 1).astype(np.int32), rng.integers(0, 1 << 17, m).astype(np.int32)
+    coef = np.ones((2, 2, 5))
+    model = lv.make_model(coef, (256, 300))
+    feat = torch.full((5, n), -1, dtype=torch.int64, device="cuda")
+    seg = torch.full((n,), 9, dtype=torch.uint8, device="cuda")
+    lv.lv_features(ctx, lv.batches_to_device(p, c, ph, off), model=model, batch_feat=feat, batch_seg=seg)
+    assert ctx.status() == lv.LV_OK
+    want, want_seg = oracle.batch_features(off, p, c, ph, (256, 300))
+    assert np.array_equal(feat.cpu().numpy(), want) and np.array_equal(seg.cpu().numpy(), want_seg)
