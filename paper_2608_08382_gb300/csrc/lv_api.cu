@@ -21,6 +21,15 @@
 
 using namespace lv;
 
+// A fit's results as its last kernel writes them.
+struct FitHost {
+  union {
+    FitOut out[4 * kFitMaxY];
+    VtcOut vtc[kFitMaxY];
+  };
+  int status;
+};
+
 struct lv_ctx {
   int device = 0;
   int sms = 0;
@@ -40,7 +49,7 @@ struct lv_ctx {
   cudaEvent_t ev_built = nullptr;
   cudaEvent_t ev_used = nullptr;
   cudaStream_t ktab_stream = nullptr;
-  void *d_fit = nullptr;      // fit partials + solve output
+  void *d_fit = nullptr;      // fit partials and totals, the batches' sums
   size_t fit_cap = 0;
   std::vector<std::pair<uint64_t, int>> occ;  // (mode << 32 | dynamic smem) -> k_tiles CTAs per SM
   void *d_wi = nullptr;       // what-if per-candidate / per-pending tables
@@ -49,6 +58,8 @@ struct lv_ctx {
   size_t acc_cap = 0;
   bool ten_attr = false;      // k_tenant_acc's shared-memory limit is set
   int acc_occ = 0;            // CTAs per SM of the accuracy kernel (0: not yet queried)
+  FitHost *h_fit = nullptr;   // a fit's results and status: pinned host memory the kernels write (mapped)
+  FitHost *hd_fit = nullptr;
   double *h_acc = nullptr;    // accuracy results: pinned host memory the kernel writes (mapped)
   double *hd_acc = nullptr;   // its device address
   void *d_probe = nullptr;    // barrier self-test: arrivals, generation, error word
@@ -535,21 +546,37 @@ lv_status run_attr(lv_ctx *ctx, TileArgs &a, int mode, lv_tenant_acc *acc, cudaS
   return acc && !a.ten_state ? fold_tenants(ctx, acc, stream) : LV_OK;
 }
 
+// Pinned host memory that kernels write, allocated at its first use; *dev: its
+// device address.
+template <class T>
+lv_status map_host(T **host, T **dev, size_t bytes) {
+  if (*host) return LV_OK;
+  void *h = nullptr, *d = nullptr;
+  if (cudaHostAlloc(&h, bytes, cudaHostAllocMapped) != cudaSuccess) return LV_ENOMEM;
+  if (cudaHostGetDevicePointer(&d, h, 0) != cudaSuccess) {
+    cudaFreeHost(h);
+    return LV_ECUDA;
+  }
+  *host = static_cast<T *>(h);
+  *dev = static_cast<T *>(d);
+  return LV_OK;
+}
+
 // The exact pass of lv_fit and lv_fit_vtc: per-CTA partials of the fit
-// statistics, reduced into totals[4 * NE]; *out points at room for the solves'
-// outputs (4 * kFitMaxY FitOut).
+// statistics, reduced into totals[4 * NE].
 lv_status fit_pass(lv_ctx *ctx, const lv_batches *b, const double *y, int32_t n_y, const int64_t split[2],
-                   cudaStream_t stream, FitAcc **totals_out, FitOut **out_out) {
+                   cudaStream_t stream, FitAcc **totals_out) {
   lv_status st = check_batches(b, false);
   if (st != LV_OK) return st;
   if (b->n_batch > 0 && (!y || !aligned(y, 8))) return LV_EINVAL;
-  // scratch: per-CTA partials, totals, solve output, each batch's sums and segment
+  st = map_host(&ctx->h_fit, &ctx->hd_fit, sizeof(FitHost));
+  if (st != LV_OK) return st;
+  // scratch: per-CTA partials, totals, each batch's sums and segment
   const int NE = fit_entries(n_y), n_ent = 4 * NE;
   const int rows = std::max(1, 2 * ctx->sms / (1 + n_y));  // two CTAs per SM over the kinds of entry
   const size_t nb = (size_t)b->n_batch;
   const size_t o_tot = ((size_t)rows * n_ent * sizeof(FitAcc) + 255) & ~(size_t)255;
-  const size_t o_out = (o_tot + (size_t)n_ent * sizeof(FitAcc) + 255) & ~(size_t)255;
-  const size_t o_feat = (o_out + sizeof(FitOut) * 4 * kFitMaxY + 255) & ~(size_t)255;
+  const size_t o_feat = (o_tot + (size_t)n_ent * sizeof(FitAcc) + 255) & ~(size_t)255;
   const size_t o_seg = o_feat + 4 * sizeof(int64_t) * nb;
   const size_t need = o_seg + nb;
   if (need > ctx->fit_cap) {
@@ -563,7 +590,6 @@ lv_status fit_pass(lv_ctx *ctx, const lv_batches *b, const double *y, int32_t n_
   unsigned char *base = static_cast<unsigned char *>(ctx->d_fit);
   FitAcc *partial = reinterpret_cast<FitAcc *>(base);
   FitAcc *totals = reinterpret_cast<FitAcc *>(base + o_tot);
-  FitOut *out = reinterpret_cast<FitOut *>(base + o_out);
   int64_t *feat = reinterpret_cast<int64_t *>(base + o_feat);
   uint8_t *seg = base + o_seg;
 
@@ -587,16 +613,15 @@ lv_status fit_pass(lv_ctx *ctx, const lv_batches *b, const double *y, int32_t n_
   st = launch_after(k_fit_reduce, n_ent, kFitRedThreads, 0, stream, partial, rows, n_ent, totals);
   if (st != LV_OK) return st;
   *totals_out = totals;
-  *out_out = out;
   return LV_OK;
 }
 
-// Reads and clears the sticky status after a synchronous fit (syncs `stream`).
+// The sticky status that a synchronous fit's last kernel handed over (syncs
+// `stream`).  It and the results come through mapped host memory: two copies
+// and a memset behind the kernels took about 20 us of a call.
 lv_status fit_status(lv_ctx *ctx, cudaStream_t stream) {
-  int hs = 0;
-  LV_CUDA(cudaMemcpyAsync(&hs, ctx->d_status, sizeof(int), cudaMemcpyDeviceToHost, stream));
-  LV_CUDA(cudaMemsetAsync(ctx->d_status, 0, sizeof(int), stream));
   LV_CUDA(cudaStreamSynchronize(stream));
+  const int hs = ctx->h_fit->status;
   if (hs & kStatusData) return LV_EDATA;
   if (hs & kStatusOverflow) return LV_EOVERFLOW;
   return LV_OK;
@@ -768,6 +793,7 @@ void lv_ctx_destroy(lv_ctx *ctx) {
   if (ctx->d_fit) cudaFree(ctx->d_fit);
   if (ctx->d_wi) cudaFree(ctx->d_wi);
   if (ctx->d_acc) cudaFree(ctx->d_acc);
+  if (ctx->h_fit) cudaFreeHost(ctx->h_fit);
   if (ctx->h_acc) cudaFreeHost(ctx->h_acc);
   if (ctx->d_probe) cudaFree(ctx->d_probe);
   if (ctx->ev_built) cudaEventDestroy(ctx->ev_built);
@@ -1059,15 +1085,14 @@ lv_status lv_fit(lv_ctx *ctx, const lv_batches *b, const double *y, int32_t n_y,
     if (inout[k].split[0] != inout[0].split[0] || inout[k].split[1] != inout[0].split[1]) return LV_EINVAL;
   cudaStream_t stream = (cudaStream_t)stream_;
   FitAcc *totals = nullptr;
-  FitOut *out = nullptr;
-  lv_status st = fit_pass(ctx, b, y, n_y, inout[0].split, stream, &totals, &out);
+  lv_status st = fit_pass(ctx, b, y, n_y, inout[0].split, stream, &totals);
   if (st != LV_OK) return st;
-  st = launch_after(k_fit_solve, 4 * kFitMaxY, 64, 0, stream, totals, n_y, out);
+  st = launch_after(k_fit_solve, 4 * kFitMaxY, 64, 0, stream, totals, n_y, ctx->hd_fit->out, ctx->d_status,
+                    &ctx->hd_fit->status);
   if (st != LV_OK) return st;
-  FitOut h[4 * kFitMaxY];
-  LV_CUDA(cudaMemcpyAsync(h, out, sizeof(FitOut) * 4 * (size_t)n_y, cudaMemcpyDeviceToHost, stream));
   st = fit_status(ctx, stream);
   if (st != LV_OK) return st;
+  const FitOut *h = ctx->h_fit->out;
   for (int k = 0; k < n_y; ++k) {
     for (int g = 0; g < 4; ++g) {
       const FitOut &o = h[k * 4 + g];
@@ -1096,18 +1121,14 @@ lv_status lv_fit_vtc(lv_ctx *ctx, const lv_batches *b, const double *y, int32_t 
   if (!ctx || !coef || !status || n_y < 1 || n_y > kFitMaxY) return LV_EINVAL;
   cudaStream_t stream = (cudaStream_t)stream_;
   FitAcc *totals = nullptr;
-  FitOut *out = nullptr;
   const int64_t split[2] = {0, 0};  // the groups do not matter: the line pools all four
-  lv_status st = fit_pass(ctx, b, y, n_y, split, stream, &totals, &out);
+  lv_status st = fit_pass(ctx, b, y, n_y, split, stream, &totals);
   if (st != LV_OK) return st;
-  static_assert(sizeof(VtcOut) * kFitMaxY <= sizeof(FitOut) * 4 * kFitMaxY, "VTC output fits the solve area");
-  VtcOut *vo = reinterpret_cast<VtcOut *>(out);
-  k_vtc_solve<<<1, 32, 0, stream>>>(totals, n_y, vo);
+  k_vtc_solve<<<1, 32, 0, stream>>>(totals, n_y, ctx->hd_fit->vtc, ctx->d_status, &ctx->hd_fit->status);
   LV_CUDA(cudaGetLastError());
-  VtcOut h[kFitMaxY];
-  LV_CUDA(cudaMemcpyAsync(h, vo, sizeof(VtcOut) * (size_t)n_y, cudaMemcpyDeviceToHost, stream));
   st = fit_status(ctx, stream);
   if (st != LV_OK) return st;
+  const VtcOut *h = ctx->h_fit->vtc;
   for (int k = 0; k < n_y; ++k) {
     status[k] = h[k].status;
     if (count) count[k] = h[k].n;
@@ -1129,16 +1150,8 @@ lv_status lv_accuracy(lv_ctx *ctx, const double *y, const double *T, int64_t n, 
   rep->r2_ssr = rep->r2_corr = rep->mean_rel = rep->p50 = rep->p90 = rep->p99 = nan;
   if (n == 0) return LV_OK;
   cudaStream_t stream = (cudaStream_t)stream_;
-  if (!ctx->h_acc) {
-    void *h = nullptr, *d = nullptr;
-    if (cudaHostAlloc(&h, 16 * sizeof(double), cudaHostAllocMapped) != cudaSuccess) return LV_ENOMEM;
-    if (cudaHostGetDevicePointer(&d, h, 0) != cudaSuccess) {
-      cudaFreeHost(h);
-      return LV_ECUDA;
-    }
-    ctx->h_acc = static_cast<double *>(h);
-    ctx->hd_acc = static_cast<double *>(d);
-  }
+  const lv_status st = map_host(&ctx->h_acc, &ctx->hd_acc, 16 * sizeof(double));
+  if (st != LV_OK) return st;
   constexpr size_t acc_dyn = kAccStage * sizeof(uint64_t);
   if (ctx->acc_occ == 0) {
     LV_CUDA(cudaFuncSetAttribute(k_acc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)acc_dyn));

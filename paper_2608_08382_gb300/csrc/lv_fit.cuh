@@ -176,8 +176,9 @@ struct GramSmem {
 
 // kGram: the Gram matrix and the flag, else the latency vector k.
 template <bool kGram>
-__device__ __forceinline__ void fit_rows(GramSmem &sm, const int64_t *feat, const uint8_t *seg, int64_t nb, const double *__restrict__ y,
-                                         int n_y, int k, FitAcc *__restrict__ partial, int *status) {
+__device__ __forceinline__ void fit_rows(GramSmem &sm, const int64_t *feat, const uint8_t *seg, int64_t nb,
+                                         const double *__restrict__ y, int n_y, int k, FitAcc *__restrict__ partial,
+                                         int *status) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int NE = fit_entries(n_y);
   const int64_t stride = (int64_t)gridDim.x * kGramWarps * kGramScan * 32;
@@ -443,6 +444,11 @@ struct FitOut {
   int32_t status, dropped;
 };
 
+// The status word's bits for the host, and the word cleared for the next call.
+__device__ __forceinline__ void hand_status(int *status, int *host) {
+  *host = atomicExch(status, 0);
+}
+
 // Index of Gram pair (a, b) in the accumulator order (row-major upper triangle).
 __host__ __device__ constexpr int gram_idx(int a, int b) {
   return a <= b ? a * 5 - a * (a - 1) / 2 + (b - a) : b * 5 - b * (b - 1) / 2 + (a - b);
@@ -472,8 +478,10 @@ __device__ __forceinline__ dd dd_sub(dd x, dd y) { return dd_add(x, dd_neg(y)); 
 // solves to 0).  Bound by the latency of that chain (one warp, 22 us;
 // with a left-looking Cholesky factorisation, one lane on the pivot, 79).  Loops
 // stay rolled: the kernel runs once per fit, so its code is fetched cold.
-__global__ void __launch_bounds__(64) k_fit_solve(const FitAcc *totals, int n_y, FitOut *__restrict__ out) {
+__global__ void __launch_bounds__(64) k_fit_solve(const FitAcc *totals, int n_y, FitOut *__restrict__ out,
+                                                   int *status, int *host_status) {
   wait_previous();
+  if (blockIdx.x == 0 && threadIdx.x == 0) hand_status(status, host_status);
   __shared__ dd G[15], R[5], A[15], B[5], inv[5];
   __shared__ dd YY, SST;
   __shared__ double cf[5];

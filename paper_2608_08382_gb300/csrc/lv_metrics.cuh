@@ -1235,7 +1235,9 @@ struct VtcOut {
   int32_t status, pad;
 };
 
-__global__ void __launch_bounds__(32) k_vtc_solve(const FitAcc *__restrict__ totals, int n_y, VtcOut *__restrict__ out) {
+__global__ void __launch_bounds__(32) k_vtc_solve(const FitAcc *__restrict__ totals, int n_y, VtcOut *__restrict__ out,
+                                                   int *status, int *host_status) {
+  if (threadIdx.x == 0) hand_status(status, host_status);
   const int k = threadIdx.x;
   if (k >= n_y) return;
   const int NE = fit_entries(n_y);

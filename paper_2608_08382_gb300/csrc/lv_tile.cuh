@@ -333,7 +333,8 @@ __device__ __forceinline__ TileRec tile_record(const TileArgs &a, const TSmem<MO
 
 // A batch's outputs.
 template <int MODE>
-__device__ __forceinline__ void tile_emit(const TileArgs &a, const TSmem<MODE> &ts, int64_t b, const BatchAgg &g, int s) {
+__device__ __forceinline__ void tile_emit(const TileArgs &a, const TSmem<MODE> &ts, int64_t b, const BatchAgg &g,
+                                          int s) {
   if ((MODE & M_ATTR) && (MODE & M_F32)) {
     if (a.T32) {
       const float *k = ts.cf[s];
@@ -368,8 +369,8 @@ __device__ __forceinline__ TenTab tile_table(const TileArgs &a, const TSmem<MODE
 // The general path of one request.  Out of line: the fast path leaves it the
 // rare ones (fp64 mode, values out of range).
 template <int MODE>
-__device__ __noinline__ void tile_slow(const TileArgs &a, const TSmem<MODE> &ts, const TileRec &rec, int64_t n, int64_t i,
-                                       int32_t p, int32_t c, int32_t u) {
+__device__ __noinline__ void tile_slow(const TileArgs &a, const TSmem<MODE> &ts, const TileRec &rec, int64_t n,
+                                       int64_t i, int32_t p, int32_t c, int32_t u) {
   const int s = (int)(rec.a.z & 3u);
   const bool slow = (rec.a.z & 4u) != 0u;
   const SegS &sg = ts.seg[s];
@@ -466,8 +467,8 @@ __device__ __forceinline__ int tile_rank(const WarpTile<MODE> &wt, int e) {
 // The tile's n listed requests, one per lane: prefills, tenants and values off
 // the common path, with every lane busy.
 template <int MODE>
-__device__ __forceinline__ void tile_rest(const TileArgs &a, const TenTab &tt, const TSmem<MODE> &ts, const WarpTile<MODE> &wt,
-                                          const TileSrc &src, int64_t rbase, int n, int lane) {
+__device__ __forceinline__ void tile_rest(const TileArgs &a, const TenTab &tt, const TSmem<MODE> &ts,
+                                          const WarpTile<MODE> &wt, const TileSrc &src, int64_t rbase, int n, int lane) {
   __syncwarp();
   int bad = 0;
 #pragma unroll 1
@@ -495,8 +496,8 @@ __device__ __forceinline__ void tile_rest(const TileArgs &a, const TenTab &tt, c
 // them goes to the list.  vec: the share array allows 32-byte (fp32: 16-byte)
 // stores.
 template <int MODE, bool kPer>
-__device__ __forceinline__ void tile_shares(const TileArgs &a, const TenTab &tt, const TSmem<MODE> &ts, WarpTile<MODE> &wt,
-                                            const TileSrc &src, int64_t rbase, int first, int cnt, bool vec,
+__device__ __forceinline__ void tile_shares(const TileArgs &a, const TenTab &tt, const TSmem<MODE> &ts,
+                                            WarpTile<MODE> &wt, const TileSrc &src, int64_t rbase, int first, int cnt, bool vec,
                                             int lane) {
   constexpr bool kTen = (MODE & M_TEN) != 0, kF32 = (MODE & M_F32) != 0;
   if (!(MODE & (M_FIX | M_F32))) {

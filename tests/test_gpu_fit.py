@@ -195,3 +195,25 @@ def test_fit_errors(lv, ctx):
         lv.lv_fit(ctx, big, torch.ones((1, 1), dtype=torch.float64, device="cuda"), [m((1, 1))])
     assert ei.value.status == lv.LV_EOVERFLOW
     assert ctx.status() == lv.LV_OK  # the sticky status was consumed by lv_fit
+
+
+def test_status_of_a_failed_fit_is_its_own(lv, ctx):
+    """The status word goes to the host with the results and is cleared: a fit or a token-count
+    fit after a failed one is unaffected, and nothing is left for the context's status."""
+    import torch
+    w = workloads.config(2, scale=0.001)
+    T, _ = oracle.attribute(w.offsets, w.p, w.c, w.phase, w.split, w.coef)
+    b = lv.batches_to_device(w.p, w.c, w.phase, w.offsets)
+    bad = T.copy()
+    bad[3] = np.inf
+    good, _ = _gpu_fit(lv, ctx, w.offsets, w.p, w.c, w.phase, T, w.split)
+    vtc = lv.lv_fit_vtc(ctx, b, torch.as_tensor(T[None], device="cuda"))
+    for call in (lambda y: lv.lv_fit(ctx, b, y, [lv.make_model(np.zeros((4, 5)), w.split)]),
+                 lambda y: lv.lv_fit_vtc(ctx, b, y)):
+        with pytest.raises(lv.LVError) as ei:
+            call(torch.as_tensor(bad[None], device="cuda"))
+        assert ei.value.status == lv.LV_EDATA
+        assert ctx.status() == lv.LV_OK
+        again, _ = _gpu_fit(lv, ctx, w.offsets, w.p, w.c, w.phase, T, w.split)
+        assert np.array_equal(again, good, equal_nan=True)
+        assert lv.lv_fit_vtc(ctx, b, torch.as_tensor(T[None], device="cuda")) == vtc
