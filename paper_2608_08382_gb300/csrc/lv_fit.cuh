@@ -31,7 +31,7 @@ namespace lv {
 // y, one flag (some batch has S1 != S3).
 // Bound by instruction issue (16 warps per SM at 128 registers; the products
 // are carry-chained 32-bit multiply-adds, a quarter fewer instructions than
-// 64-bit ones): 2e6 batches with two vectors take 117 us; 150 with 64-bit
+// 64-bit ones): 2e6 batches with two vectors take 111 us; 150 with 64-bit
 // products, 245 with, besides, one row of 32 segments looked at per turn and
 // nothing loaded ahead.  With one entry per lane and all lanes on one batch,
 // inside the kernel over the requests, the same sums took about 0.35 of 0.96 ms.
@@ -43,13 +43,26 @@ constexpr int kGramScan = 8;  // rows of 32 batches looked at together
 // v += o for W 32-bit words (modulo 2^(32 W)).
 template <int W>
 __device__ __forceinline__ void add_words(uint32_t *v, const uint32_t *o) {
-  uint64_t c = 0;
-#pragma unroll
-  for (int w = 0; w < W; ++w) {
-    c += (uint64_t)v[w] + o[w];
-    v[w] = (uint32_t)c;
-    c >>= 32;
-  }
+  static_assert(W == 3 || W == 4 || W == 6 || W == 8, "");
+  if constexpr (W == 3)
+    asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
+        : "+r"(v[0]), "+r"(v[1]), "+r"(v[2])
+        : "r"(o[0]), "r"(o[1]), "r"(o[2]));
+  else if constexpr (W == 4)
+    asm("add.cc.u32 %0, %0, %4;\n\taddc.cc.u32 %1, %1, %5;\n\taddc.cc.u32 %2, %2, %6;\n\taddc.u32 %3, %3, %7;"
+        : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3])
+        : "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]));
+  else if constexpr (W == 6)
+    asm("add.cc.u32 %0, %0, %6;\n\taddc.cc.u32 %1, %1, %7;\n\taddc.cc.u32 %2, %2, %8;\n\t"
+        "addc.cc.u32 %3, %3, %9;\n\taddc.cc.u32 %4, %4, %10;\n\taddc.u32 %5, %5, %11;"
+        : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5])
+        : "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]), "r"(o[4]), "r"(o[5]));
+  else
+    asm("add.cc.u32 %0, %0, %8;\n\taddc.cc.u32 %1, %1, %9;\n\taddc.cc.u32 %2, %2, %10;\n\t"
+        "addc.cc.u32 %3, %3, %11;\n\taddc.cc.u32 %4, %4, %12;\n\taddc.cc.u32 %5, %5, %13;\n\t"
+        "addc.cc.u32 %6, %6, %14;\n\taddc.u32 %7, %7, %15;"
+        : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7])
+        : "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]), "r"(o[4]), "r"(o[5]), "r"(o[6]), "r"(o[7]));
 }
 
 // Sum over the warp of a W-word integer (modulo 2^(32 W)), into dst (lane 0),
