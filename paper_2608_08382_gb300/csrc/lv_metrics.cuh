@@ -40,10 +40,12 @@
 //           first samples in a bucket; the block of each target then picks its
 //           second digit and ranks the bin's samples (from the bucket, or the
 //           blocks' segments when the bin outgrew it).
-// On 2e6 samples the call takes 79 us (93 with an emulated 64-bit reciprocal in
-// the division), 240 us on 8e6 (558 before the buckets grew with the count):
-// the instructions of the exact pass, then the barriers, about 23 us at
-// any size; the 32 MB of 2e6 samples take 5 us at the copy rate.
+// On 2e6 samples the call takes 75 us, on 8e6 223, on 2e4 35 (94, 558 and 41
+// with a 64-bit reciprocal in the division, 64 samples a bucket at any count
+// and the digits picked by one warp).  At 2e6: the instructions of the exact
+// pass, 22 us; about 18 us of barriers and short phases at any size; 20 us of
+// launch and wait on the host's side.  The 32 MB of 2e6 samples take 5 us at the
+// copy rate.
 #pragma once
 
 #include <cstdint>
@@ -556,16 +558,31 @@ __device__ __forceinline__ void acc_exact_loop(const double *__restrict__ y, con
                                                int64_t hi, int S, uint64_t *__restrict__ relbits, uint64_t *stage,
                                                uint64_t *w, unsigned int *h1, const AccKey &K, double &srel,
                                                bool &lost) {
-  for (int64_t i0 = lo + threadIdx.x; i0 < hi; i0 += 4 * kAccBlock) {
-    uint64_t yb[4], tb[4];  // four elements' loads in flight (a pattern of 0 is not a sample)
+  // kN elements at a time, the next ones' loads in flight (a pattern of 0 is not a
+  // sample): 2e6 samples as fast as with four loaded together and none ahead, 8e6
+  // 223 us instead of 234
+  constexpr int kN = 2;
+  uint64_t yn[kN], tn[kN];
+  auto load = [&](int64_t i0) {
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
+    for (int k = 0; k < kN; ++k) {
       const int64_t i = i0 + k * kAccBlock;
-      yb[k] = i < hi ? (uint64_t)__double_as_longlong(__ldg(y + i)) : 0ull;
-      tb[k] = i < hi ? (uint64_t)__double_as_longlong(__ldg(T + i)) : 0ull;
+      yn[k] = i < hi ? (uint64_t)__double_as_longlong(__ldg(y + i)) : 0ull;
+      tn[k] = i < hi ? (uint64_t)__double_as_longlong(__ldg(T + i)) : 0ull;
     }
+  };
+  load(lo + threadIdx.x);
+#pragma unroll 1
+  for (int64_t i0 = lo + threadIdx.x; i0 < hi; i0 += kN * kAccBlock) {
+    uint64_t yb[kN], tb[kN];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
+    for (int k = 0; k < kN; ++k) {
+      yb[k] = yn[k];
+      tb[k] = tn[k];
+    }
+    load(i0 + kN * kAccBlock);
+#pragma unroll
+    for (int k = 0; k < kN; ++k) {
       const int64_t i = i0 + k * kAccBlock;
       uint64_t rb = ~0ull;  // not a sample
       if (acc_is_sample(yb[k])) {
@@ -638,10 +655,60 @@ __device__ __forceinline__ void acc_block_sort(const uint64_t *__restrict__ relb
   __syncthreads();
 }
 
-// Pick the digit of a histogram in shared memory (kSelBins bins) that holds
-// rank r: bin, count below it, its count.  One warp; valid in every lane.
-__device__ __forceinline__ void acc_pick1(const unsigned int *h, int64_t r, int &bin, int64_t &below, int64_t &cnt) {
-  acc_scan_pick(h, r, bin, below, cnt);
+// A kSelBins-bin histogram in global memory over the block, kBlockBins
+// consecutive bins per thread: their counts, the count below them and the total
+// (below 2^32).  One round of loads and one scan by all warps: by one warp, which
+// read 64 bins a lane from a copy in shared memory, the first digit took 4.5 us.
+constexpr int kBlockBins = kSelBins / kAccBlock;
+struct AccBins {
+  unsigned int c[kBlockBins], below, total;
+};
+
+__device__ __forceinline__ AccBins acc_block_bins(const unsigned int *__restrict__ h) {
+  static_assert(kBlockBins == 8, "two 16-byte loads per thread");
+  __shared__ unsigned int wsum[kAccBlock / 32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const uint4 u = __ldcg(reinterpret_cast<const uint4 *>(h) + 2 * threadIdx.x),
+              v = __ldcg(reinterpret_cast<const uint4 *>(h) + 2 * threadIdx.x + 1);
+  AccBins r{{u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w}, 0u, 0u};
+  unsigned int s = 0u;
+#pragma unroll
+  for (int k = 0; k < kBlockBins; ++k) s += r.c[k];
+  unsigned int inc = s;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const unsigned int o = __shfl_up_sync(0xffffffffu, inc, d);
+    if (lane >= d) inc += o;
+  }
+  __syncthreads();
+  if (lane == 31) wsum[wid] = inc;
+  __syncthreads();
+  r.below = inc - s;
+#pragma unroll
+  for (int w = 0; w < kAccBlock / 32; ++w) {
+    const unsigned int o = wsum[w];
+    r.total += o;
+    if (w < wid) r.below += o;
+  }
+  return r;
+}
+
+// The thread whose bins hold rank r (1-based, at most the total): true there,
+// with the bin, the count below it and its own count.
+__device__ __forceinline__ bool acc_bin_of(const AccBins &h, int64_t r, int &bin, int64_t &below, int64_t &cnt) {
+  unsigned int b = h.below;
+  bool found = false;
+#pragma unroll
+  for (int k = 0; k < kBlockBins; ++k) {
+    if (!found && (int64_t)b < r && r <= (int64_t)b + h.c[k]) {
+      found = true;
+      bin = kBlockBins * threadIdx.x + k;
+      below = b;
+      cnt = h.c[k];
+    }
+    b += h.c[k];
+  }
+  return found;
 }
 
 // The r-th smallest (1-based) of the samples in `list` (c patterns) whose
@@ -879,21 +946,6 @@ __device__ __forceinline__ void acc_exact_totals(const AccArgs &a, uint64_t *red
   if (q == 0) a.res[0] = (double)m;
 }
 
-// The samples of the block's segment for first-digit bin `bin` (the block's
-// sorted range), visited by the whole block with eight loads in flight per
-// thread.
-template <class F>
-__device__ __forceinline__ void acc_for_segment(const uint64_t *__restrict__ seg, int cnt, F &&visit) {
-  for (int i0 = threadIdx.x; i0 < cnt; i0 += 8 * kAccBlock) {
-    uint64_t v[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) v[k] = i0 + k * kAccBlock < cnt ? __ldcg(seg + i0 + k * kAccBlock) : ~0ull;
-#pragma unroll
-    for (int k = 0; k < 8; ++k)
-      if (i0 + k * kAccBlock < cnt) visit(v[k]);
-  }
-}
-
 // The whole accuracy computation of one call; a cooperative launch of at
 // most as many blocks as fit at once.  Block b owns the elements [lo, hi).
 __global__ void __launch_bounds__(kAccBlock) k_acc(AccArgs a) {
@@ -993,8 +1045,7 @@ __global__ void __launch_bounds__(kAccBlock) k_acc(AccArgs a) {
     else
       acc_exact_loop<false>(a.y, a.T, lo, hi, path[2], a.relbits, stage, w, bh1, K, srel, lost);
     if (__syncthreads_or(lost) && tid == 0) atomicOr(a.lost, 1);
-    acc_block_sort(a.relbits, stage, sorted, lo, hi, bh1, bof1, sh, K);
-    for (int i = tid; i < kSelBins; i += kAccBlock) {
+    for (int i = tid; i < kSelBins; i += kAccBlock) {  // before the sort, which hides their latency
       const unsigned int c = bh1[i];
       if (c) atomicAdd(a.hist1 + i, c);
     }
@@ -1006,6 +1057,7 @@ __global__ void __launch_bounds__(kAccBlock) k_acc(AccArgs a) {
 #pragma unroll
       for (int j = 0; j < kAccWords; ++j) mine[kPX + j] = w[j];
     }
+    acc_block_sort(a.relbits, stage, sorted, lo, hi, bh1, bof1, sh, K);
     if (!grid_barrier(a.bar, err)) return acc_left(a);
     fp64 = __ldcg(a.lost) != 0;  // a value off the wide grid: redo the call in fp64
   }
@@ -1094,37 +1146,28 @@ __global__ void __launch_bounds__(kAccBlock) k_acc(AccArgs a) {
   // ---- first digit: the sample count (the histogram's total), then each
   // target's bin (every block)
   {
-    const unsigned int *h1 = a.hist1 + (fp64 ? kSelBins : 0);
-    for (int i = tid; i < kSelBins; i += kAccBlock) sh[i] = __ldcg(h1 + i);
-    __syncthreads();
-    if (wid == 0) {
-      unsigned long long c = 0ull;
-      for (int i = lane; i < kSelBins; i += 32) c += sh[i];
-#pragma unroll
-      for (int d = 16; d; d >>= 1) c += __shfl_xor_sync(0xffffffffu, c, d);
-      if (lane == 0) {
-        const int64_t m = (int64_t)c;
-        L.m = m;
-        L.shift = 52 - K.kbits;
-        for (int t = 0; t < kAccTargets; ++t) {
-          const int64_t q = t == 0 ? 50 : t == 1 ? 90 : 99;
-          L.rk[t] = (q * m + 99) / 100;
-        }
-      }
+    const AccBins h1 = acc_block_bins(a.hist1 + (fp64 ? kSelBins : 0));
+    const int64_t m = h1.total;
+    if (tid == 0) {
+      L.m = m;
+      L.shift = 52 - K.kbits;
     }
-    __syncthreads();
-    int bin = 0;
-    int64_t below = 0, c1 = 0;
-    if (wid < kAccTargets && L.m > 0) acc_pick1(sh, L.rk[wid], bin, below, c1);
-    if (wid < kAccTargets && lane == 0) {
-      L.bin[wid] = bin;
-      if (L.m == 0 || (K.exact && bin == 0)) {
-        L.pf[wid] = ~0ull;  // settled: rel = 0 (or no sample)
-        L.cnt[wid] = 0;
-      } else {
-        L.pf[wid] = K.exact ? (uint64_t)(bin - 1) + ((uint64_t)(1023 + K.elo) << K.kbits) : (uint64_t)bin;
-        L.rk[wid] -= below;
-        L.cnt[wid] = c1;
+#pragma unroll
+    for (int t = 0; t < kAccTargets; ++t) {
+      const int64_t q = t == 0 ? 50 : t == 1 ? 90 : 99, rk = (q * m + 99) / 100;
+      int bin = 0;
+      int64_t below = 0, c1 = 0;
+      if (m > 0 ? acc_bin_of(h1, rk, bin, below, c1) : tid == 0) {
+        L.bin[t] = bin;
+        if (m == 0 || (K.exact && bin == 0)) {
+          L.pf[t] = ~0ull;  // settled: rel = 0 (or no sample)
+          L.rk[t] = rk;
+          L.cnt[t] = 0;
+        } else {
+          L.pf[t] = K.exact ? (uint64_t)(bin - 1) + ((uint64_t)(1023 + K.elo) << K.kbits) : (uint64_t)bin;
+          L.rk[t] = rk - below;
+          L.cnt[t] = c1;
+        }
       }
     }
     __syncthreads();
@@ -1143,21 +1186,46 @@ __global__ void __launch_bounds__(kAccBlock) k_acc(AccArgs a) {
   // bin's first 2^lb samples in a bucket and publishing where its
   // segments lie
   {
+    // the targets' segments one after the other, so that all their loads and
+    // atomics are in flight together
     const int lo2 = L.shift - kSelBits;
+    int c[kAccTargets], o[kAccTargets], all3 = 0;
+#pragma unroll
     for (int t = 0; t < kAccTargets; ++t) {
-      if (L.slot[t] != t || L.pf[t] == ~0ull) continue;  // the same in every block
-      const int b = L.bin[t];
-      unsigned int *h2 = a.hist2 + t * kSelBins;
-      uint64_t *bk = a.bucket + ((int64_t)t * kSelBins << a.lb);
-      acc_for_segment(sorted + lo + bof1[b], (int)bh1[b], [&](uint64_t v) {
-        const int d = (int)((v >> lo2) & (uint64_t)(kSelBins - 1));
-        const unsigned int p = atomicAdd(h2 + d, 1u);
-        if (p < (1u << a.lb)) bk[(d << a.lb) + p] = v;  // the bin's first samples, kept for the finish
-      });
-      if (tid == 0) {
-        a.segs[2 * (blockIdx.x * kAccTargets + t)] = (uint64_t)(lo + bof1[b]);
-        a.segs[2 * (blockIdx.x * kAccTargets + t) + 1] = bh1[b];
+      const bool on = L.slot[t] == t && L.pf[t] != ~0ull;  // the same in every block
+      o[t] = on ? (int)bof1[L.bin[t]] : 0;
+      c[t] = on ? (int)bh1[L.bin[t]] : 0;
+      all3 += c[t];
+      if (on && tid == 0) {
+        a.segs[2 * (blockIdx.x * kAccTargets + t)] = (uint64_t)(lo + o[t]);
+        a.segs[2 * (blockIdx.x * kAccTargets + t) + 1] = (uint64_t)c[t];
       }
+    }
+    for (int i0 = tid; i0 < all3; i0 += 4 * kAccBlock) {
+      uint64_t v[4];
+      int tg[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        int i = i0 + k * kAccBlock;
+        const bool in = i < all3;
+        tg[k] = 0;
+#pragma unroll
+        for (int t = 0; t < kAccTargets - 1; ++t)
+          if (tg[k] == t && i >= c[t]) {
+            i -= c[t];
+            tg[k] = t + 1;
+          }
+        const int at = tg[k] == 0 ? o[0] : tg[k] == 1 ? o[1] : o[2];
+        v[k] = in ? __ldcg(sorted + lo + at + i) : 0ull;
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (i0 + k * kAccBlock < all3) {
+          const int d = (int)((v[k] >> lo2) & (uint64_t)(kSelBins - 1)), at = tg[k] * kSelBins + d;
+          const unsigned int p = atomicAdd(a.hist2 + at, 1u);
+          // the bin's first samples, kept for the finish
+          if (p < (1u << a.lb)) a.bucket[((int64_t)at << a.lb) + p] = v[k];
+        }
     }
   }
   if (!grid_barrier(a.bar, err)) return acc_left(a);
@@ -1170,17 +1238,13 @@ __global__ void __launch_bounds__(kAccBlock) k_acc(AccArgs a) {
     uint64_t r = 0ull;
     if (L.pf[t] != ~0ull) {
       const int s = L.slot[t];
-      for (int i = tid; i < kSelBins; i += kAccBlock) sh[i] = __ldcg(a.hist2 + s * kSelBins + i);
-      __syncthreads();
-      if (wid == 0) {
-        int bin;
-        int64_t below, c2;
-        acc_pick1(sh, L.rk[t], bin, below, c2);
-        if (lane == 0) {
-          F.pf[t] = (L.pf[t] << kSelBits) | (uint64_t)bin;
-          F.rk[t] = L.rk[t] - below;
-          F.cnt[t] = c2;
-        }
+      const AccBins h2 = acc_block_bins(a.hist2 + s * kSelBins);
+      int bin = 0;
+      int64_t below = 0, c2 = 0;
+      if (acc_bin_of(h2, L.rk[t], bin, below, c2)) {
+        F.pf[t] = (L.pf[t] << kSelBits) | (uint64_t)bin;
+        F.rk[t] = L.rk[t] - below;
+        F.cnt[t] = c2;
       }
       __syncthreads();
       const int cur = L.shift - kSelBits;
