@@ -50,7 +50,7 @@ METRIC = "attributed requests/sec on 1 GB300; achieved HBM GB/s vs ~8 TB/s peak"
 KERNEL_SOURCES = ["paper_2608_08382_gb300/csrc/lv_kernels.cuh", "paper_2608_08382_gb300/csrc/lv_fixed.cuh",
                   "paper_2608_08382_gb300/csrc/lv_api.cu", "paper_2608_08382_gb300/csrc/lv_fit.cuh",
                   "paper_2608_08382_gb300/csrc/lv_whatif.cuh", "paper_2608_08382_gb300/csrc/lv_step.cuh",
-                  "paper_2608_08382_gb300/csrc/lv_tile.cuh",
+                  "paper_2608_08382_gb300/csrc/lv_tile.cuh", "paper_2608_08382_gb300/csrc/lv_tenant.cuh",
                   "paper_2608_08382_gb300/csrc/lv_metrics.cuh"]
 
 
@@ -296,7 +296,8 @@ def _setup_attr(lv, ctx, w, stream, f32=False):
 
     return dict(step=step, e2e_step=e2e_step, units=w.n_req, unit="requests/s", metric=METRIC,
                 h2d=h2d,
-                d2h=(4 if f32 else 8) * (w.n_req + w.n_batch) + 8 * w.n_tenants, launches_per_step=4,
+                d2h=(4 if f32 else 8) * (w.n_req + w.n_batch) + 8 * w.n_tenants,
+                launches_per_step=4 if w.n_tenants > 2048 else 3,  # more tenants: a fold of their own
                 kernel="k_tiles", time_mask=lv.LV_TIME_TILES,
                 bytes_per_launch=(20.0 if f32 else 24.0) * w.n_req + (12.0 if f32 else 16.0) * w.n_batch,
                 bytes_rule=("20 B/request (p, c, phase, tenant read; fp32 share written) + 12 B/batch (offset read; "

@@ -31,10 +31,10 @@
 // and small enough for the instruction cache (unrolled twice it took a third
 // longer).
 // Against a kernel that walked one batch per warp (one call, GB300): 1.36e8
-// requests in batches of 16 to 256, fp64 shares, 256 tenants, 1,130 us before
-// and 880 now; 3.25e7 in batches of 1 to 64, 16 tenants, 583 and 301; 6.5e5, 113
-// and 30; 2.6e7 in Pareto batches, 65,536 tenants, 816 and 575; fp32, 4.1e7 in
-// batches of 16 to 256, 323 and 244.
+// requests in batches of 16 to 256, fp64 shares, 256 tenants, 1,134 us before
+// and 846 now; 3.25e7 in batches of 1 to 64, 16 tenants, 583 and 297; 6.5e5, 114
+// and 20; 2.6e7 in Pareto batches, 65,536 tenants, 816 and 584; fp32, 4.1e7 in
+// batches of 16 to 256, 323 and 229.
 #pragma once
 
 #include "lv_step.cuh"
@@ -54,8 +54,8 @@ constexpr uint32_t kTSmall = 1u << 23;     // p and c of a tile on the common pa
 
 // A tile's size.  The passes that write only batch features keep no records, so
 // their tiles can be twice as large and leave the L1 more.  2.57e8 requests take
-// 508 us (6.1 TB/s); a whole fit 766 us, 780 with the other passes' shape, 764
-// with 3,256 positions, 802 with 4,064, 788 with 24 warps, 792 with 16.
+// 508 us (6.1 TB/s), 14 us less than with the other passes' shape; tiles of
+// 3,256 positions 1 us less still, of 4,064 36 more, 24 warps 22 more, 16 warps 26.
 template <int MODE>
 struct Geo {
   static constexpr bool kAttr = (MODE & M_ATTR) != 0;
