@@ -409,7 +409,7 @@ lv_status run_tiles_mode(lv_ctx *ctx, int sms, TileArgs &a, void *bound, int64_t
     } else if (plan.n_tiles + 1 > bound_cap) {
       return LV_EINVAL;
     }
-    const int64_t blocks = std::min<int64_t>((a.n_batch + 1 + 255) / 256, (int64_t)sms * 16);
+    const int64_t blocks = std::min<int64_t>(a.n_batch / 1024 + 1, (int64_t)sms * 16);
     if (a.n_batch < (1ll << 32)) {
       a.bound32 = static_cast<uint32_t *>(bound);
       k_tile_bounds<uint32_t><<<(unsigned)blocks, 256, 0, stream>>>(a.off, a.n_batch, a.n_req, plan.n_tiles,

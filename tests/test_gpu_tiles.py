@@ -78,7 +78,7 @@ def test_features_match_attribution_sums(lv, ctx):
     assert np.array_equal(bf.cpu().numpy(), feat) and np.array_equal(bs.cpu().numpy(), seg)
 
 
-@pytest.mark.parametrize("lo,hi,n,cut", [(0, 1, 1_200_000, 1), (1, 40, 300_000, 0), (2470, 2500, 4000, 3),
+@pytest.mark.parametrize("lo,hi,n,cut", [(0, 1, 1_200_001, 1), (1, 40, 300_002, 0), (2470, 2500, 4003, 3),
                                          (2548, 2566, 3500, 1), (3000, 6000, 60, 0)])
 def test_feature_sizes_around_the_tile(lv, ctx, lo, hi, n, cut):
     """The feature pass has tiles of its own: exact sums at the edges of their positions and
@@ -100,3 +100,21 @@ def test_feature_sizes_around_the_tile(lv, ctx, lo, hi, n, cut):
     assert ctx.status() == lv.LV_OK
     want, want_seg = oracle.batch_features(off, p, c, ph, (256, 300))
     assert np.array_equal(feat.cpu().numpy(), want) and np.array_equal(seg.cpu().numpy(), want_seg)
+
+
+@pytest.mark.parametrize("at", [0, 1, 2, 499_996, 499_997, 499_998, 499_999, 1_000_001, 1_000_002])
+def test_offsets_out_of_order_are_seen(lv, ctx, at):
+    """One offset below the one before it, in each place of a thread's four and in the last ones (an input
+    whose tile bounds have a kernel of their own)."""
+    import torch
+    n = 1_000_002
+    off = np.arange(n + 1, dtype=np.int64)
+    one, zero = np.ones(n, np.int32), np.zeros(n, np.int32)
+    feat = torch.zeros((5, n), dtype=torch.int64, device="cuda")
+    seg = torch.zeros(n, dtype=torch.uint8, device="cuda")
+    model = lv.make_model(np.ones((2, 2, 5)), (256, 300))
+    for bad in (off[at] - 2, None):
+        o = off.copy()
+        o[at] = off[at] if bad is None else bad
+        lv.lv_features(ctx, lv.batches_to_device(one, zero, zero, o), model=model, batch_feat=feat, batch_seg=seg)
+        assert ctx.status() == (lv.LV_OK if bad is None else lv.LV_EDATA)
