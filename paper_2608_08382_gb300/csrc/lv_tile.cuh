@@ -18,9 +18,9 @@
 // no lane idles on a batch's remainder.  The requests are read twice, the
 // second time from L1 or L2.  A batch that reaches past a tile's requests
 // is walked by its warp alone, or, above kTAlone requests, by the whole CTA
-// after its tiles (a warp alone on a batch of 4,096 set the time of a small
-// input).  All sums are exact integers, so results do not depend on the
-// schedule.
+// after its tiles (1e6 Pareto batches of up to 4,096: 88 us, 196 if their warps
+// walk them all).  All sums are exact integers, so results do not depend on
+// the schedule.
 //
 // What bounds it: instruction issue and the integer pipe (about 170 warp
 // instructions per 32 requests), not HBM.  The shape follows from that: 20 warps
@@ -32,9 +32,9 @@
 // longer).
 // Against a kernel that walked one batch per warp (one call, GB300): 1.36e8
 // requests in batches of 16 to 256, fp64 shares, 256 tenants, 1,134 us before
-// and 846 now; 3.25e7 in batches of 1 to 64, 16 tenants, 583 and 297; 6.5e5, 114
-// and 20; 2.6e7 in Pareto batches, 65,536 tenants, 816 and 584; fp32, 4.1e7 in
-// batches of 16 to 256, 323 and 229.
+// and 840 now; 3.25e7 in batches of 1 to 64, 16 tenants, 583 and 290; 6.5e5, 113
+// and 20; 2.6e7 in Pareto batches, 65,536 tenants, 817 and 566; fp32, 4.1e7 in
+// batches of 16 to 256, 322 and 222.
 #pragma once
 
 #include "lv_step.cuh"
@@ -46,7 +46,6 @@ constexpr int kTThreads = 640;             // threads of a CTA, one CTA per SM (
 constexpr int kTWarps = kTThreads / 32;
 constexpr int kTW = 8;                     // merge positions a batch takes besides its requests
 constexpr int kTDMin = 128;
-constexpr int kTDense = 40;                // batches of fewer requests on average: a record per request in step 3
 constexpr int64_t kTAlone = 512;           // requests a warp walks alone
 constexpr int kTBigs = 64;                 // larger batches a CTA keeps for later
 constexpr int kTabN = 4096;                // batch sizes of the K table
@@ -480,7 +479,8 @@ __device__ __forceinline__ int tile_rank(const WarpTile<MODE> &wt, int e) {
 // the common path, with every lane busy.
 template <int MODE>
 __device__ __forceinline__ void tile_rest(const TileArgs &a, const TenTab &tt, const TSmem<MODE> &ts,
-                                          const WarpTile<MODE> &wt, const TileSrc &src, int64_t rbase, int n, int lane) {
+                                          const WarpTile<MODE> &wt, const TileSrc &src, int64_t rbase, int n,
+                                          int lane) {
   __syncwarp();
   int bad = 0;
 #pragma unroll 1
@@ -502,15 +502,16 @@ __device__ __forceinline__ void tile_rest(const TileArgs &a, const TenTab &tt, c
 
 // The tile's shares, four consecutive requests per lane and step.  The loop
 // takes decode requests (p = 1; fp32 variant: any) on the common path, without a
-// branch or a call; the rest goes to the warp's list, worked off after it.
-// kPer: a record per request (tiles of small batches); otherwise the lane's
-// four share the first one's record, and what lies past a batch's start among
-// them goes to the list.  vec: the share array allows 32-byte (fp32: 16-byte)
+// call; the rest goes to the warp's list, worked off after it.  A lane loads
+// another record where a batch starts among its four (leaving what lies past
+// the start to the list, where batches average 40 requests and more, was
+// no faster: 1.36e8 requests of batches of 16 to 256, 840 us either way, and the
+// second copy of the loop cost the fp32 variant 3 %).  vec: the share array allows 32-byte (fp32: 16-byte)
 // stores.
-template <int MODE, bool kPer>
+template <int MODE>
 __device__ __forceinline__ void tile_shares(const TileArgs &a, const TenTab &tt, const TSmem<MODE> &ts,
-                                            WarpTile<MODE> &wt, const TileSrc &src, int64_t rbase, int first, int cnt, bool vec,
-                                            int lane) {
+                                            WarpTile<MODE> &wt, const TileSrc &src, int64_t rbase, int first, int cnt,
+                                            bool vec, int lane) {
   constexpr bool kTen = (MODE & M_TEN) != 0, kF32 = (MODE & M_F32) != 0;
   if (!(MODE & (M_FIX | M_F32))) {
     // fp64 mode has no common path: one request per lane, in order
@@ -529,13 +530,12 @@ __device__ __forceinline__ void tile_shares(const TileArgs &a, const TenTab &tt,
     if (b + 128 < cnt) nx = load_quad<kTen>(src.p, src.c, src.u, e + 128, src.lim);
     const int32_t p[4] = {v.p.x, v.p.y, v.p.z, v.p.w}, c[4] = {v.c.x, v.c.y, v.c.z, v.c.w};
     const uint32_t u[4] = {(uint32_t)v.x.x, (uint32_t)v.x.y, (uint32_t)v.x.z, (uint32_t)v.x.w};
-    // the quad's requests that are the tile's, and those before the next head
+    // the quad's requests that are the tile's
     const int hi = min(max(cnt - e, 0), 4), lo = max(first - e, 0);
     const uint32_t vm = ((1u << hi) - 1u) & (15u << lo);
     const uint32_t word = wt.bits[b / 32 + (lane >> 3)];
     const int sh = e & 31;
     const uint32_t hb = (word >> sh) & 14u;
-    const uint32_t run = kPer ? vm : vm & ((hb & (0u - hb)) - 1u);  // no head: all four
     // record of the first request; -1 before the tile's first batch
     const int r0 = min((int)wt.rank[b / 32 + (lane >> 3)] + __popc(word & ((2u << sh) - 1u)), Geo<MODE>::kRec - 4) - 1;
     TileRec rec = wt.rec[max(r0, 0)];
@@ -544,8 +544,8 @@ __device__ __forceinline__ void tile_shares(const TileArgs &a, const TenTab &tt,
     float f[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      if (kPer && k > 0) rec = wt.rec[max(r0 + __popc(hb & ((2u << k) - 1u)), 0)];
-      go[k] = ((run >> k) & 1u) != 0u && (kPer || r0 >= 0);
+      if (k > 0 && ((hb >> k) & 1u)) rec = wt.rec[max(r0 + __popc(hb & ((2u << k) - 1u)), 0)];
+      go[k] = ((vm >> k) & 1u) != 0u;
       if (kF32) {
         const Share32 q{__uint_as_float(rec.k.x), __uint_as_float(rec.k.y), __uint_as_float(rec.k.z),
                         __uint_as_float(rec.k.w)};
@@ -799,10 +799,7 @@ __global__ void __launch_bounds__(kTThreads, 1) k_tiles(const TileArgs a) {
 
     // 3. requests
     if ((MODE & M_ATTR) && !wide && (kTen || a.share || a.share32)) {
-      if (!(MODE & (M_FIX | M_F32)) || before * kTDense <= cnt)
-        tile_shares<MODE, false>(a, tt, ts, wt, src, rbase, first, cnt, vec, lane);
-      else
-        tile_shares<MODE, true>(a, tt, ts, wt, src, rbase, first, cnt, vec, lane);
+      tile_shares<MODE>(a, tt, ts, wt, src, rbase, first, cnt, vec, lane);
     }
     if (direct) {
       // the last batch; every batch of a wide tile

@@ -86,10 +86,11 @@ __device__ __forceinline__ i128 cand_const(const ModelP &mp, int s, int half, in
 // pass and k_wi_cand: a planning call's few hundred to few thousand candidates
 // are bound by the chain of launches and of dependent loads (1,024
 // candidates of 144 requests: 29 us for that chain).  With more than
-// kWiDirectPerSm candidates per SM the tile pass, which packs small
-// batches, is as fast and takes over.
+// kWiDirectPerSm candidates per SM the tile pass, which packs batches, takes
+// over (whole calls by blocks and by tiles: 1,024 candidates 27 and 35 us, 10,000
+// 41.5 and 43.5, 40,000 83 and 56).
 constexpr int kWiCandThreads = 128;
-constexpr int kWiDirectPerSm = 16;
+constexpr int kWiDirectPerSm = 64;
 __global__ void __launch_bounds__(kWiCandThreads) k_wi_cand_direct(ModelP mp, const int32_t *__restrict__ p,
                                                                   const int32_t *__restrict__ c,
                                                                   const int32_t *__restrict__ ph,

@@ -53,7 +53,7 @@ def test_values_beyond_the_prefix_words(lv, ctx, field):
     _check(lv, ctx, w)
 
 
-@pytest.mark.parametrize("nt", [1, 511, 512, 513, 3000])
+@pytest.mark.parametrize("nt", [1, 511, 512, 513, 1536, 1537, 3000])
 @pytest.mark.parametrize("scale", [1e-4, 1.0, 300.0])
 def test_tenants_and_share_magnitudes(lv, ctx, nt, scale):
     """Shares below 2^-20 s (rounded to the 2^-72 s grid), common ones, and ones of 2^-9 s and

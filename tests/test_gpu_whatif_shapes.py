@@ -40,7 +40,8 @@ def _whatif(lv, ctx, w, p, c, ph, adm=None):
     return T.cpu().numpy(), S.cpu().numpy(), A
 
 
-@pytest.mark.parametrize("nc,npend", [(1, 1), (5, 700), (31, 33), (33, 5), (65, 130), (129, 40), (2433, 3), (300, 1000)])
+@pytest.mark.parametrize("nc,npend", [(1, 1), (5, 700), (31, 33), (33, 5), (65, 130), (129, 40), (2433, 3), (9728, 2), (9729, 3),
+                                     (300, 1000)])
 def test_shapes(lv, ctx, nc, npend):
     rng = np.random.default_rng(nc * 1000 + npend)
     sizes = rng.integers(0, 300, nc)
