@@ -1082,7 +1082,9 @@ __global__ void __launch_bounds__(kAccBlock) k_acc(AccArgs a) {
         ++cnt;
         sy += yv;
         st += tv;
-        bits = (uint64_t)__double_as_longlong(__ddiv_rn(fabs(__dsub_rn(tv, yv)), yv));
+        // the sign cleared after the division too: inf / inf may give a NaN of either
+        // sign, and the first digit below has to be one of the kSelBins
+        bits = (uint64_t)__double_as_longlong(fabs(__ddiv_rn(fabs(__dsub_rn(tv, yv)), yv)));
         atomicAdd(&bh1[(int)(bits >> 52)], 1u);
         srel += __longlong_as_double((long long)bits);
       }

@@ -35,3 +35,24 @@ def test_bucket_sizes(lv, ctx, n):  # noqa: F811
     T = rng.lognormal(-3.0, 0.6, n)
     y = T * rng.lognormal(0.0, 0.1, n)
     _check_accuracy(lv.lv_accuracy(ctx, _dev(y), _dev(T)), oracle.accuracy(y, T))
+
+
+@pytest.mark.parametrize("n,k", [(1, 1), (50, 1), (50, 30), (20_000, 7), (20_000, 500), (300_000, 100_000)])
+@pytest.mark.parametrize("T_inf", [False, True])
+def test_infinite_latencies(lv, ctx, n, k, T_inf):  # noqa: F811
+    """y = +inf counts as a sample; its relative error is a NaN (inf / inf, or inf - inf), which ranks above
+    every number, whatever sign the arithmetic gives it."""
+    rng = np.random.default_rng(n + k)
+    T = rng.lognormal(-3.0, 0.6, n)
+    y = T * rng.lognormal(0.0, 0.1, n)
+    at = rng.choice(n, k, replace=False)
+    y[at] = np.inf
+    if T_inf:
+        T[at[::2]] = np.inf
+    g = lv.lv_accuracy(ctx, _dev(y), _dev(T))
+    with np.errstate(invalid="ignore"):
+        rel = np.sort(np.abs(T - y) / y)  # NaN last
+    assert g["n"] == n and np.isnan(g["mean_rel"]) and np.isnan(g["r2_ssr"]) and np.isnan(g["r2_corr"])
+    for name, q in (("p50", 50), ("p90", 90), ("p99", 99)):
+        want = rel[-(-q * n // 100) - 1]
+        assert g[name] == want or (np.isnan(g[name]) and np.isnan(want)), name
