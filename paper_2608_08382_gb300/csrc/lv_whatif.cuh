@@ -270,8 +270,10 @@ __global__ void __launch_bounds__(kWiThreads) k_wi_pairs(ModelP mp, const CandP 
   if (!cb->slow && !rslow) {
     // every V of the block below 2^95 and p at most 2^24: with U and W in
     // [2^64, 2^95), three words hold the sums and one rounding form does
-    const int32_t thr0 = (int32_t)clampi(sp0 - s1, INT32_MIN, INT32_MAX),
-                  thr1 = (int32_t)clampi(sp1 - s1, INT32_MIN, INT32_MAX);
+    // s1 + p >= split as p >= split - s1; a negative split, met by every batch,
+    // counts as 0, so that the difference cannot wrap
+    const int32_t thr0 = (int32_t)clampi(max(sp0, (int64_t)0) - s1, INT32_MIN, INT32_MAX),
+                  thr1 = (int32_t)clampi(max(sp1, (int64_t)0) - s1, INT32_MIN, INT32_MAX);
     const int64_t slo_key = bound_key(adm.slo);
     double *Tp = T_new ? T_new + o : nullptr, *Sp = share_new ? share_new + o : nullptr;
     uint8_t *Ap = adm.admit ? adm.admit + o : nullptr;

@@ -53,6 +53,18 @@ def test_shapes(lv, ctx, nc, npend):
     assert np.max(np.abs(T - T_o) / T_o) <= 1e-12 and np.max(np.abs(S - S_o) / S_o) <= 1e-12
 
 
+@pytest.mark.parametrize("split", [-2 ** 63, -2 ** 63 + 1, -1, 0, 1, 2 ** 31, 2 ** 63 - 1])
+def test_extreme_splits(lv, ctx, split):
+    """Splits that every batch or none meets: the regime is S1 + p >= split in 64 bits."""
+    rng = np.random.default_rng(43)
+    w = base._from_sizes(rng, rng.integers(0, 60, 70), pre=0.05)
+    w.split[:] = split
+    p, c, ph = _pending(rng, 90)
+    T, S, _ = _whatif(lv, ctx, w, p, c, ph)
+    T_o, S_o = oracle.whatif(w.offsets, w.p, w.c, w.phase, p, c, ph, w.split, w.coef)
+    assert np.max(np.abs(T - T_o) / T_o) <= 1e-12 and np.max(np.abs(S - S_o) / S_o) <= 1e-12
+
+
 @pytest.mark.parametrize("slo", [0.004, 0.0, -0.0, float("nan"), float("inf"), float("-inf")])
 def test_admission_edges(lv, ctx, slo):
     rng = np.random.default_rng(41)
