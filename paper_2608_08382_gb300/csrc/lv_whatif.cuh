@@ -246,12 +246,16 @@ __global__ void __launch_bounds__(kWiThreads) k_wi_pairs(ModelP mp, const CandP 
       sp[r].phase = ph;
       sp[r].slow = slow;
       if (adm.admit) {
-        // a tenant id out of range makes every pair of the request inadmissible: NaN compares false
+        // a tenant id out of range, and a total that is a NaN of either sign, make
+        // every pair of the request inadmissible: a NaN budget compares false, and
+        // with the total at infinity no sum's key is as low as its bound's
         const int32_t u = adm.tenant[j];
         const bool in = u >= 0 && u < adm.n_tenants;
         if (!in) bad = 1;
-        sp[r].Lu = in ? adm.L[u] : __longlong_as_double(0x7ff8000000000000ll);
-        sp[r].Bu = in ? adm.budget[u] : 0.0;
+        const double Lu = in ? adm.L[u] : 0.0;
+        const bool ok = in && Lu == Lu;
+        sp[r].Lu = ok ? Lu : __longlong_as_double(0x7ff0000000000000ll);
+        sp[r].Bu = ok ? adm.budget[u] : __longlong_as_double(0x7ff8000000000000ll);
         sp[r].Bk = bound_key(sp[r].Bu);
       }
       if (bad) flag(status, kStatusData);
@@ -308,7 +312,7 @@ __global__ void __launch_bounds__(kWiThreads) k_wi_pairs(ModelP mp, const CandP 
       }
       // comparisons as integers: with two fp64 ones per pair as well as the
       // addition, the fp64 pipe took longer than the stores (4.2e6 pairs: 52
-      // us a call, 34 so).  A NaN sum has the largest key.
+      // us a call, 34 so).  No sum is a NaN: totals are not (above), shares are finite.
       if (Ap) {
         *Ap = (order_key(__dadd_rn(sp[r].Lu, sh)) <= sp[r].Bk && order_key(T) <= slo_key) ? 1 : 0;
         Ap += ostep;

@@ -71,8 +71,9 @@ def test_admission_edges(lv, ctx, slo):
     w = base._from_sizes(rng, rng.integers(1, 60, 70), pre=0.02)
     p, c, ph = _pending(rng, 90)
     inf, nan = float("inf"), float("nan")
-    L = np.array([0.0, -0.0, 1e-3, nan, inf, -inf, 5.0, 0.0, 1e-3])
-    B = np.array([0.0, -0.0, 2e-3, 1.0, inf, inf, nan, 1e-3, -inf])
+    neg_nan, full_nan = np.array([0xfff8000000000000, 0xffffffffffffffff], np.uint64).view(np.float64)
+    L = np.array([0.0, -0.0, 1e-3, nan, inf, -inf, 5.0, 0.0, 1e-3, neg_nan, full_nan, neg_nan, 0.0])
+    B = np.array([0.0, -0.0, 2e-3, 1.0, inf, inf, nan, 1e-3, -inf, 1.0, inf, full_nan, full_nan])
     ten = rng.integers(0, len(L), len(p)).astype(np.int32)
     T, S, _ = _whatif(lv, ctx, w, p, c, ph)
     B[7], L[7] = S[ten == 7][0, 3], 0.0   # a budget met exactly
