@@ -311,8 +311,9 @@ lv_status timing_end(cudaEvent_t stop, cudaStream_t stream) {
   return LV_OK;
 }
 
-// Occupancy of k_tiles<MODE> for launches without a context, by (mode << 32 |
-// dynamic shared memory); the kernel attributes are process-wide as well.
+// Occupancy of k_tiles<MODE> for launches without a context, by (device << 40 |
+// mode << 32 | dynamic shared memory): a kernel's attributes belong to the
+// device they were set on.
 template <int MODE>
 std::vector<std::pair<uint64_t, int>> &free_occ() {
   static std::vector<std::pair<uint64_t, int>> v;
@@ -349,10 +350,12 @@ TilePlan plan_tiles(int64_t n_batch, int64_t n_req, int64_t warps, int64_t d_max
 }
 
 // Kernel attributes and CTAs per SM of k_tiles<MODE>, once per (context or,
-// without one, process; shared-memory size).
+// without one, device; shared-memory size).
 template <int MODE>
 lv_status tiles_occupancy(lv_ctx *ctx, size_t smem, int *per_sm) {
-  const uint64_t key = ((uint64_t)MODE << 32) | smem;
+  int dev = 0;
+  if (!ctx) LV_CUDA(cudaGetDevice(&dev));
+  const uint64_t key = ((uint64_t)dev << 40) | ((uint64_t)MODE << 32) | smem;
   *per_sm = 0;
   if (ctx) {
     for (const auto &e : ctx->occ)

@@ -108,3 +108,34 @@ def test_binding_constants_match_header(lv):
     assert len(defs) >= 13
     for name, value in defs.items():
         assert getattr(lv, name) == int(value), name
+
+
+def test_noalloc_configures_its_kernels_on_each_device(lv, tmp_path):
+    """lv_attribute_noalloc's kernel needs more shared memory than a kernel gets unasked, and that is set per device:
+    a second device's first call sets it again.  On a stand-in for the runtime with two devices, in a process of its
+    own."""
+    import shutil
+    import subprocess
+    import sys
+    if shutil.which("gcc") is None:
+        pytest.skip("no C compiler")
+    fake = str(tmp_path / "libfake.so")
+    subprocess.run(["gcc", "-shared", "-fPIC", "-o", fake, os.path.join(ROOT, "tests", "fake_cudart.c")], check=True)
+    code = """
+import ctypes, sys
+import numpy as np
+import paper_2608_08382_gb300 as lv
+rt = ctypes.CDLL(sys.argv[1])
+m = lv.make_model(np.ones((4, 5)), (1, 1))
+at = ctypes.c_void_p(1 << 20)
+for n_req in (1000, 50_000_000):  # one tile per warp, and many
+    b = lv.lv_batches(at, at, at, None, at, n_req, 1000, 0, 0)
+    for dev in (0, 1, 0):
+        rt.fake_set_device(dev)
+        rc = lv.lib().lv_attribute_noalloc(ctypes.byref(m), ctypes.byref(b), at, at, at, None)
+        assert rc == lv.LV_OK, (n_req, dev, rc)
+assert rt.fake_launches(0) > 0 and rt.fake_launches(1) > 0
+"""
+    r = subprocess.run([sys.executable, "-c", code, fake], cwd=ROOT, env={**os.environ, "LD_PRELOAD": fake},
+                       capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
