@@ -530,7 +530,7 @@ struct AccKey {
 };
 
 __device__ __forceinline__ int acc_key1(uint64_t rb, const AccKey &K) {
-  if (!K.exact) return (int)(rb >> 52);
+  if (!K.exact) return (int)(rb >> 52) & (kSelBins - 1);  // the sign is clear
   if (rb == 0) return 0;
   const int64_t k = (int64_t)(rb >> (52 - K.kbits)) - ((int64_t)(1023 + K.elo) << K.kbits) + 1;
   return (int)min(max(k, (int64_t)1), (int64_t)kSelBins - 1);  // within range by construction
@@ -1082,10 +1082,12 @@ __global__ void __launch_bounds__(kAccBlock) k_acc(AccArgs a) {
         ++cnt;
         sy += yv;
         st += tv;
-        // the sign cleared after the division too: inf / inf may give a NaN of either
-        // sign, and the first digit below has to be one of the kSelBins
-        bits = (uint64_t)__double_as_longlong(fabs(__ddiv_rn(fabs(__dsub_rn(tv, yv)), yv)));
-        atomicAdd(&bh1[(int)(bits >> 52)], 1u);
+        // inf / inf (and inf - inf) give a NaN whose sign may be set; it is cleared as an
+        // integer, out of the compiler's sight: fabs of a quotient of two values that are
+        // not negative may be left out, as the sign of a NaN counts for nothing there
+        const double rel = __ddiv_rn(fabs(__dsub_rn(tv, yv)), yv);
+        asm("and.b64 %0, %1, 0x7fffffffffffffff;" : "=l"(bits) : "l"(__double_as_longlong(rel)));
+        atomicAdd(&bh1[acc_key1(bits, K)], 1u);
         srel += __longlong_as_double((long long)bits);
       }
       a.relbits[i] = bits;
