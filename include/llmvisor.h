@@ -130,8 +130,12 @@ typedef struct lv_tenant_acc lv_tenant_acc;
 #define LV_ARITH_AUTO 0
 #define LV_ARITH_FP64 1
 
-/* Create a context on the current CUDA device.  It owns a small device scratch
- * area and a sticky status word.  Returns LV_ECUDA/LV_ENOMEM on failure. */
+/* Create a context on the current CUDA device.  It owns a device scratch area
+ * that its calls grow to the largest input they have seen and keep (the first
+ * batch of each tile of about 1,200 to 2,500 requests, 4 bytes; lv_whatif: 192
+ * bytes a candidate; lv_fit: 33 bytes a batch, for 2^22 batches at most, 138 MB;
+ * lv_accuracy: about 20 bytes a batch) and a sticky status word.  Returns
+ * LV_ECUDA/LV_ENOMEM on failure. */
 lv_status lv_ctx_create(lv_ctx **out);
 void lv_ctx_destroy(lv_ctx *ctx);
 /* Select LV_ARITH_AUTO (default) or LV_ARITH_FP64. */

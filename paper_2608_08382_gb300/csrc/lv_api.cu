@@ -394,53 +394,72 @@ lv_status ensure_bound(lv_ctx *ctx, int64_t n) {
   return LV_OK;
 }
 
-// Bounds and tile kernel for the given batches.  Without a context, `bound`
-// has room for the tiles' bounds (bound_cap 32-bit entries).
+// A launch of k_tiles.
+struct TileLaunch {
+  unsigned grid;
+  size_t smem;
+  bool search;
+};
+
+// Tiles of the given batches and, unless the warps find them, their bounds.
+// Without a context, `bound` has room for the tiles' bounds (bound_cap 32-bit
+// entries).
 template <int MODE>
-lv_status run_tiles_mode(lv_ctx *ctx, int sms, TileArgs &a, void *bound, int64_t bound_cap, cudaStream_t stream) {
-  const size_t smem = sizeof(TSmem<MODE>) + ((MODE & M_TEN) ? ten_table_bytes(kHotMax) : 0);
+lv_status bound_tiles(lv_ctx *ctx, int sms, TileArgs &a, void *bound, int64_t bound_cap, cudaStream_t stream,
+                      TileLaunch *tl) {
+  tl->smem = sizeof(TSmem<MODE>) + ((MODE & M_TEN) ? ten_table_bytes(kHotMax) : 0);
   int per_sm = 0;
-  lv_status st = tiles_occupancy<MODE>(ctx, smem, &per_sm);
+  lv_status st = tiles_occupancy<MODE>(ctx, tl->smem, &per_sm);
   if (st != LV_OK) return st;
   const int64_t ctas = (int64_t)sms * per_sm;
   const TilePlan plan = plan_tiles(a.n_batch, a.n_req, ctas * kTWarps, Geo<MODE>::kD);
+  tl->grid = (unsigned)std::min<int64_t>(plan.n_tiles, ctas);
+  tl->search = plan.search;
   a.n_tiles = plan.n_tiles;
   a.D = plan.search ? plan.D : 0;
-  if (!plan.search) {
-    if (ctx) {
-      st = ensure_bound(ctx, plan.n_tiles + 1);
-      if (st != LV_OK) return st;
-      bound = ctx->d_bound;
-    } else if (plan.n_tiles + 1 > bound_cap) {
-      return LV_EINVAL;
-    }
-    const int64_t blocks = std::min<int64_t>(a.n_batch / 1024 + 1, (int64_t)sms * 16);
-    if (a.n_batch < (1ll << 32)) {
-      a.bound32 = static_cast<uint32_t *>(bound);
-      k_tile_bounds<uint32_t><<<(unsigned)blocks, 256, 0, stream>>>(a.off, a.n_batch, a.n_req, plan.n_tiles,
-                                                                    plan.magic, static_cast<uint32_t *>(bound),
-                                                                    a.status);
-    } else {
-      a.bound = static_cast<int64_t *>(bound);
-      k_tile_bounds<int64_t><<<(unsigned)blocks, 256, 0, stream>>>(a.off, a.n_batch, a.n_req, plan.n_tiles, plan.magic,
-                                                                   static_cast<int64_t *>(bound), a.status);
-    }
-    LV_CUDA(cudaGetLastError());
-  }
-  cudaEvent_t stop = nullptr;
+  if (plan.search) return LV_OK;
   if (ctx) {
-    st = timing_begin(ctx, LV_TIME_TILES, stream, &stop);
+    st = ensure_bound(ctx, plan.n_tiles + 1);
     if (st != LV_OK) return st;
+    bound = ctx->d_bound;
+  } else if (plan.n_tiles + 1 > bound_cap) {
+    return LV_EINVAL;
   }
-  const unsigned grid = (unsigned)std::min<int64_t>(plan.n_tiles, ctas);
-  if (plan.search) {
-    k_tiles<MODE><<<grid, kTThreads, smem, stream>>>(a);
+  const int64_t blocks = std::min<int64_t>(a.n_batch / 1024 + 1, (int64_t)sms * 16);
+  if (a.n_batch < (1ll << 32)) {
+    a.bound32 = static_cast<uint32_t *>(bound);
+    k_tile_bounds<uint32_t><<<(unsigned)blocks, 256, 0, stream>>>(a.off, a.n_batch, a.n_req, plan.n_tiles, plan.magic,
+                                                                  static_cast<uint32_t *>(bound), a.status);
+  } else {
+    a.bound = static_cast<int64_t *>(bound);
+    k_tile_bounds<int64_t><<<(unsigned)blocks, 256, 0, stream>>>(a.off, a.n_batch, a.n_req, plan.n_tiles, plan.magic,
+                                                                 static_cast<int64_t *>(bound), a.status);
+  }
+  LV_CUDA(cudaGetLastError());
+  return LV_OK;
+}
+
+template <int MODE>
+lv_status launch_tiles(lv_ctx *ctx, const TileArgs &a, const TileLaunch &tl, cudaStream_t stream) {
+  cudaEvent_t stop = nullptr;
+  lv_status st = ctx ? timing_begin(ctx, LV_TIME_TILES, stream, &stop) : LV_OK;
+  if (st != LV_OK) return st;
+  if (tl.search) {
+    k_tiles<MODE><<<tl.grid, kTThreads, tl.smem, stream>>>(a);
     LV_CUDA(cudaGetLastError());
   } else {
-    st = launch_after(k_tiles<MODE>, grid, kTThreads, smem, stream, a);
+    st = launch_after(k_tiles<MODE>, tl.grid, kTThreads, tl.smem, stream, a);
     if (st != LV_OK) return st;
   }
   return ctx ? timing_end(stop, stream) : LV_OK;
+}
+
+// Bounds and tile kernel for the given batches.
+template <int MODE>
+lv_status run_tiles_mode(lv_ctx *ctx, int sms, TileArgs &a, void *bound, int64_t bound_cap, cudaStream_t stream) {
+  TileLaunch tl;
+  const lv_status st = bound_tiles<MODE>(ctx, sms, a, bound, bound_cap, stream, &tl);
+  return st == LV_OK ? launch_tiles<MODE>(ctx, a, tl, stream) : st;
 }
 
 lv_status run_tiles(lv_ctx *ctx, TileArgs &a, int mode, cudaStream_t stream) {
@@ -454,7 +473,6 @@ lv_status run_tiles(lv_ctx *ctx, TileArgs &a, int mode, cudaStream_t stream) {
     case M_ATTR | M_F32: return run_tiles_mode<M_ATTR | M_F32>(ctx, sms, a, nullptr, 0, stream);
     case M_ATTR | M_TEN | M_F32: return run_tiles_mode<M_ATTR | M_TEN | M_F32>(ctx, sms, a, nullptr, 0, stream);
     case M_FEAT: return run_tiles_mode<M_FEAT>(ctx, sms, a, nullptr, 0, stream);
-    case M_FIT: return run_tiles_mode<M_FIT>(ctx, sms, a, nullptr, 0, stream);
     default: return LV_EINVAL;
   }
 }
@@ -576,14 +594,17 @@ lv_status fit_pass(lv_ctx *ctx, const lv_batches *b, const double *y, int32_t n_
   if (b->n_batch > 0 && (!y || !aligned(y, 8))) return LV_EINVAL;
   st = map_host(&ctx->h_fit, &ctx->hd_fit, sizeof(FitHost));
   if (st != LV_OK) return st;
-  // scratch: per-CTA partials, totals, each batch's sums and segment
+  // scratch: per-CTA partials, totals, a range's first and last batch, its batches' sums and segments
   const int NE = fit_entries(n_y), n_ent = 4 * NE;
   const int rows = std::max(1, 2 * ctx->sms / (1 + n_y));  // two CTAs per SM over the kinds of entry
-  const size_t nb = (size_t)b->n_batch;
+  const int64_t nb = b->n_batch;
+  const bool ranged = nb > kFitRange;
+  const int64_t stride = ranged ? kFitRange + Geo<M_FIT>::kNb : nb;  // a tile reaches past its range
   const size_t o_tot = ((size_t)rows * n_ent * sizeof(FitAcc) + 255) & ~(size_t)255;
-  const size_t o_feat = (o_tot + (size_t)n_ent * sizeof(FitAcc) + 255) & ~(size_t)255;
-  const size_t o_seg = o_feat + 4 * sizeof(int64_t) * nb;
-  const size_t need = o_seg + nb;
+  const size_t o_range = o_tot + (size_t)n_ent * sizeof(FitAcc);
+  const size_t o_feat = (o_range + 2 * sizeof(int64_t) + 255) & ~(size_t)255;
+  const size_t o_seg = o_feat + 4 * sizeof(int64_t) * (size_t)stride;
+  const size_t need = o_seg + (size_t)stride;
   if (need > ctx->fit_cap) {
     LV_CUDA(cudaDeviceSynchronize());
     if (ctx->d_fit) cudaFree(ctx->d_fit);
@@ -595,8 +616,6 @@ lv_status fit_pass(lv_ctx *ctx, const lv_batches *b, const double *y, int32_t n_
   unsigned char *base = static_cast<unsigned char *>(ctx->d_fit);
   FitAcc *partial = reinterpret_cast<FitAcc *>(base);
   FitAcc *totals = reinterpret_cast<FitAcc *>(base + o_tot);
-  int64_t *feat = reinterpret_cast<int64_t *>(base + o_feat);
-  uint8_t *seg = base + o_seg;
 
   TileArgs a{};
   a.p = b->p;
@@ -604,17 +623,31 @@ lv_status fit_pass(lv_ctx *ctx, const lv_batches *b, const double *y, int32_t n_
   a.ph = b->phase;
   a.off = b->offsets;
   a.n_req = b->n_req;
-  a.n_batch = b->n_batch;
+  a.n_batch = nb;
   a.status = ctx->d_status;
   a.mp.split[0] = split[0];
   a.mp.split[1] = split[1];
-  a.bfeat = feat;
-  a.bseg = seg;
-  st = run_tiles(ctx, a, M_FIT, stream);
-  if (st != LV_OK) return st;
-  st = launch_after(k_fit_gram, dim3((unsigned)rows, 1 + n_y), kGramThreads, 0, stream, feat, seg, b->n_batch, y, n_y,
-                    partial, ctx->d_status);
-  if (st != LV_OK) return st;
+  a.bfeat = reinterpret_cast<int64_t *>(base + o_feat);
+  a.bseg = base + o_seg;
+  a.f_stride = stride;
+  a.f_range = ranged ? reinterpret_cast<int64_t *>(base + o_range) : nullptr;
+  FitRange fr{a.bfeat, a.bseg, stride, 0, nb, a.f_range};
+  TileLaunch tl;
+  if (nb > 0) {
+    st = bound_tiles<M_FIT>(ctx, ctx->sms, a, nullptr, 0, stream, &tl);
+    if (st != LV_OK) return st;
+  }
+  for (int64_t lo = 0; lo == 0 || lo < nb; lo += kFitRange) {
+    a.f_lo = fr.lo = lo;
+    a.f_hi = std::min(nb, lo + kFitRange);
+    if (nb > 0) {
+      st = launch_tiles<M_FIT>(ctx, a, tl, stream);
+      if (st != LV_OK) return st;
+    }
+    st = launch_after(k_fit_gram, dim3((unsigned)rows, 1 + n_y), kGramThreads, 0, stream, fr, y, n_y, partial,
+                      ctx->d_status);
+    if (st != LV_OK) return st;
+  }
   st = launch_after(k_fit_reduce, n_ent, kFitRedThreads, 0, stream, partial, rows, n_ent, totals);
   if (st != LV_OK) return st;
   *totals_out = totals;

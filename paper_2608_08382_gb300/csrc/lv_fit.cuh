@@ -182,6 +182,20 @@ __device__ __forceinline__ void fit_y_add(FitYAcc &g, const Feat48 *x, i128 Y) {
   add_words<8>(g.yy, o);
 }
 
+// The batches of one launch.  Their sums and segments come from the tile kernel
+// through a scratch of bounded size, so a fit of more than kFitRange batches is
+// worked off in ranges of tiles that start in kFitRange batches each.  A range
+// of 2^22 costs two launches and a search of the tiles, about 15 us, against 0.6
+// ms for its batches' requests at 64 each, and 138 MB.
+constexpr int64_t kFitRange = 1ll << 22;
+struct FitRange {
+  const int64_t *feat;   // [4][stride] S1, S2, S3, n of batches lo and up
+  const uint8_t *seg;    // [stride]
+  int64_t stride, lo;
+  int64_t n_batch;       // of the whole input (y's rows)
+  const int64_t *range;  // first batch and the one past the last, from lo; null: all
+};
+
 struct GramSmem {
   int64_t queue[kGramWarps][32 * (kGramScan + 1)];
   FitAcc part[kGramWarps][kGramMax];
@@ -189,15 +203,17 @@ struct GramSmem {
 
 // kGram: the Gram matrix and the flag, else the latency vector k.
 template <bool kGram>
-__device__ __forceinline__ void fit_rows(GramSmem &sm, const int64_t *feat, const uint8_t *seg, int64_t nb,
-                                         const double *__restrict__ y, int n_y, int k, FitAcc *__restrict__ partial,
-                                         int *status) {
+__device__ __forceinline__ void fit_rows(GramSmem &sm, const FitRange &fr, const double *__restrict__ y, int n_y,
+                                         int k, FitAcc *__restrict__ partial, int *status) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int NE = fit_entries(n_y);
   const int64_t stride = (int64_t)gridDim.x * kGramWarps * kGramScan * 32;
   int64_t *q = sm.queue[wid];
   int bad = 0;
-  const double *yk = y + (int64_t)k * nb;
+  const int64_t *feat = fr.feat;
+  const uint8_t *seg = fr.seg;
+  const int64_t fs = fr.stride, first = fr.range ? fr.range[0] : 0, nb = fr.range ? fr.range[1] : fr.n_batch;
+  const double *yk = y + (int64_t)k * fr.n_batch + fr.lo;
   int s[kGramScan];
   auto scan = [&](int64_t i0) {  // segments of kGramScan rows of 32 batches, their loads in flight together
 #pragma unroll
@@ -229,7 +245,7 @@ __device__ __forceinline__ void fit_rows(GramSmem &sm, const int64_t *feat, cons
       }
     };
     int qn = 0;
-    int64_t i0 = ((int64_t)blockIdx.x * kGramWarps + wid) * kGramScan * 32;
+    int64_t i0 = first + ((int64_t)blockIdx.x * kGramWarps + wid) * kGramScan * 32;
     scan(i0);
     while (i0 < nb || qn > 0) {
       const bool rest = i0 >= nb;  // no batches left: work off the queue
@@ -252,9 +268,9 @@ __device__ __forceinline__ void fit_rows(GramSmem &sm, const int64_t *feat, cons
         if (lane < take) {
           const int64_t b = q[qn - take + lane];
           nx.s1 = feat[b];
-          nx.s2 = feat[nb + b];
-          nx.s3 = feat[2 * nb + b];
-          nx.n = feat[3 * nb + b];
+          nx.s2 = feat[fs + b];
+          nx.s3 = feat[2 * fs + b];
+          nx.n = feat[3 * fs + b];
           if (!kGram) nx.y = yk[b];
         }
         qn -= take;
@@ -284,7 +300,13 @@ __device__ __forceinline__ void fit_rows(GramSmem &sm, const int64_t *feat, cons
     if ((int)threadIdx.x < ne) {
       const int e = threadIdx.x;
       const bool is_flag = kGram && e == 15;
+      const int at = kGram ? (is_flag ? NE - 1 : e) : e < 5 ? 15 + 5 * k + e : 15 + 5 * n_y + k;
+      FitAcc *out = partial + (int64_t)blockIdx.x * (4 * NE) + g * NE + at;
       FitAcc s{{0ull, 0ull, 0ull, 0ull}};
+      if (fr.lo > 0) {  // added to what the ranges before gave
+#pragma unroll
+        for (int w = 0; w < 4; ++w) s.w[w] = __ldcg(reinterpret_cast<unsigned long long *>(out->w) + w);
+      }
       for (int w = 0; w < kGramWarps; ++w) {
         const FitAcc &v = sm.part[w][e];
         if (is_flag)
@@ -292,8 +314,7 @@ __device__ __forceinline__ void fit_rows(GramSmem &sm, const int64_t *feat, cons
         else
           acc_add256(s.w, v.w[0], v.w[1], v.w[2], v.w[3]);
       }
-      const int at = kGram ? (is_flag ? NE - 1 : e) : e < 5 ? 15 + 5 * k + e : 15 + 5 * n_y + k;
-      partial[(int64_t)blockIdx.x * (4 * NE) + g * NE + at] = s;
+      *out = s;
     }
     __syncthreads();
   }
@@ -301,15 +322,14 @@ __device__ __forceinline__ void fit_rows(GramSmem &sm, const int64_t *feat, cons
 }
 
 __global__ void __launch_bounds__(kGramThreads, 2)
-    k_fit_gram(const int64_t *feat, const uint8_t *seg, int64_t nb, const double *__restrict__ y, int n_y,
-               FitAcc *__restrict__ partial, int *status) {
+    k_fit_gram(const FitRange fr, const double *__restrict__ y, int n_y, FitAcc *__restrict__ partial, int *status) {
   __shared__ GramSmem sm;
   let_next();
   wait_previous();
   if (blockIdx.y == 0)
-    fit_rows<true>(sm, feat, seg, nb, y, n_y, 0, partial, status);
+    fit_rows<true>(sm, fr, y, n_y, 0, partial, status);
   else
-    fit_rows<false>(sm, feat, seg, nb, y, n_y, (int)blockIdx.y - 1, partial, status);
+    fit_rows<false>(sm, fr, y, n_y, (int)blockIdx.y - 1, partial, status);
 }
 
 // ---------------------------------------------------------------- reduction across CTAs

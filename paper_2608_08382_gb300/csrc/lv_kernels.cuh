@@ -97,8 +97,10 @@ struct TileArgs {
   int64_t D;             // merge positions per tile where the warps find their bounds themselves, or 0
   double *T, *share;
   float *T32, *share32;  // fp32 variant (M_F32): T and shares as float, or null
-  int64_t *bfeat;   // [5][n_batch] or null; M_FIT: [4][n_batch] S1, S2, S3, n
-  uint8_t *bseg;    // [n_batch] or null; M_FIT: 255 for an empty batch
+  int64_t *bfeat;   // [5][n_batch] or null; M_FIT: [4][f_stride] S1, S2, S3, n of batches f_lo and up
+  uint8_t *bseg;    // [n_batch] or null; M_FIT: 255 for an empty batch, from f_lo
+  int64_t f_lo, f_hi, f_stride;  // M_FIT: the tiles that start in batches [f_lo, f_hi)
+  int64_t *f_range;  // M_FIT: their first batch and the one past their last, from f_lo; null: all batches
   unsigned long long *ten_pend;  // [n_tenants][4] 32-bit limbs in 64-bit words, or null
   i128 *ten_state;               // the tenants' exact state where the kernel folds it, or null
   unsigned *ten_ticket;          // CTAs done (zero between launches)

@@ -158,20 +158,17 @@ __device__ __forceinline__ int64_t tile_bound(const TileArgs &a, int64_t t) {
   return a.bound32 ? (int64_t)a.bound32[t] : a.bound[t];
 }
 
-// The bounds of tile t by a warp's own search, for inputs of at most one tile
-// per warp: 16 offsets are looked at per round and bound, so 20,000 batches
-// take four rounds of one load each, less than k_tile_bounds and the gap after
-// it.  (Lanes 0..15 look for bound t, the others for t + 1.)
-__device__ __forceinline__ void tile_search(const TileArgs &a, int64_t t, int lane, int64_t *b0, int64_t *b1) {
+// The smallest m in [lo, hi] for which at(m) holds (hi where none does), for
+// two searches by a warp at once: lanes 0..15 make the first, the others the
+// second.  16 values are looked at per round and search.
+template <class F>
+__device__ __forceinline__ int64_t half_warp_search(int lane, int64_t lo, int64_t hi, F &&at) {
   const int half = lane >> 4, l = lane & 15;
-  const int64_t target = (t + half) * a.D;
-  int64_t lo = 0, hi = a.n_batch;  // the bound is in [lo, hi]; tile n_tiles ends at n_batch
-  if (t + half >= a.n_tiles) lo = hi;
   while (__any_sync(kFull, lo < hi)) {
     const int64_t m = lo + (((hi - lo) * l) >> 4);
-    const bool at = lo >= hi || kTW * m + clampi(a.off[m], 0, a.n_req) >= target;
-    const uint32_t bal = (__ballot_sync(kFull, at) >> (16 * half)) & 0xffffu;
-    const int c = bal ? __ffs(bal) - 1 : 16;  // the first c probes lie before the bound
+    const bool in = lo >= hi || at(m);
+    const uint32_t bal = (__ballot_sync(kFull, in) >> (16 * half)) & 0xffffu;
+    const int c = bal ? __ffs(bal) - 1 : 16;  // the first c probes lie before the result
     const int64_t before = __shfl_sync(kFull, m, 16 * half + max(c - 1, 0)),
                   after = __shfl_sync(kFull, m, 16 * half + min(c, 15));
     if (lo < hi) {
@@ -179,8 +176,19 @@ __device__ __forceinline__ void tile_search(const TileArgs &a, int64_t t, int la
       lo = c > 0 ? before + 1 : hi;
     }
   }
-  *b0 = __shfl_sync(kFull, lo, 0);
-  *b1 = __shfl_sync(kFull, lo, 16);
+  return lo;
+}
+
+// The bounds of tile t by a warp's own search, for inputs of at most one tile
+// per warp: 20,000 batches take four rounds of one load each, less than
+// k_tile_bounds and the gap after it.
+__device__ __forceinline__ void tile_search(const TileArgs &a, int64_t t, int lane, int64_t *b0, int64_t *b1) {
+  const int64_t tile = t + (lane >> 4), target = tile * a.D;
+  const int64_t b = half_warp_search(lane, tile < a.n_tiles ? 0 : a.n_batch, a.n_batch, [&](int64_t m) {
+    return kTW * m + clampi(a.off[m], 0, a.n_req) >= target;
+  });  // tile n_tiles ends at n_batch
+  *b0 = __shfl_sync(kFull, b, 0);
+  *b1 = __shfl_sync(kFull, b, 16);
 }
 
 // ---------------------------------------------------------------- loads
@@ -358,11 +366,12 @@ __device__ __forceinline__ void tile_emit(const TileArgs &a, const TSmem<MODE> &
   } else if ((MODE & M_ATTR) && (MODE & M_FIX)) {
     if (a.T) a.T[b] = eq1_exact(a.mp, ts.fx[s], ts.seg[s].t32, s, g);
   } else if (MODE & M_FIT) {
-    a.bfeat[b] = g.s1;
-    a.bfeat[a.n_batch + b] = g.s2;
-    a.bfeat[2 * a.n_batch + b] = g.s3;
-    a.bfeat[3 * a.n_batch + b] = g.n;
-    a.bseg[b] = g.n > 0 ? (uint8_t)s : (uint8_t)255;
+    const int64_t i = b - a.f_lo;
+    a.bfeat[i] = g.s1;
+    a.bfeat[a.f_stride + i] = g.s2;
+    a.bfeat[2 * a.f_stride + i] = g.s3;
+    a.bfeat[3 * a.f_stride + i] = g.n;
+    a.bseg[i] = g.n > 0 ? (uint8_t)s : (uint8_t)255;
   } else {
     emit_batch<MODE>(a, b, g, s, nullptr);
   }
@@ -686,8 +695,21 @@ __global__ void __launch_bounds__(kTThreads, 1) k_tiles(const TileArgs a) {
   // tile t's batches [b0, b1) and requests [r0, r1) are fetched while the tile
   // before it is worked on
   const int64_t stride = (int64_t)gridDim.x * kTWarps;
-  int64_t t = (int64_t)wid * gridDim.x + blockIdx.x;
+  int64_t t = (int64_t)wid * gridDim.x + blockIdx.x, t_end = a.n_tiles;
   int64_t b0 = 0, b1 = 0, r0 = 0, r1 = 0;
+  // a fit of many batches: the tiles whose first batch is in the range
+  const bool ranged = (MODE & M_FIT) && a.f_range != nullptr;
+  if (ranged) {
+    const int64_t from = lane < 16 ? a.f_lo : a.f_hi;
+    const int64_t x = half_warp_search(lane, 0, a.n_tiles, [&](int64_t m) { return tile_bound(a, m) >= from; });
+    const int64_t t_lo = __shfl_sync(kFull, x, 0);
+    t_end = __shfl_sync(kFull, x, 16);
+    t += t_lo;
+    if (blockIdx.x == 0 && tid == 0) {
+      a.f_range[0] = clampi(tile_bound(a, t_lo) - a.f_lo, 0, a.f_stride);
+      a.f_range[1] = clampi(tile_bound(a, t_end) - a.f_lo, a.f_range[0], a.f_stride);
+    }
+  }
   if (a.D) {
     // k_tile_bounds' checks of the offsets
     const int64_t threads = (int64_t)gridDim.x * kTThreads;
@@ -695,22 +717,22 @@ __global__ void __launch_bounds__(kTThreads, 1) k_tiles(const TileArgs a) {
       if (a.off[i] > a.off[i + 1]) bad = 1;
     if (blockIdx.x == 0 && tid == 0 && (a.off[0] != 0 || a.off[a.n_batch] != a.n_req)) bad = 1;
   }
-  if (t < a.n_tiles) {
+  if (t < t_end) {
     if (a.D) {
       tile_search(a, t, lane, &b0, &b1);
     } else {
       b0 = tile_bound(a, t);
       b1 = tile_bound(a, t + 1);
     }
-    b0 = clampi(b0, 0, a.n_batch);
+    b0 = clampi(b0, ranged ? a.f_lo : 0, ranged ? a.f_hi : a.n_batch);
     b1 = clampi(b1, b0, a.n_batch);
     r0 = clampi(a.off[b0], 0, a.n_req);
     r1 = clampi(a.off[b1], r0, a.n_req);
   }
-  while (t < a.n_tiles) {
+  while (t < t_end) {
     const int64_t tn = t + stride;
     int64_t n0 = 0, n1 = 0;
-    if (tn < a.n_tiles) {
+    if (tn < t_end) {
       n0 = tile_bound(a, tn);
       n1 = tile_bound(a, tn + 1);
     }
@@ -742,7 +764,7 @@ __global__ void __launch_bounds__(kTThreads, 1) k_tiles(const TileArgs a) {
     }
     const bool wide = tile_prefix(wt, src, cnt, lane);
     __syncwarp();
-    n0 = clampi(n0, 0, a.n_batch);
+    n0 = clampi(n0, ranged ? a.f_lo : 0, ranged ? a.f_hi : a.n_batch);
     n1 = clampi(n1, n0, a.n_batch);
     int64_t nr0 = a.off[n0], nr1 = a.off[n1];
 

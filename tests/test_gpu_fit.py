@@ -217,3 +217,37 @@ def test_status_of_a_failed_fit_is_its_own(lv, ctx):
         again, _ = _gpu_fit(lv, ctx, w.offsets, w.p, w.c, w.phase, T, w.split)
         assert np.array_equal(again, good, equal_nan=True)
         assert lv.lv_fit_vtc(ctx, b, torch.as_tensor(T[None], device="cuda")) == vtc
+
+
+@pytest.mark.parametrize("n_base,n_y", [(1_100_003, 2), (5_000_001, 1)])
+def test_fit_in_ranges_of_batches(lv, n_base, n_y):
+    """A fit of many batches is worked off in ranges of them.  The same batches four times over (18e6 and more with
+    requests of their own) have four times the normal equations, a power of two in every scaled entry, so the
+    coefficients agree bit for bit however the ranges cut them; and the context's scratch does not grow with them."""
+    import torch
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n_base)
+    size = torch.randint(0, 4, (n_base,), generator=g, device="cuda")
+    m = int(size.sum())
+    ph = torch.repeat_interleave((torch.rand(n_base, generator=g, device="cuda") < 0.4).int(), size)
+    p = torch.randint(1, 300, (m,), generator=g, device="cuda").int()
+    c = torch.randint(0, 9000, (m,), generator=g, device="cuda").int()
+    y = torch.rand((n_y, n_base), generator=g, device="cuda", dtype=torch.float64) + 1e-3
+    ctx, out = lv.Context(), []
+    torch.cuda.synchronize()
+    for k in (1, 4):
+        off = torch.cat([torch.zeros(1, dtype=torch.int64, device="cuda"), torch.cumsum(size.repeat(k), 0)])
+        b = lv.Batches(p.repeat(k), c.repeat(k), ph.repeat(k), off)
+        yk = y.repeat(1, k).contiguous()
+        models = [lv.make_model(np.full((4, 5), np.nan), (150, 200)) for _ in range(n_y)]
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        reps = lv.lv_fit(ctx, b, yk, models)
+        assert free - torch.cuda.mem_get_info()[0] < 200 << 20
+        out.append(([lv.model_coef(v) for v in models], reps))
+    (c1, r1), (c4, r4) = out
+    for a, b in zip(c1, c4):
+        assert np.all(np.isfinite(a)) and np.array_equal(a.view(np.int64), b.view(np.int64))
+    for a, b in zip(r1, r4):
+        assert [4 * v for v in a["n"]] == b["n"] and a["dropped"] == b["dropped"] and a["r2"] == b["r2"]
+        assert a["status"] == b["status"] == [0] * 4 and [4 * v for v in a["ssr"]] == b["ssr"]
