@@ -596,7 +596,7 @@ lv_status fit_pass(lv_ctx *ctx, const lv_batches *b, const double *y, int32_t n_
   if (st != LV_OK) return st;
   // scratch: per-CTA partials, totals, a range's first and last batch, its batches' sums and segments
   const int NE = fit_entries(n_y), n_ent = 4 * NE;
-  const int rows = std::max(1, 2 * ctx->sms / (1 + n_y));  // two CTAs per SM over the kinds of entry
+  const int rows = std::max(kGramMinRows, 2 * ctx->sms / (1 + n_y));  // two CTAs per SM over the kinds of entry
   const int64_t nb = b->n_batch;
   const bool ranged = nb > kFitRange;
   const int64_t stride = ranged ? kFitRange + Geo<M_FIT>::kNb : nb;  // a tile reaches past its range

@@ -7,8 +7,9 @@
 // matrix X^T X and X^T y per group.  Both are accumulated EXACTLY:
 //   - X^T X in 128-bit integers (features are integers below 2^48, so each
 //     product is below 2^96);
-//   - X^T y in 256-bit fixed point with y rounded to a multiple of 2^-100 s
-//     (exact for any latency whose lowest bit is at least 2^-100 s).
+//   - X^T y in fixed point with y rounded to a multiple of 2^-100 s (exact for any
+//     latency whose lowest bit is at least 2^-100 s), in 256 bits: a lane's and a
+//     warp's sums in 192, which hold a launch's share of the batches.
 // The tile kernel writes each batch's sums and segment, and k_fit_gram adds the
 // products with one lane per batch.  CTA partials are reduced exactly (integer
 // adds) and each group's small system is solved in double-double (about
@@ -188,6 +189,13 @@ __device__ __forceinline__ void fit_y_add(FitYAcc &g, const Feat48 *x, i128 Y) {
 // of 2^22 costs two launches and a search of the tiles, about 15 us, against 0.6
 // ms for its batches' requests at 64 each, and 138 MB.
 constexpr int64_t kFitRange = 1ll << 22;
+// Rows of blocks, at least.  A product of a feature (below 2^48) and a latency
+// (2^100 y, below 2^125) is below 2^173, so a warp's signed sum in 192 bits holds
+// 2^18 of them; with this many rows a warp meets fewer than 2^17 + 2^10 batches
+// of a range (the tiles that start in it reach less than 2^10 past it), rounded
+// up to its turns of 2^8.
+constexpr int kGramMinRows = 4;
+static_assert(kFitRange / (kGramMinRows * kGramWarps) + (1 << 11) < (1 << 18), "X^T y of a warp fits 192 bits");
 struct FitRange {
   const int64_t *feat;   // [4][stride] S1, S2, S3, n of batches lo and up
   const uint8_t *seg;    // [stride]

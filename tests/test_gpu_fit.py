@@ -251,3 +251,37 @@ def test_fit_in_ranges_of_batches(lv, n_base, n_y):
     for a, b in zip(r1, r4):
         assert [4 * v for v in a["n"]] == b["n"] and a["dropped"] == b["dropped"] and a["r2"] == b["r2"]
         assert a["status"] == b["status"] == [0] * 4 and [4 * v for v in a["ssr"]] == b["ssr"]
+
+
+def test_fit_of_many_extreme_batches(lv):
+    """X^T y stays exact at the limits that lv_fit states: 1.4e8 batches of one request of 2^24 - 1 tokens (S3 just
+    below 2^48) and a latency just below 2^25 s reach 2^200 in units of 2^-100 s.  With 64 ordinary batches the
+    normal equations are solved exactly from one row of each kind."""
+    import torch
+    from fractions import Fraction
+    from oracle.fit import _solve_exact
+    rng = np.random.default_rng(77)
+    big, p_big, y_big, few = 140_000_000, (1 << 24) - 1, 2.0 ** 25 - 0.75, 64
+    sizes = rng.integers(1, 7, few)
+    m = int(sizes.sum())
+    p, c = rng.integers(1, 1 << 20, m).astype(np.int32), rng.integers(0, 1 << 30, m).astype(np.int32)
+    c[:3] = 0
+    y = rng.uniform(1.0, 10.0, few)
+    d = lambda a: torch.as_tensor(a, device="cuda")  # noqa: E731
+    full = lambda v, t: torch.full((big,), v, dtype=t, device="cuda")  # noqa: E731
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    doff = torch.cat([d(off), m + 1 + torch.arange(big, device="cuda")])
+    b = lv.Batches(torch.cat([d(p), full(p_big, torch.int32)]), torch.cat([d(c), full(0, torch.int32)]),
+                   torch.ones(m + big, dtype=torch.int32, device="cuda"), doff)
+    yd = torch.cat([d(y), full(y_big, torch.float64)]).repeat(4, 1)
+    models = [lv.make_model(np.full((4, 5), np.nan), (1 << 40, 1 << 40)) for _ in range(4)]
+    reps = lv.lv_fit(lv.Context(), b, yd, models)
+    feat, _ = oracle.batch_features(off, p, c, np.ones(m, np.int32), (1 << 40, 1 << 40))
+    rows = [([1] + [int(v) for v in feat[[0, 1, 2, 4], k]], Fraction(y[k]), 1) for k in range(few)]
+    rows.append(([1, p_big, 0, p_big * p_big, 1], Fraction(y_big), big))
+    G = [[sum(w * x[i] * x[j] for x, _, w in rows) for j in range(5)] for i in range(5)]
+    want = [float(v) for v in _solve_exact(G, [sum(w * x[i] * t for x, t, w in rows) for i in range(5)])]
+    for k in range(4):
+        assert reps[k]["status"][2] == lv.LV_OK and reps[k]["n"][2] == big + few
+        got = lv.model_coef(models[k])[2]
+        assert np.max(np.abs(got - want) / np.abs(want)) <= COEF_TOL, (got, want)
