@@ -131,8 +131,8 @@ typedef struct lv_tenant_acc lv_tenant_acc;
 #define LV_ARITH_FP64 1
 
 /* Create a context on the current CUDA device.  It owns a device scratch area
- * that its calls grow to the largest input they have seen and keep (the first
- * batch of each tile of about 1,200 to 2,500 requests, 4 bytes; lv_whatif: 192
+ * that its calls grow to the largest input they have seen and keep (the tile
+ * pass: about 1 byte per 150 requests and batches; lv_whatif: 192
  * bytes a candidate; lv_fit: 33 bytes a batch, for 2^22 batches at most, 138 MB;
  * lv_accuracy: about 20 bytes a batch) and a sticky status word.  Returns
  * LV_ECUDA/LV_ENOMEM on failure. */
@@ -338,7 +338,7 @@ lv_status lv_whatif_admit(lv_ctx *ctx, const lv_model *model, const lv_batches *
  * Computes exactly what lv_attribute computes for T and share (no tenant
  * accumulation), with default arithmetic, using instead of an lv_ctx a fixed
  * scratch area that lives in the library image as a static device array
- * (about 2.3 MB on every GPU that loads the library, held until the process
+ * (about 2.5 MB on every GPU that loads the library, held until the process
  * exits).  It calls no cudaMalloc, cudaFree or other allocating routine.
  *  - Limit: n_batch + n_req must not exceed 67,108,864; larger inputs return
  *    LV_EINVAL before anything is launched.

@@ -35,8 +35,8 @@ struct lv_ctx {
   int sms = 0;
   int arith = LV_ARITH_AUTO;
   int *d_status = nullptr;
-  int64_t *d_bound = nullptr;  // first batch of each tile (k_tiles)
-  int64_t bound_cap = 0;
+  unsigned char *d_bound = nullptr;  // k_tiles' queue counters (zero between calls), first batch of each tile, queue
+  size_t bound_cap = 0;
   KEntry *d_ktab = nullptr;
   int ktab_nk = 0;
   bool ktab_valid = false;
@@ -80,6 +80,14 @@ struct lv_tenant_acc {
 namespace {
 
 constexpr int kKTableN = kTabN;
+constexpr size_t kBoundHead = 64;  // bytes of the queue's counters before the tiles' bounds
+static_assert(kQueueWords * sizeof(unsigned) <= kBoundHead, "queue counters");
+
+// Most batches that no tile of the mode holds.
+template <int MODE>
+constexpr int64_t queue_room(int64_t n_req) {
+  return n_req / (Geo<MODE>::kCap + 1) + 1;
+}
 
 #define LV_CUDA(call)                          \
   do {                                         \
@@ -379,18 +387,44 @@ lv_status tiles_occupancy(lv_ctx *ctx, size_t smem, int *per_sm) {
   return LV_OK;
 }
 
-lv_status ensure_bound(lv_ctx *ctx, int64_t n) {
-  if (n <= ctx->bound_cap) return LV_OK;
+lv_status ensure_bound(lv_ctx *ctx, size_t bytes) {
+  if (bytes <= ctx->bound_cap) return LV_OK;
   LV_CUDA(cudaDeviceSynchronize());
   if (ctx->d_bound) cudaFree(ctx->d_bound);
   ctx->d_bound = nullptr;
   ctx->bound_cap = 0;
-  const int64_t cap = std::max<int64_t>(n, 1 << 16);
-  if (cudaMalloc(&ctx->d_bound, cap * sizeof(int64_t)) != cudaSuccess) {
+  const size_t cap = std::max<size_t>(bytes, 1 << 19);
+  if (cudaMalloc(&ctx->d_bound, cap) != cudaSuccess) {
     ctx->d_bound = nullptr;
     return LV_ENOMEM;
   }
+  LV_CUDA(cudaMemset(ctx->d_bound, 0, kBoundHead));
+  LV_CUDA(cudaDeviceSynchronize());
   ctx->bound_cap = cap;
+  return LV_OK;
+}
+
+// Launches k_tile_bounds into scratch of [counters][bounds][queue], in 32 or 64
+// bits; queue_cap: entries of the queue, or 0.
+template <class V>
+lv_status launch_bounds(const TilePlan &plan, TileArgs &a, unsigned char *scratch, int64_t queue_cap, int64_t most,
+                        int sms, cudaStream_t stream) {
+  V *bound = reinterpret_cast<V *>(scratch + kBoundHead);
+  TileQueue<V> q{nullptr, 0, INT64_MAX, nullptr};
+  if (queue_cap > 0) {
+    q = TileQueue<V>{bound + plan.n_tiles + 1, queue_cap, most, reinterpret_cast<unsigned *>(scratch)};
+    a.queue = q.queue;
+    a.queue_cap = queue_cap;
+    a.queue_ctr = q.ctr;
+  }
+  if (sizeof(V) == 4)
+    a.bound32 = reinterpret_cast<const uint32_t *>(bound);
+  else
+    a.bound = reinterpret_cast<const int64_t *>(bound);
+  const int64_t blocks = std::min<int64_t>(a.n_batch / 1024 + 1, (int64_t)sms * 16);
+  k_tile_bounds<V><<<(unsigned)blocks, 256, 0, stream>>>(a.off, a.n_batch, a.n_req, plan.n_tiles, plan.magic, bound, q,
+                                                         a.status);
+  LV_CUDA(cudaGetLastError());
   return LV_OK;
 }
 
@@ -401,12 +435,13 @@ struct TileLaunch {
   bool search;
 };
 
-// Tiles of the given batches and, unless the warps find them, their bounds.
-// Without a context, `bound` has room for the tiles' bounds (bound_cap 32-bit
-// entries).
+// Tiles of the given batches and, unless the warps find them, their bounds and
+// the queue of the batches that no tile holds (not for a fit in ranges, whose
+// launches would each have to pick theirs).  Without a context, `scratch` holds
+// scratch_cap bytes.
 template <int MODE>
-lv_status bound_tiles(lv_ctx *ctx, int sms, TileArgs &a, void *bound, int64_t bound_cap, cudaStream_t stream,
-                      TileLaunch *tl) {
+lv_status bound_tiles(lv_ctx *ctx, int sms, TileArgs &a, unsigned char *scratch, size_t scratch_cap,
+                      cudaStream_t stream, TileLaunch *tl) {
   tl->smem = sizeof(TSmem<MODE>) + ((MODE & M_TEN) ? ten_table_bytes(kHotMax) : 0);
   int per_sm = 0;
   lv_status st = tiles_occupancy<MODE>(ctx, tl->smem, &per_sm);
@@ -418,25 +453,19 @@ lv_status bound_tiles(lv_ctx *ctx, int sms, TileArgs &a, void *bound, int64_t bo
   a.n_tiles = plan.n_tiles;
   a.D = plan.search ? plan.D : 0;
   if (plan.search) return LV_OK;
+  const bool narrow = a.n_batch < (1ll << 32);
+  const int64_t queue_cap = a.f_range ? 0 : queue_room<MODE>(a.n_req);
+  const size_t need = kBoundHead + (narrow ? sizeof(uint32_t) : sizeof(int64_t)) * (size_t)(plan.n_tiles + 1 + queue_cap);
   if (ctx) {
-    st = ensure_bound(ctx, plan.n_tiles + 1);
+    st = ensure_bound(ctx, need);
     if (st != LV_OK) return st;
-    bound = ctx->d_bound;
-  } else if (plan.n_tiles + 1 > bound_cap) {
+    scratch = ctx->d_bound;
+  } else if (need > scratch_cap || !narrow) {
     return LV_EINVAL;
   }
-  const int64_t blocks = std::min<int64_t>(a.n_batch / 1024 + 1, (int64_t)sms * 16);
-  if (a.n_batch < (1ll << 32)) {
-    a.bound32 = static_cast<uint32_t *>(bound);
-    k_tile_bounds<uint32_t><<<(unsigned)blocks, 256, 0, stream>>>(a.off, a.n_batch, a.n_req, plan.n_tiles, plan.magic,
-                                                                  static_cast<uint32_t *>(bound), a.status);
-  } else {
-    a.bound = static_cast<int64_t *>(bound);
-    k_tile_bounds<int64_t><<<(unsigned)blocks, 256, 0, stream>>>(a.off, a.n_batch, a.n_req, plan.n_tiles, plan.magic,
-                                                                 static_cast<int64_t *>(bound), a.status);
-  }
-  LV_CUDA(cudaGetLastError());
-  return LV_OK;
+  const int64_t most = Geo<MODE>::kCap;
+  return narrow ? launch_bounds<uint32_t>(plan, a, scratch, queue_cap, most, sms, stream)
+                : launch_bounds<int64_t>(plan, a, scratch, queue_cap, most, sms, stream);
 }
 
 template <int MODE>
@@ -456,9 +485,10 @@ lv_status launch_tiles(lv_ctx *ctx, const TileArgs &a, const TileLaunch &tl, cud
 
 // Bounds and tile kernel for the given batches.
 template <int MODE>
-lv_status run_tiles_mode(lv_ctx *ctx, int sms, TileArgs &a, void *bound, int64_t bound_cap, cudaStream_t stream) {
+lv_status run_tiles_mode(lv_ctx *ctx, int sms, TileArgs &a, unsigned char *scratch, size_t scratch_cap,
+                         cudaStream_t stream) {
   TileLaunch tl;
-  const lv_status st = bound_tiles<MODE>(ctx, sms, a, bound, bound_cap, stream, &tl);
+  const lv_status st = bound_tiles<MODE>(ctx, sms, a, scratch, scratch_cap, stream, &tl);
   return st == LV_OK ? launch_tiles<MODE>(ctx, a, tl, stream) : st;
 }
 
@@ -1316,10 +1346,12 @@ namespace {
 constexpr int64_t kNoAllocMaxUnits = 65536 * 1024;  // n_batch + n_req
 // most tiles: every unit an empty batch, and a partial round of 32 warps on each of 256 SMs
 constexpr int64_t kNoAllocBounds = kTW * kNoAllocMaxUnits / Geo<M_ATTR>::kD + 32 * 256 + 2;
-constexpr size_t kNoAllocTabOffset = (sizeof(uint32_t) * (size_t)kNoAllocBounds + 255) & ~(size_t)255;
+constexpr size_t kNoAllocTiles =
+    kBoundHead + sizeof(uint32_t) * (size_t)(kNoAllocBounds + queue_room<M_ATTR>(kNoAllocMaxUnits));
+constexpr size_t kNoAllocTabOffset = (kNoAllocTiles + 255) & ~(size_t)255;
 constexpr size_t kNoAllocBytes = kNoAllocTabOffset + sizeof(KEntry) * 4 * (kKTableN + 1);
-// the size stated in include/llmvisor.h ("about 2.3 MB")
-static_assert(kNoAllocBytes > 2250000 && kNoAllocBytes < 2350000, "no-alloc scratch size as documented");
+// the size stated in include/llmvisor.h ("about 2.5 MB")
+static_assert(kNoAllocBytes > 2450000 && kNoAllocBytes < 2550000, "no-alloc scratch size as documented");
 
 }  // namespace
 
@@ -1392,6 +1424,7 @@ extern "C" lv_status lv_attribute_noalloc(const lv_model *model, const lv_batche
   a.status = status;
   a.mp = mp;
   static_assert(kNoAllocMaxUnits < (1ll << 32), "32-bit tile bounds");
-  return mp.fixed ? run_tiles_mode<M_ATTR | M_FIX>(nullptr, sms, a, scratch, kNoAllocBounds, stream)
-                  : run_tiles_mode<M_ATTR>(nullptr, sms, a, scratch, kNoAllocBounds, stream);
+  unsigned char *tiles = static_cast<unsigned char *>(scratch);  // its counters start at zero, as static memory does
+  return mp.fixed ? run_tiles_mode<M_ATTR | M_FIX>(nullptr, sms, a, tiles, kNoAllocTiles, stream)
+                  : run_tiles_mode<M_ATTR>(nullptr, sms, a, tiles, kNoAllocTiles, stream);
 }

@@ -87,6 +87,10 @@ __device__ __forceinline__ i128 y_fixed(double y, bool *ovf) {
   return double_to_fix(y, kFitYLsb, ovf);
 }
 
+// Counters of the queue of batches that no tile holds: medium and large ones
+// queued, medium and large ones taken, CTAs done with it.
+enum : int { kQMedium, kQLarge, kQTakenM, kQTakenL, kQDone, kQueueWords };
+
 struct TileArgs {
   const int32_t *p, *c, *ph, *ten;
   const int64_t *off;
@@ -95,6 +99,11 @@ struct TileArgs {
   const uint32_t *bound32;  // the same in 32 bits (fewer than 2^32 batches)
   int64_t n_tiles;
   int64_t D;             // merge positions per tile where the warps find their bounds themselves, or 0
+  // batches that no tile holds, found with the bounds (null: none are queued): the
+  // medium ones from the front, the large ones from the back, in the bounds' type
+  const void *queue;
+  int64_t queue_cap;
+  unsigned *queue_ctr;   // [kQueueWords], zero between calls
   double *T, *share;
   float *T32, *share32;  // fp32 variant (M_F32): T and shares as float, or null
   int64_t *bfeat;   // [5][n_batch] or null; M_FIT: [4][f_stride] S1, S2, S3, n of batches f_lo and up

@@ -118,3 +118,96 @@ def test_offsets_out_of_order_are_seen(lv, ctx, at):
         o[at] = off[at] if bad is None else bad
         lv.lv_features(ctx, lv.batches_to_device(one, zero, zero, o), model=model, batch_feat=feat, batch_seg=seg)
         assert ctx.status() == (lv.LV_OK if bad is None else lv.LV_EDATA)
+
+
+def _queued(kind):
+    """Sizes of an input of more than one tile per warp (3.8e6 positions) with batches that no tile holds."""
+    rng = np.random.default_rng(50)
+    small = rng.integers(0, 9, 460_000)
+    edges = np.array([1533, 1536, 1537, 1540, 8191, 8192, 8193, 65_535, 65_536, 65_537, 100_001])
+    if kind == "few":
+        s = np.concatenate([small, edges, rng.integers(1500, 70_000, 20)])
+    elif kind == "medium":
+        s = rng.integers(1500, 1800, 3_500)     # enough for every warp of the chip
+    elif kind == "large":
+        s = rng.integers(8193, 9000, 800)       # enough for every team
+    else:
+        s = np.concatenate([small[:1000], edges, rng.integers(1537, 1600, 3_300), rng.integers(8193, 9000, 790)])
+    rng.shuffle(s)
+    return s
+
+
+@pytest.mark.parametrize("kind", ["few", "medium", "large", "all"])
+@pytest.mark.parametrize("mode", ["f64", "f64_unaligned", "fp64_arith", "f32", "f32_unaligned"])
+def test_queued_batches(lv, ctx, kind, mode):
+    """Batches that no tile holds, by warps, teams and whole CTAs.  Each call twice: the queue of the second starts
+    where the first left it.  fp32: within 1e-5, the stated bound."""
+    import torch
+    rng = np.random.default_rng(51)
+    w = base._from_sizes(rng, _queued(kind), nt=600, pre=0.02)
+    b, model = base._dev(lv, w), lv.make_model(w.coef, w.split)
+    f32, at = mode.startswith("f32"), 1 if "unaligned" in mode else 0
+    dt = torch.float32 if f32 else torch.float64
+    outs = []
+    for _ in range(2):
+        T = torch.full((w.n_batch + at,), float("nan"), dtype=dt, device="cuda")[at:]
+        S = torch.full((w.n_req + at,), float("nan"), dtype=dt, device="cuda")[at:]
+        acc = lv.TenantAcc(ctx, w.n_tenants)
+        ctx.set_arith(1 if mode == "fp64_arith" else 0)
+        (lv.lv_attribute_f32 if f32 else lv.lv_attribute)(ctx, model, b, T, S, acc)
+        L = torch.empty(w.n_tenants, dtype=torch.float64, device="cuda")
+        lv.lv_tenant_totals(ctx, acc, L)
+        assert ctx.status() == lv.LV_OK
+        ctx.set_arith(0)
+        outs.append([x.cpu().numpy().astype(np.float64) for x in (T, S, L)])
+    for x, y in zip(*outs):
+        assert np.array_equal(x, y)
+    T, S, L = outs[0]
+    if not f32:
+        base._check_parity(w, T, S, L)
+        return
+    T_o, s_o = oracle.attribute(w.offsets, w.p, w.c, w.phase, w.split, w.coef)
+    nz = T_o != 0
+    assert np.all(T[~nz] == 0) and np.max(np.abs(T[nz] - T_o[nz]) / T_o[nz]) <= 1e-5
+    assert np.max(np.abs(S - s_o) / s_o) <= 1e-5
+    L_o = oracle.tenant_totals(s_o, w.tenant, w.n_tenants)
+    assert np.max(np.abs(L - L_o) / L_o) <= 1e-5
+
+
+@pytest.mark.parametrize("kind", ["few", "medium", "large", "all"])
+def test_queued_batches_features_and_noalloc(lv, ctx, kind):
+    """The same inputs' batch features, and lv_attribute_noalloc's T and shares bit for bit those of lv_attribute."""
+    import ctypes
+    import torch
+    w = base._from_sizes(np.random.default_rng(52), np.concatenate([_queued(kind)] * 2), pre=0.02)
+    b, model = base._dev(lv, w, tenant=False), lv.make_model(w.coef, w.split)
+    bf = torch.empty((5, w.n_batch), dtype=torch.int64, device="cuda")
+    bs = torch.empty(w.n_batch, dtype=torch.uint8, device="cuda")
+    lv.lv_features(ctx, b, model=model, batch_feat=bf, batch_seg=bs)
+    feat, seg = oracle.batch_features(w.offsets, w.p, w.c, w.phase, w.split)
+    assert ctx.status() == lv.LV_OK
+    assert np.array_equal(bf.cpu().numpy(), feat) and np.array_equal(bs.cpu().numpy(), seg)
+    T, S = base._run(lv, ctx, w, acc=False)[:2]
+    status = torch.full((1,), -1, dtype=torch.int32, device="cuda")
+    bst = b.struct()
+    for _ in range(2):
+        Tn = torch.full((w.n_batch,), float("nan"), dtype=torch.float64, device="cuda")
+        Sn = torch.full((w.n_req,), float("nan"), dtype=torch.float64, device="cuda")
+        rc = lv.lib().lv_attribute_noalloc(ctypes.byref(model), ctypes.byref(bst), Tn.data_ptr(), Sn.data_ptr(),
+                                           status.data_ptr(), torch.cuda.current_stream().cuda_stream)
+        assert rc == lv.LV_OK and int(status.item()) == 0
+        assert np.array_equal(Tn.cpu().numpy(), T) and np.array_equal(Sn.cpu().numpy(), S)
+
+
+@pytest.mark.parametrize("kind", ["few", "large"])
+def test_invalid_values_in_queued_batches(lv, ctx, kind):
+    """Negative p and c count as 0, tenants out of range as the nearest; the call reports them."""
+    rng = np.random.default_rng(53)
+    w = base._from_sizes(rng, _queued(kind), nt=7, pre=0.02)
+    big = np.flatnonzero(np.diff(w.offsets) > 1536)
+    at = w.offsets[rng.choice(big, 30)] + rng.integers(0, 1537, 30)
+    w.p[at[:10]], w.c[at[10:20]], w.tenant[at[20:25]], w.tenant[at[25:]] = -5, -(1 << 31), -1, 7
+    T, S, L, st = base._run(lv, ctx, w)
+    assert st == lv.LV_EDATA
+    w.p[:], w.c[:], w.tenant[:] = np.maximum(w.p, 0), np.maximum(w.c, 0), np.clip(w.tenant, 0, 6)
+    base._check_parity(w, T, S, L)
