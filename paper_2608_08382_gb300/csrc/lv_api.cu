@@ -731,8 +731,10 @@ lv_status whatif_run(lv_ctx *ctx, const lv_model *model, const lv_batches *cand,
   if (by_block) {
     st = timing_begin(ctx, LV_TIME_TILES, stream, &stop);
     if (st != LV_OK) return st;
-    k_wi_cand_direct<<<(unsigned)nc, kWiCandThreads, 0, stream>>>(mp, cand->p, cand->c, cand->phase, cand->offsets,
-                                                                  cand->n_req, nc, candp, ctx->d_status);
+    const bool wide = nc <= 2 * ctx->sms && cand->n_req > (int64_t)kWiWide * nc;
+    auto *kernel = wide ? k_wi_cand_direct<512, 4> : k_wi_cand_direct<128, 2>;
+    kernel<<<(unsigned)nc, wide ? 512 : 128, 0, stream>>>(mp, cand->p, cand->c, cand->phase, cand->offsets,
+                                                         cand->n_req, nc, candp, ctx->d_status);
     LV_CUDA(cudaGetLastError());
     st = timing_end(stop, stream);
     if (st != LV_OK) return st;

@@ -89,15 +89,20 @@ __device__ __forceinline__ i128 cand_const(const ModelP &mp, int s, int half, in
 // kWiDirectPerSm candidates per SM the tile pass, which packs batches, takes
 // over (whole calls by blocks and by tiles: 1,024 candidates 27 and 35 us, 10,000
 // 41.5 and 43.5, 40,000 83 and 56).
-constexpr int kWiCandThreads = 128;
-constexpr int kWiDirectPerSm = 64;
-__global__ void __launch_bounds__(kWiCandThreads) k_wi_cand_direct(ModelP mp, const int32_t *__restrict__ p,
-                                                                  const int32_t *__restrict__ c,
-                                                                  const int32_t *__restrict__ ph,
-                                                                  const int64_t *__restrict__ off, int64_t n_req,
-                                                                  int64_t nc, CandP *__restrict__ out, int *status) {
+// A candidate is one block's chain of loads, so a few large ones (at most two per
+// SM, of more than kWiWide requests each on average) get blocks of 512 threads
+// with four 16-byte loads of every array in flight each: 24 candidates of 1e6
+// requests 255 us, 1,310 with 128 threads and four 4-byte loads; one of 5e6 1.0
+// ms, 2.3.  The others get 128 threads with two such loads, few enough registers
+// for ten blocks per SM (5,000 of 3,000: 47 us, 111 with 512 threads).
+constexpr int kWiDirectPerSm = 64, kWiWide = 4096;
+template <int kThreads, int kQuads>
+__global__ void __launch_bounds__(kThreads, kThreads == 128 ? 10 : 1)
+    k_wi_cand_direct(ModelP mp, const int32_t *__restrict__ p,
+                     const int32_t *__restrict__ c, const int32_t *__restrict__ ph, const int64_t *__restrict__ off,
+                     int64_t n_req, int64_t nc, CandP *__restrict__ out, int *status) {
   let_next();
-  __shared__ Sums red[kWiCandThreads / 32];
+  __shared__ Sums red[kThreads / 32];
   const int64_t b = blockIdx.x;
   const int tid = threadIdx.x;
   int bad = 0;
@@ -105,22 +110,29 @@ __global__ void __launch_bounds__(kWiCandThreads) k_wi_cand_direct(ModelP mp, co
   const int64_t r0 = clampi(o0, 0, n_req), r1 = clampi(o1, r0, n_req);
   if (r0 != o0 || r1 != o1 || (b == 0 && o0 != 0) || (b == nc - 1 && o1 != n_req)) bad = 1;
   Sums acc{0, 0, 0, 0};
-  for (int64_t i = r0 + tid; i < r1; i += 4 * kWiCandThreads) {
-    int32_t pv[4], cv[4], fv[4];
+  for (int64_t q0 = (r0 & ~(int64_t)3) + 4 * tid; q0 < r1; q0 += 4 * kQuads * kThreads) {
+    Quad v[kQuads];  // all loads in flight
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int64_t j = i + k * kWiCandThreads;
-      pv[k] = j < r1 ? p[j] : 0;
-      cv[k] = j < r1 ? c[j] : 0;
-      fv[k] = j < r1 ? ph[j] : 0;
+    for (int h = 0; h < kQuads; ++h) {
+      const int64_t q = q0 + 4 * kThreads * h, left = n_req - q;
+      v[h].p = v[h].c = v[h].x = make_int4(0, 0, 0, 0);
+      if (q < r1) v[h] = load_quad<true>(p + q, c + q, ph + q, 0, left < 4 ? (int)left : 4);
     }
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      check_req(pv[k], cv[k], fv[k], &bad);
-      acc.s1 += pv[k];
-      acc.s2 += cv[k];
-      acc.s3 += (int64_t)pv[k] * pv[k];
-      acc.ph |= fv[k];
+    for (int h = 0; h < kQuads; ++h) {
+      const int64_t q = q0 + 4 * kThreads * h;
+      if (q >= r1) break;
+      int32_t pv[4] = {v[h].p.x, v[h].p.y, v[h].p.z, v[h].p.w}, cv[4] = {v[h].c.x, v[h].c.y, v[h].c.z, v[h].c.w},
+              fv[4] = {v[h].x.x, v[h].x.y, v[h].x.z, v[h].x.w};
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (q + k < r0 || q + k >= r1) pv[k] = cv[k] = fv[k] = 0;
+        check_req(pv[k], cv[k], fv[k], &bad);
+        acc.s1 += pv[k];
+        acc.s2 += cv[k];
+        acc.s3 += (int64_t)pv[k] * pv[k];
+        acc.ph |= fv[k];
+      }
     }
   }
   acc = warp_sum(acc);
@@ -130,7 +142,7 @@ __global__ void __launch_bounds__(kWiCandThreads) k_wi_cand_direct(ModelP mp, co
   if (tid >= 32) return;
   acc = red[0];
 #pragma unroll
-  for (int w = 1; w < kWiCandThreads / 32; ++w) acc = add_sums(acc, red[w]);
+  for (int w = 1; w < kThreads / 32; ++w) acc = add_sums(acc, red[w]);
   bool slow = !mp.fixed;
   if (tid < 8 && mp.fixed) {
     const i128 v = cand_const(mp, tid & 3, tid >> 2, acc.s1, acc.s2, acc.s3, r1 - r0, &slow);

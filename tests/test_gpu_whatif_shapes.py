@@ -53,6 +53,19 @@ def test_shapes(lv, ctx, nc, npend):
     assert np.max(np.abs(T - T_o) / T_o) <= 1e-12 and np.max(np.abs(S - S_o) / S_o) <= 1e-12
 
 
+@pytest.mark.parametrize("sizes", [[4097, 0, 4096, 4099], [1, 1023, 1024, 1025, 1026, 2047, 2049], [8191, 8192, 8193, 8195],
+                                   [300_001], [3, 5, 100_002], [4096] * 305])
+def test_large_candidates(lv, ctx, sizes):
+    """Candidates of one and of several turns of a block's loads, in blocks of 128 and of 512 threads, and arrays that
+    end inside a quad."""
+    rng = np.random.default_rng(len(sizes))
+    w = base._from_sizes(rng, np.array(sizes), pre=0.02)
+    p, c, ph = _pending(rng, 40)
+    T, S, _ = _whatif(lv, ctx, w, p, c, ph)
+    T_o, S_o = oracle.whatif(w.offsets, w.p, w.c, w.phase, p, c, ph, w.split, w.coef)
+    assert np.max(np.abs(T - T_o) / T_o) <= 1e-12 and np.max(np.abs(S - S_o) / S_o) <= 1e-12
+
+
 @pytest.mark.parametrize("split", [-2 ** 63, -2 ** 63 + 1, -1, 0, 1, 2 ** 31, 2 ** 63 - 1])
 def test_extreme_splits(lv, ctx, split):
     """Splits that every batch or none meets: the regime is S1 + p >= split in 64 bits."""
