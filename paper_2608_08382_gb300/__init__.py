@@ -135,19 +135,23 @@ def _ptr(t):
     return None if t is None else t.data_ptr()
 
 
-_torch = None  # set once torch's CUDA state exists
+_raw_stream = _device = None  # set once torch's CUDA state exists
 
 
 def _stream(stream):
     """The stream's handle; None is torch's current stream.  A serving step's call is bound by its
-    host side, so the current stream is taken as a bare handle, without a torch.cuda.Stream object."""
-    global _torch
+    host side, so the current stream is taken as a bare handle, without a torch.cuda.Stream object,
+    where torch has the two functions for that."""
+    global _raw_stream, _device
     if stream is None:
-        if _torch is None:
+        if _raw_stream is None:
             import torch
             torch.cuda.current_stream()
-            _torch = torch
-        return _torch._C._cuda_getCurrentRawStream(_torch._C._cuda_getDevice())
+            raw, _device = (getattr(torch._C, n, None) for n in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
+            if raw is None or _device is None:
+                raw, _device = (lambda _: torch.cuda.current_stream().cuda_stream), (lambda: None)
+            _raw_stream = raw
+        return _raw_stream(_device())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 

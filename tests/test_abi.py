@@ -110,6 +110,25 @@ def test_binding_constants_match_header(lv):
         assert getattr(lv, name) == int(value), name
 
 
+@pytest.mark.parametrize("missing", [(), ("_cuda_getCurrentRawStream",), ("_cuda_getDevice",)])
+def test_current_stream_with_and_without_the_short_way(lv, monkeypatch, missing):
+    torch = pytest.importorskip("torch")
+
+    class Stream:
+        cuda_stream = 4711
+
+    monkeypatch.setattr(lv, "_raw_stream", None)
+    monkeypatch.setattr(lv, "_device", None)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: Stream)
+    monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", lambda dev: 100 + dev, raising=False)
+    monkeypatch.setattr(torch._C, "_cuda_getDevice", lambda: 3, raising=False)
+    for name in missing:
+        monkeypatch.delattr(torch._C, name)
+    for _ in range(2):
+        assert lv._stream(None) == (4711 if missing else 103)
+    assert lv._stream(Stream) == 4711 and lv._stream(7) == 7
+
+
 def test_noalloc_configures_its_kernels_on_each_device(lv, tmp_path):
     """lv_attribute_noalloc's kernel needs more shared memory than a kernel gets unasked, and that is set per device:
     a second device's first call sets it again.  On a stand-in for the runtime with two devices, in a process of its
