@@ -37,6 +37,13 @@
  *    16-byte aligned (so that kernels may read them with 16-byte vector loads),
  *    fp64 outputs 8-byte aligned; otherwise LV_EINVAL.
  *  - One lv_ctx must not be used from two host threads at once.
+ *  - Streams: the calls of one context share its scratch, and the calls into one
+ *    accumulator its state.  Issue them on one stream, or order their work
+ *    across streams (events), so that no two of them overlap on the GPU.  Calls
+ *    that overlap can give wrong results; into one accumulator they can lose
+ *    shares, of that call and of later ones until lv_tenant_acc_reset or
+ *    lv_tenant_acc_import.  Several contexts, each with accumulators of its own,
+ *    may work at the same time.
  *  - CUDA graphs: lv_features, lv_batch_latency, lv_attribute,
  *    lv_attribute_step, lv_tenant_acc_reset, lv_tenant_accumulate,
  *    lv_tenant_totals, lv_whatif
@@ -132,10 +139,10 @@ typedef struct lv_tenant_acc lv_tenant_acc;
 
 /* Create a context on the current CUDA device.  It owns a device scratch area
  * that its calls grow to the largest input they have seen and keep (the tile
- * pass: about 1 byte per 150 requests and batches; lv_whatif: 192
- * bytes a candidate; lv_fit: 33 bytes a batch, for 2^22 batches at most, 138 MB;
- * lv_accuracy: about 20 bytes a batch) and a sticky status word.  Returns
- * LV_ECUDA/LV_ENOMEM on failure. */
+ * pass: about 1 byte per 150 requests; lv_whatif: about 220 bytes a candidate;
+ * lv_fit: 33 bytes a batch, for 2^22 batches at most, 138 MB; lv_accuracy: about
+ * 20 bytes a batch) and a sticky status word.  Returns LV_ECUDA/LV_ENOMEM on
+ * failure. */
 lv_status lv_ctx_create(lv_ctx **out);
 void lv_ctx_destroy(lv_ctx *ctx);
 /* Select LV_ARITH_AUTO (default) or LV_ARITH_FP64. */

@@ -1138,8 +1138,7 @@ lv_status lv_tenant_acc_export(lv_tenant_acc *acc, void *host_state, int64_t byt
 
 lv_status lv_tenant_acc_import(lv_tenant_acc *acc, const void *host_state, int64_t bytes, void *stream) {
   if (!acc || !host_state || bytes != lv_tenant_acc_state_bytes(acc)) return LV_EINVAL;
-  LV_CUDA(cudaMemsetAsync(acc->d_pend, 0, sizeof(unsigned long long) * 4 * (size_t)acc->n_tenants,
-                          (cudaStream_t)stream));
+  LV_CUDA(cudaMemsetAsync(acc->d_pend, 0, acc->bytes, (cudaStream_t)stream));  // the ticket too
   LV_CUDA(cudaMemcpyAsync(acc->d_state, host_state, (size_t)bytes, cudaMemcpyHostToDevice, (cudaStream_t)stream));
   LV_CUDA(cudaStreamSynchronize((cudaStream_t)stream));
   return LV_OK;
