@@ -38,7 +38,6 @@ struct lv_ctx {
   unsigned char *d_bound = nullptr;  // k_tiles' queue counters (zero between calls), first batch of each tile, queue
   size_t bound_cap = 0;
   KEntry *d_ktab = nullptr;
-  int ktab_nk = 0;
   bool ktab_valid = false;
   lv_model ktab_model{};
   bool mp_valid = false;  // parameters of the previous call's model

@@ -11,7 +11,6 @@
 
 namespace lv {
 
-constexpr int kBlock = 256;                        // threads per CTA of the small kernels
 constexpr int kHotMax = 512;                       // tenants kept in shared memory per CTA
 constexpr int64_t kPMaxFix = 1ll << 24;            // p beyond this uses the fp64 share path
 constexpr int kTenLsb = -72;                       // tenant totals: shares rounded to 2^-72 s, summed exactly
@@ -80,11 +79,6 @@ __device__ __forceinline__ void acc_add256(uint64_t *w, uint64_t a0, uint64_t a1
   c3 |= (s < c2) ? 1ull : 0ull;
   w[2] = s;
   w[3] = w[3] + a3 + c3;
-}
-
-// Exact y * 2^100 as a signed 128-bit integer (round to nearest even below 2^-100).
-__device__ __forceinline__ i128 y_fixed(double y, bool *ovf) {
-  return double_to_fix(y, kFitYLsb, ovf);
 }
 
 // Counters of the queue of batches that no tile holds: medium and large ones
