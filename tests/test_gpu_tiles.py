@@ -137,14 +137,12 @@ def _queued(kind):
     return s
 
 
-@pytest.mark.parametrize("kind", ["few", "medium", "large", "all"])
-@pytest.mark.parametrize("mode", ["f64", "f64_unaligned", "fp64_arith", "f32", "f32_unaligned"])
-def test_queued_batches(lv, ctx, kind, mode):
-    """Batches that no tile holds, by warps, teams and whole CTAs.  Each call twice: the queue of the second starts
-    where the first left it.  fp32: within 1e-5, the stated bound."""
+_MODES = ["f64", "f64_unaligned", "fp64_arith", "f32", "f32_unaligned"]
+
+
+def _check_mode(lv, ctx, w, mode):
+    """Two calls, alike bit for bit, against the oracle.  fp32: within 1e-5, the stated bound."""
     import torch
-    rng = np.random.default_rng(51)
-    w = base._from_sizes(rng, _queued(kind), nt=600, pre=0.02)
     b, model = base._dev(lv, w), lv.make_model(w.coef, w.split)
     f32, at = mode.startswith("f32"), 1 if "unaligned" in mode else 0
     dt = torch.float32 if f32 else torch.float64
@@ -172,6 +170,23 @@ def test_queued_batches(lv, ctx, kind, mode):
     assert np.max(np.abs(S - s_o) / s_o) <= 1e-5
     L_o = oracle.tenant_totals(s_o, w.tenant, w.n_tenants)
     assert np.max(np.abs(L - L_o) / L_o) <= 1e-5
+
+
+@pytest.mark.parametrize("kind", ["few", "medium", "large", "all"])
+@pytest.mark.parametrize("mode", _MODES)
+def test_queued_batches(lv, ctx, kind, mode):
+    """Batches that no tile holds, by warps, teams and whole CTAs.  Each call twice: the queue of the second starts
+    where the first left it."""
+    rng = np.random.default_rng(51)
+    _check_mode(lv, ctx, base._from_sizes(rng, _queued(kind), nt=600, pre=0.02), mode)
+
+
+@pytest.mark.parametrize("lo,hi,n", [(0, 2, 9000), (1, 8, 6000), (30, 50, 900), (1240, 1256, 200), (1528, 1544, 150),
+                                     (513, 5000, 200)])
+@pytest.mark.parametrize("mode", _MODES[1:])
+def test_modes_around_the_tile(lv, ctx, lo, hi, n, mode):
+    rng = np.random.default_rng(hi)
+    _check_mode(lv, ctx, base._from_sizes(rng, rng.integers(lo, hi + 1, n), nt=9, pre=0.1), mode)
 
 
 @pytest.mark.parametrize("kind", ["few", "medium", "large", "all"])
