@@ -82,10 +82,14 @@ constexpr int kKTableN = kTabN;
 constexpr size_t kBoundHead = 64;  // bytes of the queue's counters before the tiles' bounds
 static_assert(kQueueWords * sizeof(unsigned) <= kBoundHead, "queue counters");
 
-// Most batches that no tile of the mode holds.
+// The queue's lists, with room for the batches that no tile of the mode holds:
+// where each class's starts, for c = kQClasses where the last one ends.
 template <int MODE>
-constexpr int64_t queue_room(int64_t n_req) {
-  return n_req / (Geo<MODE>::kCap + 1) + 1;
+constexpr int64_t queue_at(int64_t n_req, int c) {
+  constexpr int64_t from[kQClasses] = {Geo<MODE>::kCap, kQWarp, kQTeam};  // more requests than these
+  int64_t at = 0;
+  for (int k = 0; k < c; ++k) at += n_req / (from[k] + 1) + 1;
+  return at;
 }
 
 #define LV_CUDA(call)                          \
@@ -404,25 +408,23 @@ lv_status ensure_bound(lv_ctx *ctx, size_t bytes) {
 }
 
 // Launches k_tile_bounds into scratch of [counters][bounds][queue], in 32 or 64
-// bits; queue_cap: entries of the queue, or 0.
-template <class V>
-lv_status launch_bounds(const TilePlan &plan, TileArgs &a, unsigned char *scratch, int64_t queue_cap, int64_t most,
-                        int sms, cudaStream_t stream) {
+// bits.
+template <class V, int MODE>
+lv_status launch_bounds(const TilePlan &plan, TileArgs &a, unsigned char *scratch, bool queue, int sms,
+                        cudaStream_t stream) {
   V *bound = reinterpret_cast<V *>(scratch + kBoundHead);
-  TileQueue<V> q{nullptr, 0, INT64_MAX, nullptr};
-  if (queue_cap > 0) {
-    q = TileQueue<V>{bound + plan.n_tiles + 1, queue_cap, most, reinterpret_cast<unsigned *>(scratch)};
-    a.queue = q.queue;
-    a.queue_cap = queue_cap;
-    a.queue_ctr = q.ctr;
+  if (queue) {
+    a.queue.list = bound + plan.n_tiles + 1;
+    a.queue.ctr = reinterpret_cast<unsigned *>(scratch);
+    for (int c = 0; c <= kQClasses; ++c) a.queue.at[c] = queue_at<MODE>(a.n_req, c);
   }
   if (sizeof(V) == 4)
     a.bound32 = reinterpret_cast<const uint32_t *>(bound);
   else
     a.bound = reinterpret_cast<const int64_t *>(bound);
   const int64_t blocks = std::min<int64_t>(a.n_batch / 1024 + 1, (int64_t)sms * 16);
-  k_tile_bounds<V><<<(unsigned)blocks, 256, 0, stream>>>(a.off, a.n_batch, a.n_req, plan.n_tiles, plan.magic, bound, q,
-                                                         a.status);
+  k_tile_bounds<V><<<(unsigned)blocks, 256, 0, stream>>>(a.off, a.n_batch, a.n_req, plan.n_tiles, plan.magic, bound,
+                                                         a.queue, queue ? Geo<MODE>::kCap : INT64_MAX, a.status);
   LV_CUDA(cudaGetLastError());
   return LV_OK;
 }
@@ -453,8 +455,9 @@ lv_status bound_tiles(lv_ctx *ctx, int sms, TileArgs &a, unsigned char *scratch,
   a.D = plan.search ? plan.D : 0;
   if (plan.search) return LV_OK;
   const bool narrow = a.n_batch < (1ll << 32);
-  const int64_t queue_cap = a.f_range ? 0 : queue_room<MODE>(a.n_req);
-  const size_t need = kBoundHead + (narrow ? sizeof(uint32_t) : sizeof(int64_t)) * (size_t)(plan.n_tiles + 1 + queue_cap);
+  const bool queue = a.f_range == nullptr;
+  const int64_t entries = plan.n_tiles + 1 + (queue ? queue_at<MODE>(a.n_req, kQClasses) : 0);
+  const size_t need = kBoundHead + (narrow ? sizeof(uint32_t) : sizeof(int64_t)) * (size_t)entries;
   if (ctx) {
     st = ensure_bound(ctx, need);
     if (st != LV_OK) return st;
@@ -462,9 +465,8 @@ lv_status bound_tiles(lv_ctx *ctx, int sms, TileArgs &a, unsigned char *scratch,
   } else if (need > scratch_cap || !narrow) {
     return LV_EINVAL;
   }
-  const int64_t most = Geo<MODE>::kCap;
-  return narrow ? launch_bounds<uint32_t>(plan, a, scratch, queue_cap, most, sms, stream)
-                : launch_bounds<int64_t>(plan, a, scratch, queue_cap, most, sms, stream);
+  return narrow ? launch_bounds<uint32_t, MODE>(plan, a, scratch, queue, sms, stream)
+                : launch_bounds<int64_t, MODE>(plan, a, scratch, queue, sms, stream);
 }
 
 template <int MODE>
@@ -1347,7 +1349,7 @@ constexpr int64_t kNoAllocMaxUnits = 65536 * 1024;  // n_batch + n_req
 // most tiles: every unit an empty batch, and a partial round of 32 warps on each of 256 SMs
 constexpr int64_t kNoAllocBounds = kTW * kNoAllocMaxUnits / Geo<M_ATTR>::kD + 32 * 256 + 2;
 constexpr size_t kNoAllocTiles =
-    kBoundHead + sizeof(uint32_t) * (size_t)(kNoAllocBounds + queue_room<M_ATTR>(kNoAllocMaxUnits));
+    kBoundHead + sizeof(uint32_t) * (size_t)(kNoAllocBounds + queue_at<M_ATTR>(kNoAllocMaxUnits, kQClasses));
 constexpr size_t kNoAllocTabOffset = (kNoAllocTiles + 255) & ~(size_t)255;
 constexpr size_t kNoAllocBytes = kNoAllocTabOffset + sizeof(KEntry) * 4 * (kKTableN + 1);
 // the size stated in include/llmvisor.h ("about 2.5 MB")

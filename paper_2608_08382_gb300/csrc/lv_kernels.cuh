@@ -81,9 +81,16 @@ __device__ __forceinline__ void acc_add256(uint64_t *w, uint64_t a0, uint64_t a1
   w[3] = w[3] + a3 + c3;
 }
 
-// Counters of the queue of batches that no tile holds: medium and large ones
-// queued, medium and large ones taken, CTAs done with it.
-enum : int { kQMedium, kQLarge, kQTakenM, kQTakenL, kQDone, kQueueWords };
+// The queue of the batches that no tile holds: one list per class of sizes, one
+// after the other, in the bounds' type.  Counters: batches listed and taken, by
+// class, and CTAs done with them; zero between calls.
+constexpr int kQClasses = 3;
+enum : int { kQListed, kQTaken = kQClasses, kQDone = 2 * kQClasses, kQueueWords };
+struct TileQueue {
+  void *list;             // null: nothing is queued
+  unsigned *ctr;          // [kQueueWords]
+  int64_t at[kQClasses + 1];  // where each class's list starts; the end
+};
 
 struct TileArgs {
   const int32_t *p, *c, *ph, *ten;
@@ -93,11 +100,7 @@ struct TileArgs {
   const uint32_t *bound32;  // the same in 32 bits (fewer than 2^32 batches)
   int64_t n_tiles;
   int64_t D;             // merge positions per tile where the warps find their bounds themselves, or 0
-  // batches that no tile holds, found with the bounds (null: none are queued): the
-  // medium ones from the front, the large ones from the back, in the bounds' type
-  const void *queue;
-  int64_t queue_cap;
-  unsigned *queue_ctr;   // [kQueueWords], zero between calls
+  TileQueue queue;
   double *T, *share;
   float *T32, *share32;  // fp32 variant (M_F32): T and shares as float, or null
   int64_t *bfeat;   // [5][n_batch] or null; M_FIT: [4][f_stride] S1, S2, S3, n of batches f_lo and up

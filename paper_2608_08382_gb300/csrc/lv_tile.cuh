@@ -20,12 +20,11 @@
 // walked on its own afterwards: one of more requests than a tile holds comes
 // from a queue that k_tile_bounds has filled, so that such batches spread over
 // the chip wherever they start (walk_queue); a smaller one by its warp at once,
-// or, above kTAlone requests, by the CTA that met it (1e6 Pareto batches of up to
-// 4,096: 88 us, 196 if their warps
-// walk them all).  All sums are exact integers, so results do not depend on
-// the schedule.
+// or, above kTAlone requests, by the CTA that met it, once its tiles are done (1e6
+// Pareto batches: 85 us, 119 if their warps walk them; 1e7: 538 and 600).  All
+// sums are exact integers, so results do not depend on the schedule.
 //
-// What bounds it: instruction issue and the integer pipe (about 170 warp
+// What bounds it: instruction issue and the integer pipe (about 143 warp
 // instructions per 32 requests), not HBM.  The shape follows from that: 20 warps
 // per SM with 96 registers each spill little (24 warps of 80 took 9 % longer,
 // 32 of 64 a third), and the largest tile whose shared memory (182 KB) leaves the
@@ -36,8 +35,8 @@
 // Against a kernel that walked one batch per warp (one call, GB300): 1.36e8
 // requests in batches of 16 to 256, fp64 shares, 256 tenants, 1,134 us before
 // and 840 now; 3.25e7 in batches of 1 to 64, 16 tenants, 583 and 290; 6.5e5, 113
-// and 20; 2.6e7 in Pareto batches, 65,536 tenants, 817 and 566; fp32, 4.1e7 in
-// batches of 16 to 256, 322 and 222.
+// and 20; 2.6e7 in Pareto batches, 65,536 tenants, 817 and 541; fp32, 4.1e7 in
+// batches of 16 to 256, 322 and 224; 5e7 in batches of 4,096, 531 and 407.
 #pragma once
 
 #include "lv_step.cuh"
@@ -51,8 +50,8 @@ constexpr int kTW = 8;                     // merge positions a batch takes besi
 constexpr int kTDMin = 128;
 constexpr int64_t kTAlone = 512;           // requests a warp walks alone where nothing is queued
 constexpr int kTBigs = 64;                 // larger batches a CTA keeps for later
-constexpr int64_t kQWarp = 8192;           // requests of a medium queued batch, at most
-constexpr int64_t kQTeam = 65536;          // and of one that a team walks
+constexpr int64_t kQWarp = 4096;           // requests of a queued batch that a warp walks, at most
+constexpr int64_t kQTeam = 24576;          // that a team walks
 constexpr int kTTeam = 128, kTTeams = kTThreads / kTTeam;
 static_assert(3 * kTTeams <= kTBigs, "a turn of the queue fits the list's memory");
 constexpr int kTabN = 4096;                // batch sizes of the K table
@@ -108,7 +107,7 @@ struct TSmem {
   alignas(16) Sums red[kTWarps];
   alignas(16) int64_t big[kTBigs];    // batches left for the whole CTA
   int n_big;
-  unsigned queued[2];                 // medium and large batches in the queue
+  unsigned queued[kQClasses];         // batches in the queue
 };
 
 // ---------------------------------------------------------------- bounds
@@ -118,46 +117,40 @@ __device__ __forceinline__ int64_t div_magic(int64_t x, uint64_t magic) {
   return (int64_t)__umul64hi((uint64_t)x, magic);
 }
 
-// part[t] = the first batch whose start position kTW * b + off[b] is at least
-// t * D, for t in [0, n_tiles); part[n_tiles] = n_batch.  Batch b writes the t
-// in (f(b-1) / D, f(b) / D], so every entry is written once.  Checks the
-// offsets, and queues the batches of more than `most` requests, which no tile
-// holds (q.queue null: none).  HBM-bound: 8 B per batch; four batches per thread
-// from two 16-byte loads, and the divisions are multiplications (1e7 batches
-// take 30 us; one batch per thread 18 us more; a test that skips the four
-// divisions of batches within one tile 3 us more).
+// Lists the warp's batches b0 + k for which bit k of `mask` is set.
 template <class V>
-struct TileQueue {
-  V *queue;
-  int64_t cap, most;
-  unsigned *ctr;
-};
-
-// Adds the warp's batches b0 + k for which bit k of `mask` is set to one end of the queue.
-template <class V>
-__device__ __forceinline__ void queue_add(const TileQueue<V> &q, int which, uint32_t mask, int64_t b0, int lane) {
-  int at = __popc(mask), total = at;
+__device__ __forceinline__ void queue_add(const TileQueue &q, int cls, uint32_t mask, int64_t b0, int lane) {
+  const int own = __popc(mask);
+  int end = own;
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
-    const int o = __shfl_up_sync(kFull, at, d);
-    if (lane >= d) at += o;
+    const int o = __shfl_up_sync(kFull, end, d);
+    if (lane >= d) end += o;
   }
-  total = __shfl_sync(kFull, at, 31);
+  const int total = __shfl_sync(kFull, end, 31);
   if (total == 0) return;
   unsigned base = 0;
-  if (lane == 0) base = atomicAdd(q.ctr + which, (unsigned)total);
-  int64_t i = (int64_t)__shfl_sync(kFull, base, 0) + at - __popc(mask);
+  if (lane == 0) base = atomicAdd(q.ctr + kQListed + cls, (unsigned)total);
+  int64_t i = q.at[cls] + __shfl_sync(kFull, base, 0) + end - own;
 #pragma unroll
   for (int k = 0; k < 4; ++k)
     if ((mask >> k) & 1u) {
-      if (i < q.cap) q.queue[which == kQLarge ? q.cap - 1 - i : i] = (V)(b0 + k);  // always, for valid offsets
+      if (i < q.at[cls + 1]) static_cast<V *>(q.list)[i] = (V)(b0 + k);  // always, for valid offsets
       ++i;
     }
 }
 
+// part[t] = the first batch whose start position kTW * b + off[b] is at least
+// t * D, for t in [0, n_tiles); part[n_tiles] = n_batch.  Batch b writes the t
+// in (f(b-1) / D, f(b) / D], so every entry is written once.  Checks the
+// offsets, and queues the batches of more than `most` requests, which no tile
+// holds.  HBM-bound: 8 B per batch; four batches per thread from two 16-byte
+// loads, and the divisions are multiplications (1e7 batches take 30 us; one batch
+// per thread 18 us more; a test that skips the four divisions of batches within
+// one tile 3 us more).
 template <class V>
 __global__ void k_tile_bounds(const int64_t *__restrict__ off, int64_t n_batch, int64_t n_req, int64_t n_tiles,
-                              uint64_t magic, V *__restrict__ part, const TileQueue<V> q, int *status) {
+                              uint64_t magic, V *__restrict__ part, const TileQueue q, int64_t most, int *status) {
   let_next();
   int bad = 0;
   const int lane = threadIdx.x & 31;
@@ -181,14 +174,16 @@ __global__ void k_tile_bounds(const int64_t *__restrict__ off, int64_t n_batch, 
     if (b0 == 0 && v[1] != 0) bad = 1;
     int64_t c = clampi(v[0], 0, n_req);
     int64_t t0 = b0 > 0 ? div_magic(kTW * (b0 - 1) + c, magic) : -1;
-    uint32_t medium = 0, large = 0;  // bit k: batch b0 - 1 + k
+    uint32_t big[kQClasses] = {};  // bit k: batch b0 - 1 + k
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const int64_t b = b0 + k;
       if (b > n_batch) break;
       if (b > 0 && v[k] > v[k + 1]) bad = 1;
       const int64_t cb = clampi(v[k + 1], 0, n_req), n = cb - c;
-      if (b > 0 && n > q.most) (n > kQWarp ? large : medium) |= 1u << k;
+      if (b > 0 && n > most) big[0] |= 1u << k;
+      if (b > 0 && n > most && n > kQWarp) big[1] |= 1u << k;
+      if (b > 0 && n > most && n > kQTeam) big[2] |= 1u << k;
       const int64_t tb = div_magic(kTW * b + cb, magic);
       if (b == n_batch && v[k + 1] != n_req) bad = 1;
       const int64_t tmax = b == n_batch ? n_tiles : min(tb, n_tiles);
@@ -196,9 +191,10 @@ __global__ void k_tile_bounds(const int64_t *__restrict__ off, int64_t n_batch, 
       t0 = tb;
       c = cb;
     }
-    if (__any_sync(kFull, (medium | large) != 0u)) {
-      queue_add(q, kQMedium, medium, b0 - 1, lane);
-      queue_add(q, kQLarge, large, b0 - 1, lane);
+    if (__any_sync(kFull, big[0] != 0u)) {
+#pragma unroll
+      for (int k = 0; k < kQClasses; ++k)
+        queue_add<V>(q, k, big[k] & ~(k + 1 < kQClasses ? big[k + 1 < kQClasses ? k + 1 : 0] : 0u), b0 - 1, lane);
     }
   }
   if (bad) flag(status, kStatusData);
@@ -206,8 +202,8 @@ __global__ void k_tile_bounds(const int64_t *__restrict__ off, int64_t n_batch, 
 
 // Entry i of the queue.
 __device__ __forceinline__ int64_t queued_batch(const TileArgs &a, int64_t i) {
-  const int64_t b = a.bound32 ? (int64_t)static_cast<const uint32_t *>(a.queue)[i]
-                              : static_cast<const int64_t *>(a.queue)[i];
+  const int64_t b = a.bound32 ? (int64_t)static_cast<const uint32_t *>(a.queue.list)[i]
+                              : static_cast<const int64_t *>(a.queue.list)[i];
   return clampi(b, 0, a.n_batch - 1);
 }
 
@@ -572,8 +568,8 @@ __device__ __forceinline__ void tile_rest(const TileArgs &a, const TenTab &tt, c
 // another record where a batch starts among its four (leaving what lies past
 // the start to the list, where batches average 40 requests and more, was
 // no faster: 1.36e8 requests of batches of 16 to 256, 840 us either way, and the
-// second copy of the loop cost the fp32 variant 3 %).  vec: the share array allows 32-byte (fp32: 16-byte)
-// stores.  kWalk: a part of a batch of n_walk requests on its own, whose values may
+// second copy of the loop cost the fp32 variant 3 %).  vec: the share array allows
+// 32-byte (fp32: 16-byte) stores.  kWalk: a part of a batch of n_walk requests on its own, whose values may
 // be negative (walk_batch).
 template <int MODE, bool kWalk>
 __device__ __forceinline__ void tile_shares(const TileArgs &a, const TenTab &tt, const TSmem<MODE> &ts,
@@ -824,72 +820,76 @@ __device__ __forceinline__ void walk_list(const TileArgs &a, TSmem<MODE> &ts, in
   }
 }
 
-// The queued batches, first the large ones, then the medium ones.  A batch is
-// walked by the whole CTA where there are few; by a team where there are enough
-// for every team, five at a time, unless one is so large that the others would
-// wait for it; medium ones by a warp where there are enough for every warp.  The
-// last CTA out leaves the counters at zero for the next call.  5e7 requests in
-// batches of 4,096, 9,976 and 49,912: 399, 385 and 479 us, about 310 in batches
-// that fit their tiles; 1,307, 930 and 905 when each CTA walked those that start
-// in its tiles, one request per thread and turn.
-template <int MODE>
-__device__ __noinline__ void walk_queue(const TileArgs &a, TSmem<MODE> &ts, unsigned n_medium, unsigned n_large) {
-  const int tid = threadIdx.x, lane = tid & 31, team = tid / kTTeam;
-  const bool by_warp = n_medium >= gridDim.x * kTWarps;
-  const int64_t med = min((int64_t)n_medium, a.queue_cap), lar = min((int64_t)n_large, a.queue_cap);
-  const int64_t n_cta = lar + (by_warp ? 0 : med);
-  const int step = n_cta >= (int64_t)gridDim.x * kTTeams ? kTTeams : 1;
-  // the turn's batches, their first requests and sizes (-1: none), by the first warp
-  int64_t *turn = ts.big;
+// One class of the queue, each team or CTA taking one batch at a time.
+template <int MODE, int kThreads>
+__device__ __forceinline__ void walk_class(const TileArgs &a, TSmem<MODE> &ts, int cls, int64_t count) {
+  int64_t *turn = ts.big + 3 * ((int)threadIdx.x / kThreads);  // batch, first request, requests
   for (;;) {
-    __syncthreads();
-    if (tid < 32) {
-      unsigned nx = 0;
-      if (lane == 0) nx = atomicAdd(a.queue_ctr + kQTakenL, (unsigned)step);
-      const int64_t i = (int64_t)__shfl_sync(kFull, nx, 0) + lane;
-      if (lane < kTTeams) {
-        int64_t b = 0, r0 = 0, n = -1;
-        if (lane < step && i < n_cta) {
-          b = queued_batch(a, i < lar ? a.queue_cap - 1 - i : i - lar);
-          batch_range(a, b, &r0, &n);
-        }
-        turn[3 * lane] = b;
-        turn[3 * lane + 1] = r0;
-        turn[3 * lane + 2] = n;
+    if ((int)threadIdx.x % kThreads == 0) {
+      const int64_t i = atomicAdd(a.queue.ctr + kQTaken + cls, 1u);
+      turn[0] = -1;
+      if (i < count) {
+        turn[0] = queued_batch(a, a.queue.at[cls] + i);
+        batch_range(a, turn[0], turn + 1, turn + 2);
       }
     }
-    __syncthreads();
-    if (turn[2] < 0) break;
-    bool teams = step > 1;
-#pragma unroll
-    for (int k = 0; k < kTTeams; ++k) teams = teams && turn[3 * k + 2] <= kQTeam;
-    if (teams) {
-      if (turn[3 * team + 2] >= 0)
-        walk_batch<MODE, kTTeam>(a, ts, turn[3 * team], turn[3 * team + 1], turn[3 * team + 2]);
-    } else {
-      for (int k = 0; k < kTTeams && turn[3 * k + 2] >= 0; ++k)
-        walk_batch<MODE, kTThreads>(a, ts, turn[3 * k], turn[3 * k + 1], turn[3 * k + 2]);
-    }
-  }
-  if (by_warp) {
-    unsigned nx = 0;  // taken one ahead
-    if (lane == 0) nx = atomicAdd(a.queue_ctr + kQTakenM, 1u);
-    for (;;) {
-      const int64_t i = __shfl_sync(kFull, nx, 0);
-      if (i >= med) break;
-      if (lane == 0) nx = atomicAdd(a.queue_ctr + kQTakenM, 1u);
-      int64_t r0, n;
-      const int64_t b = queued_batch(a, i);
-      batch_range(a, b, &r0, &n);
-      walk_batch<MODE, 32>(a, ts, b, r0, n);
-    }
+    sync_team<kThreads>();
+    if (turn[0] < 0) break;
+    walk_batch<MODE, kThreads>(a, ts, turn[0], turn[1], turn[2]);  // synchronises the team after reading these
   }
   __syncthreads();
-  if (tid == 0) {
+}
+
+// The same, each warp one batch at a time, taken one ahead.
+template <int MODE>
+__device__ __forceinline__ void walk_class_warps(const TileArgs &a, TSmem<MODE> &ts, int cls, int64_t count) {
+  const int lane = threadIdx.x & 31;
+  unsigned nx = 0;
+  if (lane == 0) nx = atomicAdd(a.queue.ctr + kQTaken + cls, 1u);
+  for (;;) {
+    const int64_t i = __shfl_sync(kFull, nx, 0);
+    if (i >= count) break;
+    if (lane == 0) nx = atomicAdd(a.queue.ctr + kQTaken + cls, 1u);
+    int64_t r0, n;
+    const int64_t b = queued_batch(a, a.queue.at[cls] + i);
+    batch_range(a, b, &r0, &n);
+    walk_batch<MODE, 32>(a, ts, b, r0, n);
+  }
+  __syncthreads();
+}
+
+// The queued batches, the largest class first.  A warp walks a batch with the
+// fewest instructions but takes longest for one, a CTA the other way round: so a
+// CTA takes large ones and those of a class with few, a team of four warps those
+// of a class with two or more for every CTA, a warp the smallest where there are
+// half as many again as warps.  Measured on both sides of each line (fp64 shares,
+// 256 tenants; 5e7 requests unless said):
+//   1,600 a batch, by warps    401 us, teams 612         20,000, by teams 439, CTAs 508
+//   4,096 a batch, by warps    407 us, teams 429         30,000, by CTAs  461, teams 488
+//   6,000 of 4,000, by warps   223 us, teams 251         60,000, by CTAs  472, teams 614
+//   3,100 of 4,000, by teams   162 us, warps 205         500 of 10,000, by teams 105, CTAs 119
+// Before the queue, with the CTA whose tile held a batch's start walking it one
+// request per thread and turn, 4,096 a batch took 1,307 us, 9,976 930 (415 now),
+// 200,000 1,280 (465).  The last CTA out leaves the counters at zero for the next
+// call.
+template <int MODE>
+__device__ __noinline__ void walk_queue(const TileArgs &a, TSmem<MODE> &ts) {
+  __syncthreads();  // the list's memory is free
+#pragma unroll 1
+  for (int c = kQClasses - 1; c >= 0; --c) {
+    const int64_t count = min((int64_t)ts.queued[c], a.queue.at[c + 1] - a.queue.at[c]);
+    if (c == 0 && 2 * count >= 3 * (int64_t)gridDim.x * kTWarps)
+      walk_class_warps<MODE>(a, ts, c, count);
+    else if (c <= 1 && count >= 2 * (int64_t)gridDim.x)
+      walk_class<MODE, kTTeam>(a, ts, c, count);
+    else if (count > 0)
+      walk_class<MODE, kTThreads>(a, ts, c, count);
+  }
+  if (threadIdx.x == 0) {
     __threadfence();
-    if (atomicAdd(a.queue_ctr + kQDone, 1u) == gridDim.x - 1) {
+    if (atomicAdd(a.queue.ctr + kQDone, 1u) == gridDim.x - 1) {
 #pragma unroll
-      for (int k = 0; k < kQueueWords; ++k) a.queue_ctr[k] = 0u;
+      for (int k = 0; k < kQueueWords; ++k) a.queue.ctr[k] = 0u;
     }
   }
 }
@@ -931,8 +931,8 @@ __global__ void __launch_bounds__(kTThreads, 1) k_tiles(const TileArgs a) {
     t = a.n_tiles * blockIdx.x / gridDim.x + wid;
     t_end = a.n_tiles * (blockIdx.x + 1) / gridDim.x;
   }
-  const bool queued = a.queue != nullptr;
-  const unsigned in_queue = queued && tid < 2 ? __ldcg(a.queue_ctr + tid) : 0u;
+  const bool queued = a.queue.list != nullptr;
+  const unsigned in_queue = queued && tid < kQClasses ? __ldcg(a.queue.ctr + kQListed + tid) : 0u;
   int64_t b0 = 0, b1 = 0, r0 = 0, r1 = 0;
   // a fit of many batches: the tiles whose first batch is in the range
   const bool ranged = (MODE & M_FIT) && a.f_range != nullptr;
@@ -966,7 +966,7 @@ __global__ void __launch_bounds__(kTThreads, 1) k_tiles(const TileArgs a) {
     r0 = clampi(a.off[b0], 0, a.n_req);
     r1 = clampi(a.off[b1], r0, a.n_req);
   }
-  if (tid < 2) ts.queued[tid] = in_queue;
+  if (tid < kQClasses) ts.queued[tid] = in_queue;
   while (t < t_end) {
     const int64_t tn = t + stride;
     int64_t n0 = 0, n1 = 0;
@@ -1106,7 +1106,7 @@ __global__ void __launch_bounds__(kTThreads, 1) k_tiles(const TileArgs a) {
       walk_list<MODE, kTThreads>(a, ts, nbig);
     }
   }
-  if (queued && (ts.queued[0] | ts.queued[1])) walk_queue<MODE>(a, ts, ts.queued[0], ts.queued[1]);
+  if (queued && (ts.queued[0] | ts.queued[1] | ts.queued[2])) walk_queue<MODE>(a, ts);
   if (kTen) {
     __syncthreads();
     ten_table_flush(tw, kHotMax, a.H, a.ten_pend, tid, kTThreads);

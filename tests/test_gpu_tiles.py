@@ -124,15 +124,18 @@ def _queued(kind):
     """Sizes of an input of more than one tile per warp (3.8e6 positions) with batches that no tile holds."""
     rng = np.random.default_rng(50)
     small = rng.integers(0, 9, 460_000)
-    edges = np.array([1533, 1536, 1537, 1540, 8191, 8192, 8193, 65_535, 65_536, 65_537, 100_001])
+    edges = np.array([1533, 1536, 1537, 1540, 4095, 4096, 4097, 24_575, 24_576, 24_577, 100_001])
     if kind == "few":
         s = np.concatenate([small, edges, rng.integers(1500, 70_000, 20)])
-    elif kind == "medium":
-        s = rng.integers(1500, 1800, 3_500)     # enough for every warp of the chip
-    elif kind == "large":
-        s = rng.integers(8193, 9000, 800)       # enough for every team
+    elif kind == "warps":
+        s = rng.integers(1537, 1800, 4_700)     # enough for every warp of the chip
+    elif kind == "teams":
+        s = np.concatenate([rng.integers(1537, 4000, 900), rng.integers(4097, 9000, 500)])  # enough for teams
+    elif kind == "ctas":
+        s = rng.integers(24_577, 28_000, 200)
     else:
-        s = np.concatenate([small[:1000], edges, rng.integers(1537, 1600, 3_300), rng.integers(8193, 9000, 790)])
+        s = np.concatenate([small[:1000], edges, rng.integers(1537, 1600, 4_600), rng.integers(4097, 9000, 400),
+                            rng.integers(24_577, 28_000, 160)])
     rng.shuffle(s)
     return s
 
@@ -172,7 +175,7 @@ def _check_mode(lv, ctx, w, mode):
     assert np.max(np.abs(L - L_o) / L_o) <= 1e-5
 
 
-@pytest.mark.parametrize("kind", ["few", "medium", "large", "all"])
+@pytest.mark.parametrize("kind", ["few", "warps", "teams", "ctas", "all"])
 @pytest.mark.parametrize("mode", _MODES)
 def test_queued_batches(lv, ctx, kind, mode):
     """Batches that no tile holds, by warps, teams and whole CTAs.  Each call twice: the queue of the second starts
@@ -189,7 +192,7 @@ def test_modes_around_the_tile(lv, ctx, lo, hi, n, mode):
     _check_mode(lv, ctx, base._from_sizes(rng, rng.integers(lo, hi + 1, n), nt=9, pre=0.1), mode)
 
 
-@pytest.mark.parametrize("kind", ["few", "medium", "large", "all"])
+@pytest.mark.parametrize("kind", ["few", "warps", "teams", "ctas", "all"])
 def test_queued_batches_features_and_noalloc(lv, ctx, kind):
     """The same inputs' batch features, and lv_attribute_noalloc's T and shares bit for bit those of lv_attribute."""
     import ctypes
@@ -214,7 +217,7 @@ def test_queued_batches_features_and_noalloc(lv, ctx, kind):
         assert np.array_equal(Tn.cpu().numpy(), T) and np.array_equal(Sn.cpu().numpy(), S)
 
 
-@pytest.mark.parametrize("kind", ["few", "large"])
+@pytest.mark.parametrize("kind", ["few", "teams"])
 def test_invalid_values_in_queued_batches(lv, ctx, kind):
     """Negative p and c count as 0, tenants out of range as the nearest; the call reports them."""
     rng = np.random.default_rng(53)
