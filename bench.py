@@ -36,6 +36,7 @@ import argparse
 import hashlib
 import json
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -60,6 +61,12 @@ def kernel_hash() -> str:
         with open(os.path.join(ROOT, f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
+
+
+def fold_inline() -> int:
+    """The most tenants whose shares the attribution kernel folds itself, from the kernel sources."""
+    with open(os.path.join(ROOT, "paper_2608_08382_gb300", "csrc", "lv_tenant.cuh")) as f:
+        return int(re.search(r"constexpr int kFoldInline = (\d+);", f.read()).group(1))
 
 
 def measured_peaks():
@@ -297,7 +304,7 @@ def _setup_attr(lv, ctx, w, stream, f32=False):
     return dict(step=step, e2e_step=e2e_step, units=w.n_req, unit="requests/s", metric=METRIC,
                 h2d=h2d,
                 d2h=(4 if f32 else 8) * (w.n_req + w.n_batch) + 8 * w.n_tenants,
-                launches_per_step=4 if w.n_tenants > 1536 else 3,  # more tenants: a fold of their own
+                launches_per_step=4 if w.n_tenants > fold_inline() else 3,  # more tenants: a fold of their own
                 kernel="k_tiles", time_mask=lv.LV_TIME_TILES,
                 bytes_per_launch=(20.0 if f32 else 24.0) * w.n_req + (12.0 if f32 else 16.0) * w.n_batch,
                 bytes_rule=("20 B/request (p, c, phase, tenant read; fp32 share written) + 12 B/batch (offset read; "

@@ -30,10 +30,10 @@ namespace lv {
 // Gram's in 128 bits, X^T y modulo 2^192, y'y in 256).  Entry order
 // in `partial`: 15 Gram pairs (a <= b, row order), 5 X^T y per y, one y'y per
 // y, one flag (some batch has S1 != S3).
-// Bound by instruction issue (16 warps per SM at 128 registers; the products
-// are carry-chained 32-bit multiply-adds, a quarter fewer instructions than
-// 64-bit ones): 2e6 batches with two vectors take 111 us; 150 with 64-bit
-// products, 245 with, besides, one row of 32 segments looked at per turn and
+// Bound by latency at 16 warps per SM (128 registers): the products are chains of
+// 32-bit multiply-adds through the carry, a quarter fewer instructions than
+// 64-bit ones, issued in 58 % of the slots.  2e6 batches with two vectors take 111
+// us; 150 with 64-bit products, 245 with, besides, one row of 32 segments looked at per turn and
 // nothing loaded ahead.  With one entry per lane and all lanes on one batch,
 // inside the kernel over the requests, the same sums took about 0.35 of 0.96 ms.
 constexpr int kGramThreads = 256;

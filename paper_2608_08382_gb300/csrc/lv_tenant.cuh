@@ -52,9 +52,11 @@ __device__ __forceinline__ void ten_table_flush(const uint32_t *smem, int cap, i
 
 // The fold by the last CTA to finish (every CTA calls this once its additions
 // to the pending counters are issued): for few tenants one CTA's pass over them
-// costs less than a launch of k_tenant_fold (a call on 6.5e5 requests with and
+// costs less than a launch of k_tenant_fold.  A call on 6.5e5 requests with and
 // without that launch: 16 tenants 22.6 and 21.1 us, 600 44.2 and 42.5, 1,280 34.2
-// and 33.8, 2,048 35.6 and 36.9).
+// and 33.8, 2,048 35.6 and 36.9.  (Between the counts the time goes into the cold
+// tenants' global atomics, most where a few of them share all of those: 512
+// tenants 28 us, 520 34, 600 42, 800 38.)
 constexpr int kFoldInline = 1536;
 __device__ __forceinline__ void ten_fold_last(unsigned long long *pend, i128 *state, unsigned *ticket, int n,
                                               int *status, int tid, int threads) {

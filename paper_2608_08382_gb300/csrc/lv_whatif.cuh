@@ -220,8 +220,10 @@ constexpr int kWiRows = 32;      // pending requests per block, at most
 // so).  The block's rows get their V here, one thread per row and segment; a
 // candidate's U and W of the segment in use stay in registers (they change with
 // the row only where the merged batch crosses the split or turns prefill), so a
-// pair reads one V from shared memory.  Bound by the stores: 16-17 B a pair
-// (4.2e6 pairs, 67 MB: 21.5 us, 24.4 with U and W read per pair).
+// pair reads one V from shared memory.  Bound by the integer ALU pipe (75 % busy
+// at 66 % issue: about 125 warp instructions per 32 pairs, most of them the two
+// roundings' shifts and logic), ahead of the stores, 16-17 B a pair (4.2e6 pairs,
+// 67 MB into L2: 21.5 us, 24.4 with U and W read per pair).
 __global__ void __launch_bounds__(kWiThreads) k_wi_pairs(ModelP mp, const CandP *cand, int64_t nc,
                                                          const int32_t *__restrict__ p_new,
                                                          const int32_t *__restrict__ c_new,
@@ -323,7 +325,7 @@ __global__ void __launch_bounds__(kWiThreads) k_wi_pairs(ModelP mp, const CandP 
         Sp += ostep;
       }
       // comparisons as integers: with two fp64 ones per pair as well as the
-      // addition, the fp64 pipe took longer than the stores (4.2e6 pairs: 52
+      // addition, the fp64 pipe took longer than all the rest (4.2e6 pairs: 52
       // us a call, 34 so).  No sum is a NaN: totals are not (above), shares are finite.
       if (Ap) {
         *Ap = (order_key(__dadd_rn(sp[r].Lu, sh)) <= sp[r].Bk && order_key(T) <= slo_key) ? 1 : 0;
