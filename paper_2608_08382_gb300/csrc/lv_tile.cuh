@@ -721,10 +721,12 @@ __device__ __noinline__ void walk_alone(const TileArgs &a, TSmem<MODE> &ts, int6
 // A barrier of `kThreads` consecutive threads of the CTA (all of it, or a team).
 template <int kThreads>
 __device__ __forceinline__ void sync_team() {
-  if (kThreads == kTThreads)
+  if (kThreads == kTThreads) {
     __syncthreads();
-  else
+  } else {
+    __syncwarp();  // the barrier counts whole warps
     asm volatile("bar.sync %0, %1;" ::"r"(1 + (int)threadIdx.x / kThreads), "n"(kThreads) : "memory");
+  }
 }
 
 // One batch walked by `kThreads` threads (a warp, a team, or the CTA) from global
