@@ -930,8 +930,9 @@ __global__ void __launch_bounds__(kTThreads, 1) k_tiles(const TileArgs a) {
   if (a.D) {
     // at most one tile per warp: a CTA takes neighbours, so that batches that reach
     // past their tiles, which it walks afterwards, are spread over the CTAs
-    t = a.n_tiles * blockIdx.x / gridDim.x + wid;
-    t_end = a.n_tiles * (blockIdx.x + 1) / gridDim.x;
+    const unsigned n = (unsigned)a.n_tiles;  // at most kTWarps a CTA
+    t = n * blockIdx.x / gridDim.x + wid;
+    t_end = n * (blockIdx.x + 1) / gridDim.x;
   }
   const bool queued = a.queue.list != nullptr;
   const unsigned in_queue = queued && tid < kQClasses ? __ldcg(a.queue.ctr + kQListed + tid) : 0u;
