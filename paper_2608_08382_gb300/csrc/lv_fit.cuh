@@ -32,7 +32,7 @@ namespace lv {
 // y, one flag (some batch has S1 != S3).
 // Bound by latency at 16 warps per SM (128 registers): the products are chains of
 // 32-bit multiply-adds through the carry, a quarter fewer instructions than
-// 64-bit ones, issued in 58 % of the slots.  2e6 batches with two vectors take 111
+// 64-bit ones, issued in 57 % of the slots.  2e6 batches with two vectors take 111
 // us; 150 with 64-bit products, 245 with, besides, one row of 32 segments looked at per turn and
 // nothing loaded ahead.  With one entry per lane and all lanes on one batch,
 // inside the kernel over the requests, the same sums took about 0.35 of 0.96 ms.
@@ -186,8 +186,9 @@ __device__ __forceinline__ void fit_y_add(FitYAcc &g, const Feat48 *x, i128 Y) {
 // The batches of one launch.  Their sums and segments come from the tile kernel
 // through a scratch of bounded size, so a fit of more than kFitRange batches is
 // worked off in ranges of tiles that start in kFitRange batches each.  A range
-// of 2^22 costs two launches and a search of the tiles, about 15 us, against 0.6
-// ms for its batches' requests at 64 each, and 138 MB.
+// of 2^22 takes 138 MB and costs about 37 us (two launches, a search of the tiles,
+// both kernels' ends): 8e6 batches of 1 to 64 requests 1,156 us, 1,117 with a
+// scratch for all of them.
 constexpr int64_t kFitRange = 1ll << 22;
 // Rows of blocks, at least.  A product of a feature (below 2^48) and a latency
 // (2^100 y, below 2^125) is below 2^173, so a warp's signed sum in 192 bits holds

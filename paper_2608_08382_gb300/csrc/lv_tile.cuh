@@ -24,7 +24,7 @@
 // Pareto batches: 85 us, 119 if their warps walk them; 1e7: 538 and 600).  All
 // sums are exact integers, so results do not depend on the schedule.
 //
-// What bounds it: instruction issue and the integer pipe (about 143 warp
+// What bounds it: instruction issue and the integer pipe (about 148 warp
 // instructions per 32 requests), not HBM.  The shape follows from that: 20 warps
 // per SM with 96 registers each spill little (24 warps of 80 took 9 % longer,
 // 32 of 64 a third), and the largest tile whose shared memory (182 KB) leaves the

@@ -221,7 +221,7 @@ constexpr int kWiRows = 32;      // pending requests per block, at most
 // candidate's U and W of the segment in use stay in registers (they change with
 // the row only where the merged batch crosses the split or turns prefill), so a
 // pair reads one V from shared memory.  Bound by the integer ALU pipe (75 % busy
-// at 66 % issue: about 125 warp instructions per 32 pairs, most of them the two
+// at 65 % issue: about 129 warp instructions per 32 pairs, most of them the two
 // roundings' shifts and logic), ahead of the stores, 16-17 B a pair (4.2e6 pairs,
 // 67 MB into L2: 21.5 us, 24.4 with U and W read per pair).
 __global__ void __launch_bounds__(kWiThreads) k_wi_pairs(ModelP mp, const CandP *cand, int64_t nc,

@@ -53,6 +53,27 @@ def test_values_beyond_the_prefix_words(lv, ctx, field):
     _check(lv, ctx, w)
 
 
+@pytest.mark.parametrize("p_max", [1, 8192, 8193, 1 << 23])
+@pytest.mark.parametrize("share", [1e-3, 1.0])
+@pytest.mark.parametrize("lo,hi,n", [(0, 9, 9000), (1, 300, 900), (900, 1530, 60)])
+def test_long_contexts(lv, ctx, p_max, share, lo, hi, n):
+    """Contexts of 2^23 tokens and more, up to the type's largest, in some tiles and in all, beside prefills of
+    several lengths."""
+    import torch
+    rng = np.random.default_rng(p_max + hi)
+    w = base._from_sizes(rng, rng.integers(lo, hi + 1, n), nt=20, pre=0.3)
+    at = rng.random(w.n_req) < share
+    w.c[at] = rng.integers(1 << 23, 1 << 31, int(at.sum()))
+    w.c[rng.integers(0, w.n_req, 50)] = (1 << 31) - 1
+    w.p[w.phase == 1] = np.where(rng.random(int((w.phase == 1).sum())) < 0.9, p_max, 2)
+    _check(lv, ctx, w)
+    b = base._dev(lv, w, tenant=False)
+    bf = torch.empty((5, w.n_batch), dtype=torch.int64, device="cuda")
+    lv.lv_features(ctx, b, model=lv.make_model(w.coef, w.split), batch_feat=bf)
+    assert ctx.status() == lv.LV_OK
+    assert np.array_equal(bf.cpu().numpy(), oracle.batch_features(w.offsets, w.p, w.c, w.phase, w.split)[0])
+
+
 @pytest.mark.parametrize("nt", [1, 511, 512, 513, 1536, 1537, 3000])
 @pytest.mark.parametrize("scale", [1e-4, 1.0, 300.0])
 def test_tenants_and_share_magnitudes(lv, ctx, nt, scale):
